@@ -206,3 +206,88 @@ def tolerance(case):
     if case["kind"] == "fit":
         return {"rel": 1e-5}
     return {"rel": 1e-5, "max": 1e-4, "differ": 0.0} if case["dtype"] == "f32" else {"rel": 4e-3, "max": 2e-2, "differ": 0.0}
+
+
+# ---- the same results in 64 bits ----
+# Plain torch, one operation after another; the only rounding is the one the method states: keys and values of a bf16
+# decoder are bf16 numbers in the cache.
+
+def _norm(x, gain):
+    return x * torch.rsqrt((x * x).mean(-1, keepdim=True) + 1e-5) * gain
+
+
+def _rotate(x, pos):  # x [T, heads, head_dim]
+    half = x.shape[-1] // 2
+    angle = pos.double()[:, None] * (10000.0 ** (-torch.arange(half, device=x.device, dtype=torch.float64) / half))[None]
+    c, s = torch.cos(angle).float().double()[:, None], torch.sin(angle).float().double()[:, None]  # tables of 32-bit numbers
+    a, b = x[..., :half], x[..., half:]
+    return torch.cat([a * c - b * s, b * c + a * s], -1)
+
+
+class _Exact:
+    def __init__(self, case, weights, grad=False):
+        self.case, self.w, self.cache, self.grad = case, weights, [None] * case["layers"], grad
+
+    def _attend(self, l, q, k, v):
+        heads, hd = self.case["heads"], self.case["head_dim"]
+        q, k, v = (t.view(len(t), heads, hd) for t in (q, k, v))
+        before = 0 if self.cache[l] is None else len(self.cache[l][0])
+        pos = torch.arange(before, before + len(q), device=q.device)
+        q, k = _rotate(q, pos), _rotate(k, pos)
+        if not self.grad:
+            if self.case["dtype"] != "f32":
+                k, v = k.bfloat16().double(), v.bfloat16().double()
+            if before:
+                k, v = torch.cat([self.cache[l][0], k]), torch.cat([self.cache[l][1], v])
+            self.cache[l] = (k, v)
+        see = torch.arange(len(k), device=q.device)[None] <= pos[:, None]
+        out = [torch.softmax((q[:, h] @ k[:, h].t() / math.sqrt(hd)).masked_fill(~see, -math.inf), -1) @ v[:, h] for h in range(heads)]
+        return torch.cat(out, -1)
+
+    def logits(self, tokens, rows, layers=None):
+        """Logits of the last `rows` of these tokens, which follow what the cache holds."""
+        h = self.w["tok_embed"][torch.as_tensor(tokens, device="cuda").long()].double()
+        for l in range(self.case["layers"]):
+            lw = layers[l] if layers else {n: t.double() for n, t in self.w["layers"][l].items()}
+            x = _norm(h, lw["attn_norm"])
+            h = h + self._attend(l, x @ lw["wq"].t(), x @ lw["wk"].t(), x @ lw["wv"].t()) @ lw["wo"].t()
+            x = _norm(h, lw["ffn_norm"])
+            h = h + (torch.nn.functional.silu(x @ lw["w_gate"].t()) * (x @ lw["w_up"].t())) @ lw["w_down"].t()
+        return _norm(h[len(h) - rows:], self.w["final_norm"].double()) @ self.w["lm_head"].double().t()
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits.  The logits behind a greedy text follow the text that 64-bit arithmetic decodes; sampled
+    tokens hang on the library's own random numbers and have no such value."""
+    if case["kind"] == "generate" and case["temperature"] > 0.0:
+        return None
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(int(seed) * 7919 + 17)
+    rng = np.random.RandomState(int(seed) % (2**31 - 1))
+    w = _weights(case, gen)
+    if case["kind"] == "fit":
+        tokens = rng.randint(0, case["vocab"], (case["sequences"], case["length"])).astype(np.int32)
+        layers = [{n: t.double().requires_grad_(True) for n, t in lw.items()} for lw in w["layers"]]
+        trace, fit = np.zeros(case["layers"]), np.zeros(case["layers"])
+        for seq in tokens:
+            out = _Exact(case, w, grad=True).logits(seq[:-1], len(seq) - 1, layers)
+            torch.nn.functional.cross_entropy(out, torch.as_tensor(seq[1:], device="cuda").long()).backward()
+            for l, lw in enumerate(layers):
+                for t in lw.values():
+                    g = float((t.grad * t.grad).sum()) / len(tokens)
+                    trace[l] += g
+                    fit[l] += g * float((t.detach() * t.detach()).mean())
+                    t.grad = None
+        return {"trace": trace, "fit": fit}
+    with torch.no_grad():
+        m = _Exact(case, w)
+        if case["kind"] == "score":
+            tokens = rng.randint(0, case["vocab"], case["length"]).astype(np.int32)
+            out = m.logits(tokens, len(tokens)).cpu().numpy()
+            return [out[i:i + 80] for i in range(0, len(tokens), 80)]
+        text = list(rng.randint(0, case["vocab"], (case["batch"], case["prompt"])).astype(np.int32)[0])
+        last = [m.logits(text, min(TAIL_ROWS, len(text)))]
+        for _ in range(case["new"]):
+            text.append(int(last[-1][-1].argmax()))
+            last.append(m.logits(text[-1:], 1))
+        return {"tokens": None, "rounds": None, "logits": torch.cat(last)[-min(TAIL_ROWS, len(text)):].cpu().numpy()}
