@@ -175,7 +175,14 @@ int check_device(sdfp_ctx* c, const char* who) {
 template <typename T>
 int dev_alloc(sdfp_ctx* c, T** p, size_t n, bool zero = false) {
   void* q = nullptr;
-  CU_OK(c, cudaMalloc(&q, std::max<size_t>(n * sizeof(T), 16)));
+  const size_t bytes = std::max<size_t>(n * sizeof(T), 16);
+  cudaError_t e = cudaMalloc(&q, bytes);
+  if (e == cudaErrorMemoryAllocation) {  // what sdfp_fit_scores keeps between calls goes back first
+    cudaGetLastError();
+    fit::fit_pool_trim(c->device);
+    e = cudaMalloc(&q, bytes);
+  }
+  CU_OK(c, e);
   c->allocs.push_back(q);
   if (zero) CU_OK(c, cudaMemsetAsync(q, 0, std::max<size_t>(n * sizeof(T), 16), c->stream));
   *p = reinterpret_cast<T*>(q);
@@ -806,6 +813,7 @@ extern "C" void sdfp_destroy(sdfp_ctx* c) {
   cudaStreamSynchronize(c->stream);
   for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second.exec);
   for (void* p : c->allocs) cudaFree(p);
+  fit::fit_pool_trim(c->device);
   if (c->pinned_flag) cudaFreeHost(c->pinned_flag);
   for (auto& e : c->ev)
     if (e) cudaEventDestroy(e);

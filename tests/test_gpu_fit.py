@@ -54,6 +54,31 @@ def test_fit_scores_tiny_config_and_ranking(shape):
     assert same_T == got_T                                   # run to run: bit-identical
 
 
+@pytest.mark.parametrize("d,heads,ffn,vocab,n_seq,seq_len,dtype", [
+    (32, 2, 40, 50, 3, 2, "f32"),        # one token per sequence, a vocabulary that is no multiple of 8
+    (36, 2, 41, 64, 2, 34, "f32"),       # rows that are no whole 16-byte pieces, two Gram tiles with a remainder
+    (128, 2, 264, 96, 11, 66, "bf16"),   # more rows than go through at a time: a full and a smaller group
+    (136, 1, 72, 130, 1, 130, "bf16"),   # one head wider than a block, five Gram tiles, cut contractions
+    (64, 4, 2048, 4096, 2, 18, "f32"),   # long contractions over few tiles: the widest split
+])
+def test_fit_scores_at_the_edges(d, heads, ffn, vocab, n_seq, seq_len, dtype):
+    """Tile remainders, unaligned rows, groups of sequences and split contractions against the fp64 oracle.  The fp32
+    forward and backward sums are off by a few 1e-6 (2^-24 times the root of the longest sum, two passes); 1e-4
+    leaves room for tensors whose gradients nearly cancel."""
+    shape = si.ModelShape("edge", 2, d, heads, d // heads, ffn, vocab, dtype=dtype)
+    w = si.make_weights(shape, [], random_gains=True)
+    for lw in w["layers"]:
+        for k in lw:
+            if k.startswith("w"):
+                lw[k] *= 4.0
+    calib = si.make_prompts(shape.vocab, n_seq, seq_len, seed=5)
+    got_T, got_F, ref_T, ref_F = _both(shape, w, calib)
+    assert got_T == pytest.approx(ref_T, rel=1e-4)
+    assert got_F == pytest.approx(ref_F, rel=1e-4)
+    back_T, _ = pkg.sdfp_fit_scores(shape, si.weights_to(w, "cuda:0"), calib[::-1].copy())
+    assert back_T == pytest.approx(got_T, rel=1e-12)   # a sequence's numbers do not depend on its group
+
+
 def test_fit_scores_drive_the_draft_mask():
     """Stage A feeding Stage B: the prune set chosen from the GPU scores is handed to
     sdfp_set_draft_layers and the speculative output stays the target's."""
