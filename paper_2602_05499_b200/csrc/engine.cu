@@ -128,7 +128,9 @@ struct sdfp_ctx {
   int* um_flags_dummy = nullptr;          // failure-path test hook: where posts go to be lost
   unsigned long long um_expire_ns = 0;    // hook armed: the next sdfp_forward_logits call runs with ...
   unsigned long long um_sabotage_ns = 0;  // ... lost posts and this wait limit
+  bool prompt_grouped = false;            // the running prompt pass carries prompts of at most one row block (launch_dense)
   int rows_cap = kMaxRows;         // rows the activation buffers h, q, att, u and the row plan hold
+  int prompt_rows = 0;             // rows of short prompts the dense path takes together
   int max_smem_optin = 0;
   bool own_stream = false;
   sdfp_timing timing{};
@@ -236,15 +238,22 @@ UmmaParams dense_params(const sdfp_ctx* c, const void* w_img, const unsigned cha
 // One CTA per SM.  Launched with the programmatic-dependent-launch attribute like every other
 // kernel: the kernel requests its first weights before it waits for its predecessor.
 cudaError_t launch_dense(sdfp_ctx* c, const UmmaParams& p) {
-  return launch(c, umma_linear_kernel, dim3(c->num_sms), dim3(kUmThreads), umma_smem_bytes(p.RB, p.n_stages), p);
+  return launch(c, c->prompt_grouped ? umma_linear_kernel<true> : umma_linear_kernel<false>, dim3(c->num_sms), dim3(kUmThreads),
+                umma_smem_bytes(p.RB, p.n_stages), p);
 }
 
 // Linear layer on the tcgen05 path from fp32 rows: activation image (RMSNorm folded in) by a
 // conversion kernel, then the stream-K kernel.  (The prompt pass; decode passes on the dense path
 // chain the kernels image to image instead, see enqueue_dense_pass.)
+// posts (partial accumulators and their flags) a launch can have: one per CTA and row block of a prompt group
+size_t um_posts(const sdfp_ctx* c) { return (size_t)c->num_sms * std::max(1, (c->prompt_rows + kUmMaxRB - 1) / kUmMaxRB); }
+
+// Row block of a pass of `rows` rows: 128 once they fill one, else the rows rounded up to the MMA's granularity
+int dense_row_block(int rows) { return rows >= kUmMaxRB ? kUmMaxRB : ((rows + 15) / 16) * 16; }
+
 cudaError_t run_dense_linear(sdfp_ctx* c, const void* w_img, const float* x, int ldx, int rows, int K, int n_pairs,
                              const float* gain, const EpiParams& ep) {
-  const int RB = rows >= kUmMaxRB ? kUmMaxRB : ((rows + 15) / 16) * 16;
+  const int RB = dense_row_block(rows);
   const int KB = (K + kUmBK - 1) / kUmBK;
   cudaError_t e = launch(c, prep_rows_kernel, dim3((rows + 7) / 8), dim3(kPrepThreads), 0, x, ldx, rows, K, gain, c->cfg.rms_eps,
                          c->um_x, RB, KB);
@@ -506,6 +515,14 @@ cudaError_t run_pass(sdfp_ctx* c, bool draft, int rows, int rows_per_seq, bool w
 
 // ---- one forward pass ------------------------------------------------------------------
 
+// Rows of short prompts (at most one row block each) that share a sweep of the weights: beyond eight row
+// blocks a sweep is bound by the MMAs and no longer by the weights, and the partial sums of cut tiles
+// (one buffer per CTA and row block) grow with them.
+constexpr int kPromptRows = 8 * kUmMaxRB;
+// ... and the longest prompt that does.  Going through the row blocks inside a piece pays with partial sums
+// per row block; at 202 tokens a prompt alone would take 1.62 ms instead of 1.26 (4 layers d 4096), eight of
+// them together 11.0 instead of 10.0, and the rule must be the same for both.
+constexpr int kGroupedPrompt = kUmMaxRB;
 // prompts shorter than this go through the decode kernels in chunks (a handful of launches)
 constexpr int kDenseMinRows = 16;
 
@@ -903,8 +920,10 @@ extern "C" int sdfp_create(const sdfp_config* cfg, const sdfp_weights* w, void* 
   c->use_dense = c->use_mma && !(g.flags & SDFP_FLAG_NO_DENSE);
   c->dense_decode = c->use_dense && !c->use_pass && !(g.flags & SDFP_FLAG_NO_PASS_KERNEL);
   if (c->use_dense) {
-    c->rows_cap = std::max((int)kMaxRows, g.max_seq);
-    if (cudaFuncSetAttribute(umma_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
+    c->prompt_rows = std::min((int)kPromptRows, g.max_batch * std::min((int)kGroupedPrompt, g.max_seq));
+    c->rows_cap = std::max(std::max((int)kMaxRows, g.max_seq), c->prompt_rows);
+    if (cudaFuncSetAttribute(umma_linear_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
+        cudaFuncSetAttribute(umma_linear_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess ||
         cudaFuncSetAttribute(prefill_attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)prefill_attention_smem<64>()) != cudaSuccess ||
         cudaFuncSetAttribute(prefill_attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -988,9 +1007,9 @@ extern "C" int sdfp_create(const sdfp_config* cfg, const sdfp_weights* w, void* 
     const size_t kd64 = (size_t)(((g.d_model + kUmBK - 1) / kUmBK) * kUmBK), kf64 = (size_t)(((g.d_ffn + kUmBK - 1) / kUmBK) * kUmBK);
     if ((r = dev_alloc(c, &c->um_x, rows128 * kmax * 4, true)) || (r = dev_alloc(c, &c->um_pa, rows128 * kd64 * 4, true)) ||
         (r = dev_alloc(c, &c->um_pu, rows128 * kf64 * 4, true)) ||
-        (r = dev_alloc(c, &c->um_partial, (size_t)c->num_sms * kUmMaxRB * kUmFeat)) ||
-        (r = dev_alloc(c, &c->um_flags, (size_t)c->num_sms, true)) || (r = dev_alloc(c, &c->um_error, 1, true)) ||
-        (r = dev_alloc(c, &c->um_flags_dummy, (size_t)c->num_sms, true)) ||
+        (r = dev_alloc(c, &c->um_partial, um_posts(c) * kUmMaxRB * kUmFeat)) ||
+        (r = dev_alloc(c, &c->um_flags, um_posts(c), true)) || (r = dev_alloc(c, &c->um_error, 1, true)) ||
+        (r = dev_alloc(c, &c->um_flags_dummy, um_posts(c), true)) ||
         (r = dev_alloc(c, &c->h_fork, R * g.d_model)))
       return bail(r);
     if (c->dense_decode) {
@@ -1078,8 +1097,8 @@ int check_dense_error(sdfp_ctx* c) {
   CU_OK(c, cudaStreamSynchronize(c->stream));
   if (e == 0) return 0;
   cudaMemsetAsync(c->um_error, 0, sizeof(int), c->stream);
-  cudaMemsetAsync(c->um_flags, 0, (size_t)c->num_sms * sizeof(int), c->stream);
-  cudaMemsetAsync(c->um_flags_dummy, 0, (size_t)c->num_sms * sizeof(int), c->stream);
+  cudaMemsetAsync(c->um_flags, 0, um_posts(c) * sizeof(int), c->stream);
+  cudaMemsetAsync(c->um_flags_dummy, 0, um_posts(c) * sizeof(int), c->stream);
   cudaStreamSynchronize(c->stream);
   static const char* const what[] = {"", "pipeline stage never freed", "pipeline stage never filled", "accumulator never freed",
                                      "accumulator never finished", "partial accumulator of a cut tile never posted"};
@@ -1145,21 +1164,25 @@ int forward_logits_passes_inner(sdfp_ctx* c, bool draft, const int32_t* tokens, 
 
 namespace {
 
-// Feed tokens [from, to) of sequence b (already in seq_tok) through target or draft to fill its cache.
-int prefill_range(sdfp_ctx* c, bool draft, int b, int from, int to) {
-  const int chunk = c->use_pass ? kPassMaxRows : 32;
-  for (int s = from; s < to; s += chunk) {
-    const int cnt = std::min(chunk, to - s);
-    PassDesc pd{};
-    pd.kind = PASS_TOKENS;
-    pd.seq = b;
-    pd.start = s;
-    pd.count = cnt;
-    pd.src = c->seq_tok + (size_t)b * c->cfg.max_seq + s;
-    const int rps = std::min(cnt, kAttnMaxR);
-    const int rows = ((cnt + rps - 1) / rps) * rps;  // whole attention groups; extra rows carry nothing
+// Feed the first `len` prompt tokens of every sequence (already in seq_tok) through target or draft to
+// fill its cache: passes of the widest kind, of as many positions and then of as many sequences as
+// fit.  A row's numbers do not depend on the pass it sits in.
+int prefill_passes(sdfp_ctx* c, bool draft, int batch, int len) {
+  const int widest = c->use_pass ? kPassMaxRows : kMaxRows;
+  for (int s = 0; s < len;) {
+    // rows of a sequence: as many whole attention groups as fit, or what is left of the prompt
+    const int left = std::min(widest, len - s), cnt = left > kAttnMaxR ? left / kAttnMaxR * kAttnMaxR : left;
+    const int group = std::min(batch, widest / cnt);
     const int n_chunks = (s + cnt + kAttnChunk - 1) / kAttnChunk;
-    if (int r = enqueue_pass(c, pd, draft, rows, rps, n_chunks, DECIDE_NONE)) return r;
+    for (int b = 0; b < batch; b += group) {
+      PassDesc pd{};
+      pd.kind = PASS_PROMPT;
+      pd.seq = b;
+      pd.start = s;
+      pd.count = cnt;
+      if (int r = enqueue_pass(c, pd, draft, cnt * std::min(group, batch - b), std::min(cnt, (int)kAttnMaxR), n_chunks, DECIDE_NONE)) return r;
+    }
+    s += cnt;
   }
   return 0;
 }
@@ -1189,16 +1212,17 @@ int dense_ffn_block(sdfp_ctx* c, const LayerWeights& lw, int rows, int RB, int K
   return 0;
 }
 
-int dense_layer(sdfp_ctx* c, const KvCache& kv, int l, int b, int rows, bool run_attn, bool run_ffn) {
+// nb sequences from slot b on, rows_seq rows each, one after the other
+int dense_layer(sdfp_ctx* c, const KvCache& kv, int l, int b, int nb, int rows_seq, bool run_attn, bool run_ffn) {
+  const int rows = nb * rows_seq;
   const sdfp_config& g = c->cfg;
   const int d = g.d_model, f = g.d_ffn;
   const LayerWeights& lw = c->layers[l];
   if (run_ffn && !run_attn) {
-    const int RB0 = rows >= kUmMaxRB ? kUmMaxRB : ((rows + 15) / 16) * 16;
-    return dense_ffn_block(c, lw, rows, RB0, (f + kUmBK - 1) / kUmBK);
+    return dense_ffn_block(c, lw, rows, dense_row_block(rows), (f + kUmBK - 1) / kUmBK);
   }
   if (!run_attn) return 0;
-  const int RB = rows >= kUmMaxRB ? kUmMaxRB : ((rows + 15) / 16) * 16;  // as run_dense_linear chooses it
+  const int RB = dense_row_block(rows);
   const int KBd = (d + kUmBK - 1) / kUmBK, KBf = (f + kUmBK - 1) / kUmBK;
   EpiParams qkv = base_epi(c, EPI_QKV, c->q, d);
   qkv.kcache = kv.k[l];
@@ -1206,15 +1230,15 @@ int dense_layer(sdfp_ctx* c, const KvCache& kv, int l, int b, int rows, bool run
   CU_OK(c, run_dense_linear(c, lw.um_qkv, c->h, d, rows, d, 3 * d / 2, lw.attn_gain, qkv));
   // the attention output and the SwiGLU output are written as operand images by their producers
   const float scale = 1.0f / std::sqrt((float)g.head_dim);
-  const dim3 grid((rows + kPfaQ - 1) / kPfaQ, g.n_heads);
+  const dim3 grid((rows_seq + kPfaQ - 1) / kPfaQ, g.n_heads, nb);
   const __nv_bfloat16* kc = reinterpret_cast<const __nv_bfloat16*>(kv.k[l]);
   const __nv_bfloat16* vc = reinterpret_cast<const __nv_bfloat16*>(kv.v[l]);
   if (g.head_dim == 128)
     CU_OK(c, launch(c, prefill_attention_kernel<128>, grid, dim3(kPfaThreads), prefill_attention_smem<128>(), (const float*)c->q, kc,
-                    vc, c->att, rows, g.n_heads, g.max_seq, b, scale, c->um_pa, RB, KBd));
+                    vc, c->att, rows_seq, g.n_heads, g.max_seq, b, scale, c->um_pa, RB, KBd));
   else
     CU_OK(c, launch(c, prefill_attention_kernel<64>, grid, dim3(kPfaThreads), prefill_attention_smem<64>(), (const float*)c->q, kc, vc,
-                    c->att, rows, g.n_heads, g.max_seq, b, scale, c->um_pa, RB, KBd));
+                    c->att, rows_seq, g.n_heads, g.max_seq, b, scale, c->um_pa, RB, KBd));
   CU_OK(c, launch_dense(c, dense_params(c, lw.um_wo, c->um_pa, rows, RB, KBd, d / 2, base_epi(c, EPI_RESID, c->h, d))));
   if (!run_ffn) return 0;
   return dense_ffn_block(c, lw, rows, RB, KBf);
@@ -1226,43 +1250,58 @@ int first_pruned_layer(const sdfp_ctx* c) {
   return c->cfg.n_layers;
 }
 
-// rows_t rows through the target and, when with_draft, rows_d <= rows_t rows through the draft
-int prefill_dense(sdfp_ctx* c, int b, int rows_t, int rows_d, bool with_draft) {
+// Prompts of nb sequences from slot b on, `rows` rows each, through the target and, with_draft, through
+// the draft.  (The draft needs one row less; the entry its last row leaves is the first that its first
+// decode pass writes again.)
+//
+// Prompts of at most one row block go together: one sweep of the weights for all of them, where the
+// sweep of a short prompt costs what its weights cost (4 layers d 4096: 16 prompts of 44 rows 11.1 ms one after
+// the other, 4.8 together; 8 of 29 rows 4.8 and 1.7; 8 of 99 rows 7.1 and 5.5).  Their pieces of work are cut as for one sequence alone
+// (UmmaParams::rb_inner), so a sequence's cache does not depend on what else is in the batch.
+int prefill_dense(sdfp_ctx* c, int b, int nb, int rows, bool with_draft) {
   const sdfp_config& g = c->cfg;
-  const int d = g.d_model;
+  const int d = g.d_model, total = nb * rows;
   PassDesc pd{};
-  pd.kind = PASS_TOKENS;
+  pd.kind = PASS_PROMPT;
   pd.seq = b;
   pd.start = 0;
-  pd.count = rows_t;
-  pd.src = c->seq_tok + (size_t)b * g.max_seq;
-  CU_OK(c, launch(c, plan_embed_kernel<__nv_bfloat16>, dim3(rows_t), dim3(128), 0, pd, (const GenState*)c->gs, (const int*)c->seq_tok,
+  pd.count = rows;
+  CU_OK(c, launch(c, plan_embed_kernel<__nv_bfloat16>, dim3(total), dim3(128), 0, pd, (const GenState*)c->gs, (const int*)c->seq_tok,
                   g.max_seq, (const int*)c->draft_tok, c->plan, reinterpret_cast<const __nv_bfloat16*>(c->embed), c->h, d, EmbedImage{}));
   const int fork = with_draft ? first_pruned_layer(c) : -1;  // the draft's residual rows leave the target's after this many layers
-  const size_t fork_bytes = (size_t)rows_d * d * sizeof(float);
-  if (fork == 0 && rows_d > 0) CU_OK(c, cudaMemcpyAsync(c->h_fork, c->h, fork_bytes, cudaMemcpyDeviceToDevice, c->stream));
+  const size_t fork_bytes = (size_t)total * d * sizeof(float);
+  if (fork == 0) CU_OK(c, cudaMemcpyAsync(c->h_fork, c->h, fork_bytes, cudaMemcpyDeviceToDevice, c->stream));
   for (int l = 0; l < g.n_layers; ++l) {
-    if (int r = dense_layer(c, c->cache_t, l, b, rows_t, true, true)) return r;
-    if (l + 1 == fork && rows_d > 0) CU_OK(c, cudaMemcpyAsync(c->h_fork, c->h, fork_bytes, cudaMemcpyDeviceToDevice, c->stream));
+    if (int r = dense_layer(c, c->cache_t, l, b, nb, rows, true, true)) return r;
+    if (l + 1 == fork) CU_OK(c, cudaMemcpyAsync(c->h_fork, c->h, fork_bytes, cudaMemcpyDeviceToDevice, c->stream));
   }
-  if (!with_draft || rows_d <= 0) return 0;
-  // K/V of the shared layers: per head one contiguous run of rows_d positions
-  const size_t pitch = (size_t)g.max_seq * g.head_dim * c->esz, width = (size_t)rows_d * g.head_dim * c->esz;
+  if (!with_draft) return 0;
+  // K/V of the shared layers: per (sequence, head) one contiguous run of positions
+  const size_t pitch = (size_t)g.max_seq * g.head_dim * c->esz, width = (size_t)rows * g.head_dim * c->esz;
   const size_t seq_off = (size_t)b * g.n_heads * pitch;
   for (int l = 0; l < std::min(fork, g.n_layers); ++l) {
     CU_OK(c, cudaMemcpy2DAsync((unsigned char*)c->cache_d.k[l] + seq_off, pitch, (const unsigned char*)c->cache_t.k[l] + seq_off, pitch,
-                               width, g.n_heads, cudaMemcpyDeviceToDevice, c->stream));
+                               width, (size_t)nb * g.n_heads, cudaMemcpyDeviceToDevice, c->stream));
     CU_OK(c, cudaMemcpy2DAsync((unsigned char*)c->cache_d.v[l] + seq_off, pitch, (const unsigned char*)c->cache_t.v[l] + seq_off, pitch,
-                               width, g.n_heads, cudaMemcpyDeviceToDevice, c->stream));
+                               width, (size_t)nb * g.n_heads, cudaMemcpyDeviceToDevice, c->stream));
   }
   bool any = false;
   for (int l = fork; l < g.n_layers; ++l) any = any || c->keep_attn[l] || c->keep_ffn[l];
   if (!any) return 0;
   CU_OK(c, cudaMemcpyAsync(c->h, c->h_fork, fork_bytes, cudaMemcpyDeviceToDevice, c->stream));
-  pd.count = rows_d;  // the row plan of the draft's rows (positions 0..rows_d-1 are already right; rows beyond carry nothing)
   for (int l = fork; l < g.n_layers; ++l)
-    if (int r = dense_layer(c, c->cache_d, l, b, rows_d, c->keep_attn[l] != 0, c->keep_ffn[l] != 0)) return r;
+    if (int r = dense_layer(c, c->cache_d, l, b, nb, rows, c->keep_attn[l] != 0, c->keep_ffn[l] != 0)) return r;
   return 0;
+}
+
+// The prompts of all sequences, `rows` rows each, on the dense path
+int prefill_dense_all(sdfp_ctx* c, int batch, int rows, bool with_draft) {
+  c->prompt_grouped = rows <= kGroupedPrompt;
+  const int group = c->prompt_grouped ? std::max(1, std::min(batch, c->prompt_rows / rows)) : 1;
+  int r = 0;
+  for (int b = 0; b < batch && r == 0; b += group) r = prefill_dense(c, b, std::min(group, batch - b), rows, with_draft);
+  c->prompt_grouped = false;
+  return r;
 }
 
 }  // namespace
@@ -1308,15 +1347,13 @@ extern "C" int sdfp_generate(sdfp_ctx* c, const int32_t* prompts, int32_t batch,
   // prefill: the target caches positions 0..P-2, the draft 0..P-3 (its first pass of a
   // round always feeds the last two committed tokens)
   CU_OK(c, cudaEventRecord(c->ev[0], st));
-  for (int b = 0; b < batch; ++b) {
-    const bool draft_prompt = k > 0 && !c->share_kv;  // a sharing draft has no prompt pass of its own
-    if (c->use_dense && prompt_len - 1 >= kDenseMinRows) {
-      if (int r = prefill_dense(c, b, prompt_len - 1, prompt_len - 2, draft_prompt)) return r;
-      continue;
-    }
-    if (int r = prefill_range(c, false, b, 0, prompt_len - 1)) return r;
+  const bool draft_prompt = k > 0 && !c->share_kv;  // a sharing draft has no prompt pass of its own
+  if (c->use_dense && prompt_len - 1 >= kDenseMinRows) {
+    if (int r = prefill_dense_all(c, batch, prompt_len - 1, draft_prompt)) return r;
+  } else {
+    if (int r = prefill_passes(c, false, batch, prompt_len - 1)) return r;
     if (draft_prompt)
-      if (int r = prefill_range(c, true, b, 0, prompt_len - 2)) return r;
+      if (int r = prefill_passes(c, true, batch, prompt_len - 2)) return r;
   }
   CU_OK(c, cudaEventRecord(c->ev[1], st));
 

@@ -27,12 +27,13 @@ enum PassKind {
   PASS_TOKENS = 0,       // rows r = 0..count-1 of one sequence: token src[r], position start + r
   PASS_DRAFT_FIRST = 1,  // rows_per_seq (2, or 1 when the draft shares the target's cache) rows per sequence: the last committed tokens
   PASS_DRAFT_NEXT = 2,   // 1 row per sequence: draft token number `step` (1-based step >= 1)
+  PASS_PROMPT = 4,       // `count` rows per sequence from slot seq on: prompt tokens at positions start..start+count-1
   PASS_VERIFY = 3        // k+1 rows per sequence: last committed token, then the k drafts
 };
 
 struct PassDesc {
   int kind, step, rows_per_seq, n_seq;
-  int seq, start, count;  // PASS_TOKENS
+  int seq, start, count;  // PASS_TOKENS, PASS_PROMPT
   const int* src;         // PASS_TOKENS: device token ids
   // Greedy decision fused into the lm-head (whole-pass kernel): the previous pass left, per row and
   // per 128-feature group of the vocabulary, the largest logit and its index; the kernel that needs
@@ -118,6 +119,10 @@ plan_embed_kernel(PassDesc pd, const GenState* gs, const int* seq_tok, int max_s
         tok = ld_act(pd.src + m);
         pos = pd.start + m;
       }
+    } else if (pd.kind == PASS_PROMPT) {
+      seq = pd.seq + m / pd.count;
+      pos = pd.start + m % pd.count;
+      tok = ld_act(seq_tok + (size_t)seq * max_seq + pos);
     } else {
       const int R = pd.rows_per_seq;
       const int b = m / R, i = m - b * R;

@@ -1,8 +1,8 @@
-// Causal attention over a whole prompt (the pass that fills the KV cache, Section II-A), one
-// sequence at a time: row m (position m) attends keys 0..m of the cache the QKV epilogue of the
-// same layer has just written.
+// Causal attention over whole prompts (the pass that fills the KV cache, Section II-A), of M tokens
+// each, sequences seq, seq + 1, ... (blockIdx.z): row m of a sequence (position m) attends keys 0..m of the
+// cache the QKV epilogue of the same layer has just written; sequence z's rows are rows z*M .. of q and out.
 //
-// One CTA = (block of 64 query rows, head); its four warps own 16 query rows each and walk the key
+// One CTA = (block of 64 query rows, head, sequence); its four warps own 16 query rows each and walk the key
 // blocks 0..diagonal with the usual running max / running sum per row (exact softmax, rescaled as
 // the maximum grows).  Both products run on mma.sync.m16n8k16 with fp32 accumulators:
 //   S = Q K^T    Q is fp32: split q = hi + lo into bf16, two MMAs; K is bf16 in the cache
@@ -52,6 +52,8 @@ __global__ void __launch_bounds__(kPfaThreads)
 prefill_attention_kernel(const float* __restrict__ q, const __nv_bfloat16* __restrict__ kcache,
                          const __nv_bfloat16* __restrict__ vcache, float* __restrict__ out, int M, int n_heads, int max_seq,
                          int seq, float scale, unsigned char* __restrict__ img, int img_rb, int img_kb) {
+  seq += blockIdx.z;
+  const int row_base = blockIdx.z * M;
   constexpr int LD = HD + 8;
   extern __shared__ __align__(16) unsigned char pfa_smem[];
   __nv_bfloat16* sQh = reinterpret_cast<__nv_bfloat16*>(pfa_smem);
@@ -93,7 +95,7 @@ prefill_attention_kernel(const float* __restrict__ q, const __nv_bfloat16* __res
   for (int e = tid; e < kPfaQ * (HD / 4); e += kPfaThreads) {
     const int i = e / (HD / 4), d = (e - i * (HD / 4)) * 4;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (q0 + i < M) v = ld_act4(q + (size_t)(q0 + i) * d_model + head * HD + d);
+    if (q0 + i < M) v = ld_act4(q + (size_t)(row_base + q0 + i) * d_model + head * HD + d);
     uint2 hi, lo;
     split_pack(v.x, v.y, hi.x, lo.x);
     split_pack(v.z, v.w, hi.y, lo.y);
@@ -214,6 +216,7 @@ prefill_attention_kernel(const float* __restrict__ q, const __nv_bfloat16* __res
   // O-projection on the dense path: bf16 hi + lo, two neighbouring columns per 4-byte store (layout
   // as in attn_store of attention.cuh: row block img_rb, img_kb k blocks of 64).
   auto put = [&](int m, int col, float x0, float x1) {
+    m += row_base;
     if (img == nullptr) {
       *reinterpret_cast<float2*>(out + (size_t)m * d_model + col) = make_float2(x0, x1);
       return;

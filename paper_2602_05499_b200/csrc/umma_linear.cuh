@@ -87,8 +87,8 @@ struct UmmaParams {
   int M;                   // valid rows (<= n_rb * RB)
   int n_pairs;             // valid output pairs (<= 64 * n_ft)
   int n_stages;
-  float* partial;          // [grid][RB * 128] partial accumulators of cut tiles
-  int* flags;              // [grid], zero between launches: "CTA c has posted its partial accumulator"
+  float* partial;          // [grid][row blocks if RB_INNER][RB * 128] partial accumulators of cut tiles
+  int* flags;              // [grid][row blocks if RB_INNER], zero between launches: "CTA c has posted its partial accumulator"
   int* flags_post;         // where a CTA raises its flag: flags, except under the failure-path test hook
   int* error;              // first UmmaError seen, sticky
   unsigned long long wait_limit_ns;  // after this long a wait gives up (kWaitLimitNs unless the test hook shortens it)
@@ -215,6 +215,10 @@ struct UmSeg {
   int tile, kb0, kb1;
 };
 
+// RB_INNER false: one list of (feature tile, row block) tiles is cut over the CTAs.  true: a list of feature
+// tiles is, and a CTA takes each of its pieces through all row blocks before the next piece; where the
+// cuts lie, and so the order of a row's sums, then does not depend on how many rows there are.
+template <bool RB_INNER>
 __global__ void __launch_bounds__(kUmThreads, 1) umma_linear_kernel(UmmaParams p) {
   extern __shared__ unsigned char um_smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(um_smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -224,7 +228,8 @@ __global__ void __launch_bounds__(kUmThreads, 1) umma_linear_kernel(UmmaParams p
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int cta = blockIdx.x, n_cta = gridDim.x;
   const int KB = p.KB;
-  const long long n_units = (long long)p.n_ft * p.n_rb * KB;
+  const int n_in = RB_INNER ? p.n_rb : 1, n_outer = RB_INNER ? 1 : p.n_rb;  // row blocks per piece; per feature tile in the list
+  const long long n_units = (long long)p.n_ft * n_outer * KB;
   long long ub, ue;
   unit_range(n_units, cta, n_cta, ub, ue);
 
@@ -282,33 +287,37 @@ __global__ void __launch_bounds__(kUmThreads, 1) umma_linear_kernel(UmmaParams p
         phase = 0;
         for (long long u = ub; u < ue && ok;) {
           const UmSeg s = next_seg(u);
-          const int ft = s.tile / p.n_rb, rb = s.tile - ft * p.n_rb;
-          const unsigned char* wsrc = p.W + ((size_t)ft * KB + s.kb0) * kUmABytes;
-          const unsigned char* xsrc = p.X + ((size_t)rb * KB + s.kb0) * um_b_stage_bytes(p.RB);
-          for (int kb = s.kb0; kb < s.kb1; ++kb, ++i) {
-            const bool early = i < (unsigned)p.n_stages;  // first use of its stage: nothing to wait for
-            if (pass == 0 && !early) break;
-            unsigned char* dst = smem + (size_t)stage * stage_bytes;
-            if (pass == 0) {
-              mbar_arrive_expect_tx(&sh->full[stage], (unsigned)stage_bytes);
-              bulk_load(dst, wsrc, kUmABytes, &sh->full[stage], pol);
-              ++issued;
-            } else if (early) {
-              bulk_load(dst + kUmABytes, xsrc, (unsigned)um_b_stage_bytes(p.RB), &sh->full[stage], pol_x);
-            } else {
-              ok = um_wait([&] { return mbar_try_wait(&sh->empty[stage], phase ^ 1u); }, p.error, s_abort, UMMA_ERR_STAGE_EMPTY, p.wait_limit_ns);
-              if (!ok) break;
-              mbar_arrive_expect_tx(&sh->full[stage], (unsigned)stage_bytes);
-              bulk_load(dst, wsrc, kUmABytes, &sh->full[stage], pol);
-              bulk_load(dst + kUmABytes, xsrc, (unsigned)um_b_stage_bytes(p.RB), &sh->full[stage], pol_x);
-              ++issued;
+          const int ft = s.tile / n_outer, rb0 = s.tile - ft * n_outer;
+          for (int rin = 0; rin < n_in && ok; ++rin) {
+            const unsigned char* wsrc = p.W + ((size_t)ft * KB + s.kb0) * kUmABytes;
+            const unsigned char* xsrc = p.X + ((size_t)(rb0 + rin) * KB + s.kb0) * um_b_stage_bytes(p.RB);
+            const uint64_t pol_w = rin + 1 < n_in ? pol_x : pol;  // a weight that comes back for the next row block stays in L2
+            for (int kb = s.kb0; kb < s.kb1; ++kb, ++i) {
+              const bool early = i < (unsigned)p.n_stages;  // first use of its stage: nothing to wait for
+              if (pass == 0 && !early) break;
+              unsigned char* dst = smem + (size_t)stage * stage_bytes;
+              if (pass == 0) {
+                mbar_arrive_expect_tx(&sh->full[stage], (unsigned)stage_bytes);
+                bulk_load(dst, wsrc, kUmABytes, &sh->full[stage], pol_w);
+                ++issued;
+              } else if (early) {
+                bulk_load(dst + kUmABytes, xsrc, (unsigned)um_b_stage_bytes(p.RB), &sh->full[stage], pol_x);
+              } else {
+                ok = um_wait([&] { return mbar_try_wait(&sh->empty[stage], phase ^ 1u); }, p.error, s_abort, UMMA_ERR_STAGE_EMPTY, p.wait_limit_ns);
+                if (!ok) break;
+                mbar_arrive_expect_tx(&sh->full[stage], (unsigned)stage_bytes);
+                bulk_load(dst, wsrc, kUmABytes, &sh->full[stage], pol_w);
+                bulk_load(dst + kUmABytes, xsrc, (unsigned)um_b_stage_bytes(p.RB), &sh->full[stage], pol_x);
+                ++issued;
+              }
+              wsrc += kUmABytes;
+              xsrc += um_b_stage_bytes(p.RB);
+              if (++stage == p.n_stages) {
+                stage = 0;
+                phase ^= 1u;
+              }
             }
-            wsrc += kUmABytes;
-            xsrc += um_b_stage_bytes(p.RB);
-            if (++stage == p.n_stages) {
-              stage = 0;
-              phase ^= 1u;
-            }
+            if (pass == 0 && i >= (unsigned)p.n_stages) break;
           }
           if (pass == 0 && i >= (unsigned)p.n_stages) break;
           u += s.kb1 - s.kb0;
@@ -336,31 +345,33 @@ __global__ void __launch_bounds__(kUmThreads, 1) umma_linear_kernel(UmmaParams p
       bool ok = true;
       for (long long u = ub; u < ue && ok;) {
         const UmSeg s = next_seg(u);
-        ok = um_wait([&] { return mbar_try_wait(&sh->acc_empty[buf], acc_phase ^ 1u); }, p.error, s_abort, UMMA_ERR_ACC_EMPTY, p.wait_limit_ns);
-        if (!ok) break;
-        um_fence_after();
-        const uint32_t tmem_d = tmem_base + (uint32_t)(buf * 2 * p.RB);
-        for (int kb = s.kb0; kb < s.kb1; ++kb) {
-          ok = um_wait([&] { return mbar_try_wait(&sh->full[stage], phase); }, p.error, s_abort, UMMA_ERR_STAGE_FULL, p.wait_limit_ns);
+        for (int rin = 0; rin < n_in && ok; ++rin) {
+          ok = um_wait([&] { return mbar_try_wait(&sh->acc_empty[buf], acc_phase ^ 1u); }, p.error, s_abort, UMMA_ERR_ACC_EMPTY, p.wait_limit_ns);
           if (!ok) break;
           um_fence_after();
-          const uint32_t a0 = smem_u32(smem + (size_t)stage * stage_bytes);
-          const uint32_t b0 = a0 + kUmABytes;
+          const uint32_t tmem_d = tmem_base + (uint32_t)(buf * 2 * p.RB);
+          for (int kb = s.kb0; kb < s.kb1; ++kb) {
+            ok = um_wait([&] { return mbar_try_wait(&sh->full[stage], phase); }, p.error, s_abort, UMMA_ERR_STAGE_FULL, p.wait_limit_ns);
+            if (!ok) break;
+            um_fence_after();
+            const uint32_t a0 = smem_u32(smem + (size_t)stage * stage_bytes);
+            const uint32_t b0 = a0 + kUmABytes;
 #pragma unroll
-          for (int st = 0; st < kUmBK / 16; ++st) {
-            const uint64_t ad = um_desc(a0 + st * 4096u, 2048u, 128u);
-            const uint64_t bd = um_desc(b0 + st * 2u * lbo_b, lbo_b, 128u);
-            um_mma(tmem_d, ad, bd, idesc, (kb > s.kb0 || st > 0) ? 1u : 0u);
+            for (int st = 0; st < kUmBK / 16; ++st) {
+              const uint64_t ad = um_desc(a0 + st * 4096u, 2048u, 128u);
+              const uint64_t bd = um_desc(b0 + st * 2u * lbo_b, lbo_b, 128u);
+              um_mma(tmem_d, ad, bd, idesc, (kb > s.kb0 || st > 0) ? 1u : 0u);
+            }
+            um_commit(&sh->empty[stage]);  // the stage is free once these MMAs have read it
+            if (++stage == p.n_stages) {
+              stage = 0;
+              phase ^= 1u;
+            }
           }
-          um_commit(&sh->empty[stage]);  // the stage is free once these MMAs have read it
-          if (++stage == p.n_stages) {
-            stage = 0;
-            phase ^= 1u;
-          }
+          if (!ok) break;
+          um_commit(&sh->acc_full[buf]);
+          if ((buf ^= 1) == 0) acc_phase ^= 1u;
         }
-        if (!ok) break;
-        um_commit(&sh->acc_full[buf]);
-        if ((buf ^= 1) == 0) acc_phase ^= 1u;
         u += s.kb1 - s.kb0;
       }
     }
@@ -398,164 +409,171 @@ __global__ void __launch_bounds__(kUmThreads, 1) umma_linear_kernel(UmmaParams p
       um_epi_sync();
       inv_rb = rb_;
     };
-    if (ub < ue) ensure_inv(next_seg(ub).tile % p.n_rb);
-    for (long long u = ub; u < ue;) {
+    if (ub < ue) ensure_inv(next_seg(ub).tile % n_outer);
+    bool alive = true;
+    for (long long u = ub; u < ue && alive;) {
       const UmSeg s = next_seg(u);
-      const int ft = s.tile / p.n_rb, rb = s.tile - ft * p.n_rb;
-      const bool starts = s.kb0 == 0, whole = starts && s.kb1 == KB;
-      const bool owner = starts && !whole;
-      const bool okw = um_wait([&] { return mbar_try_wait(&sh->acc_full[buf], acc_phase); }, p.error, s_abort, UMMA_ERR_ACC_FULL, p.wait_limit_ns);
-      (void)okw;
-      if (owner && et == 0) {
-        // the rest of the tile lies at the start of the ranges of the CTAs that follow
-        const long long tile_end = (long long)(s.tile + 1) * KB;
-        int n = 0;
-        for (int c2 = cta + 1; c2 < n_cta; ++c2) {
-          long long b2, e2;
-          unit_range(n_units, c2, n_cta, b2, e2);
-          if (b2 >= tile_end) break;
-          if (e2 > b2) {
-            um_wait([&] { return ld_acquire(p.flags + c2) != 0; }, p.error, s_abort, UMMA_ERR_POST, p.wait_limit_ns);
-            sh->posts[n++] = c2;
-          }
-        }
-        sh->n_posts = n;
-      }
-      um_epi_sync();
-      if (et == 0) sh->decision = sh->abort;
-      um_epi_sync();
-      if (sh->decision) break;
-      um_fence_after();
-      const int n_posts = owner ? sh->n_posts : 0;
-      const int row0 = rb * RB;
-      ensure_inv(rb);
-      float* my_post = p.partial + (size_t)cta * (RB * kUmFeat);
-      // the output pair this thread finishes, located once per piece (not once per row)
-      const int pg = ft * 64 + pl;
-      int q_t = 0, q_head = 0, q_i = 0;
-      if (p.ep.mode == EPI_QKV) {
-        const int hp = p.ep.head_dim >> 1, per_tensor = p.ep.n_heads * hp;
-        q_t = pg / per_tensor;
-        const int rem = pg - q_t * per_tensor;
-        q_head = rem / hp;
-        q_i = rem - q_head * hp;
-      }
-      for (int c = chalf; c < RB / kUmChunk; c += 2) {
-        if (row0 + c * kUmChunk >= p.M) break;  // rows that carry nothing (uniform over the warp)
-        float hi[16], lo[16];
-        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 2 * RB + c * kUmChunk);
-        um_ld16(taddr, hi);
-        um_ld16(taddr + (uint32_t)RB, lo);
-#pragma unroll
-        for (int t = 0; t < 16; ++t) hi[t] += lo[t];
-        if (!starts) {  // a piece from the middle or the end of a tile: post it
-#pragma unroll
-          for (int t = 0; t < 16; ++t) my_post[(size_t)(c * kUmChunk + t) * kUmFeat + R] = hi[t];
-          continue;
-        }
-        for (int k2 = 0; k2 < n_posts; ++k2) {
-          const float* src = p.partial + (size_t)sh->posts[k2] * (RB * kUmFeat) + (size_t)(c * kUmChunk) * kUmFeat + R;
-#pragma unroll
-          for (int t = 0; t < 16; ++t) hi[t] += __ldcg(src + t * kUmFeat);
-        }
-        // The two features of an output pair sit 16 lanes apart in the same warp: one shuffle per
-        // row brings them together, and thread (pair, half) finishes rows half*8 .. half*8+7.
-        const bool want_img = p.img_out != nullptr;
-        float keep0[8], keep1[8];  // results this thread owes the output image
-#pragma unroll
-        for (int t8 = 0; t8 < 8; ++t8) {
-          const float own_lo = hi[t8], own_hi = hi[8 + t8];  // rows 0..7 and 8..15 of the chunk, this lane's feature
-          const float oth_lo = __shfl_xor_sync(0xffffffffu, own_lo, 16), oth_hi = __shfl_xor_sync(0xffffffffu, own_hi, 16);
-          float v0 = half ? oth_hi : own_lo, v1 = half ? own_hi : oth_lo;
-          const int t = half * 8 + t8;
-          const int m = row0 + c * kUmChunk + t;
-          keep0[t8] = 0.f;
-          keep1[t8] = 0.f;
-          if (m < p.M && pg < p.n_pairs) {
-            if (p.ssq_in != nullptr) {
-              const float inv = sh->inv[c * kUmChunk + t];
-              v0 *= inv;
-              v1 *= inv;
-            }
-            if (p.ep.mode == EPI_RESID && want_img) {
-              const int r0 = ((pg >> 3) << 4) + (pg & 7);
-              float* hp = p.ep.out + (size_t)m * p.ep.out_ld;
-              keep0[t8] = ld_act(hp + r0) + v0;
-              keep1[t8] = ld_act(hp + r0 + 8) + v1;
-              hp[r0] = keep0[t8];
-              hp[r0 + 8] = keep1[t8];
-            } else if (p.ep.mode == EPI_SWIGLU && want_img) {
-              keep0[t8] = (v0 / (1.0f + __expf(-v0))) * v1;
-              if (p.ep.out != nullptr) p.ep.out[(size_t)m * p.ep.out_ld + pg] = keep0[t8];
-            } else if (p.ep.mode == EPI_QKV) {
-              um_qkv_epilogue(p.ep, q_t, q_head, q_i, m, v0, v1);
-            } else {
-              apply_epilogue<__nv_bfloat16>(p.ep, pg, m, v0, v1);
+      const int ft = s.tile / n_outer, rb0 = s.tile - ft * n_outer;
+      for (int rin = 0; rin < n_in; ++rin) {
+        const int rb = rb0 + rin;
+        const bool starts = s.kb0 == 0, whole = starts && s.kb1 == KB;
+        const bool owner = starts && !whole;
+        const bool okw = um_wait([&] { return mbar_try_wait(&sh->acc_full[buf], acc_phase); }, p.error, s_abort, UMMA_ERR_ACC_FULL, p.wait_limit_ns);
+        (void)okw;
+        if (owner && et == 0) {
+          // the rest of the tile lies at the start of the ranges of the CTAs that follow
+          const long long tile_end = (long long)(s.tile + 1) * KB;
+          int n = 0;
+          for (int c2 = cta + 1; c2 < n_cta; ++c2) {
+            long long b2, e2;
+            unit_range(n_units, c2, n_cta, b2, e2);
+            if (b2 >= tile_end) break;
+            if (e2 > b2) {
+              um_wait([&] { return ld_acquire(p.flags + c2 * n_in + rin) != 0; }, p.error, s_abort, UMMA_ERR_POST, p.wait_limit_ns);
+              sh->posts[n++] = c2;
             }
           }
+          sh->n_posts = n;
         }
-        if (want_img) {
-          // Results into this warp's own piece of shared memory as [feature][row], then out as 16-byte
-          // pieces of the image (8 consecutive features of one row, high parts and low parts).  A warp
-          // covers 32 consecutive features of the residual stream, or 16 consecutive columns of u.
-          const bool resid = p.ep.mode == EPI_RESID;
-          float* exw = ex + ew * (32 * kUmExLd);
-          const int li = lane & 15;
-          const int f0 = resid ? ((li >> 3) << 4) + (li & 7) : li;
-          __syncwarp();
+        um_epi_sync();
+        if (et == 0) sh->decision = sh->abort;
+        um_epi_sync();
+        if (sh->decision) {
+          alive = false;
+          break;
+        }
+        um_fence_after();
+        const int n_posts = owner ? sh->n_posts : 0;
+        const int row0 = rb * RB;
+        ensure_inv(rb);
+        float* my_post = p.partial + ((size_t)cta * n_in + rin) * (RB * kUmFeat);
+        // the output pair this thread finishes, located once per piece (not once per row)
+        const int pg = ft * 64 + pl;
+        int q_t = 0, q_head = 0, q_i = 0;
+        if (p.ep.mode == EPI_QKV) {
+          const int hp = p.ep.head_dim >> 1, per_tensor = p.ep.n_heads * hp;
+          q_t = pg / per_tensor;
+          const int rem = pg - q_t * per_tensor;
+          q_head = rem / hp;
+          q_i = rem - q_head * hp;
+        }
+        for (int c = chalf; c < RB / kUmChunk; c += 2) {
+          if (row0 + c * kUmChunk >= p.M) break;  // rows that carry nothing (uniform over the warp)
+          float hi[16], lo[16];
+          const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 2 * RB + c * kUmChunk);
+          um_ld16(taddr, hi);
+          um_ld16(taddr + (uint32_t)RB, lo);
+#pragma unroll
+          for (int t = 0; t < 16; ++t) hi[t] += lo[t];
+          if (!starts) {  // a piece from the middle or the end of a tile: post it
+#pragma unroll
+            for (int t = 0; t < 16; ++t) my_post[(size_t)(c * kUmChunk + t) * kUmFeat + R] = hi[t];
+            continue;
+          }
+          for (int k2 = 0; k2 < n_posts; ++k2) {
+            const float* src = p.partial + ((size_t)sh->posts[k2] * n_in + rin) * (RB * kUmFeat) + (size_t)(c * kUmChunk) * kUmFeat + R;
+#pragma unroll
+            for (int t = 0; t < 16; ++t) hi[t] += __ldcg(src + t * kUmFeat);
+          }
+          // The two features of an output pair sit 16 lanes apart in the same warp: one shuffle per
+          // row brings them together, and thread (pair, half) finishes rows half*8 .. half*8+7.
+          const bool want_img = p.img_out != nullptr;
+          float keep0[8], keep1[8];  // results this thread owes the output image
 #pragma unroll
           for (int t8 = 0; t8 < 8; ++t8) {
-            exw[f0 * kUmExLd + half * 8 + t8] = keep0[t8];
-            if (resid) exw[(f0 + 8) * kUmExLd + half * 8 + t8] = keep1[t8];
-          }
-          __syncwarp();
-          const int t = lane & 15, m = row0 + c * kUmChunk + t;
-          const int n_kg = resid ? 4 : 2, feat0 = resid ? ft * 128 + quarter * 32 : ft * 64 + quarter * 16;
-          if (m < p.M) {
-            for (int kgl = lane >> 4; kgl < n_kg; kgl += 2) {
-              float v[8];
-#pragma unroll
-              for (int e = 0; e < 8; ++e) v[e] = exw[(kgl * 8 + e) * kUmExLd + t];
-              const int k0 = feat0 + kgl * 8;  // first feature of the piece = column of the next layer's input
-              if (k0 >= p.img_KB * kUmBK) continue;
-              if (p.gain_out != nullptr) {
-                const float4 g0 = __ldg(reinterpret_cast<const float4*>(p.gain_out + k0)), g1 = __ldg(reinterpret_cast<const float4*>(p.gain_out + k0 + 4));
-                v[0] *= g0.x; v[1] *= g0.y; v[2] *= g0.z; v[3] *= g0.w;
-                v[4] *= g1.x; v[5] *= g1.y; v[6] *= g1.z; v[7] *= g1.w;
+            const float own_lo = hi[t8], own_hi = hi[8 + t8];  // rows 0..7 and 8..15 of the chunk, this lane's feature
+            const float oth_lo = __shfl_xor_sync(0xffffffffu, own_lo, 16), oth_hi = __shfl_xor_sync(0xffffffffu, own_hi, 16);
+            float v0 = half ? oth_hi : own_lo, v1 = half ? own_hi : oth_lo;
+            const int t = half * 8 + t8;
+            const int m = row0 + c * kUmChunk + t;
+            keep0[t8] = 0.f;
+            keep1[t8] = 0.f;
+            if (m < p.M && pg < p.n_pairs) {
+              if (p.ssq_in != nullptr) {
+                const float inv = sh->inv[c * kUmChunk + t];
+                v0 *= inv;
+                v1 *= inv;
               }
-              uint4 h4, l4;
-              split_pack(v[0], v[1], h4.x, l4.x);
-              split_pack(v[2], v[3], h4.y, l4.y);
-              split_pack(v[4], v[5], h4.z, l4.z);
-              split_pack(v[6], v[7], h4.w, l4.w);
-              unsigned char* dst = p.img_out + um_img_offset(RB, p.img_KB, m, k0 >> 3);
-              *reinterpret_cast<uint4*>(dst) = h4;
-              *reinterpret_cast<uint4*>(dst + um_img_lo(RB)) = l4;
+              if (p.ep.mode == EPI_RESID && want_img) {
+                const int r0 = ((pg >> 3) << 4) + (pg & 7);
+                float* hp = p.ep.out + (size_t)m * p.ep.out_ld;
+                keep0[t8] = ld_act(hp + r0) + v0;
+                keep1[t8] = ld_act(hp + r0 + 8) + v1;
+                hp[r0] = keep0[t8];
+                hp[r0 + 8] = keep1[t8];
+              } else if (p.ep.mode == EPI_SWIGLU && want_img) {
+                keep0[t8] = (v0 / (1.0f + __expf(-v0))) * v1;
+                if (p.ep.out != nullptr) p.ep.out[(size_t)m * p.ep.out_ld + pg] = keep0[t8];
+              } else if (p.ep.mode == EPI_QKV) {
+                um_qkv_epilogue(p.ep, q_t, q_head, q_i, m, v0, v1);
+              } else {
+                apply_epilogue<__nv_bfloat16>(p.ep, pg, m, v0, v1);
+              }
             }
           }
-          if (resid && p.ssq_out != nullptr && lane < 16 && m < p.M) {
-            float ssum = 0.f;  // this warp's 32 features of row `lane`, in feature order
-            for (int fl = 0; fl < 32; ++fl) {
-              const float x = exw[fl * kUmExLd + lane];
-              ssum = fmaf(x, x, ssum);
+          if (want_img) {
+            // Results into this warp's own piece of shared memory as [feature][row], then out as 16-byte
+            // pieces of the image (8 consecutive features of one row, high parts and low parts).  A warp
+            // covers 32 consecutive features of the residual stream, or 16 consecutive columns of u.
+            const bool resid = p.ep.mode == EPI_RESID;
+            float* exw = ex + ew * (32 * kUmExLd);
+            const int li = lane & 15;
+            const int f0 = resid ? ((li >> 3) << 4) + (li & 7) : li;
+            __syncwarp();
+#pragma unroll
+            for (int t8 = 0; t8 < 8; ++t8) {
+              exw[f0 * kUmExLd + half * 8 + t8] = keep0[t8];
+              if (resid) exw[(f0 + 8) * kUmExLd + half * 8 + t8] = keep1[t8];
             }
-            p.ssq_out[(size_t)(ft * 4 + quarter) * p.ssq_ld + m] = ssum;
+            __syncwarp();
+            const int t = lane & 15, m = row0 + c * kUmChunk + t;
+            const int n_kg = resid ? 4 : 2, feat0 = resid ? ft * 128 + quarter * 32 : ft * 64 + quarter * 16;
+            if (m < p.M) {
+              for (int kgl = lane >> 4; kgl < n_kg; kgl += 2) {
+                float v[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = exw[(kgl * 8 + e) * kUmExLd + t];
+                const int k0 = feat0 + kgl * 8;  // first feature of the piece = column of the next layer's input
+                if (k0 >= p.img_KB * kUmBK) continue;
+                if (p.gain_out != nullptr) {
+                  const float4 g0 = __ldg(reinterpret_cast<const float4*>(p.gain_out + k0)), g1 = __ldg(reinterpret_cast<const float4*>(p.gain_out + k0 + 4));
+                  v[0] *= g0.x; v[1] *= g0.y; v[2] *= g0.z; v[3] *= g0.w;
+                  v[4] *= g1.x; v[5] *= g1.y; v[6] *= g1.z; v[7] *= g1.w;
+                }
+                uint4 h4, l4;
+                split_pack(v[0], v[1], h4.x, l4.x);
+                split_pack(v[2], v[3], h4.y, l4.y);
+                split_pack(v[4], v[5], h4.z, l4.z);
+                split_pack(v[6], v[7], h4.w, l4.w);
+                unsigned char* dst = p.img_out + um_img_offset(RB, p.img_KB, m, k0 >> 3);
+                *reinterpret_cast<uint4*>(dst) = h4;
+                *reinterpret_cast<uint4*>(dst + um_img_lo(RB)) = l4;
+              }
+            }
+            if (resid && p.ssq_out != nullptr && lane < 16 && m < p.M) {
+              float ssum = 0.f;  // this warp's 32 features of row `lane`, in feature order
+              for (int fl = 0; fl < 32; ++fl) {
+                const float x = exw[fl * kUmExLd + lane];
+                ssum = fmaf(x, x, ssum);
+              }
+              p.ssq_out[(size_t)(ft * 4 + quarter) * p.ssq_ld + m] = ssum;
+            }
           }
         }
+        // tensor memory of this accumulator has been read: hand it back to the MMA warp
+        um_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh->acc_empty[buf]);
+        if (!starts) {
+          __threadfence();
+          um_epi_sync();
+          if (et == 0) st_release(p.flags_post + cta * n_in + rin, 1);
+        } else if (owner) {
+          um_epi_sync();  // every thread has read the posts
+          if (et < n_posts) p.flags[sh->posts[et] * n_in + rin] = 0;
+        }
+        if ((buf ^= 1) == 0) acc_phase ^= 1u;
       }
-      // tensor memory of this accumulator has been read: hand it back to the MMA warp
-      um_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sh->acc_empty[buf]);
-      if (!starts) {
-        __threadfence();
-        um_epi_sync();
-        if (et == 0) st_release(p.flags_post + cta, 1);
-      } else if (owner) {
-        um_epi_sync();  // every thread has read the posts
-        if (et < n_posts) p.flags[sh->posts[et]] = 0;
-      }
-      if ((buf ^= 1) == 0) acc_phase ^= 1u;
       u += s.kb1 - s.kb0;
     }
   }

@@ -860,6 +860,46 @@ def test_time_linear_hook_on_both_bf16_paths():
             eng.close()
 
 
+@pytest.mark.parametrize("batch,prompt_len", [
+    (3, 17),     # the shortest prompts on the dense path: 48 rows, one row block
+    (8, 18),     # 136 rows: a sequence across two row blocks
+    (12, 101),   # 1200 rows: a group of ten prompts and one of two
+    (4, 129),    # one whole row block each
+    (4, 130),    # one row more than a block: one prompt after the other
+])
+def test_grouped_prompts_equal_solo_runs(batch, prompt_len):
+    """Prompts that share a sweep of the weights: every sequence's tokens and acceptance counts are those of its solo run
+    in the same context, for the target's cache (autoregressive) and the draft's (speculative)."""
+    eng, m, _ = make_pair(si.TINY_BF16, (1, 2), max_seq=prompt_len + 24, max_batch=batch, k_max=4)
+    try:
+        prompts = si.make_prompts(m.vocab, batch, prompt_len, seed=70 + batch)
+        spec, ar = eng.sdfp_generate(prompts, 4, 16), eng.sdfp_generate(prompts, 0, 16)
+        for b in range(batch):
+            assert spec.tokens[b] == ar.tokens[b]
+        for b in (0, 1, batch - 1):
+            solo = eng.sdfp_generate(prompts[b:b + 1], 4, 16)
+            assert solo.tokens[0] == spec.tokens[b]
+            n = solo.n_rounds
+            assert spec.stats[:n, b, 1].tolist() == solo.stats[:, 0, 1].tolist()
+    finally:
+        eng.close()
+
+
+@pytest.mark.parametrize("batch,prompt_len,dtype", [(5, 40, "f32"), (2, 9, "bf16"), (16, 6, "bf16"), (3, 100, "f32")])
+def test_prompt_passes_of_a_batch_equal_solo_runs(batch, prompt_len, dtype):
+    """Prompts that go through the decode passes (fp32 models, prompts of a few tokens), several sequences to a pass."""
+    eng, m, _ = make_pair(si.TINY if dtype == "f32" else si.TINY_BF16, (1, 2), max_seq=prompt_len + 24, max_batch=batch, k_max=4)
+    try:
+        prompts = si.make_prompts(m.vocab, batch, prompt_len, seed=90 + batch)
+        out = eng.sdfp_generate(prompts, 4, 12)
+        for b in range(batch):
+            solo = eng.sdfp_generate(prompts[b:b + 1], 4, 12)
+            assert solo.tokens[0] == out.tokens[b]
+            assert out.stats[:solo.n_rounds, b, 1].tolist() == solo.stats[:, 0, 1].tolist()
+    finally:
+        eng.close()
+
+
 def test_largest_batch_and_row_count():
     """The library's limits in one context: 16 sequences, k = 4, 80 rows in a verify pass (row block of
     80 rows = MMA width 160), 32 rows in the first draft pass; prompts of one token (nothing to cache
