@@ -206,9 +206,16 @@ struct LinearCall {
   EpiParams ep;
 };
 
-int linear_grid_fma(const sdfp_ctx* c, int n_pairs) {
-  const int want = (n_pairs + 7) / 8;
-  return std::max(1, std::min(want, c->num_sms * 8));
+// P pairs per warp: more share the reads of the rows, fewer spread a small matrix over the SMs
+template <typename WT>
+cudaError_t launch_linear_fma(sdfp_ctx* c, const LinearCall& lc) {
+  const int row_groups = (lc.rows + kFmaRows - 1) / kFmaRows;
+  const long long ctas4 = (long long)((lc.n_pairs + 4 * kFmaWarps - 1) / (4 * kFmaWarps)) * row_groups;
+  const int P = ctas4 >= 2LL * c->num_sms ? 4 : ctas4 >= c->num_sms ? 2 : 1;
+  auto kernel = P == 4 ? linear_fma_kernel<WT, WT, 4> : P == 2 ? linear_fma_kernel<WT, WT, 2> : linear_fma_kernel<WT, WT, 1>;
+  const dim3 grid((lc.n_pairs + P * kFmaWarps - 1) / (P * kFmaWarps), row_groups);
+  return launch(c, kernel, grid, dim3(kFmaThreads), 0, reinterpret_cast<const WT*>(lc.w), lc.x, lc.ldx, lc.rows, lc.K, lc.n_pairs,
+                lc.gain, c->cfg.rms_eps, lc.ep);
 }
 
 UmmaParams dense_params(const sdfp_ctx* c, const void* w_img, const unsigned char* x_img, int rows, int RB, int KB, int n_pairs,
@@ -267,13 +274,7 @@ cudaError_t run_linear(sdfp_ctx* c, const LinearCall& lc) {
     return run_dense_linear(c, lc.w, lc.x, lc.ldx, lc.rows, lc.K, lc.n_pairs, lc.gain, lc.ep);
   if (c->use_mma)
     return launch_linear_mma(c->L, c->num_sms, lc.w, lc.x, lc.ldx, lc.rows, lc.K, lc.n_pairs, lc.gain, c->cfg.rms_eps, lc.ep);
-  const dim3 grid(linear_grid_fma(c, lc.n_pairs)), block(kFmaThreads);
-  if (c->bf16)
-    return launch(c, linear_fma_kernel<__nv_bfloat16, __nv_bfloat16>, grid, block, 0,
-                  reinterpret_cast<const __nv_bfloat16*>(lc.w), lc.x, lc.ldx, lc.rows, lc.K, lc.n_pairs, lc.gain,
-                  c->cfg.rms_eps, lc.ep);
-  return launch(c, linear_fma_kernel<float, float>, grid, block, 0, reinterpret_cast<const float*>(lc.w), lc.x,
-                lc.ldx, lc.rows, lc.K, lc.n_pairs, lc.gain, c->cfg.rms_eps, lc.ep);
+  return c->bf16 ? launch_linear_fma<__nv_bfloat16>(c, lc) : launch_linear_fma<float>(c, lc);
 }
 
 EpiParams base_epi(const sdfp_ctx* c, int mode, float* out, int ld) {

@@ -1,11 +1,18 @@
-// CUDA-core weight-streaming linear kernel: Y = [RMSNorm](X) · Wᵀ with a fused epilogue.
+// CUDA-core linear kernel: Y = [RMSNorm](X) · Wᵀ with a fused epilogue.
 //
 // Used for fp32 models (the tiny configuration) and, on request, for bf16 models as
 // the comparison path of the tensor-core kernel.  Weights are stored pair-major,
-// W[pair][2][K] (see EpiMode in common.cuh for what a pair is).  One warp owns one
-// pair at a time and sweeps K with 128-bit loads; lanes reduce with a fixed xor
-// tree.  A row's result does not depend on how many rows the launch carries:
-// every row runs the same instruction sequence on its own accumulators.
+// W[pair][2][K] (see EpiMode in common.cuh for what a pair is).
+//
+// A CTA takes eight rows and 8 P pairs.  The rows are brought into shared memory once for all its warps
+// (normalised there), a warp owns P pairs and sweeps K with its lanes, 128-bit loads, and the lanes' sums
+// are added in the fixed xor tree.  What bounds it: at a few rows the chain of round trips from the
+// previous kernel's end to this one's (the weights of the first steps are therefore asked for before
+// the wait), at many rows the FMAs.  When every warp read the rows from L2 itself and re-read its weights for
+// every eight rows, that traffic cost more than either: speculative decoding of 16 sequences, 6 layers d 768,
+// FFN 2352, vocabulary 8192, k = 4: 147 -> 24.5 ms; of one, 4 layers d 256: 10.0 -> 6.7 ms.
+// A row's result does not depend on how many rows the launch carries or on P: every (row, feature) runs
+// the same additions in the same order.
 #pragma once
 
 #include "common.cuh"
@@ -13,80 +20,161 @@
 namespace sdfp {
 
 constexpr int kFmaThreads = 256;
+constexpr int kFmaWarps = kFmaThreads / 32;
+constexpr int kFmaRows = 8;      // rows of a CTA
+constexpr int kFmaCols = 1024;   // columns staged at a time (32 KB of rows)
+constexpr int kFmaAhead = 2;     // k steps (128 columns) whose weights are requested before the wait on the preceding kernel
 
-// inv_rms[m] = 1/sqrt(mean_k x[m,k]^2 + eps), computed redundantly by every CTA in a
-// fixed order: lane-strided sequential sums, then the xor tree.
-__device__ __forceinline__ void cta_inv_rms(const float* X, int ldx, int M, int K, float eps, float* inv_rms) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  for (int m = warp; m < M; m += nwarps) {
-    const float* x = X + (size_t)m * ldx;
-    float s = 0.f;
-    for (int k = lane * 4; k < K; k += 128) {
-      const float4 v = ld_act4(x + k);
-      s = fmaf(v.x, v.x, s);
-      s = fmaf(v.y, v.y, s);
-      s = fmaf(v.z, v.z, s);
-      s = fmaf(v.w, v.w, s);
+// Sum over the warp of N values per lane, N = 2, 4, ... 32: value i ends in the lanes with (lane * N / 32) == i (returned).
+// Each value is added in the xor tree of warp_sum; halving the values with the lanes takes N - 1 + log2(32 / N)
+// shuffles instead of 5 N.
+template <int N>
+__device__ __forceinline__ float warp_sum_scatter(float (&v)[N]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16, n = N; o > 0; o >>= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool up = (lane & o) != 0;  // this lane keeps the upper half of the values
+#pragma unroll
+      for (int i = 0; i < N / 2; ++i)
+        if (i < n) {
+          const float keep = up ? v[i + n] : v[i], give = up ? v[i] : v[i + n];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
     }
-    s = warp_sum(s);
-    if (lane == 0) inv_rms[m] = rsqrtf(s / (float)K + eps);
   }
+  return v[0];
 }
 
-template <typename WT, typename KT>
+template <typename WT, typename KT, int P>
 __global__ void __launch_bounds__(kFmaThreads)
 linear_fma_kernel(const WT* __restrict__ W, const float* __restrict__ X, int ldx, int M, int K, int n_pairs,
                   const float* __restrict__ gain, float eps, EpiParams ep) {
-  __shared__ float inv_rms[kMaxRows];
+  __shared__ __align__(16) float xs[kFmaRows][kFmaCols];
+  __shared__ float s_inv[kFmaRows];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m0 = blockIdx.y * kFmaRows, rows = min(kFmaRows, M - m0);
+  const int p0 = (blockIdx.x * kFmaWarps + warp) * P;  // this warp's first pair
+  const WT* wp[P][2];
+#pragma unroll
+  for (int j = 0; j < P; ++j) {  // pairs beyond the last repeat it; their sums are not used
+    wp[j][0] = W + (size_t)min(p0 + j, n_pairs - 1) * 2 * K;
+    wp[j][1] = wp[j][0] + K;
+  }
+  float4 wq[kFmaAhead][P][2];
+#pragma unroll
+  for (int a = 0; a < kFmaAhead; ++a) {
+    const int k = a * 128 + lane * 4;
+#pragma unroll
+    for (int j = 0; j < P; ++j)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) wq[a][j][h] = k < K ? load4(wp[j][h] + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   pdl_wait();
   pdl_launch_dependents();
-  if (gain != nullptr) {
-    cta_inv_rms(X, ldx, M, K, eps, inv_rms);
-    __syncthreads();
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int p = blockIdx.x * (kFmaThreads / 32) + warp; p < n_pairs; p += gridDim.x * (kFmaThreads / 32)) {
-    const WT* w0p = W + (size_t)p * 2 * K;
-    const WT* w1p = w0p + K;
-    for (int m0 = 0; m0 < M; m0 += 8) {
-      float a0[8], a1[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) a0[i] = a1[i] = 0.f;
+  if (gain != nullptr && K > kFmaCols) {  // rows that do not fit: their norm first
+    if (warp < rows) {
+      const float* x = X + (size_t)(m0 + warp) * ldx;
+      float s = 0.f;
       for (int k = lane * 4; k < K; k += 128) {
-        const float4 w0 = load4(w0p + k);
-        const float4 w1 = load4(w1p + k);
-        float4 g = make_float4(1.f, 1.f, 1.f, 1.f);
-        if (gain != nullptr) g = load4(gain + k);
+        const float4 v = ld_act4(x + k);
+        s = fmaf(v.x, v.x, s);
+        s = fmaf(v.y, v.y, s);
+        s = fmaf(v.z, v.z, s);
+        s = fmaf(v.w, v.w, s);
+      }
+      s = warp_sum(s);
+      if (lane == 0) s_inv[warp] = rsqrtf(s / (float)K + eps);
+    }
+  }
+  float acc[kFmaRows * P * 2];  // [row][pair][half]
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int m = m0 + i;
-          if (m < M) {
-            float4 x = ld_act4(X + (size_t)m * ldx + k);
-            if (gain != nullptr) {
-              const float r = inv_rms[m];
-              x.x = x.x * r * g.x;
-              x.y = x.y * r * g.y;
-              x.z = x.z * r * g.z;
-              x.w = x.w * r * g.w;
-            }
-            a0[i] = fmaf(w0.x, x.x, a0[i]);
-            a0[i] = fmaf(w0.y, x.y, a0[i]);
-            a0[i] = fmaf(w0.z, x.z, a0[i]);
-            a0[i] = fmaf(w0.w, x.w, a0[i]);
-            a1[i] = fmaf(w1.x, x.x, a1[i]);
-            a1[i] = fmaf(w1.y, x.y, a1[i]);
-            a1[i] = fmaf(w1.z, x.z, a1[i]);
-            a1[i] = fmaf(w1.w, x.w, a1[i]);
-          }
+  for (int i = 0; i < kFmaRows * P * 2; ++i) acc[i] = 0.f;
+  for (int c0 = 0; c0 < K; c0 += kFmaCols) {
+    const int nc = min(kFmaCols, K - c0);
+    __syncthreads();  // the previous columns are no longer read (and s_inv is written)
+    // warp r stages row r, each lane the columns it will read itself
+    if (warp < rows) {
+      const float* x = X + (size_t)(m0 + warp) * ldx + c0;
+      float s = 0.f;
+#pragma unroll 4
+      for (int k = lane * 4; k < nc; k += 128) {
+        const float4 v = ld_act4(x + k);
+        *reinterpret_cast<float4*>(&xs[warp][k]) = v;
+        s = fmaf(v.x, v.x, s);
+        s = fmaf(v.y, v.y, s);
+        s = fmaf(v.z, v.z, s);
+        s = fmaf(v.w, v.w, s);
+      }
+      if (gain != nullptr) {
+        float r;
+        if (K <= kFmaCols)
+          r = rsqrtf(warp_sum(s) / (float)K + eps);
+        else
+          r = s_inv[warp];
+        for (int k = lane * 4; k < nc; k += 128) {
+          float4 v = *reinterpret_cast<const float4*>(&xs[warp][k]);
+          const float4 g = load4(gain + c0 + k);
+          v.x = v.x * r * g.x;
+          v.y = v.y * r * g.y;
+          v.z = v.z * r * g.z;
+          v.w = v.w * r * g.w;
+          *reinterpret_cast<float4*>(&xs[warp][k]) = v;
         }
       }
+    } else {
+      for (int k = lane * 4; k < nc; k += 128) *reinterpret_cast<float4*>(&xs[warp][k]) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    for (int k = lane * 4; k < nc; k += 128) {
+      const int kg = c0 + k;
+      float4 w[P][2];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float s0 = warp_sum(a0[i]);
-        const float s1 = warp_sum(a1[i]);
-        if (lane == i && m0 + i < M) apply_epilogue<KT>(ep, p, m0 + i, s0, s1);
+      for (int j = 0; j < P; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) w[j][h] = wq[0][j][h];
+#pragma unroll
+      for (int a = 0; a + 1 < kFmaAhead; ++a)
+#pragma unroll
+        for (int j = 0; j < P; ++j)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) wq[a][j][h] = wq[a + 1][j][h];
+      const int kn = kg + kFmaAhead * 128;
+#pragma unroll
+      for (int j = 0; j < P; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) wq[kFmaAhead - 1][j][h] = kn < K ? load4(wp[j][h] + kn) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < kFmaRows; ++i) {
+        if (i < rows) {
+          const float4 x = *reinterpret_cast<const float4*>(&xs[i][k]);
+#pragma unroll
+          for (int j = 0; j < P; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              float& a = acc[(i * P + j) * 2 + h];
+              a = fmaf(w[j][h].x, x.x, a);
+              a = fmaf(w[j][h].y, x.y, a);
+              a = fmaf(w[j][h].z, x.z, a);
+              a = fmaf(w[j][h].w, x.w, a);
+            }
+        }
       }
     }
+  }
+  // lane groups end up with one (row, pair, half) each; the two halves of a pair sit next to each other
+#pragma unroll
+  for (int b = 0; b < kFmaRows * P * 2; b += 16) {
+    float part[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) part[i] = acc[b + i];
+    const float mine = warp_sum_scatter<16>(part);  // value lane / 2
+    const float other = __shfl_xor_sync(0xffffffffu, mine, 2);
+    const int v = (b + (lane >> 1)) >> 1, row = v / P, pair = p0 + v % P;
+    if ((lane & 3) == 0 && row < rows && pair < n_pairs) apply_epilogue<KT>(ep, pair, m0 + row, mine, other);
   }
 }
 

@@ -900,6 +900,29 @@ def test_prompt_passes_of_a_batch_equal_solo_runs(batch, prompt_len, dtype):
         eng.close()
 
 
+@pytest.mark.parametrize("d_heads,ffn,vocab,rows,flags", [
+    (1, 16, 16, 9, 0),           # fewer columns than one step of a warp, fewer pairs than warps; a second row group of one
+    (9, 1040, 528, 16, 0),       # 1040 columns: more than are staged at a time, by one step's remainder
+    (18, 2064, 1040, 80, 0),     # rows that do not fit the staged columns under a norm (d 1152); the widest pass, four pairs per warp
+    (5, 336, 208, 5, "fma"),     # bf16 weights on the same kernel
+])
+def test_fma_linear_at_the_edges(d_heads, ffn, vocab, rows, flags):
+    """Logits of the fp32 linear kernel at its column, pair and row remainders against the oracle (fp32 sums: 1e-4, bf16
+    cache: 1e-2), and every row alone gives the bits it has in the full pass."""
+    bf16 = flags == "fma"
+    shape = si.ModelShape("edge", 2, 64 * d_heads, d_heads, 64, ffn, vocab, dtype="bf16" if bf16 else "f32")
+    eng, m, _ = make_pair(shape, (), max_seq=96, max_batch=max(1, rows // 5), k_max=4, flags=pkg.FLAG_FMA_GEMM if bf16 else 0)
+    try:
+        toks = si.make_prompts(shape.vocab, 1, rows, seed=3)[0].tolist()
+        got = eng.sdfp_forward_logits(toks, 0).astype(np.float64)
+        want = orc.forward_nocache(m, toks).detach().numpy().astype(np.float64)
+        assert np.linalg.norm(got - want) <= (1e-2 if bf16 else 1e-4) * np.linalg.norm(want)
+        for i in (0, rows // 2, rows - 1):
+            assert np.array_equal(eng.sdfp_forward_logits(toks[i:i + 1], i)[0], got[i].astype(np.float32))
+    finally:
+        eng.close()
+
+
 def test_largest_batch_and_row_count():
     """The library's limits in one context: 16 sequences, k = 4, 80 rows in a verify pass (row block of
     80 rows = MMA width 160), 32 rows in the first draft pass; prompts of one token (nothing to cache
