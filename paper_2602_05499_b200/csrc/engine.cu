@@ -103,6 +103,7 @@ struct sdfp_ctx {
   // persistent pass kernel (bf16 tensor path, passes of up to kPassMaxRows rows)
   bool use_pass = false;
   StageDesc *prog_t = nullptr, *prog_d = nullptr;  // device: stage lists of the target and of the draft
+  StageShare *shares_t = nullptr, *shares_d = nullptr;   // ... and every CTA's share of their stages
   int n_prog_t = 0, n_prog_d = 0;
   PassSync* psync = nullptr;
   ulonglong2* split_partials = nullptr;
@@ -371,7 +372,7 @@ StageDesc linear_desc(const void* w, const float* x, int K, int n_pairs, const f
 // The stage list of one forward pass: the target runs every layer, the draft the kept ones
 // (Algorithm 1: the draft is the model with the pruned layers removed).  The lm-head is the
 // last stage, so a pass that needs no logits runs the list without its last entry.
-int build_program(sdfp_ctx* c, bool draft, StageDesc** dev, int* n_out) {
+int build_program(sdfp_ctx* c, bool draft, StageDesc** dev, StageShare** dev_shares, int* n_out) {
   const sdfp_config& g = c->cfg;
   const int d = g.d_model, f = g.d_ffn;
   const int resid_groups = (d / 16 + kUnitTiles - 1) / kUnitTiles;  // groups of the stages that write the residual stream
@@ -406,16 +407,23 @@ int build_program(sdfp_ctx* c, bool draft, StageDesc** dev, int* n_out) {
   for (StageDesc& sd : prog) sd.ssq_groups = resid_groups;
   if (*dev == nullptr)
     if (int r = dev_alloc(c, dev, (size_t)5 * g.n_layers + 1)) return r;
+  const size_t grid = (size_t)c->pass_grid;
+  if (*dev_shares == nullptr)
+    if (int r = dev_alloc(c, dev_shares, ((size_t)5 * g.n_layers + 1) * grid)) return r;
+  std::vector<StageShare> shares(prog.size() * grid);
+  for (size_t i = 0; i < prog.size(); ++i)
+    if (prog[i].kind == ST_LINEAR) stage_shares(shares.data() + i * grid, prog[i].n_groups, prog[i].KT, (int)grid);
   CU_OK(c, cudaMemcpyAsync(*dev, prog.data(), prog.size() * sizeof(StageDesc), cudaMemcpyHostToDevice, c->stream));
-  CU_OK(c, cudaStreamSynchronize(c->stream));  // prog is a local
+  CU_OK(c, cudaMemcpyAsync(*dev_shares, shares.data(), shares.size() * sizeof(StageShare), cudaMemcpyHostToDevice, c->stream));
+  CU_OK(c, cudaStreamSynchronize(c->stream));  // both are locals
   *n_out = (int)prog.size();
   return 0;
 }
 
 int build_programs(sdfp_ctx* c) {
   if (!c->use_pass) return 0;
-  if (int r = build_program(c, false, &c->prog_t, &c->n_prog_t)) return r;
-  return build_program(c, true, &c->prog_d, &c->n_prog_d);
+  if (int r = build_program(c, false, &c->prog_t, &c->shares_t, &c->n_prog_t)) return r;
+  return build_program(c, true, &c->prog_d, &c->shares_d, &c->n_prog_d);
 }
 
 template <int CG, int HD>
@@ -494,6 +502,7 @@ cudaError_t launch_pass_t(sdfp_ctx* c, const PassParams& pp) {
 cudaError_t run_pass(sdfp_ctx* c, bool draft, int rows, int rows_per_seq, bool with_lm_head, bool fused_argmax = false) {
   PassParams pp{};
   pp.prog = draft ? c->prog_d : c->prog_t;
+  pp.shares = draft ? c->shares_d : c->shares_t;
   pp.n_stages = (draft ? c->n_prog_d : c->n_prog_t) - (with_lm_head ? 0 : 1);
   pp.M = rows;
   pp.rows_per_seq = rows_per_seq;

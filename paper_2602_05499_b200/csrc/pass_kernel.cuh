@@ -36,6 +36,8 @@
 // bit-identical whether it is computed alone (autoregressive step) or among k+1 rows (verify).
 #pragma once
 
+#include <algorithm>
+
 #include "attention.cuh"
 #include "common.cuh"
 #include "linear_mma.cuh"
@@ -102,8 +104,17 @@ struct PassSync {                // one per context, in global memory, zero-init
   unsigned pad2[28];
 };
 
+// A CTA's share of a linear stage: units ub .. ub + n - 1, and into how many further pieces the group is cut that
+// its last unit belongs to, if it holds that group's beginning (the next CTAs hold them).  Worked out on the
+// host once: two 64-bit divisions per look would sit on the stage boundary's critical path, here and for
+// every CTA an owner looks for.
+struct StageShare {
+  int ub, n, posters, pad;
+};
+
 struct PassParams {
   const StageDesc* prog;
+  const StageShare* shares;  // [stage][grid]
   int n_stages;
   int M;             // rows in this pass (<= kPassMaxRows); rows beyond carry nothing
   int rows_per_seq;  // attention: rows m0..m0+R-1 of a group belong to one sequence
@@ -217,6 +228,7 @@ struct PassShared {
   uint64_t empty[8];
   StageDesc st;       // the running stage
   StageDesc st_next;  // the next one, fetched while the running stage works
+  StageShare share, share_next;  // this CTA's share of them
   float inv_rms[kPassMaxRows];
   int row_pos[kPassMaxRows], row_seq[kPassMaxRows];  // fixed for the whole pass
   unsigned long long bar_base;
@@ -224,8 +236,6 @@ struct PassShared {
   int abort;     // set by whichever thread gives up a wait
   int decision;  // abort as sampled by thread 0 between two consumer barriers: uniform for all
   float attn_m[2][kPassAttnR], attn_l[2][kPassAttnR], attn_a[2][kPassAttnR];
-  int n_parts;
-  int parts[160];  // CTAs that post a partial for the group this CTA finishes
 };
 
 // All consumer threads learn the same answer to "has anything failed": thread 0 samples the
@@ -302,6 +312,49 @@ __device__ __forceinline__ bool grid_barrier(PassSync* sync, unsigned long long 
 __device__ __forceinline__ void unit_range(long long n_units, int cta, int n_cta, long long& ub, long long& ue) {
   ub = n_units * cta / n_cta;
   ue = n_units * (cta + 1) / n_cta;
+}
+
+// How the units of a linear stage are dealt to the CTAs, fixed by the matrix and the grid.  0: the whole list cut
+// evenly.  s > 0: every group of 128 features cut into s pieces, a CTA each, the CTAs beyond them idle.
+//
+// The rule: time of a stage in us, fitted to measurements.  A unit costs what streaming it costs; a group in
+// pieces costs its owner a wait and one L2 round trip per further piece, which it collects one after the
+// other.  With two units and more per class of every CTA the even cut wins: the pieces are few and all CTAs
+// stream (O-projection at d 3328, 36 units per CTA, as 5 pieces per group: 3 us longer at five rows).  A small
+// matrix cut evenly leaves a unit or a few per CTA and up to sixteen pieces per group, most of the
+// stage's time: pass of one row, 4 layers, d 256, FFN 688, vocabulary 2048: 246 -> 127 us; d 1024, FFN 2816: 196 -> 160.
+inline int stage_split(int n_groups, int KT, int grid) {
+  constexpr float kUnit = 0.14f, kPost = 2.0f, kPiece = 0.7f;
+  const float even = (float)n_groups * KT / grid;
+  if (even >= 2.0f * kClasses) return 0;
+  float best = even * kUnit + kPost + kPiece * std::max(1.0f, (float)KT / std::max(1.0f, even));
+  int split = 0;
+  for (int s = 1; s * n_groups <= grid && s <= KT; ++s) {
+    const float cost = (float)((KT + s - 1) / s) * kUnit + (s > 1 ? kPost + kPiece * (float)(s - 1) : 0.f);
+    if (cost < best) {
+      best = cost;
+      split = s;
+    }
+  }
+  return split;
+}
+inline void stage_shares(StageShare* out, int n_groups, int KT, int grid) {
+  const int split = stage_split(n_groups, KT, grid);
+  const long long total = (long long)n_groups * KT;
+  auto begin = [&](int cta) -> long long {
+    if (cta >= grid) return total;
+    if (split == 0) return total * cta / grid;
+    const int grp = cta / split;
+    return grp >= n_groups ? total : (long long)grp * KT + (long long)KT * (cta - grp * split) / split;
+  };
+  for (int c = 0; c < grid; ++c) {
+    const long long ub = begin(c), ue = begin(c + 1);
+    out[c] = StageShare{(int)ub, (int)(ue - ub), 0, 0};
+    if (ue == ub || ue % KT == 0) continue;
+    const long long grp_begin = ue / KT * KT, grp_end = grp_begin + KT;
+    if (grp_begin < ub) continue;  // this CTA's own last piece is one to post
+    for (int c2 = c + 1; c2 < grid && begin(c2) < grp_end; ++c2) out[c].posters += 1;  // (an even cut of a list no shorter than the grid leaves no CTA empty)
+  }
 }
 
 // ---- one linear stage, consumer side -------------------------------------------------------------
@@ -394,15 +447,13 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
   const int cls = warp & (kClasses - 1), th = warp / kClasses;
   const int KT = st.KT, M = pp.M, NT = st.NT;
   const int epi_mode = st.ep.mode;
-  const int cta = blockIdx.x, n_cta = gridDim.x;
-  const long long n_units = (long long)st.n_groups * KT;
-  long long ub64, ue64;
-  unit_range(n_units, cta, n_cta, ub64, ue64);
-  const int nun = (int)(ue64 - ub64);  // units of this CTA; below, units are numbered from ub64
+  const int cta = blockIdx.x;
+  const StageShare share = sh->share;
+  const int nun = share.n;  // units of this CTA; below, units are numbered from share.ub
   const int n_chunks = (nun + kChunkUnits - 1) / kChunkUnits;
   const int my_n = nun > cls ? (nun - cls + kChunkUnits - 1) / kChunkUnits : 0;
-  const int grp0 = (int)(ub64 / KT);
-  const int kt_first = (int)(ub64 - (long long)grp0 * KT);  // k-tile of unit 0
+  const int grp0 = share.ub / KT;
+  const int kt_first = share.ub - grp0 * KT;  // k-tile of unit 0
   // ring position of this stage's first chunk; advanced by one slot per unit of this warp
   unsigned slot = chunk_base % (unsigned)n_slots, parity = (chunk_base / (unsigned)n_slots) & 1u;
 
@@ -548,7 +599,7 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
   }
 
   int i = 0;          // my next unit is number cls + kChunkUnits * i
-  int seg_begin = 0;  // in units from ub64
+  int seg_begin = 0;  // in units from share.ub
   int grp = grp0;
   int seg_kt0 = kt_first;  // k-tile at seg_begin
   while (seg_begin < nun) {
@@ -638,32 +689,17 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
         red[((cls * kUnitTiles + th * 4 + r) * CG + cg) * 32 + lane] =
             make_float4(acc[r][cg][0], acc[r][cg][1], acc[r][cg][2], acc[r][cg][3]);
     if (owner && warp == 0) {
-      // The rest of the group sits at the beginning of the ranges of the CTAs that follow; every
-      // lane looks at one candidate and waits for that CTA's flag, so the waits overlap.
-      const long long grp_end = (long long)(grp + 1) * KT;
-      int n = 0;
-      bool more = true;
-      for (int base = cta + 1; more; base += 32) {
-        const int c2 = base + lane;
-        long long b2 = grp_end, e2 = grp_end;
-        if (c2 < n_cta) unit_range(n_units, c2, n_cta, b2, e2);
-        const bool beyond = (c2 >= n_cta) || (b2 >= grp_end);
-        const bool part = !beyond && e2 > b2;  // an empty range posts nothing
-        // one lane per posting CTA waits for the packet that CTA's last thread writes; the others
-        // are then there too or about to be, and every reader checks its own packets anyway
-        if (part) wait_packet(pp.split_partials + (size_t)c2 * (kUnitTiles * CG * 64) + (kPassConsumerThreads * CG - 1), epoch, pp.sync, &sh->abort);
-        const unsigned mask = __ballot_sync(0xffffffffu, part);
-        if (part) sh->parts[n + __popc(mask & ((1u << lane) - 1u))] = c2;
-        n += __popc(mask);
-        more = !__any_sync(0xffffffffu, beyond);
-      }
-      if (lane == 0) sh->n_parts = n;
+      // The rest of the group sits at the beginning of the ranges of the CTAs that follow: a lane waits
+      // for each, for the packet that CTA's last thread writes; the others are then there too or about to be,
+      // and every reader checks its own packets anyway.
+      for (int k2 = lane; k2 < share.posters; k2 += 32)
+        wait_packet(pp.split_partials + (size_t)(cta + 1 + k2) * (kUnitTiles * CG * 64) + (kPassConsumerThreads * CG - 1), epoch, pp.sync, &sh->abort);
     }
     if (!consumers_agree_ok(sh)) return;
 
     {
       ulonglong2* my_post = pp.split_partials + (size_t)cta * (kUnitTiles * CG * 64);
-      const int n_parts = owner ? sh->n_parts : 0;
+      const int n_parts = owner ? share.posters : 0;
 #pragma unroll
       for (int j = 0; j < CG; ++j) {
         const int it = tid + j * kPassConsumerThreads;
@@ -683,7 +719,7 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
           continue;
         }
         for (int k2 = 0; k2 < n_parts; ++k2) {
-          const ulonglong2* src = pp.split_partials + (size_t)sh->parts[k2] * (kUnitTiles * CG * 64) + it;
+          const ulonglong2* src = pp.split_partials + (size_t)(cta + 1 + k2) * (kUnitTiles * CG * 64) + it;
           ulonglong2 pk = ld_packet(src);
           if (!packet_is(pk, epoch)) pk = wait_packet(src, epoch, pp.sync, &sh->abort);
           v0 += __uint_as_float((unsigned)pk.x);
@@ -746,7 +782,7 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
         pp.amax_part[grp * kPassMaxRows + tid] = make_int2(__float_as_int(best), bi);
       }
     }
-    consumer_sync();  // red and parts may be rewritten
+    consumer_sync();  // red may be rewritten
     seg_begin = seg_end;
     seg_kt0 = 0;
     ++grp;
@@ -1020,17 +1056,16 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, in
       struct Cursor {
         int s;
         const unsigned char* src;
-        long long left;
+        int left;
       };
       auto advance = [&](Cursor& c) {  // to the next linear stage that has units for this CTA
         while (c.left == 0 && c.s < pp.n_stages) {
           if (++c.s == pp.n_stages) break;
           const StageDesc& st = pp.prog[c.s];
           if (st.kind != ST_LINEAR) continue;
-          long long ub, ue;
-          unit_range((long long)st.n_groups * st.KT, blockIdx.x, gridDim.x, ub, ue);
-          c.src = reinterpret_cast<const unsigned char*>(st.W) + (size_t)ub * kUnitBytes;
-          c.left = ue - ub;
+          const int2 own = __ldg(reinterpret_cast<const int2*>(pp.shares + (size_t)c.s * gridDim.x + blockIdx.x));  // ub, n
+          c.src = reinterpret_cast<const unsigned char*>(st.W) + (size_t)own.x * kUnitBytes;
+          c.left = own.y;
         }
       };
       const uint64_t pol_first = l2_policy_evict_first();  // a weight is read once per pass
@@ -1082,14 +1117,17 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, in
   unsigned chunk_base = 0;
   bool ok = true;
   constexpr int kDescWords = (int)(sizeof(StageDesc) / sizeof(int));
-  static_assert(kDescWords <= 64, "two warps fetch a stage descriptor");
+  static_assert(kDescWords < 64, "two warps fetch a stage descriptor and the CTA's share");
   const int desc_w = tid - (kPassConsumerThreads - 64);  // the last two warps fetch descriptors, one word per thread
+  const bool share_thread = desc_w == kDescWords;
   for (int s = 0; s < pp.n_stages && ok; ++s) {
     if (s == 0) {
       if (desc_w >= 0 && desc_w < kDescWords)
         reinterpret_cast<int*>(&sh->st)[desc_w] = reinterpret_cast<const int*>(pp.prog)[desc_w];
+      if (share_thread) sh->share = pp.shares[blockIdx.x];
     } else {
       if (desc_w >= 0 && desc_w < kDescWords) reinterpret_cast<int*>(&sh->st)[desc_w] = reinterpret_cast<const int*>(&sh->st_next)[desc_w];
+      if (share_thread) sh->share = sh->share_next;
     }
     consumer_sync();
     // the next stage's descriptor: asked for now, stored at the end of this stage, so that the
@@ -1097,6 +1135,8 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, in
     int next_word = 0;
     if (s + 1 < pp.n_stages && desc_w >= 0 && desc_w < kDescWords)
       next_word = reinterpret_cast<const int*>(pp.prog + s + 1)[desc_w];
+    StageShare next_share{};
+    if (s + 1 < pp.n_stages && share_thread) next_share = pp.shares[(size_t)(s + 1) * gridDim.x + blockIdx.x];
     if (sh->st.kind == ST_LINEAR) {
       // The posts of split groups carry a number no stage of any launch shares.  Barrier serials
       // advance by n_stages - 1 per launch, so stage s gets (bar_base + s) * 2 + (1 if it is the
@@ -1108,9 +1148,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, in
       } else {
         // fold the attention partials into shared memory first if the columns this CTA's units
         // use fit beside the other work buffers (they do for passes of a few rows)
-        long long ub, ue;
-        unit_range((long long)sh->st.n_groups * sh->st.KT, blockIdx.x, gridDim.x, ub, ue);
-        const long long kts = ue - ub < sh->st.KT ? ue - ub : sh->st.KT;
+        const int kts = min(sh->share.n, sh->st.KT);
         const size_t need = (size_t)pp.M * (size_t)(kts * 16 + 8) * sizeof(float);
         if (need <= pass_work_bytes<CG, HD>() - (size_t)work_sc_off<CG>())
           linear_stage<CG, HD, X_STAGED>(pp, sh, ring, n_slots, work, chunk_base, serial);
@@ -1136,6 +1174,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, in
       }
     }
     if (desc_w >= 0 && desc_w < kDescWords) reinterpret_cast<int*>(&sh->st_next)[desc_w] = next_word;
+    if (share_thread) sh->share_next = next_share;
     // the barrier also tells every thread whether a wait of this CTA gave up (the CTA still arrives)
     ok = (s + 1 < pp.n_stages) ? grid_barrier(pp.sync, bar_base + (unsigned long long)(s + 1), sh) : consumers_agree_ok(sh);
   }

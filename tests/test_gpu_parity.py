@@ -923,6 +923,28 @@ def test_fma_linear_at_the_edges(d_heads, ffn, vocab, rows, flags):
         eng.close()
 
 
+@pytest.mark.parametrize("heads,head_dim,ffn,vocab", [
+    (1, 64, 16, 16),        # one group of features, fewer k-tiles than classes: a CTA per group, most CTAs idle
+    (9, 64, 1552, 400),     # matrices cut into pieces per group next to evenly cut ones, a ragged last group
+    (25, 128, 272, 144),    # d 3200: the fp32 hand-over up to eight rows, fragment images above
+    (40, 64, 336, 2064),    # d 2560: fragment images at every row count
+])
+def test_pass_kernel_work_split_and_images(heads, head_dim, ffn, vocab):
+    """The whole-pass kernel over the ways its stages are cut and its activations handed on: 16, 9, 8 and 1 rows give
+    the same bits row by row, and the logits are the oracle's."""
+    shape = si.ModelShape("edge", 2, heads * head_dim, heads, head_dim, ffn, vocab, dtype="bf16")
+    eng, m, _ = make_pair(shape, (), max_seq=48, random_gains=True)
+    try:
+        toks = si.make_prompts(shape.vocab, 1, 32, seed=11)[0].tolist()
+        got = eng.sdfp_forward_logits(toks, 0)             # two passes of 16 rows
+        want = orc.forward_nocache(m, toks).detach().numpy()
+        assert rel_l2(got, want) <= 1e-2
+        for lo, hi in ((16, 25), (16, 24), (20, 25), (16, 17), (31, 32)):
+            assert np.array_equal(eng.sdfp_forward_logits(toks[lo:hi], lo), got[lo:hi])
+    finally:
+        eng.close()
+
+
 def test_largest_batch_and_row_count():
     """The library's limits in one context: 16 sequences, k = 4, 80 rows in a verify pass (row block of
     80 rows = MMA width 160), 32 rows in the first draft pass; prompts of one token (nothing to cache
