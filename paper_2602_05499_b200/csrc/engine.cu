@@ -108,10 +108,12 @@ struct sdfp_ctx {
   PassSync* psync = nullptr;
   ulonglong2* split_partials = nullptr;
   float* ssq_part = nullptr;
+  uint4 *x_h = nullptr, *x_u = nullptr;  // activations between its stages: fragment images of gain * h and of u
+  const float *first_gain_t = nullptr, *first_gain_d = nullptr;  // the gain of a pass's first norm, target and draft
   int2* amax_part = nullptr;  // greedy decision fused into the lm-head: (largest logit, index) per (group of the vocabulary, row)
   int amax_groups = 0;
   int pass_slots[3] = {0, 0, 0};  // ring slots of the instantiation with 1 and with 2 column groups
-  size_t pass_smem = 0;
+  size_t pass_smem[3] = {0, 0, 0};  // dynamic shared memory of the instantiations with 1 and with 2 column groups
   int pass_grid = 0;
   // dense path on tcgen05 (bf16 tensor path): the prompt pass of every context, and every pass of
   // a context whose widest pass does not fit the whole-pass kernel
@@ -351,7 +353,8 @@ cudaError_t configure_kernels(const sdfp_ctx* c) {
 
 // ---- persistent pass kernel: stage lists and launch ---------------------------------------------
 
-StageDesc linear_desc(const void* w, const float* x, int K, int n_pairs, const float* gain, const EpiParams& ep) {
+StageDesc linear_desc(const sdfp_ctx* c, const void* w, const float* rows, const uint4* x, int K, int n_pairs, const float* gain,
+                      const EpiParams& ep) {
   StageDesc s{};
   s.kind = ST_LINEAR;
   s.K = K;
@@ -363,8 +366,10 @@ StageDesc linear_desc(const void* w, const float* x, int K, int n_pairs, const f
   s.rms_mode = gain ? RMS_FROM_PARTS : RMS_NONE;
   s.write_ssq = ep.mode == EPI_RESID ? 1 : 0;
   s.W = reinterpret_cast<const uint4*>(w);
-  s.X = x;
+  s.X = rows;
   s.gain = gain;
+  s.x_in = x;
+  s.x_out = ep.mode == EPI_SWIGLU ? c->x_u : c->x_h;
   s.ep = ep;
   return s;
 }
@@ -378,13 +383,22 @@ int build_program(sdfp_ctx* c, bool draft, StageDesc** dev, StageShare** dev_sha
   const int resid_groups = (d / 16 + kUnitTiles - 1) / kUnitTiles;  // groups of the stages that write the residual stream
   const KvCache& kv = (draft && !c->share_kv) ? c->cache_d : c->cache_t;
   std::vector<StageDesc> prog;
+  const float** wants_gain = &(draft ? c->first_gain_d : c->first_gain_t);  // who leaves gain * h for the next norm: the embedding, then ...
+  int resid = -1;                                                          // ... the last stage that wrote the residual stream
+  auto norm_gain = [&](const float* gain) {
+    if (resid >= 0)
+      prog[resid].gain_out = gain;
+    else
+      *wants_gain = gain;
+  };
   for (int l = 0; l < g.n_layers; ++l) {
     const LayerWeights& lw = c->layers[l];
     if (!draft || c->keep_attn[l]) {  // the attention block: h += Wo * Attn(norm(h))
+      norm_gain(lw.attn_gain);
       EpiParams qkv = base_epi(c, EPI_QKV, c->q, d);
       qkv.kcache = kv.k[l];
       qkv.vcache = kv.v[l];
-      prog.push_back(linear_desc(lw.qkv, c->h, d, 3 * d / 2, lw.attn_gain, qkv));
+      prog.push_back(linear_desc(c, lw.qkv, c->h, c->x_h, d, 3 * d / 2, lw.attn_gain, qkv));
       StageDesc at{};
       at.kind = ST_ATTN;
       at.X = c->q;
@@ -393,15 +407,19 @@ int build_program(sdfp_ctx* c, bool draft, StageDesc** dev, StageShare** dev_sha
       at.ep.vcache = kv.v[l];
       prog.push_back(at);
       // the O-projection reads the attention output as kAttnSplits partials per (row, head)
-      prog.push_back(linear_desc(lw.wo, nullptr, d, d / 2, nullptr, base_epi(c, EPI_RESID, c->h, d)));
+      prog.push_back(linear_desc(c, lw.wo, nullptr, nullptr, d, d / 2, nullptr, base_epi(c, EPI_RESID, c->h, d)));
       prog.back().x_mode = X_ATTN_FOLD;
+      resid = (int)prog.size() - 1;
     }
     if (!draft || c->keep_ffn[l]) {   // the FFN block: h += Wdown * SwiGLU(norm(h))
-      prog.push_back(linear_desc(lw.gu, c->h, d, f, lw.ffn_gain, base_epi(c, EPI_SWIGLU, c->u, f)));
-      prog.push_back(linear_desc(lw.down, c->u, f, d / 2, nullptr, base_epi(c, EPI_RESID, c->h, d)));
+      norm_gain(lw.ffn_gain);
+      prog.push_back(linear_desc(c, lw.gu, c->h, c->x_h, d, f, lw.ffn_gain, base_epi(c, EPI_SWIGLU, c->u, f)));
+      prog.push_back(linear_desc(c, lw.down, c->u, c->x_u, f, d / 2, nullptr, base_epi(c, EPI_RESID, c->h, d)));
+      resid = (int)prog.size() - 1;
     }
   }
-  prog.push_back(linear_desc(c->lm_head, c->h, d, g.vocab / 2, c->final_gain, base_epi(c, EPI_LOGITS, c->logits, g.vocab)));
+  norm_gain(c->final_gain);
+  prog.push_back(linear_desc(c, c->lm_head, c->h, c->x_h, d, g.vocab / 2, c->final_gain, base_epi(c, EPI_LOGITS, c->logits, g.vocab)));
   // the embedding rows come from another kernel: the first norm of a pass sums its rows itself
   prog.front().rms_mode = RMS_DIRECT;
   for (StageDesc& sd : prog) sd.ssq_groups = resid_groups;
@@ -451,16 +469,16 @@ template <int HD>
 cudaError_t configure_pass_t(sdfp_ctx* c, int max_smem_optin) {
   c->pass_slots[1] = pass_slots_that_fit<1, HD>(max_smem_optin);
   c->pass_slots[2] = pass_slots_that_fit<2, HD>(max_smem_optin);
-  c->pass_smem = std::max(pass_smem_bytes<1, HD>(c->pass_slots[1]), pass_smem_bytes<2, HD>(c->pass_slots[2]));
-  if (c->pass_smem > (size_t)max_smem_optin) return cudaErrorLaunchOutOfResources;
-  cudaError_t e = cudaFuncSetAttribute(pass_kernel<1, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->pass_smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(pass_kernel<2, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->pass_smem);
-  if (e != cudaSuccess) return e;
+  c->pass_smem[1] = pass_smem_bytes<1, HD>(c->pass_slots[1]);
+  c->pass_smem[2] = pass_smem_bytes<2, HD>(c->pass_slots[2]);
+  if (std::max(c->pass_smem[1], c->pass_smem[2]) > (size_t)max_smem_optin) return cudaErrorLaunchOutOfResources;
+  cudaError_t e = cudaSuccess;
   // The kernel moves registers from its producer group to its consumers; the amounts are fixed
   // numbers that only add up if it was compiled to the launch size they assume.  Otherwise the
   // consumers would wait for registers that never come: refuse rather than launch.
-  for (const void* fn : {(const void*)pass_kernel<1, HD>, (const void*)pass_kernel<2, HD>}) {
+  for (const void* fn : {(const void*)pass_kernel<1, HD, false>, (const void*)pass_kernel<1, HD, true>, (const void*)pass_kernel<2, HD, true>}) {
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(c->pass_smem[1], c->pass_smem[2]));
+    if (e != cudaSuccess) return e;
     cudaFuncAttributes fa{};
     e = cudaFuncGetAttributes(&fa, fn);
     if (e != cudaSuccess) return e;
@@ -468,19 +486,35 @@ cudaError_t configure_pass_t(sdfp_ctx* c, int max_smem_optin) {
   }
   // a cooperative launch needs every CTA resident at once: one per SM
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pass_kernel<2, HD>, kPassThreads, c->pass_smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pass_kernel<2, HD, true>, kPassThreads, c->pass_smem[2]);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorLaunchOutOfResources;
   c->pass_grid = c->num_sms;
   return cudaSuccess;
 }
 
-template <int CG, int HD>
+// Whether a pass hands its activations on as fragment images.  More than eight rows: always, the loads and
+// splits of two column groups are what bounds the loop otherwise (d 4096, 12 layers, 16 rows: 2170 -> 1746 us, with the larger staging area).
+// Up to eight rows the loop of a large matrix waits for its weights either way and the images only
+// lengthen the epilogue (d 4096, one row: 1192 -> 1206 us); a small one is bound by latency and gains (d 2048, 6
+// layers, one row: 343 -> 326 us).  The results have the same bits.
+bool pass_images(const sdfp_ctx* c, int rows) { return rows > 8 || c->cfg.d_model <= 3072; }
+
+// what the embedding kernel leaves for the whole-pass kernel's first stage
+EmbedImage pass_embed_image(const sdfp_ctx* c, bool draft, int rows) {
+  EmbedImage im{};
+  if (!c->use_pass || !pass_images(c, rows)) return im;
+  im.gain = draft ? c->first_gain_d : c->first_gain_t;
+  im.frag = c->x_h;
+  return im;
+}
+
+template <int CG, int HD, bool IMG>
 cudaError_t launch_pass_t(sdfp_ctx* c, const PassParams& pp) {
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(c->pass_grid);
   lc.blockDim = dim3(kPassThreads);
-  lc.dynamicSmemBytes = c->pass_smem;
+  lc.dynamicSmemBytes = c->pass_smem[CG];
   lc.stream = c->stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -488,7 +522,7 @@ cudaError_t launch_pass_t(sdfp_ctx* c, const PassParams& pp) {
   lc.attrs = attr;
   lc.numAttrs = 1;
   c->launches += 1;
-  return cudaLaunchKernelEx(&lc, pass_kernel<CG, HD>, pp, c->pass_slots[CG]);
+  return cudaLaunchKernelEx(&lc, pass_kernel<CG, HD, IMG>, pp, c->pass_slots[CG]);
 }
 
 // Chunks (32 KB per CTA) of weights the producer asks into L2 ahead of the ring.  Measured on the
@@ -519,8 +553,9 @@ cudaError_t run_pass(sdfp_ctx* c, bool draft, int rows, int rows_per_seq, bool w
   pp.amax_part = fused_argmax ? c->amax_part : nullptr;
   pp.sync = c->psync;
   const bool hd128 = c->cfg.head_dim == 128;
-  if (rows <= 8) return hd128 ? launch_pass_t<1, 128>(c, pp) : launch_pass_t<1, 64>(c, pp);
-  return hd128 ? launch_pass_t<2, 128>(c, pp) : launch_pass_t<2, 64>(c, pp);
+  if (!pass_images(c, rows)) return hd128 ? launch_pass_t<1, 128, false>(c, pp) : launch_pass_t<1, 64, false>(c, pp);
+  if (rows <= 8) return hd128 ? launch_pass_t<1, 128, true>(c, pp) : launch_pass_t<1, 64, true>(c, pp);
+  return hd128 ? launch_pass_t<2, 128, true>(c, pp) : launch_pass_t<2, 64, true>(c, pp);
 }
 
 // ---- one forward pass ------------------------------------------------------------------
@@ -549,7 +584,7 @@ int enqueue_pass(sdfp_ctx* c, const PassDesc& pd, bool draft, int rows, int attn
   if (c->bf16)
     CU_OK(c, launch(c, plan_embed_kernel<__nv_bfloat16>, dim3(rows), dim3(128), 0, pd, (const GenState*)c->gs,
                     (const int*)c->seq_tok, g.max_seq, (const int*)c->draft_tok, c->plan,
-                    reinterpret_cast<const __nv_bfloat16*>(c->embed), c->h, d, EmbedImage{}));
+                    reinterpret_cast<const __nv_bfloat16*>(c->embed), c->h, d, pass_embed_image(c, draft, rows)));
   else
     CU_OK(c, launch(c, plan_embed_kernel<float>, dim3(rows), dim3(128), 0, pd, (const GenState*)c->gs,
                     (const int*)c->seq_tok, g.max_seq, (const int*)c->draft_tok, c->plan,
@@ -1033,6 +1068,7 @@ extern "C" int sdfp_create(const sdfp_config* cfg, const sdfp_weights* w, void* 
   if (c->use_pass) {
     if ((r = dev_alloc(c, &c->psync, 1, true)) ||
         (r = dev_alloc(c, &c->split_partials, (size_t)c->pass_grid * kUnitTiles * 2 * 64, true)) ||
+        (r = dev_alloc(c, &c->x_h, frag_image_len(g.d_model), true)) || (r = dev_alloc(c, &c->x_u, frag_image_len(g.d_ffn), true)) ||
         (r = dev_alloc(c, &c->ssq_part, (size_t)kSsqMaxGroups * kPassMaxRows, true)) ||
         (r = dev_alloc(c, &c->amax_part, (size_t)((g.vocab / 16 + kUnitTiles - 1) / kUnitTiles) * kPassMaxRows, true)) ||
         (r = build_programs(c)))
@@ -1629,7 +1665,7 @@ extern "C" int sdfp_time_pass(sdfp_ctx* c, int32_t draft, int32_t rows, int32_t 
   auto plan = [&]() -> cudaError_t {
     return launch(c, plan_embed_kernel<__nv_bfloat16>, dim3(rows), dim3(128), 0, pd, (const GenState*)c->gs,
                   (const int*)c->seq_tok, g.max_seq, (const int*)c->draft_tok, c->plan,
-                  reinterpret_cast<const __nv_bfloat16*>(c->embed), c->h, g.d_model, EmbedImage{});
+                  reinterpret_cast<const __nv_bfloat16*>(c->embed), c->h, g.d_model, pass_embed_image(c, draft != 0, rows));
   };
   for (int i = 0; i < 3 && err == cudaSuccess; ++i) {  // warm-up
     err = plan();

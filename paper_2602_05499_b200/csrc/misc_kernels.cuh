@@ -3,6 +3,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "linear_mma.cuh"
 
 namespace sdfp {
 
@@ -84,6 +85,7 @@ struct EmbedImage {
   const float* gain;
   float* ssq;          // [rows]
   int rb, kb;
+  uint4* frag;         // whole-pass kernel: its fragment image of gain * h instead (frag_index of pass_kernel.cuh); null: none
 };
 
 // One CTA per row: decide which token sits in the row and where, then gather its
@@ -156,6 +158,17 @@ plan_embed_kernel(PassDesc pd, const GenState* gs, const int* seq_tok, int max_s
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (s_pos >= 0) v = load4(e + k);
     *reinterpret_cast<float4*>(dst + k) = v;
+    if (im.frag != nullptr) {
+      const float4 g = *reinterpret_cast<const float4*>(im.gain + k);
+      uint32_t h0, h1, l0, l1;
+      split_pack(v.x * g.x, v.y * g.y, h0, l0);
+      split_pack(v.z * g.z, v.w * g.w, h1, l1);
+      uint32_t* f = reinterpret_cast<uint32_t*>(im.frag) + (((size_t)(k >> 4) * 16 + m) * 4 + ((k & 7) >> 1)) * 4 + ((k >> 3) & 1);
+      f[0] = h0;
+      f[2] = l0;
+      f[4] = h1;
+      f[6] = l1;
+    }
     if (im.img != nullptr) {
       sq = fmaf(v.x, v.x, sq);
       sq = fmaf(v.y, v.y, sq);

@@ -83,10 +83,23 @@ struct StageDesc {
   int write_ssq;      // EPI_RESID stages: leave per-group sums of squares of the new residual rows
   int ssq_groups;     // RMS_FROM_PARTS: how many group sums make a row's sum
   const uint4* W;     // unit layout
-  const float* X;     // linear: activations [rows, K]; attention: q [rows, d_model]
-  const float* gain;  // linear: RMSNorm gain or null
+  const float* X;     // fp32 activations [rows, K]; RMS_DIRECT: the rows the norm is of; attention: q [rows, d_model]
+  const float* gain;  // the norm's gain or null
+  // IMG: activations travel between the stages as the B fragments the MMA takes, split once by whoever
+  // makes them (fragment image, frag_index): x is (gain of the norm in between) * h, or u.
+  const uint4* x_in;       // X_PLAIN
+  uint4* x_out;            // EPI_RESID, EPI_SWIGLU: the next linear stage's x_in
+  const float* gain_out;   // EPI_RESID: the next norm's gain
   EpiParams ep;       // linear epilogue; attention: kcache, vcache, n_heads, max_seq
 };
+
+// Fragment image of up to kPassMaxRows activation rows: for every k-tile of 16 columns, row and quarter q
+// one uint4 = bf16 pairs {hi(2q, 2q+1), hi(2q+8, 2q+9), lo(2q, 2q+1), lo(2q+8, 2q+9)}, x = hi + lo: what lane
+// (row, q) of the MMA holds.  A fragment of eight rows is one 128-bit load per lane, 512 contiguous bytes;
+// with fp32 rows it was two 64-bit loads, two of the gain and the split, repeated by every warp of every
+// CTA that meets the columns.
+__host__ __device__ __forceinline__ size_t frag_index(int kt, int row, int q) { return ((size_t)kt * 16 + row) * 4 + q; }
+inline size_t frag_image_len(int K) { return (size_t)(K / 16) * 64; }  // in uint4
 
 // what a wait that gave up leaves in PassSync::error
 enum PassError { PASS_OK = 0, PASS_ERR_GRID_BARRIER = 1, PASS_ERR_SLOT_FULL = 2, PASS_ERR_SLOT_EMPTY = 3, PASS_ERR_SPLIT_FLAG = 4 };
@@ -358,26 +371,31 @@ inline void stage_shares(StageShare* out, int n_groups, int KT, int grid) {
 }
 
 // ---- one linear stage, consumer side -------------------------------------------------------------
-template <int CG>
+template <int CG, bool RAW>
 struct XRegs {
+  uint4 v[CG];  // fragment (frag_index) of row 8 cg + g
+};
+template <int CG>
+struct XRegs<CG, true> {    // still fp32: split when it is used
   float2 lo8[CG], hi8[CG];  // x[m][16kt + 2q .. +1] and x[m][16kt + 2q + 8 .. +9], m = 8 cg + g
   float2 g0, g1;            // the RMSNorm gain at the same columns (1 when the stage has no norm)
 };
 
 struct XSource {  // the fields of the stage an activation load needs, kept in registers
-  const float* X;  // X_STAGED: shared memory, column 0 = first column of k-tile kt0
+  const float* X;        // RAW: fp32 rows, ldx apart, and the norm's gain (or null)
   const float* gain;
+  int ldx;
+  const uint4* x;        // X_PLAIN: fragment image; X_STAGED: shared memory, first k-tile = kt0, rows ld words apart
   const float* part_o;
-  int ldx, n_heads;
+  int ld, n_heads;
   int kt0, KT;  // X_STAGED only
 };
 
 // Activation fragment of k-tile kt for every column group.  X_ATTN_FOLD: the activation is the
 // attention output, which exists only as kAttnSplits partial sums per (row, head); sc[m][head][j]
 // holds exp(m_j - max)/sum, and the fragment is the weighted sum of the partials in split order.
-template <int CG, int HD, int XM>
-__device__ __forceinline__ void load_xregs(XRegs<CG>& x, const XSource& xs, const float* sc, int M, int kt, int g, int q,
-                                           bool valid) {
+template <int CG>
+__device__ __forceinline__ void load_xraw(XRegs<CG, true>& x, const XSource& xs, int M, int kt, int g, int q, bool valid) {
   x.g0 = make_float2(1.f, 1.f);
   x.g1 = make_float2(1.f, 1.f);
   if (valid && xs.gain != nullptr) {  // asked for together with the activations: a first touch misses L1
@@ -391,16 +409,26 @@ __device__ __forceinline__ void load_xregs(XRegs<CG>& x, const XSource& xs, cons
     x.lo8[cg] = make_float2(0.f, 0.f);
     x.hi8[cg] = make_float2(0.f, 0.f);
     if (valid && m < M) {
+      const float* xp = xs.X + (size_t)m * xs.ldx + kt * 16 + 2 * q;
+      x.lo8[cg] = ld_act2(xp);
+      x.hi8[cg] = ld_act2(xp + 8);
+    }
+  }
+}
+template <int CG, int HD, int XM>
+__device__ __forceinline__ void load_xregs(XRegs<CG, false>& x, const XSource& xs, const float* sc, int M, int kt, int g, int q,
+                                           bool valid) {
+#pragma unroll
+  for (int cg = 0; cg < CG; ++cg) {
+    const int m = cg * 8 + g;
+    x.v[cg] = make_uint4(0u, 0u, 0u, 0u);
+    if (valid && m < M) {
       if (XM == X_PLAIN) {
-        const float* xp = xs.X + (size_t)m * xs.ldx + kt * 16 + 2 * q;
-        x.lo8[cg] = ld_act2(xp);
-        x.hi8[cg] = ld_act2(xp + 8);
+        x.v[cg] = __ldcg(xs.x + frag_index(kt, m, q));
       } else if (XM == X_STAGED) {
         int dk = kt - xs.kt0;
         if (dk < 0) dk += xs.KT;
-        const float* xp = xs.X + m * xs.ldx + dk * 16 + 2 * q;
-        x.lo8[cg] = *reinterpret_cast<const float2*>(xp);
-        x.hi8[cg] = *reinterpret_cast<const float2*>(xp + 8);
+        x.v[cg] = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint32_t*>(xs.x) + m * xs.ld + dk * 16 + q * 4);
       } else {
         const int k = kt * 16 + 2 * q;
         const int head = k / HD, d = k - head * HD;
@@ -417,8 +445,8 @@ __device__ __forceinline__ void load_xregs(XRegs<CG>& x, const XSource& xs, cons
           hi.x = fmaf(w, b.x, hi.x);
           hi.y = fmaf(w, b.y, hi.y);
         }
-        x.lo8[cg] = lo;
-        x.hi8[cg] = hi;
+        split_pack(lo.x, lo.y, x.v[cg].x, x.v[cg].z);
+        split_pack(hi.x, hi.y, x.v[cg].y, x.v[cg].w);
       }
     }
   }
@@ -431,11 +459,45 @@ template <int CG>
 __host__ __device__ constexpr int work_sq_off() { return work_red_bytes<CG>(); }  // squares of new residual values [it]
 template <int CG>
 __host__ __device__ constexpr int work_sc_off() { return work_sq_off<CG>() + kUnitTiles * CG * 64 * 4; }  // attention fold weights
-constexpr int kWorkScBytes = kPassMaxRows * kPassMaxHeads * kAttnSplits * 4;
+// words between the staged rows of a CTA that needs kts k-tiles: an odd number of half bank rows, so that the two rows
+// a quarter warp reads at a time lie in different halves
+__host__ __device__ constexpr int staged_row_words(int kts) { return (kts | 1) * 16; }
+// The area of the attention fold: the factors of every (row, head), or the folded columns a CTA's units use.  With two
+// column groups it is sized so that 16 rows are staged at d 5120 (87 k-tiles a CTA) beside a ring of two slots.
+template <int CG>
+__host__ __device__ constexpr int work_sc_bytes() { return CG == 1 ? kPassMaxRows * kPassMaxHeads * kAttnSplits * 4 : 92 * 1024; }
+static_assert(work_sc_bytes<2>() >= kPassMaxRows * kPassMaxHeads * kAttnSplits * 4,
+              "the fold weights of every row and head");
 
-template <int CG, int HD, int XM>
+// (max, sum) of each split's partial of one (row, head), and the factors the partials get: exp(m_j - max) / sum,
+// zero for a split that saw nothing
+struct FoldStats {
+  float2 v[kAttnSplits];
+  __device__ __forceinline__ void load(const float* ml) {
+#pragma unroll
+    for (int j = 0; j < kAttnSplits; ++j) v[j] = ld_act2(ml + 2 * j);
+  }
+  __device__ __forceinline__ void weights(float (&w)[kAttnSplits]) const {
+    float mx = -INFINITY;
+#pragma unroll
+    for (int j = 0; j < kAttnSplits; ++j)
+      if (v[j].y > 0.f) mx = fmaxf(mx, v[j].x);
+    float l = 0.f;
+#pragma unroll
+    for (int j = 0; j < kAttnSplits; ++j) {
+      w[j] = v[j].y > 0.f ? __expf(v[j].x - mx) : 0.f;
+      l = fmaf(v[j].y, w[j], l);
+    }
+    const float inv_l = l > 0.f ? 1.0f / l : 0.f;
+#pragma unroll
+    for (int j = 0; j < kAttnSplits; ++j) w[j] *= inv_l;
+  }
+};
+
+template <int CG, int HD, int XM, bool IMG>
 __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigned char* ring, int n_slots, unsigned char* work,
                              unsigned& chunk_base, unsigned epoch) {
+  constexpr bool RAW = XM == X_PLAIN && !IMG;
   const StageDesc& st = sh->st;
   float4* red = reinterpret_cast<float4*>(work);
   float* sq_buf = reinterpret_cast<float*>(work + work_sq_off<CG>());
@@ -489,37 +551,25 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
   if (XM == X_ATTN_FOLD) {
     const int n_heads = st.ep.n_heads;
     for (int e = tid; e < M * n_heads; e += kPassConsumerThreads) {
-      const float* ml = pp.part_ml + (size_t)e * kAttnSplits * 2;  // e = m * n_heads + head
-      float mj[kAttnSplits], lj[kAttnSplits];
-      float mx = -INFINITY;
+      FoldStats fs;
+      fs.load(pp.part_ml + (size_t)e * kAttnSplits * 2);  // e = m * n_heads + head
+      float w[kAttnSplits];
+      fs.weights(w);
 #pragma unroll
-      for (int j = 0; j < kAttnSplits; ++j) {
-        const float2 v = ld_act2(ml + 2 * j);
-        mj[j] = v.x;
-        lj[j] = v.y;
-        if (v.y > 0.f) mx = fmaxf(mx, v.x);
-      }
-      float l = 0.f, wj[kAttnSplits];
-#pragma unroll
-      for (int j = 0; j < kAttnSplits; ++j) {
-        wj[j] = lj[j] > 0.f ? __expf(mj[j] - mx) : 0.f;
-        l = fmaf(lj[j], wj[j], l);
-      }
-      const float inv_l = l > 0.f ? 1.0f / l : 0.f;
-#pragma unroll
-      for (int j = 0; j < kAttnSplits; ++j) sc[(size_t)e * kAttnSplits + j] = wj[j] * inv_l;
+      for (int j = 0; j < kAttnSplits; ++j) sc[(size_t)e * kAttnSplits + j] = w[j];
     }
     consumer_sync();
   }
 
   // ---- or the folded activations themselves, for the k-tiles this CTA's units use ----
-  // Every element asks for its 8 (max, sum) pairs and its 8 partial values at once, so the whole
-  // fold costs one round trip to L2, where folding inside the fragment loads costs one for the
-  // weights and one more for each of the first three fragments.  Same operations in the same
-  // order as above: the result is bit-identical whichever way a CTA takes.
-  float* const x_staged = sc;  // same place: a stage uses one or the other
-  const int staged_kts = min(nun, KT), staged_ld = staged_kts * 16 + 8;  // +8: rows start 8 banks apart
-  if (XM == X_STAGED) {
+  // Same operations in the same order as above: the result is bit-identical whichever way a CTA takes.
+  uint32_t* const x_staged = reinterpret_cast<uint32_t*>(sc);  // same place: a stage uses one or the other
+  const int staged_kts = min(nun, KT), staged_ld = staged_row_words(staged_kts);
+  auto staged_word = [&](int m, int c) { return x_staged + m * staged_ld + (c >> 4) * 16 + ((c & 7) >> 1) * 4 + ((c >> 3) & 1); };
+  if (XM == X_STAGED && CG == 1) {
+    // Few rows: every element asks for its 8 (max, sum) pairs and its 8 partial values at once, so the whole
+    // fold costs one round trip to L2, where folding inside the fragment loads costs one for the
+    // weights and one more for each of the first three fragments.
     const int n_heads = st.ep.n_heads;
     const int pairs_per_row = staged_kts * 8;
 #pragma unroll 2
@@ -530,46 +580,89 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
       const int k = kt * 16 + (c & 15);
       const int head = k / HD, d = k - head * HD;
       const size_t rh = (size_t)m * n_heads + head;
+      FoldStats fs;
+      float2 oj[kAttnSplits];
       const float* ml = pp.part_ml + rh * kAttnSplits * 2;
       const float* po = pp.part_o + rh * kAttnSplits * HD + d;
-      float mj[kAttnSplits], lj[kAttnSplits];
-      float2 oj[kAttnSplits];
 #pragma unroll
       for (int j = 0; j < kAttnSplits; ++j) {
-        const float2 v = ld_act2(ml + 2 * j);
-        mj[j] = v.x;
-        lj[j] = v.y;
+        fs.v[j] = ld_act2(ml + 2 * j);
         oj[j] = ld_act2(po + (size_t)j * HD);
       }
-      float mx = -INFINITY;
-#pragma unroll
-      for (int j = 0; j < kAttnSplits; ++j)
-        if (lj[j] > 0.f) mx = fmaxf(mx, mj[j]);
-      float l = 0.f, wj[kAttnSplits];
+      float w[kAttnSplits];
+      fs.weights(w);
+      float2 x = make_float2(0.f, 0.f);
 #pragma unroll
       for (int j = 0; j < kAttnSplits; ++j) {
-        wj[j] = lj[j] > 0.f ? __expf(mj[j] - mx) : 0.f;
-        l = fmaf(lj[j], wj[j], l);
+        x.x = fmaf(w[j], oj[j].x, x.x);
+        x.y = fmaf(w[j], oj[j].y, x.y);
       }
-      const float inv_l = l > 0.f ? 1.0f / l : 0.f;
-      float2 xv = make_float2(0.f, 0.f);
+      uint32_t* xw = staged_word(m, c);
+      split_pack(x.x, x.y, xw[0], xw[2]);
+    }
+    consumer_sync();
+  }
+  if (XM == X_STAGED && CG == 2) {
+    // Many rows: the columns lie in at most heads_here neighbouring heads (cyclically); their factors first, into
+    // the reduction area, which is idle until the first segment ends, then four columns per step.
+    const int n_heads = st.ep.n_heads;
+    float* const w8 = reinterpret_cast<float*>(red);  // [m][head - head0][kAttnSplits]
+    const int head0 = kt_first * 16 / HD;
+    const int heads_here = min(n_heads, (kt_first * 16 + staged_kts * 16 - 1) / HD - head0 + 1);
+    for (int e = tid; e < M * heads_here; e += kPassConsumerThreads) {
+      const int m = e / heads_here;
+      int head = head0 + e - m * heads_here;
+      if (head >= n_heads) head -= n_heads;
+      FoldStats fs;
+      fs.load(pp.part_ml + ((size_t)m * n_heads + head) * kAttnSplits * 2);
+      float w[kAttnSplits];
+      fs.weights(w);
+#pragma unroll
+      for (int j = 0; j < kAttnSplits; ++j) w8[(size_t)e * kAttnSplits + j] = w[j];
+    }
+    consumer_sync();
+    const int quads_per_row = staged_kts * 4;
+#pragma unroll 2
+    for (int e = tid; e < M * quads_per_row; e += kPassConsumerThreads) {
+      const int m = e / quads_per_row, c = (e - m * quads_per_row) * 4;
+      int kt = kt_first + (c >> 4), wrapped = 0;
+      if (kt >= KT) {
+        kt -= KT;
+        wrapped = n_heads;
+      }
+      const int k = kt * 16 + (c & 15);
+      const int head = k / HD, d = k - head * HD;
+      int hl = head + wrapped - head0;
+      if (hl >= heads_here) hl -= n_heads;
+      const float* po = pp.part_o + ((size_t)m * n_heads + head) * kAttnSplits * HD + d;
+      const float* w = w8 + ((size_t)m * heads_here + hl) * kAttnSplits;
+      float4 oj[kAttnSplits];
+#pragma unroll
+      for (int j = 0; j < kAttnSplits; ++j) oj[j] = ld_act4(po + (size_t)j * HD);
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int j = 0; j < kAttnSplits; ++j) {
-        const float w = wj[j] * inv_l;
-        xv.x = fmaf(w, oj[j].x, xv.x);
-        xv.y = fmaf(w, oj[j].y, xv.y);
+        x.x = fmaf(w[j], oj[j].x, x.x);
+        x.y = fmaf(w[j], oj[j].y, x.y);
+        x.z = fmaf(w[j], oj[j].z, x.z);
+        x.w = fmaf(w[j], oj[j].w, x.w);
       }
-      *reinterpret_cast<float2*>(x_staged + m * staged_ld + c) = xv;
+      uint32_t* xw = staged_word(m, c);
+      split_pack(x.x, x.y, xw[0], xw[2]);
+      split_pack(x.z, x.w, xw[4], xw[6]);
     }
     consumer_sync();
   }
 
   // activation fragments of my next three units; kt_pref = k-tile of the next unit to prefetch
-  const XSource xs{XM == X_STAGED ? x_staged : st.X, st.gain, pp.part_o, XM == X_STAGED ? staged_ld : st.ldx, st.ep.n_heads, kt_first, KT};
-  XRegs<CG> x0, x1, x2;
+  const XSource xs{st.X, st.gain, st.ldx, XM == X_STAGED ? reinterpret_cast<const uint4*>(x_staged) : st.x_in, pp.part_o, staged_ld, st.ep.n_heads, kt_first, KT};
+  XRegs<CG, RAW> x0, x1, x2;
   int kt_pref = (kt_first + cls) % KT;
-  auto prefetch = [&](XRegs<CG>& x, int i) {
-    load_xregs<CG, HD, XM>(x, xs, sc, M, kt_pref, g, q, i < my_n);
+  auto prefetch = [&](XRegs<CG, RAW>& x, int i) {
+    if constexpr (RAW)
+      load_xraw<CG>(x, xs, M, kt_pref, g, q, i < my_n);
+    else
+      load_xregs<CG, HD, XM>(x, xs, sc, M, kt_pref, g, q, i < my_n);
     kt_pref += kChunkUnits;
     if (kt_pref >= KT) kt_pref -= KT;
   };
@@ -610,9 +703,9 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
     const bool owner = starts_group && !whole;
 
     // the old residual values this thread will add to, fetched now so that they are there at the end
-    float2 hold[CG];
+    float2 hold[CG], hgain[CG];  // ... and the next norm's gain at the same features
 #pragma unroll
-    for (int j = 0; j < CG; ++j) hold[j] = make_float2(0.f, 0.f);
+    for (int j = 0; j < CG; ++j) hold[j] = hgain[j] = make_float2(0.f, 0.f);
     if (starts_group && epi_mode == EPI_RESID) {
 #pragma unroll
       for (int j = 0; j < CG; ++j) {
@@ -624,6 +717,10 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
         if (m < M && rt < NT) {
           const float* hp = st.ep.out + (size_t)m * st.ep.out_ld + 16 * rt + (ln >> 2);
           hold[j] = make_float2(ld_act(hp), ld_act(hp + 8));
+          if (IMG) {
+            const float* gp = st.gain_out + 16 * rt + (ln >> 2);
+            hgain[j] = make_float2(__ldg(gp), __ldg(gp + 8));
+          }
         }
       }
     }
@@ -648,16 +745,19 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
       uint4 a[4];
 #pragma unroll
       for (int r = 0; r < 4; ++r) a[r] = tiles[r * 32 + lane];
-      const float2 g0 = x0.g0, g1 = x0.g1;
 #pragma unroll
       for (int cg = 0; cg < CG; ++cg) {
-        uint32_t bh0, bl0, bh1, bl1;
-        split_pack(x0.lo8[cg].x * g0.x, x0.lo8[cg].y * g0.y, bh0, bl0);
-        split_pack(x0.hi8[cg].x * g1.x, x0.hi8[cg].y * g1.y, bh1, bl1);
+        uint4 b;
+        if constexpr (RAW) {
+          split_pack(x0.lo8[cg].x * x0.g0.x, x0.lo8[cg].y * x0.g0.y, b.x, b.z);
+          split_pack(x0.hi8[cg].x * x0.g1.x, x0.hi8[cg].y * x0.g1.y, b.y, b.w);
+        } else {
+          b = x0.v[cg];
+        }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          mma_bf16_16816(acc[r][cg], a[r], bh0, bh1);
-          mma_bf16_16816(acc[r][cg], a[r], bl0, bl1);
+          mma_bf16_16816(acc[r][cg], a[r], b.x, b.y);
+          mma_bf16_16816(acc[r][cg], a[r], b.z, b.w);
         }
       }
       // Hand the slot back once the tile reads above have returned: the producer's next bulk
@@ -728,15 +828,42 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
         const int m = cg * 8 + 2 * (ln & 3) + ch;
         const int rt = grp * kUnitTiles + tile;
         float sq = 0.f;
-        if (m < M && rt < NT) {
-          const float inv = sh->inv_rms[m];
-          if (epi_mode == EPI_RESID) {
-            float* hp = st.ep.out + (size_t)m * st.ep.out_ld + 16 * rt + (ln >> 2);
+        const int kk = ln >> 2;
+        const bool odd = (kk & 1) != 0, live = m < M && rt < NT;
+        if (epi_mode == EPI_RESID) {
+          float y0 = 0.f, y1 = 0.f;
+          if (live) {
+            const float inv = sh->inv_rms[m];
+            float* hp = st.ep.out + (size_t)m * st.ep.out_ld + 16 * rt + kk;
             const float n0 = hold[j].x + v0 * inv, n1 = hold[j].y + v1 * inv;
             hp[0] = n0;
             hp[8] = n1;
             sq = fmaf(n0, n0, n1 * n1);
-          } else if (fused_argmax) {
+            y0 = n0 * hgain[j].x;
+            y1 = n1 * hgain[j].y;
+          }
+          if constexpr (IMG) {
+            // neighbouring features (lanes 8 apart) make the fragment's pairs: the even one stores the high parts, the odd one the low
+            const float p0 = __shfl_xor_sync(0xffffffffu, y0, 8), p1 = __shfl_xor_sync(0xffffffffu, y1, 8);
+            uint32_t h0, h1, l0, l1;
+            split_pack(odd ? p0 : y0, odd ? y0 : p0, h0, l0);
+            split_pack(odd ? p1 : y1, odd ? y1 : p1, h1, l1);
+            if (live) reinterpret_cast<uint2*>(st.x_out + frag_index(rt, m, kk >> 1))[odd] = odd ? make_uint2(l0, l1) : make_uint2(h0, h1);
+          }
+        } else if (IMG && epi_mode == EPI_SWIGLU) {
+          float y = 0.f;
+          if (live) {
+            const float inv = sh->inv_rms[m], a = v0 * inv;
+            y = a / (1.0f + __expf(-a)) * (v1 * inv);
+          }
+          const float p = __shfl_xor_sync(0xffffffffu, y, 8);
+          uint32_t h, l;
+          split_pack(odd ? p : y, odd ? y : p, h, l);
+          // feature 8 rt + kk of u: column 8 (rt % 2) + kk of k-tile rt / 2
+          if (live) reinterpret_cast<uint32_t*>(st.x_out + frag_index(rt >> 1, m, kk >> 1))[(odd ? 2 : 0) + (rt & 1)] = odd ? l : h;
+        } else if (live) {
+          const float inv = sh->inv_rms[m];
+          if (fused_argmax) {
             const float a = v0 * inv, b2 = v1 * inv;  // logits of features 16 rt + ln/4 and + 8
             const int f0 = 16 * rt + (ln >> 2);
             sq = b2 > a ? b2 : a;
@@ -1005,12 +1132,13 @@ __host__ __device__ constexpr size_t pass_attn_smem_half() {
 
 template <int CG, int HD>
 __host__ __device__ constexpr size_t pass_work_bytes() {
-  return (size_t)(work_sc_off<CG>() + kWorkScBytes) > 2 * pass_attn_smem_half<HD>() ? (size_t)(work_sc_off<CG>() + kWorkScBytes)
+  return (size_t)(work_sc_off<CG>() + work_sc_bytes<CG>()) > 2 * pass_attn_smem_half<HD>() ? (size_t)(work_sc_off<CG>() + work_sc_bytes<CG>())
                                                                                     : 2 * pass_attn_smem_half<HD>();
 }
 
 // Dynamic shared memory: [ring: n_slots * 32 KB][work area][PassShared]
-template <int CG, int HD>
+// IMG: the activations of plain stages travel as fragment images (otherwise as fp32 rows that every load splits)
+template <int CG, int HD, bool IMG>
 __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, int n_slots) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* ring = smem;
@@ -1144,16 +1272,16 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, in
       // otherwise collide.
       const unsigned serial = 2u * ((unsigned)bar_base + (unsigned)s) + (s == 0 ? 1u : 0u) + 2u;
       if (sh->st.x_mode == X_PLAIN) {
-        linear_stage<CG, HD, X_PLAIN>(pp, sh, ring, n_slots, work, chunk_base, serial);
+        linear_stage<CG, HD, X_PLAIN, IMG>(pp, sh, ring, n_slots, work, chunk_base, serial);
       } else {
         // fold the attention partials into shared memory first if the columns this CTA's units
         // use fit beside the other work buffers (they do for passes of a few rows)
         const int kts = min(sh->share.n, sh->st.KT);
-        const size_t need = (size_t)pp.M * (size_t)(kts * 16 + 8) * sizeof(float);
+        const size_t need = (size_t)pp.M * staged_row_words(kts) * sizeof(uint32_t);
         if (need <= pass_work_bytes<CG, HD>() - (size_t)work_sc_off<CG>())
-          linear_stage<CG, HD, X_STAGED>(pp, sh, ring, n_slots, work, chunk_base, serial);
+          linear_stage<CG, HD, X_STAGED, IMG>(pp, sh, ring, n_slots, work, chunk_base, serial);
         else
-          linear_stage<CG, HD, X_ATTN_FOLD>(pp, sh, ring, n_slots, work, chunk_base, serial);
+          linear_stage<CG, HD, X_ATTN_FOLD, IMG>(pp, sh, ring, n_slots, work, chunk_base, serial);
       }
     } else {
       const int half = tid / kHalfThreads, htid = tid % kHalfThreads;
