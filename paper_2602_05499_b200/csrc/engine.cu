@@ -233,6 +233,7 @@ UmmaParams dense_params(const sdfp_ctx* c, const void* w_img, const unsigned cha
   p.M = rows;
   p.n_pairs = n_pairs;
   p.n_stages = umma_stages_for(RB, c->max_smem_optin);
+  p.n_work = umma_workers(p.n_ft * (c->prompt_grouped ? 1 : p.n_rb), KB, c->num_sms);
   p.partial = c->um_partial;
   p.flags = c->um_flags;
   p.flags_post = c->um_sabotage_ns ? c->um_flags_dummy : c->um_flags;  // test hook: posts that never arrive

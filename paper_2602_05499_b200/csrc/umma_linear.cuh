@@ -36,6 +36,8 @@
 // Every wait is bounded: a wait that runs out records an error word and the CTA winds down.
 #pragma once
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "linear_fma.cuh"
 #include "pass_kernel.cuh"
@@ -74,6 +76,16 @@ struct UmmaShared {
 inline size_t umma_smem_bytes(int RB, int n_stages) {
   return (size_t)n_stages * um_stage_bytes(RB) + (size_t)kUmEpiWarps * 32 * kUmExLd * 4 + sizeof(UmmaShared) + 1024;
 }
+// Over how many CTAs the units (weight blocks of 128 features x 64 columns) are cut: all of them while each gets
+// kUmMinUnits, but never fewer than there are tiles.  A small matrix over all CTAs leaves a block or two each and
+// a tile in as many pieces as it has blocks, which its finisher has to wait for and add.  Decoding 8
+// sequences, 6 layers d 512, FFN 1520, k = 3: 18.4 ms over all CTAs, 15.3 with at least 4 units each, 14.3 with 8; at
+// d 256 whole tiles of 4 and 11 units 6.1 ms, 8 units across them 8.5.
+constexpr int kUmMinUnits = 8;
+inline int umma_workers(int tiles, int KB, int grid) {
+  const long long fed = ((long long)tiles * KB + kUmMinUnits - 1) / kUmMinUnits;
+  return (int)std::min((long long)grid, std::max(fed, (long long)tiles));
+}
 inline int umma_stages_for(int RB, int max_smem_optin) {
   int s = kUmMaxStages;
   while (s > 2 && umma_smem_bytes(RB, s) > (size_t)max_smem_optin) --s;
@@ -87,6 +99,7 @@ struct UmmaParams {
   int M;                   // valid rows (<= n_rb * RB)
   int n_pairs;             // valid output pairs (<= 64 * n_ft)
   int n_stages;
+  int n_work;              // CTAs the list is cut over (umma_workers)
   float* partial;          // [grid][row blocks if RB_INNER][RB * 128] partial accumulators of cut tiles
   int* flags;              // [grid][row blocks if RB_INNER], zero between launches: "CTA c has posted its partial accumulator"
   int* flags_post;         // where a CTA raises its flag: flags, except under the failure-path test hook
@@ -226,12 +239,12 @@ __global__ void __launch_bounds__(kUmThreads, 1) umma_linear_kernel(UmmaParams p
   float* ex = reinterpret_cast<float*>(smem + (size_t)p.n_stages * stage_bytes);
   UmmaShared* sh = reinterpret_cast<UmmaShared*>(ex + kUmEpiWarps * 32 * kUmExLd);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int cta = blockIdx.x, n_cta = gridDim.x;
+  const int cta = blockIdx.x, n_cta = p.n_work;
   const int KB = p.KB;
   const int n_in = RB_INNER ? p.n_rb : 1, n_outer = RB_INNER ? 1 : p.n_rb;  // row blocks per piece; per feature tile in the list
   const long long n_units = (long long)p.n_ft * n_outer * KB;
-  long long ub, ue;
-  unit_range(n_units, cta, n_cta, ub, ue);
+  long long ub = n_units, ue = n_units;  // CTAs beyond n_work have nothing to do
+  if (cta < n_cta) unit_range(n_units, cta, n_cta, ub, ue);
 
   if (tid == 0) {
     for (int s = 0; s < p.n_stages; ++s) {
@@ -338,6 +351,7 @@ __global__ void __launch_bounds__(kUmThreads, 1) umma_linear_kernel(UmmaParams p
   } else if (warp == 1) {
     // ================= MMA issue =================
     if (lane == 0 && !*s_abort) {
+      pdl_wait();  // nothing arrives before: a wait limit counts from here and not from the preceding kernel's run
       const uint32_t idesc = um_idesc(2 * p.RB);
       const uint32_t lbo_b = (uint32_t)p.RB * 32u;  // 2*RB/8 row groups of 128 bytes between the k groups
       int stage = 0, buf = 0;
@@ -420,20 +434,22 @@ __global__ void __launch_bounds__(kUmThreads, 1) umma_linear_kernel(UmmaParams p
         const bool owner = starts && !whole;
         const bool okw = um_wait([&] { return mbar_try_wait(&sh->acc_full[buf], acc_phase); }, p.error, s_abort, UMMA_ERR_ACC_FULL, p.wait_limit_ns);
         (void)okw;
-        if (owner && et == 0) {
-          // the rest of the tile lies at the start of the ranges of the CTAs that follow
+        if (owner && et < 32) {
+          // the rest of the tile lies at the start of the ranges of the CTAs that follow: a lane waits for each
           const long long tile_end = (long long)(s.tile + 1) * KB;
           int n = 0;
-          for (int c2 = cta + 1; c2 < n_cta; ++c2) {
-            long long b2, e2;
-            unit_range(n_units, c2, n_cta, b2, e2);
-            if (b2 >= tile_end) break;
-            if (e2 > b2) {
-              um_wait([&] { return ld_acquire(p.flags + c2 * n_in + rin) != 0; }, p.error, s_abort, UMMA_ERR_POST, p.wait_limit_ns);
-              sh->posts[n++] = c2;
-            }
+          for (int base = cta + 1;; base += 32) {
+            const int c2 = base + et;
+            long long b2 = tile_end, e2 = tile_end;
+            if (c2 < n_cta) unit_range(n_units, c2, n_cta, b2, e2);
+            const bool part = b2 < tile_end && e2 > b2;
+            if (part) um_wait([&] { return ld_acquire(p.flags + c2 * n_in + rin) != 0; }, p.error, s_abort, UMMA_ERR_POST, p.wait_limit_ns);
+            const unsigned mask = __ballot_sync(0xffffffffu, part);
+            if (part) sh->posts[n + __popc(mask & ((1u << et) - 1u))] = c2;
+            n += __popc(mask);
+            if (__any_sync(0xffffffffu, b2 >= tile_end)) break;
           }
-          sh->n_posts = n;
+          if (et == 0) sh->n_posts = n;
         }
         um_epi_sync();
         if (et == 0) sh->decision = sh->abort;

@@ -945,6 +945,26 @@ def test_pass_kernel_work_split_and_images(heads, head_dim, ffn, vocab):
         eng.close()
 
 
+@pytest.mark.parametrize("heads,head_dim,ffn,vocab", [
+    (1, 64, 16, 16),       # one weight block per tile, one tile per matrix
+    (5, 64, 1040, 272),    # tiles of 5 and 17 blocks, a ragged last tile
+    (9, 128, 2064, 144),   # d 1152: tiles cut into pieces of eight blocks and more, fewer CTAs than the grid
+])
+def test_dense_path_small_matrices(heads, head_dim, ffn, vocab):
+    """The dense decode path where a matrix is cut over fewer CTAs than the grid has: 80 rows against the oracle, and rows
+    alone, in 16-row and in 17-row passes with the same bits."""
+    shape = si.ModelShape("edge", 2, heads * head_dim, heads, head_dim, ffn, vocab, dtype="bf16")
+    eng, m, _ = make_pair(shape, (), max_seq=96, max_batch=8, k_max=4, random_gains=True)
+    try:
+        toks = si.make_prompts(shape.vocab, 1, 80, seed=12)[0].tolist()
+        got = eng.sdfp_forward_logits(toks, 0)
+        assert rel_l2(got, orc.forward_nocache(m, toks).detach().numpy()) <= 1e-2
+        for lo, hi in ((0, 1), (40, 56), (63, 80), (79, 80)):
+            assert np.array_equal(eng.sdfp_forward_logits(toks[lo:hi], lo), got[lo:hi])
+    finally:
+        eng.close()
+
+
 def test_largest_batch_and_row_count():
     """The library's limits in one context: 16 sequences, k = 4, 80 rows in a verify pass (row block of
     80 rows = MMA width 160), 32 rows in the first draft pass; prompts of one token (nothing to cache
