@@ -965,6 +965,22 @@ def test_dense_path_small_matrices(heads, head_dim, ffn, vocab):
         eng.close()
 
 
+@pytest.mark.parametrize("head_dim", [64, 128])
+def test_per_operation_attention_around_the_first_chunk(head_dim):
+    """Passes whose rows see exactly one 64-key chunk, end on it or reach into the second: logits against the oracle, and a
+    row has the same bits whether its pass stays inside the chunk or not."""
+    shape = si.ModelShape("edge", 2, 2 * head_dim, 2, head_dim, 336, 208)
+    eng, m, _ = make_pair(shape, (), max_seq=160, max_batch=4, k_max=4)
+    try:
+        toks = si.make_prompts(shape.vocab, 1, 80, seed=13)[0].tolist()
+        got = eng.sdfp_forward_logits(toks, 0)             # 80 rows: the groups up to position 63 finish themselves
+        assert rel_l2(got, orc.forward_nocache(m, toks).detach().numpy()) <= 1e-4
+        for lo, hi in ((0, 1), (50, 64), (60, 68), (63, 64), (64, 65), (62, 66)):
+            assert np.array_equal(eng.sdfp_forward_logits(toks[lo:hi], lo), got[lo:hi])
+    finally:
+        eng.close()
+
+
 def test_largest_batch_and_row_count():
     """The library's limits in one context: 16 sequences, k = 4, 80 rows in a verify pass (row block of
     80 rows = MMA width 160), 32 rows in the first draft pass; prompts of one token (nothing to cache
