@@ -15,13 +15,18 @@
 //   * Sixteen consumer warps take the slots in order, feed the tiles to mma.sync.m16n8k16 (weights
 //     are the A operand, tokens the 8-wide B operand) and run the fused epilogues.
 //   * Stages are separated by a grid barrier (arrival counter in global memory, bounded spin).
+//     What a stage boundary costs is its chain of dependent steps, not its bytes; those that need no
+//     other CTA are kept off it: the next stage's descriptor and share are fetched during the running
+//     stage, ring positions run on from stage to stage, one barrier carries "all agree", a row's squares are
+//     added by a warp (pass of one row, 4 layers d 256 123 -> 117 us, 6 layers d 2048 313 -> 306, 12 layers
+//     d 4096 1164 -> 1157, five rows 1281 -> 1267).
 //
 // Weight layout ("unit" layout, written by pack_units_kernel): a matrix with NT 16-row tiles and
 // KT 16-column tiles is stored as units of 8 row tiles at one k-tile, 4096 contiguous bytes,
 // unit index = group * KT + kt with group = row tile / 8; inside a unit tile r at r*512 bytes in
-// the register order of the MMA A fragment.  The units of a matrix are split evenly over the
-// CTAs as contiguous ranges, so every CTA streams one contiguous byte range per stage and the
-// shares differ by at most one unit (4 KB).  A range cuts groups at arbitrary k: a group that
+// the register order of the MMA A fragment.  The units of a matrix are dealt to the CTAs as
+// contiguous ranges (evenly, to one unit of 4 KB, or for a small matrix in a few pieces per group:
+// stage_shares), so every CTA streams one contiguous byte range per stage.  An even cut cuts groups at arbitrary k: a group that
 // spans several CTAs is finished by the CTA that holds its beginning (which reaches it last),
 // after the others have posted their partial sums to global scratch; partials are added in CTA
 // order, so the result does not depend on timing.  A post is written as 64-bit words that hold a
@@ -122,7 +127,7 @@ struct PassSync {                // one per context, in global memory, zero-init
 // host once: two 64-bit divisions per look would sit on the stage boundary's critical path, here and for
 // every CTA an owner looks for.
 struct StageShare {
-  int ub, n, posters, pad;
+  int ub, n, posters, group;  // group = ub / KT
 };
 
 struct PassParams {
@@ -233,9 +238,8 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 struct PassShared {
   uint64_t full[8];
   uint64_t empty[8];
-  StageDesc st;       // the running stage
-  StageDesc st_next;  // the next one, fetched while the running stage works
-  StageShare share, share_next;  // this CTA's share of them
+  StageDesc st[2];      // stage s in st[s % 2]; the other one is the next stage's, fetched while the running stage works
+  StageShare share[2];  // this CTA's share of them
   float inv_rms[kPassMaxRows];
   int row_pos[kPassMaxRows], row_seq[kPassMaxRows];  // fixed for the whole pass
   unsigned long long bar_base;
@@ -245,13 +249,16 @@ struct PassShared {
   float attn_m[2][kPassAttnR], attn_l[2][kPassAttnR], attn_a[2][kPassAttnR];
 };
 
-// All consumer threads learn the same answer to "has anything failed": thread 0 samples the
-// flag between two barriers, so warps never disagree about leaving a loop that contains barriers.
+// A barrier of the consumer threads that also tells all of them the same answer to "has anything failed": every
+// thread brings the flag as it sees it, so warps never disagree about leaving a loop that contains barriers.
 __device__ __forceinline__ bool consumers_agree_ok(PassShared* sh) {
-  consumer_sync();
-  if (threadIdx.x == 0) sh->decision = sh->abort;
-  consumer_sync();
-  return sh->decision == 0;
+  const int seen = *reinterpret_cast<volatile int*>(&sh->abort);
+  unsigned any;
+  asm volatile("{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+               : "=r"(any)
+               : "r"(seen), "n"(kPassConsumerThreads)
+               : "memory");
+  return any == 0;
 }
 
 // Spin until pred() holds; false (and the error recorded) if the limit passes or another CTA
@@ -356,7 +363,7 @@ inline void stage_shares(StageShare* out, int n_groups, int KT, int grid) {
   };
   for (int c = 0; c < grid; ++c) {
     const long long ub = begin(c), ue = begin(c + 1);
-    out[c] = StageShare{(int)ub, (int)(ue - ub), 0, 0};
+    out[c] = StageShare{(int)ub, (int)(ue - ub), 0, (int)(ub / KT)};
     if (ue == ub || ue % KT == 0) continue;
     const long long grp_begin = ue / KT * KT, grp_end = grp_begin + KT;
     if (grp_begin < ub) continue;  // this CTA's own last piece is one to post
@@ -489,10 +496,9 @@ struct FoldStats {
 };
 
 template <int CG, int HD, int XM, bool IMG>
-__device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigned char* ring, int n_slots, unsigned char* work,
-                             unsigned& chunk_base, unsigned epoch) {
+__device__ void linear_stage(const PassParams& pp, PassShared* sh, const StageDesc& st, const StageShare share, const unsigned char* ring,
+                             int n_slots, unsigned char* work, unsigned& ring_slot, unsigned& ring_parity, unsigned epoch) {
   constexpr bool RAW = XM == X_PLAIN && !IMG;
-  const StageDesc& st = sh->st;
   float4* red = reinterpret_cast<float4*>(work);
   float* sq_buf = reinterpret_cast<float*>(work + work_sq_off<CG>());
   float* sc = reinterpret_cast<float*>(work + work_sc_off<CG>());
@@ -504,14 +510,13 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
   const int KT = st.KT, M = pp.M, NT = st.NT;
   const int epi_mode = st.ep.mode;
   const int cta = blockIdx.x;
-  const StageShare share = sh->share;
   const int nun = share.n;  // units of this CTA; below, units are numbered from share.ub
   const int n_chunks = (nun + kChunkUnits - 1) / kChunkUnits;
   const int my_n = nun > cls ? (nun - cls + kChunkUnits - 1) / kChunkUnits : 0;
-  const int grp0 = share.ub / KT;
+  const int grp0 = share.group;
   const int kt_first = share.ub - grp0 * KT;  // k-tile of unit 0
-  // ring position of this stage's first chunk; advanced by one slot per unit of this warp
-  unsigned slot = chunk_base % (unsigned)n_slots, parity = (chunk_base / (unsigned)n_slots) & 1u;
+  // ring position of this stage's first chunk; advanced by one slot per unit of this warp, and per chunk of the stage in the end
+  unsigned slot = ring_slot, parity = ring_parity;
 
   // ---- 1/rms of every row (needed only by the epilogue) ----
   if (st.rms_mode == RMS_DIRECT) {
@@ -873,14 +878,13 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
       }
     }
     if (starts_group && st.write_ssq) {
-      // one sum of squares per row over this group's 128 features, in tile-then-row order
+      // one sum of squares per row over this group's 128 features: a warp per row, two features per lane, fixed xor tree
       consumer_sync();
-      if (tid < M) {
-        const int cg = tid >> 3, qq = (tid & 7) >> 1, ch = tid & 1;
-        float s = 0.f;
-        for (int tile = 0; tile < kUnitTiles; ++tile)
-          for (int g8 = 0; g8 < 8; ++g8) s += sq_buf[(((tile * CG + cg) * 32) + g8 * 4 + qq) * 2 + ch];
-        pp.ssq_part[grp * kPassMaxRows + tid] = s;
+      if (warp < M) {
+        const int cg = warp >> 3, qq = (warp & 7) >> 1, ch = warp & 1;
+        auto at = [&](int i) { return sq_buf[((((i >> 3) * CG + cg) * 32) + (i & 7) * 4 + qq) * 2 + ch]; };  // i = tile * 8 + row of the tile
+        const float sum = warp_sum(at(lane) + at(lane + 32));
+        if (lane == 0) pp.ssq_part[grp * kPassMaxRows + warp] = sum;
       }
     }
     if (starts_group && fused_argmax) {
@@ -903,7 +907,7 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
         pp.amax_part[grp * kPassMaxRows + tid] = make_int2(__float_as_int(best), bi);
       }
     }
-    consumer_sync();  // red may be rewritten
+    if (seg_end < nun) consumer_sync();  // red may be rewritten (behind the last segment the stage's barrier says so)
     seg_begin = seg_end;
     seg_kt0 = 0;
     ++grp;
@@ -916,8 +920,13 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const unsigne
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh->empty[slot]);
     }
+    if (++slot == (unsigned)n_slots) {
+      slot = 0;
+      parity ^= 1u;
+    }
   }
-  chunk_base += (unsigned)n_chunks;
+  ring_slot = slot;
+  ring_parity = parity;
 }
 
 // ---- attention stage --------------------------------------------------------------------------
@@ -1236,22 +1245,19 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, in
   // ================= consumer warps =================
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPassConsumerRegs));
   const unsigned long long bar_base = sh->bar_base;
-  unsigned chunk_base = 0;
+  unsigned ring_slot = 0, ring_parity = 0;
   bool ok = true;
   constexpr int kDescWords = (int)(sizeof(StageDesc) / sizeof(int));
   static_assert(kDescWords < 64, "two warps fetch a stage descriptor and the CTA's share");
   const int desc_w = tid - (kPassConsumerThreads - 64);  // the last two warps fetch descriptors, one word per thread
   const bool share_thread = desc_w == kDescWords;
   for (int s = 0; s < pp.n_stages && ok; ++s) {
+    const StageDesc& st = sh->st[s & 1];
     if (s == 0) {
-      if (desc_w >= 0 && desc_w < kDescWords)
-        reinterpret_cast<int*>(&sh->st)[desc_w] = reinterpret_cast<const int*>(pp.prog)[desc_w];
-      if (share_thread) sh->share = pp.shares[blockIdx.x];
-    } else {
-      if (desc_w >= 0 && desc_w < kDescWords) reinterpret_cast<int*>(&sh->st)[desc_w] = reinterpret_cast<const int*>(&sh->st_next)[desc_w];
-      if (share_thread) sh->share = sh->share_next;
+      if (desc_w >= 0 && desc_w < kDescWords) reinterpret_cast<int*>(&sh->st[0])[desc_w] = reinterpret_cast<const int*>(pp.prog)[desc_w];
+      if (share_thread) sh->share[0] = pp.shares[blockIdx.x];
+      consumer_sync();
     }
-    consumer_sync();
     // the next stage's descriptor: asked for now, stored at the end of this stage, so that the
     // stage after a barrier starts without a round trip to global memory
     int next_word = 0;
@@ -1259,27 +1265,28 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, in
       next_word = reinterpret_cast<const int*>(pp.prog + s + 1)[desc_w];
     StageShare next_share{};
     if (s + 1 < pp.n_stages && share_thread) next_share = pp.shares[(size_t)(s + 1) * gridDim.x + blockIdx.x];
-    if (sh->st.kind == ST_LINEAR) {
+    const StageShare share = sh->share[s & 1];
+    if (st.kind == ST_LINEAR) {
       // The posts of split groups carry a number no stage of any launch shares.  Barrier serials
       // advance by n_stages - 1 per launch, so stage s gets (bar_base + s) * 2 + (1 if it is the
       // launch's first stage): only a launch's last stage and the next launch's first would
       // otherwise collide.
       const unsigned serial = 2u * ((unsigned)bar_base + (unsigned)s) + (s == 0 ? 1u : 0u) + 2u;
-      if (sh->st.x_mode == X_PLAIN) {
-        linear_stage<CG, HD, X_PLAIN, IMG>(pp, sh, ring, n_slots, work, chunk_base, serial);
+      if (st.x_mode == X_PLAIN) {
+        linear_stage<CG, HD, X_PLAIN, IMG>(pp, sh, st, share, ring, n_slots, work, ring_slot, ring_parity, serial);
       } else {
         // fold the attention partials into shared memory first if the columns this CTA's units
         // use fit beside the other work buffers (they do for passes of a few rows)
-        const int kts = min(sh->share.n, sh->st.KT);
+        const int kts = min(share.n, st.KT);
         const size_t need = (size_t)pp.M * staged_row_words(kts) * sizeof(uint32_t);
         if (need <= pass_work_bytes<CG, HD>() - (size_t)work_sc_off<CG>())
-          linear_stage<CG, HD, X_STAGED, IMG>(pp, sh, ring, n_slots, work, chunk_base, serial);
+          linear_stage<CG, HD, X_STAGED, IMG>(pp, sh, st, share, ring, n_slots, work, ring_slot, ring_parity, serial);
         else
-          linear_stage<CG, HD, X_ATTN_FOLD, IMG>(pp, sh, ring, n_slots, work, chunk_base, serial);
+          linear_stage<CG, HD, X_ATTN_FOLD, IMG>(pp, sh, st, share, ring, n_slots, work, ring_slot, ring_parity, serial);
       }
     } else {
       const int half = tid / kHalfThreads, htid = tid % kHalfThreads;
-      const int n_heads = sh->st.ep.n_heads;
+      const int n_heads = st.ep.n_heads;
       const int n_groups = (pp.M + pp.rows_per_seq - 1) / pp.rows_per_seq;
       const int items = kAttnSplits * n_heads * n_groups;
       unsigned char* my = work + (size_t)half * pass_attn_smem_half<HD>();
@@ -1288,15 +1295,15 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, in
         const int hb = it / kAttnSplits;
         const int hd_ = hb % n_heads, b_ = hb / n_heads;
         if (pp.rows_per_seq <= 2)
-          attention_item<HD, 2>(sh->st, pp, sh, my, half, htid, hd_, split, b_);
+          attention_item<HD, 2>(st, pp, sh, my, half, htid, hd_, split, b_);
         else if (pp.rows_per_seq <= 8)
-          attention_item<HD, 8>(sh->st, pp, sh, my, half, htid, hd_, split, b_);
+          attention_item<HD, 8>(st, pp, sh, my, half, htid, hd_, split, b_);
         else
-          attention_item<HD, 16>(sh->st, pp, sh, my, half, htid, hd_, split, b_);
+          attention_item<HD, 16>(st, pp, sh, my, half, htid, hd_, split, b_);
       }
     }
-    if (desc_w >= 0 && desc_w < kDescWords) reinterpret_cast<int*>(&sh->st_next)[desc_w] = next_word;
-    if (share_thread) sh->share_next = next_share;
+    if (desc_w >= 0 && desc_w < kDescWords) reinterpret_cast<int*>(&sh->st[(s + 1) & 1])[desc_w] = next_word;
+    if (share_thread) sh->share[(s + 1) & 1] = next_share;
     // the barrier also tells every thread whether a wait of this CTA gave up (the CTA still arrives)
     ok = (s + 1 < pp.n_stages) ? grid_barrier(pp.sync, bar_base + (unsigned long long)(s + 1), sh) : consumers_agree_ok(sh);
   }
