@@ -241,7 +241,7 @@ int sdfp_forward_logits_static(sdfp_ctx *ctx, int32_t draft, const int32_t *toke
 /*
  * Stage A of Algorithm 1 ("FIT-based pruning"): the layer scores from which the prune set P is
  * chosen.  No context is needed; the weights are read where the caller has them (same structure
- * and storage type as for sdfp_create, row-major [out, in]) and nothing is kept.
+ * and storage type as for sdfp_create, row-major [out, in]); the caller may free them afterwards.
  *   tokens     host int32 [n_seq, seq_len]: the calibration set D, one sequence = one sample z_i;
  *              f(z_i, theta) = mean cross-entropy of token t+1 under the logits at position t
  *   out_trace  host double [n_layers]: T_l = (1/N) sum_i ||grad_{theta_l} f(z_i, theta)||^2, the
@@ -251,13 +251,26 @@ int sdfp_forward_logits_static(sdfp_ctx *ctx, int32_t draft, const int32_t *toke
  *              the layer-wise FIT form (Eq. 7) with the perturbation of removing the layer,
  *              delta theta = -theta
  * Algorithm 1 then sorts ascending and prunes the floor(r L) lowest layers; feed the result to
- * sdfp_set_draft_layers.  One forward and one backward pass per sequence in fp32 (squared norms
- * accumulated in fp64); device memory for the activations of one sequence is allocated and freed
- * inside the call, which is synchronous.  Errors as for sdfp_create (message via
- * sdfp_last_error(NULL)).
+ * sdfp_set_draft_layers.  One forward and one backward pass in fp32 (squared norms accumulated in
+ * fp64), synchronous.  Calls may run on several threads and streams at a time.
+ * Device memory: the call works on up to 512 tokens (at least one whole sequence) at a time and holds,
+ * for R = sequences * (seq_len - 1) rows of such a group, about
+ *   4 R (n_layers (8 d_model + 3 d_ffn) + 10 d_model + 3 d_ffn + vocab) bytes of activations,
+ *   4 (n_layers + 1) R n_heads (seq_len - 1) bytes of attention probabilities,
+ * and partial sums; when the device has no room it takes fewer sequences at a time.  A working set above
+ * 256 MB is given back before the call returns.  A smaller one stays in a pool of the library (at
+ * most 256 MB per device) for the next call, until sdfp_fit_release, the next sdfp_destroy of a context on
+ * that device, or an sdfp_create that finds the device full.
+ * Errors as for sdfp_create (message via sdfp_last_error(NULL)).
  */
 int sdfp_fit_scores(const sdfp_config *cfg, const sdfp_weights *w, void *cuda_stream, const int32_t *tokens,
                     int32_t n_seq, int32_t seq_len, double *out_trace, double *out_fit);
+
+/*
+ * Give back the device memory that sdfp_fit_scores keeps between calls, on every device.  Safe at any time and from any
+ * thread: the memory of a call that is running stays.  Always 0.
+ */
+int sdfp_fit_release(void);
 
 /* Timing of the last successful sdfp_generate. */
 int sdfp_get_timing(const sdfp_ctx *ctx, sdfp_timing *out);

@@ -17,7 +17,7 @@ FLAG_NO_GRAPH, FLAG_NO_PDL, FLAG_FMA_GEMM, FLAG_NO_PASS_KERNEL, FLAG_NO_DENSE = 
 
 EXPORTS = ["sdfp_create", "sdfp_set_draft_layers", "sdfp_set_draft_sublayers", "sdfp_set_draft_kv_sharing", "sdfp_generate", "sdfp_forward_logits",
            "sdfp_forward_logits_static", "sdfp_get_timing", "sdfp_time_linear", "sdfp_time_pass",
-           "sdfp_debug_expire_next_wait", "sdfp_fit_scores", "sdfp_last_error", "sdfp_destroy"]
+           "sdfp_debug_expire_next_wait", "sdfp_fit_scores", "sdfp_fit_release", "sdfp_last_error", "sdfp_destroy"]
 
 
 class SdfpConfig(C.Structure):
@@ -97,6 +97,8 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     lib.sdfp_fit_scores.argtypes = [C.POINTER(SdfpConfig), C.POINTER(SdfpWeights), vp, C.POINTER(C.c_int32), C.c_int32, C.c_int32,
                                     C.POINTER(C.c_double), C.POINTER(C.c_double)]
     lib.sdfp_fit_scores.restype = C.c_int
+    lib.sdfp_fit_release.argtypes = []
+    lib.sdfp_fit_release.restype = C.c_int
     lib.sdfp_last_error.argtypes = [vp]
     lib.sdfp_last_error.restype = C.c_char_p
     lib.sdfp_destroy.argtypes = [vp]
@@ -150,6 +152,11 @@ def sdfp_fit_scores(shape, weights: Dict, calib) -> "tuple":
         raise SdfpError(rc, lib.sdfp_last_error(None).decode())
     del keep
     return trace.tolist(), fit.tolist()
+
+
+def sdfp_fit_release() -> None:
+    """Give back the device memory that sdfp_fit_scores keeps between calls."""
+    load_library().sdfp_fit_release()
 
 
 class GenOutput:

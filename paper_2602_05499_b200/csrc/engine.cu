@@ -1614,7 +1614,8 @@ extern "C" int sdfp_fit_scores(const sdfp_config* cfg, const sdfp_weights* w, vo
     return fail(nullptr, SDFP_EINVAL, "sdfp_fit_scores: bad model dimensions");
   if (g.dtype != SDFP_F32 && g.dtype != SDFP_BF16) return fail(nullptr, SDFP_EINVAL, "unknown dtype");
   if (!(g.rms_eps > 0.f) || !(g.rope_theta > 0.f)) return fail(nullptr, SDFP_EINVAL, "bad rms_eps or rope_theta");
-  if (n_seq < 1 || seq_len < 2 || seq_len > 4097) return fail(nullptr, SDFP_EINVAL, "sdfp_fit_scores: need n_seq >= 1 and 2 <= seq_len <= 4097");
+  if (n_seq < 1 || seq_len < 2 || seq_len > fit::kFitMaxT + 1)
+    return fail(nullptr, SDFP_EINVAL, "sdfp_fit_scores: need n_seq >= 1 and 2 <= seq_len <= %d", fit::kFitMaxT + 1);
   if (!w->tok_embed || !w->final_norm || !w->lm_head || !w->wq || !w->wk || !w->wv || !w->wo || !w->w_gate || !w->w_up || !w->w_down ||
       !w->attn_norm || !w->ffn_norm)
     return fail(nullptr, SDFP_EINVAL, "sdfp_fit_scores: NULL weight pointer");
@@ -1634,6 +1635,11 @@ extern "C" int sdfp_fit_scores(const sdfp_config* cfg, const sdfp_weights* w, vo
                                               : fit::run<float>(g, w, st, tokens, n_seq, seq_len, out_trace, out_fit);
   if (e != cudaSuccess)
     return fail(nullptr, e == cudaErrorMemoryAllocation ? SDFP_ENOMEM : SDFP_ECUDA, "sdfp_fit_scores: %s", cudaGetErrorString(e));
+  return 0;
+}
+
+extern "C" int sdfp_fit_release(void) {
+  for (int dev = 0; dev < fit::kFitPools; ++dev) fit::fit_pool_trim(dev);
   return 0;
 }
 

@@ -375,6 +375,7 @@ __global__ void rope_kernel(float* __restrict__ xq, float* __restrict__ xk, cons
 // A block takes kAtQ consecutive queries of one head of one sequence (grid: query group, head, sequence),
 // so that a key or value row is read once for all of them; sums run over the keys in order.
 constexpr int kAtQ = 8, kAtThreads = 128, kAtKeys = 32, kAtDim = 64;
+constexpr int kFitMaxT = 4096;  // positions of the longest sequence the entry point accepts
 
 inline size_t attn_smem(int T) { return (size_t)(kAtQ * T + kAtQ * kAtDim + kAtKeys * (kAtDim + 1)) * sizeof(float); }
 
@@ -781,11 +782,13 @@ static_assert(kTensors == kFitTensors, "the kernels' tensor count");
 
 constexpr int kFitRows = 512;  // calibration tokens that go through the stack together (at least one sequence)
 
-// Device memory of the calls comes from a pool of the library's own, one per device: cudaMalloc and cudaFree
-// of a call's buffers took 1 to 2 ms, as much as the whole call for a small decoder.  The pool keeps
-// at most kFitPoolKeep bytes between calls; what a call needed beyond that goes back to the device at
-// the next synchronisation, and all of it when a context is destroyed or runs out of memory (fit_pool_trim).
-constexpr unsigned long long kFitPoolKeep = 512ull << 20;
+// Device memory of a call, one allocation.  Up to kFitPoolKeep bytes come from a pool of the library's own, one per device:
+// cudaMalloc and cudaFree take 0.7 to 1.5 ms, as much as the whole call for a small decoder (4 layers d 256, 8 x 31
+// tokens: 1.07 ms from the pool, 1.82 without; 4 layers d 4096, 2 x 64 tokens, 200 MB: 12.7 and 14.3).  The pool keeps what it has
+// handed out, at most kFitPoolKeep bytes, until sdfp_fit_release, until a context is destroyed or until one runs
+// out of memory.  A larger working set is allocated and freed by the call itself: the call takes tens
+// of milliseconds, and mapping that much through the pool costs more than cudaMalloc (1.2 GB: 17.8 and 7.7 ms a call).
+constexpr unsigned long long kFitPoolKeep = 256ull << 20;
 constexpr int kFitPools = 64;
 struct FitPools {
   std::mutex lock;
@@ -823,6 +826,26 @@ inline void fit_pool_trim(int dev) {
   FitPools& f = fit_pools();
   std::lock_guard<std::mutex> g(f.lock);
   if (f.pool[dev] != nullptr && cudaMemPoolTrimTo(f.pool[dev], 0) != cudaSuccess) cudaGetLastError();
+}
+inline cudaError_t fit_alloc(void** p, size_t bytes, int dev, cudaStream_t st) {
+  if (bytes <= kFitPoolKeep) {
+    cudaMemPool_t pool;
+    const cudaError_t e = fit_pool(dev, &pool);
+    return e != cudaSuccess ? e : cudaMallocFromPoolAsync(p, bytes, pool, st);
+  }
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    fit_pool_trim(dev);
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+// after whatever is still running on the buffer; on return the memory is the pool's or the device's again
+inline cudaError_t fit_free(void* p, size_t bytes, cudaStream_t st) {
+  if (bytes > kFitPoolKeep) return cudaFree(p);
+  const cudaError_t e = cudaFreeAsync(p, st);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(st);
 }
 
 // One device allocation per call, cut into buffers: the layout runs once to learn the size and once
@@ -965,8 +988,6 @@ cudaError_t run_in(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st,
   auto W = [&](const void* const* arr, int l) { return reinterpret_cast<const WT*>(arr[l]); };
   const int eb = 4 * n_sm;  // blocks of the elementwise kernels
   const size_t att_smem = attn_smem(T);
-  FIT_OK(cudaFuncSetAttribute(attn_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_smem));
-  FIT_OK(cudaFuncSetAttribute(attn_bwd_q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_smem));
   cudaError_t ge = cudaSuccess;
 
   for (int s0 = 0; s0 < n_seq; s0 += nb) {
@@ -1068,8 +1089,9 @@ cudaError_t run(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st, co
   FIT_OK((gemm_prepare<WT, 32>(room.clusters[0])));
   FIT_OK((gemm_prepare<WT, 64>(room.clusters[1])));
   FIT_OK((gemm_prepare<WT, 128>(room.clusters[2])));
-  cudaMemPool_t pool;
-  FIT_OK(fit_pool(dev, &pool));
+  // (the limits belong to the kernels and not to this call: constants, or calls on other threads would lower them under it)
+  for (const void* k : {(const void*)attn_fwd_kernel, (const void*)attn_bwd_q_kernel})
+    FIT_OK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem(kFitMaxT)));
   // as many sequences at a time as fill kFitRows rows; fewer if the device has no room for their activations
   for (int nb = std::max(1, std::min(n_seq, kFitRows / T));; nb = (nb + 1) / 2) {
     const GramPlan gp = gram_plan(T, nb, g.d_model, g.d_ffn, n_sm);
@@ -1082,7 +1104,7 @@ cudaError_t run(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st, co
     };
     lay();
     void* p = nullptr;
-    const cudaError_t me = cudaMallocFromPoolAsync(&p, A.used, pool, st);
+    const cudaError_t me = fit_alloc(&p, A.used, dev, st);
     if (me == cudaErrorMemoryAllocation && nb > 1) {
       cudaGetLastError();
       continue;
@@ -1091,7 +1113,7 @@ cudaError_t run(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st, co
     A.base = reinterpret_cast<unsigned char*>(p);
     lay();
     const cudaError_t e = run_in<WT>(g, w, st, tokens, n_seq, seq_len, out_trace, out_fit, B, nb, n_sm, room, gp, n_slots);
-    const cudaError_t fe = cudaFreeAsync(p, st);  // after whatever is still running on these buffers
+    const cudaError_t fe = fit_free(p, A.used, st);
     return e != cudaSuccess ? e : fe;
   }
 }

@@ -1,5 +1,7 @@
 """Stage A of Algorithm 1 on the GPU (sdfp_fit_scores) against the CPU oracle's FIT scores, which
 are themselves pinned by finite differences (tests/test_oracle_fit.py)."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -77,6 +79,65 @@ def test_fit_scores_at_the_edges(d, heads, ffn, vocab, n_seq, seq_len, dtype):
     assert got_F == pytest.approx(ref_F, rel=1e-4)
     back_T, _ = pkg.sdfp_fit_scores(shape, si.weights_to(w, "cuda:0"), calib[::-1].copy())
     assert back_T == pytest.approx(got_T, rel=1e-12)   # a sequence's numbers do not depend on its group
+
+
+def test_fit_scores_on_two_threads_with_different_lengths():
+    """Calls on other threads, of other sequence lengths, do not disturb one another: a long sequence's launches go
+    through, and to the same bits, while a second thread scores sequences of a few tokens."""
+    pkg.build_library()
+    shape = si.ModelShape("threads", 8, 64, 1, 64, 80, 64)
+    w = si.weights_to(si.make_weights(shape, []), "cuda:0")
+    long_set, short_set = si.make_prompts(shape.vocab, 4, 1501, seed=1), si.make_prompts(shape.vocab, 2, 5, seed=2)
+    want = pkg.sdfp_fit_scores(shape, w, long_set)
+    stop, errors = threading.Event(), []
+
+    def score_short():
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                while not stop.is_set():
+                    pkg.sdfp_fit_scores(shape, w, short_set)
+        except Exception as e:  # noqa: BLE001 (reported by the test's own thread)
+            errors.append(e)
+
+    other = threading.Thread(target=score_short)
+    other.start()
+    try:
+        for _ in range(20):
+            assert pkg.sdfp_fit_scores(shape, w, long_set) == want
+    finally:
+        stop.set()
+        other.join()
+    assert not errors
+
+
+def test_fit_scores_give_their_memory_back():
+    """What a call holds when it returns, before anything else synchronises: nothing of a working set above 256 MB, at most
+    256 MB of a smaller one, and that until sdfp_fit_release or the end of a context."""
+    pkg.build_library()
+    small, large = si.ModelShape("small", 2, 64, 1, 64, 80, 64), si.ModelShape("large", 2, 64, 1, 64, 80, 1 << 17)
+    w_small, w_large = (si.weights_to(si.make_weights(m, []), "cuda:0") for m in (small, large))
+    sets = {m.name: si.make_prompts(m.vocab, 2, 600, seed=1) for m in (small, large)}  # large: 599 x 131072 logits, 314 MB
+    keep = 256 << 20
+
+    def kept(call):
+        call()                         # kernels and device tables loaded
+        pkg.sdfp_fit_release()
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        call()
+        return before - torch.cuda.mem_get_info()[0], before
+
+    assert kept(lambda: pkg.sdfp_fit_scores(large, w_large, sets["large"]))[0] <= 0
+    held, before = kept(lambda: pkg.sdfp_fit_scores(small, w_small, sets["small"]))
+    assert 0 < held <= keep
+    pkg.sdfp_fit_release()
+    assert torch.cuda.mem_get_info()[0] == before
+    eng = pkg.Sdfp(si.TINY, si.weights_to(si.make_weights(si.TINY, []), "cuda:0"), max_seq=64)
+    pkg.sdfp_fit_scores(small, w_small, sets["small"])
+    eng.close()
+    pkg.sdfp_fit_scores(small, w_small, sets["small"])
+    pkg.sdfp_fit_release()
+    pkg.sdfp_fit_release()             # nothing left: no error
 
 
 def test_fit_scores_drive_the_draft_mask():
