@@ -982,7 +982,6 @@ cudaError_t run_in(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st,
                    double* out_trace, double* out_fit, Buffers& B, int nb, int n_sm, const GemmRoom& room, const GramPlan& gp, int n_slots) {
   const int L = g.n_layers, d = g.d_model, f = g.d_ffn, V = g.vocab, H = g.n_heads, hd = g.head_dim, T = seq_len - 1;
   const float scale = 1.0f / std::sqrt((float)hd);
-  FIT_OK(cudaMemcpyAsync(B.tok, tokens, (size_t)n_seq * seq_len * 4, cudaMemcpyHostToDevice, st));
   FIT_OK(cudaMemsetAsync(B.slots, 0, (size_t)L * kTensors * n_slots * sizeof(double), st));
   rope_table_kernel<<<(T * (hd / 2) + 127) / 128, 128, 0, st>>>(B.cs, B.sn, T, hd, (double)g.rope_theta);
   auto W = [&](const void* const* arr, int l) { return reinterpret_cast<const WT*>(arr[l]); };
@@ -993,7 +992,8 @@ cudaError_t run_in(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st,
   for (int s0 = 0; s0 < n_seq; s0 += nb) {
     const int ns = std::min(nb, n_seq - s0), R = ns * T;
     const size_t Rf = (size_t)R * f;
-    const int* tok = B.tok + (size_t)s0 * seq_len;
+    const int* tok = B.tok;
+    FIT_OK(cudaMemcpyAsync(B.tok, tokens + (size_t)s0 * seq_len, (size_t)ns * seq_len * 4, cudaMemcpyHostToDevice, st));
     auto nt = [&](GemmArgs a, int N, int K) {
       a.R = R; a.N = N; a.K = K;
       if (ge == cudaSuccess) ge = fit_gemm_launch<WT, true>(a, nb * T, room, n_sm, st);
@@ -1100,7 +1100,7 @@ cudaError_t run(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st, co
     Arena A;
     auto lay = [&] {
       A.used = 0;
-      B.layout(A, g.n_layers, g.d_model, g.d_ffn, g.vocab, g.n_heads, g.head_dim, T, nb, n_seq * seq_len, gp.doubles(nb), n_slots);
+      B.layout(A, g.n_layers, g.d_model, g.d_ffn, g.vocab, g.n_heads, g.head_dim, T, nb, nb * seq_len, gp.doubles(nb), n_slots);
     };
     lay();
     void* p = nullptr;
