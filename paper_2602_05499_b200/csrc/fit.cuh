@@ -16,7 +16,9 @@
 // their storage type (fp32 or bf16) from the caller's row-major [out, in] matrices.  The calibration
 // sequences go through the stack together, up to kFitRows rows at a time: a GEMM then reads a weight
 // once for all of them, and a layer costs the same number of launches whatever the set's size.
-// Every reduction runs in a fixed order, so the scores are reproducible bit for bit.
+// Every reduction runs in an order fixed by the model, the sequences' length and how many of them make a full group
+// (the set's size up to kFitRows rows), so the same call gives the same bits; a sequence scored in a set of
+// another size may differ in the last places.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -942,8 +944,8 @@ cudaError_t gemm_prepare(int* clusters) {
   return cudaSuccess;
 }
 
-// plan_rows: the rows of a full group of sequences.  How a contraction is cut depends on them and not
-// on g.R, so that a sequence's numbers do not change when it sits in a last, smaller group.
+// plan_rows: the rows of a full group of sequences.  How a contraction is cut depends on them and not on g.R, so
+// that a sequence's numbers do not change when it sits in a smaller group (the last one, or where memory is short).
 template <typename WT, bool NT>
 cudaError_t fit_gemm_launch(const GemmArgs& g, int plan_rows, const GemmRoom& room, int n_sm, cudaStream_t st) {
   const int cols = NT ? g.N : g.K, inner = NT ? g.K : g.N;
@@ -979,7 +981,8 @@ cudaError_t fit_gemm_launch(const GemmArgs& g, int plan_rows, const GemmRoom& ro
 
 template <typename WT>
 cudaError_t run_in(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st, const int32_t* tokens, int n_seq, int seq_len,
-                   double* out_trace, double* out_fit, Buffers& B, int nb, int n_sm, const GemmRoom& room, const GramPlan& gp, int n_slots) {
+                   double* out_trace, double* out_fit, Buffers& B, int nb, int full, int n_sm, const GemmRoom& room, const GramPlan& gp,
+                   int n_slots) {
   const int L = g.n_layers, d = g.d_model, f = g.d_ffn, V = g.vocab, H = g.n_heads, hd = g.head_dim, T = seq_len - 1;
   const float scale = 1.0f / std::sqrt((float)hd);
   FIT_OK(cudaMemsetAsync(B.slots, 0, (size_t)L * kTensors * n_slots * sizeof(double), st));
@@ -989,18 +992,21 @@ cudaError_t run_in(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st,
   const size_t att_smem = attn_smem(T);
   cudaError_t ge = cudaSuccess;
 
-  for (int s0 = 0; s0 < n_seq; s0 += nb) {
-    const int ns = std::min(nb, n_seq - s0), R = ns * T;
+  const int gain_blocks = (d + kGainCols - 1) / kGainCols;
+  for (int s0 = 0, ns; s0 < n_seq; s0 += ns) {
+    const int z0 = s0 % full;  // place of the first sequence in its full group: its slots, whatever goes through together
+    ns = std::min(std::min(nb, full - z0), n_seq - s0);
+    const int R = ns * T;
     const size_t Rf = (size_t)R * f;
     const int* tok = B.tok;
     FIT_OK(cudaMemcpyAsync(B.tok, tokens + (size_t)s0 * seq_len, (size_t)ns * seq_len * 4, cudaMemcpyHostToDevice, st));
     auto nt = [&](GemmArgs a, int N, int K) {
       a.R = R; a.N = N; a.K = K;
-      if (ge == cudaSuccess) ge = fit_gemm_launch<WT, true>(a, nb * T, room, n_sm, st);
+      if (ge == cudaSuccess) ge = fit_gemm_launch<WT, true>(a, full * T, room, n_sm, st);
     };
     auto nn = [&](GemmArgs a, int N, int K) {
       a.R = R; a.N = N; a.K = K;
-      if (ge == cudaSuccess) ge = fit_gemm_launch<WT, false>(a, nb * T, room, n_sm, st);
+      if (ge == cudaSuccess) ge = fit_gemm_launch<WT, false>(a, full * T, room, n_sm, st);
     };
     // ---- forward ----
     embed_kernel<WT><<<R, 256, 0, st>>>(tok, reinterpret_cast<const WT*>(w->tok_embed), B.Hs[0], d, T, seq_len);
@@ -1028,7 +1034,7 @@ cudaError_t run_in(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st,
       nn({{dh}, {w->w_down[l]}, {B.du}, nullptr, 0, 0, 0, 1}, d, f);
       swiglu_bwd_kernel<<<eb, 256, 0, st>>>(B.du, B.gt[l], B.up[l], B.dgt, B.dup, Rf);
       nn({{B.dgt, B.dup}, {w->w_gate[l], w->w_up[l]}, {B.dx}, nullptr, 0, 0, 0, 2}, f, d);
-      gain_grad_sq_kernel<<<dim3((d + kGainCols - 1) / kGainCols, ns), 256, 0, st>>>(B.dx, B.Hmid[l], B.inv2[l], T, d, slots + (size_t)T_FFN_NORM * n_slots);
+      gain_grad_sq_kernel<<<dim3(gain_blocks, ns), 256, 0, st>>>(B.dx, B.Hmid[l], B.inv2[l], T, d, slots + (size_t)T_FFN_NORM * n_slots + z0 * gain_blocks);
       rmsnorm_bwd_kernel<WT><<<R, 512, 0, st>>>(B.dx, B.Hmid[l], W(w->ffn_norm, l), B.inv2[l], dh, dmid, d);  // d f / d Hmid
       // attention block: Hmid = H[l] + a Wo^T
       nn({{dmid}, {w->wo[l]}, {B.da}, nullptr, 0, 0, 0, 1}, d, d);
@@ -1036,7 +1042,7 @@ cudaError_t run_in(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st,
       attn_bwd_kv_kernel<<<dim3((T + kAtQ - 1) / kAtQ, H, ns), kAtThreads, 0, st>>>(B.da, B.q[l], B.P[l], B.dS, B.dk, B.dv, T, H, hd, scale);
       rope_kernel<<<dim3(R, 2), 128, 0, st>>>(B.dq, B.dk, B.cs, B.sn, T, H, hd, -1.f);
       nn({{B.dq, B.dk, B.dv}, {w->wq[l], w->wk[l], w->wv[l]}, {B.dx}, nullptr, 0, 0, 0, 3}, d, d);
-      gain_grad_sq_kernel<<<dim3((d + kGainCols - 1) / kGainCols, ns), 256, 0, st>>>(B.dx, B.Hs[l], B.inv1[l], T, d, slots + (size_t)T_ATTN_NORM * n_slots);
+      gain_grad_sq_kernel<<<dim3(gain_blocks, ns), 256, 0, st>>>(B.dx, B.Hs[l], B.inv1[l], T, d, slots + (size_t)T_ATTN_NORM * n_slots + z0 * gain_blocks);
       rmsnorm_bwd_kernel<WT><<<R, 512, 0, st>>>(B.dx, B.Hs[l], W(w->attn_norm, l), B.inv1[l], dmid, dnext, d);  // d f / d H[l]
       // every factor of the layer's weight gradients is at hand: all its Gram matrices, then the seven dot products
       GramArgs ga{};
@@ -1044,7 +1050,7 @@ cudaError_t run_in(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st,
       for (int i = 0; i < kGrams; ++i) ga.A[i] = src[i];
       ga.d = d; ga.f = f; ga.T = T; ga.plan = gp; ga.G = B.G;
       gram_kernel<<<dim3(gp.pairs, gp.pieces(), ns), kGramThreads, 0, st>>>(ga);
-      gram_dot_kernel<<<dim3(gp.dot_blocks, kDots, ns), 256, 0, st>>>(B.G, gp, slots, n_slots);
+      gram_dot_kernel<<<dim3(gp.dot_blocks, kDots, ns), 256, 0, st>>>(B.G, gp, slots + z0 * gp.dot_blocks, n_slots);
       std::swap(dh, dnext);
     }
     FIT_OK(ge);
@@ -1092,10 +1098,12 @@ cudaError_t run(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st, co
   // (the limits belong to the kernels and not to this call: constants, or calls on other threads would lower them under it)
   for (const void* k : {(const void*)attn_fwd_kernel, (const void*)attn_bwd_q_kernel})
     FIT_OK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem(kFitMaxT)));
-  // as many sequences at a time as fill kFitRows rows; fewer if the device has no room for their activations
-  for (int nb = std::max(1, std::min(n_seq, kFitRows / T));; nb = (nb + 1) / 2) {
-    const GramPlan gp = gram_plan(T, nb, g.d_model, g.d_ffn, n_sm);
-    const int n_slots = nb * std::max((g.d_model + kGainCols - 1) / kGainCols, gp.dot_blocks);
+  // As many sequences at a time as fill kFitRows rows; fewer if the device has no room for their activations.  How sums are
+  // cut and where they are kept follows the full group either way: free memory does not show in the results.
+  const int full = std::max(1, std::min(n_seq, kFitRows / T));
+  const GramPlan gp = gram_plan(T, full, g.d_model, g.d_ffn, n_sm);
+  const int n_slots = full * std::max((g.d_model + kGainCols - 1) / kGainCols, gp.dot_blocks);
+  for (int nb = full;; nb = (nb + 1) / 2) {
     Buffers B;
     Arena A;
     auto lay = [&] {
@@ -1112,7 +1120,7 @@ cudaError_t run(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st, co
     FIT_OK(me);
     A.base = reinterpret_cast<unsigned char*>(p);
     lay();
-    const cudaError_t e = run_in<WT>(g, w, st, tokens, n_seq, seq_len, out_trace, out_fit, B, nb, n_sm, room, gp, n_slots);
+    const cudaError_t e = run_in<WT>(g, w, st, tokens, n_seq, seq_len, out_trace, out_fit, B, nb, full, n_sm, room, gp, n_slots);
     const cudaError_t fe = fit_free(p, A.used, st);
     return e != cudaSuccess ? e : fe;
   }

@@ -140,6 +140,25 @@ def test_fit_scores_give_their_memory_back():
     pkg.sdfp_fit_release()             # nothing left: no error
 
 
+def test_fit_scores_do_not_depend_on_free_memory():
+    """With room for only some of the sequences at a time the scores have the same bits as with room for all: 8 sequences
+    of 64 tokens need 537 MB of logits, half of them fit into what a hold on the rest of the device leaves."""
+    pkg.build_library()
+    shape = si.ModelShape("memory", 3, 64, 1, 64, 336, 1 << 18)
+    w = si.weights_to(si.make_weights(shape, []), "cuda:0")
+    calib = si.make_prompts(shape.vocab, 9, 65, seed=3)  # a full group of eight and one more
+    want = pkg.sdfp_fit_scores(shape, w, calib)
+    pkg.sdfp_fit_release()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (420 << 20), dtype=torch.uint8, device="cuda:0")
+    try:
+        assert pkg.sdfp_fit_scores(shape, w, calib) == want
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+        pkg.sdfp_fit_release()
+
+
 def test_fit_scores_drive_the_draft_mask():
     """Stage A feeding Stage B: the prune set chosen from the GPU scores is handed to
     sdfp_set_draft_layers and the speculative output stays the target's."""
