@@ -209,13 +209,16 @@ struct LinearCall {
   EpiParams ep;
 };
 
-// P pairs per warp: more share the reads of the rows, fewer spread a small matrix over the SMs
+// One pair per warp while the CTAs of that, three on an SM, all run at the same time; beyond that two pairs, which share
+// the reads of the rows.  One row, bf16, us with one pair and with two: lm-head of 8192 (512 CTAs of one pair) d 1024 9.0 and 6.4,
+// d 4096 33.6 and 22.3; QKV of d 2048 (384 CTAs) 14.0 and 15.1; gate/up of d 4096 (1382 CTAs) 95.5 and 80.2.
+// Four pairs took 200 registers, one CTA on an SM, and up to 23 % longer than two.
 template <typename WT>
 cudaError_t launch_linear_fma(sdfp_ctx* c, const LinearCall& lc) {
   const int row_groups = (lc.rows + kFmaRows - 1) / kFmaRows;
-  const long long ctas4 = (long long)((lc.n_pairs + 4 * kFmaWarps - 1) / (4 * kFmaWarps)) * row_groups;
-  const int P = ctas4 >= 2LL * c->num_sms ? 4 : ctas4 >= c->num_sms ? 2 : 1;
-  auto kernel = P == 4 ? linear_fma_kernel<WT, WT, 4> : P == 2 ? linear_fma_kernel<WT, WT, 2> : linear_fma_kernel<WT, WT, 1>;
+  const long long ctas1 = (long long)((lc.n_pairs + kFmaWarps - 1) / kFmaWarps) * row_groups;
+  const int P = ctas1 > 3LL * c->num_sms ? 2 : 1;
+  auto kernel = P == 2 ? linear_fma_kernel<WT, WT, 2> : linear_fma_kernel<WT, WT, 1>;
   const dim3 grid((lc.n_pairs + P * kFmaWarps - 1) / (P * kFmaWarps), row_groups);
   return launch(c, kernel, grid, dim3(kFmaThreads), 0, reinterpret_cast<const WT*>(lc.w), lc.x, lc.ldx, lc.rows, lc.K, lc.n_pairs,
                 lc.gain, c->cfg.rms_eps, lc.ep);

@@ -49,8 +49,28 @@ __device__ __forceinline__ float warp_sum_scatter(float (&v)[N]) {
   return v[0];
 }
 
+// Four weights as they lie in memory.  A load that is converted where it is issued is waited for there: with bf16
+// weights nothing was in flight then, and a wide matrix was slower than with fp32 ones.
+template <typename WT>
+struct Raw4;
+template <>
+struct Raw4<float> {
+  float4 v;
+  __device__ __forceinline__ void load(const float* p, bool in) { v = in ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f); }
+  __device__ __forceinline__ float4 get() const { return v; }
+};
+template <>
+struct Raw4<__nv_bfloat16> {
+  uint2 v;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p, bool in) { v = in ? *reinterpret_cast<const uint2*>(p) : make_uint2(0u, 0u); }
+  __device__ __forceinline__ float4 get() const {
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+  }
+};
+
+// P pairs per warp, 1 or 2.  Registers leave room for three CTAs on an SM with one pair and for two with two.
 template <typename WT, typename KT, int P>
-__global__ void __launch_bounds__(kFmaThreads)
+__global__ void __launch_bounds__(kFmaThreads, 4 - P)
 linear_fma_kernel(const WT* __restrict__ W, const float* __restrict__ X, int ldx, int M, int K, int n_pairs,
                   const float* __restrict__ gain, float eps, EpiParams ep) {
   __shared__ __align__(16) float xs[kFmaRows][kFmaCols];
@@ -64,14 +84,14 @@ linear_fma_kernel(const WT* __restrict__ W, const float* __restrict__ X, int ldx
     wp[j][0] = W + (size_t)min(p0 + j, n_pairs - 1) * 2 * K;
     wp[j][1] = wp[j][0] + K;
   }
-  float4 wq[kFmaAhead][P][2];
+  Raw4<WT> wq[kFmaAhead][P][2];
 #pragma unroll
   for (int a = 0; a < kFmaAhead; ++a) {
     const int k = a * 128 + lane * 4;
 #pragma unroll
     for (int j = 0; j < P; ++j)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) wq[a][j][h] = k < K ? load4(wp[j][h] + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int h = 0; h < 2; ++h) wq[a][j][h].load(wp[j][h] + k, k < K);
   }
   pdl_wait();
   pdl_launch_dependents();
@@ -135,7 +155,7 @@ linear_fma_kernel(const WT* __restrict__ W, const float* __restrict__ X, int ldx
 #pragma unroll
       for (int j = 0; j < P; ++j)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) w[j][h] = wq[0][j][h];
+        for (int h = 0; h < 2; ++h) w[j][h] = wq[0][j][h].get();
 #pragma unroll
       for (int a = 0; a + 1 < kFmaAhead; ++a)
 #pragma unroll
@@ -146,7 +166,7 @@ linear_fma_kernel(const WT* __restrict__ W, const float* __restrict__ X, int ldx
 #pragma unroll
       for (int j = 0; j < P; ++j)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) wq[kFmaAhead - 1][j][h] = kn < K ? load4(wp[j][h] + kn) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int h = 0; h < 2; ++h) wq[kFmaAhead - 1][j][h].load(wp[j][h] + kn, kn < K);
 #pragma unroll
       for (int i = 0; i < kFmaRows; ++i) {
         if (i < rows) {

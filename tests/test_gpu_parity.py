@@ -903,8 +903,9 @@ def test_prompt_passes_of_a_batch_equal_solo_runs(batch, prompt_len, dtype):
 @pytest.mark.parametrize("d_heads,ffn,vocab,rows,flags", [
     (1, 16, 16, 9, 0),           # fewer columns than one step of a warp, fewer pairs than warps; a second row group of one
     (9, 1040, 528, 16, 0),       # 1040 columns: more than are staged at a time, by one step's remainder
-    (18, 2064, 1040, 80, 0),     # rows that do not fit the staged columns under a norm (d 1152); the widest pass, four pairs per warp
-    (5, 336, 208, 5, "fma"),     # bf16 weights on the same kernel
+    (18, 2064, 1040, 80, 0),     # rows that do not fit the staged columns under a norm (d 1152); the widest pass, two pairs per warp
+    (5, 336, 208, 5, "fma"),     # bf16 weights on the same kernel, one pair per warp
+    (18, 2064, 1040, 80, "fma"), # ... and two
 ])
 def test_fma_linear_at_the_edges(d_heads, ffn, vocab, rows, flags):
     """Logits of the fp32 linear kernel at its column, pair and row remainders against the oracle (fp32 sums: 1e-4, bf16
