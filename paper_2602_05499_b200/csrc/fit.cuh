@@ -552,9 +552,6 @@ __global__ void swiglu_bwd_kernel(const float* __restrict__ du, const float* __r
     dup[i] = du[i] * g * sg;
   }
 }
-__global__ void add_kernel(float* __restrict__ dst, const float* __restrict__ a, const float* __restrict__ b, size_t n) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) dst[i] = a[i] + b[i];
-}
 
 // Mean next-token cross-entropy: dlogits[t,:] = (softmax(logits[t,:]) - onehot(target_t)) / T, in place; loss[t] kept
 __global__ void __launch_bounds__(1024) ce_bwd_kernel(float* __restrict__ logits, const int* __restrict__ tok, int V, int T,
