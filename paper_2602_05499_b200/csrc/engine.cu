@@ -498,11 +498,12 @@ cudaError_t configure_pass_t(sdfp_ctx* c, int max_smem_optin) {
 }
 
 // Whether a pass hands its activations on as fragment images.  More than eight rows: always, the loads and
-// splits of two column groups are what bounds the loop otherwise (d 4096, 12 layers, 16 rows: 2170 -> 1746 us, with the larger staging area).
-// Up to eight rows the loop of a large matrix waits for its weights either way and the images only
-// lengthen the epilogue (d 4096, one row: 1192 -> 1206 us); a small one is bound by latency and gains (d 2048, 6
-// layers, one row: 343 -> 326 us).  The results have the same bits.
-bool pass_images(const sdfp_ctx* c, int rows) { return rows > 8 || c->cfg.d_model <= 3072; }
+// splits of two column groups are what bounds the loop otherwise (d 4096, 12 layers, 16 rows: 2130 -> 1746 us, with the
+// larger staging area).  Up to eight rows the loop of a large matrix waits for its weights either way and the images only
+// lengthen the epilogue; a small one is bound by latency and gains.  6 layers, vocabulary 8192, one / eight rows, images against
+// fp32 rows: d 1024 218 / 264 and 227 / 278 us, d 2048 294 / 348 and 303 / 366, d 2560 349 / 407 and 354 / 421; d 2816 381 / 442 and
+// 380 / 450, d 3072 410 / 477 and 401 / 474, d 3200 426 / 493 and 421 / 493, d 4096 562 / 655 and 562 / 645.  The results have the same bits.
+bool pass_images(const sdfp_ctx* c, int rows) { return rows > 8 || c->cfg.d_model <= 2688; }
 
 // what the embedding kernel leaves for the whole-pass kernel's first stage
 EmbedImage pass_embed_image(const sdfp_ctx* c, bool draft, int rows) {
