@@ -10,7 +10,7 @@
 // previous kernel's end to this one's (the weights of the first steps are therefore asked for before
 // the wait), at many rows the FMAs.  When every warp read the rows from L2 itself and re-read its weights for
 // every eight rows, that traffic cost more than either: speculative decoding of 16 sequences, 6 layers d 768,
-// FFN 2352, vocabulary 8192, k = 4: 147 -> 24.5 ms; of one, 4 layers d 256: 10.0 -> 6.7 ms.
+// FFN 2352, vocabulary 8192, k = 4: 147 -> 24.5 ms; of one, 4 layers d 256: 10.5 -> 7.0 ms.
 // A row's result does not depend on how many rows the launch carries or on P: every (row, feature) runs
 // the same additions in the same order.
 #pragma once

@@ -18,8 +18,8 @@
 //     What a stage boundary costs is its chain of dependent steps, not its bytes; those that need no
 //     other CTA are kept off it: the next stage's descriptor and share are fetched during the running
 //     stage, ring positions run on from stage to stage, one barrier carries "all agree", a row's squares are
-//     added by a warp (pass of one row, 4 layers d 256 123 -> 117 us, 6 layers d 2048 313 -> 306, 12 layers
-//     d 4096 1164 -> 1157, five rows 1281 -> 1267).
+//     added by a warp (pass of one row, 4 layers d 256 121 -> 115 us, 6 layers d 2048 312 -> 302, 12 layers
+//     d 4096 1164 -> 1155, five rows 1287 -> 1271).
 //
 // Weight layout ("unit" layout, written by pack_units_kernel): a matrix with NT 16-row tiles and
 // KT 16-column tiles is stored as units of 8 row tiles at one k-tile, 4096 contiguous bytes,
@@ -336,7 +336,7 @@ __device__ __forceinline__ void unit_range(long long n_units, int cta, int n_cta
 // other.  With two units and more per class of every CTA the even cut wins: the pieces are few and all CTAs
 // stream (O-projection at d 3328, 36 units per CTA, as 5 pieces per group: 3 us longer at five rows).  A small
 // matrix cut evenly leaves a unit or a few per CTA and up to sixteen pieces per group, most of the
-// stage's time: pass of one row, 4 layers, d 256, FFN 688, vocabulary 2048: 246 -> 127 us; d 1024, FFN 2816: 196 -> 160.
+// stage's time: pass of one row, 4 layers, d 256, FFN 688, vocabulary 2048: 246 -> 127 us; d 1024, FFN 2816: 196 -> 163.
 inline int stage_split(int n_groups, int KT, int grid) {
   constexpr float kUnit = 0.14f, kPost = 2.0f, kPiece = 0.7f;
   const float even = (float)n_groups * KT / grid;
@@ -733,7 +733,6 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const StageDe
         for (int e = 0; e < 4; ++e) acc[r][cg][e] = 0.f;
 
     bool warp_ok = true;
-    int kt = seg_kt0 + (cls + kChunkUnits * i - seg_begin);  // k-tile of my next unit while it lies in this segment
     while (warp_ok && i < my_n && cls + kChunkUnits * i < seg_end) {
       // Lanes leave the polling loop at different times.  mma.sync needs the whole warp
       // converged, so the vote below is both the warp-uniform outcome and the reconvergence point.
@@ -777,7 +776,6 @@ __device__ void linear_stage(const PassParams& pp, PassShared* sh, const StageDe
       x1 = x2;
       prefetch(x2, i + 3);
       ++i;
-      kt += kChunkUnits;
     }
 
     // ---- end of the segment: add the class partials, then finish the group or post ----
@@ -1276,7 +1274,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) pass_kernel(PassParams pp, in
         linear_stage<CG, HD, X_PLAIN, IMG>(pp, sh, st, share, ring, n_slots, work, ring_slot, ring_parity, serial);
       } else {
         // fold the attention partials into shared memory first if the columns this CTA's units
-        // use fit beside the other work buffers (they do for passes of a few rows)
+        // use fit beside the other work buffers (one column group: 6 rows at d 4096, 4 at d 5120; two: all 16)
         const int kts = min(share.n, st.KT);
         const size_t need = (size_t)pp.M * staged_row_words(kts) * sizeof(uint32_t);
         if (need <= pass_work_bytes<CG, HD>() - (size_t)work_sc_off<CG>())
