@@ -841,11 +841,14 @@ inline cudaError_t fit_alloc(void** p, size_t bytes, int dev, cudaStream_t st) {
   }
   return e;
 }
-// after whatever is still running on the buffer; on return the memory is the pool's or the device's again
+// behind whatever is still running on the buffer, and waited for: on return the results are there and the memory is the
+// pool's or the device's again
 inline cudaError_t fit_free(void* p, size_t bytes, cudaStream_t st) {
-  if (bytes > kFitPoolKeep) return cudaFree(p);
-  const cudaError_t e = cudaFreeAsync(p, st);
-  return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+  const bool pooled = bytes <= kFitPoolKeep;
+  const cudaError_t pe = pooled ? cudaFreeAsync(p, st) : cudaSuccess;
+  const cudaError_t se = cudaStreamSynchronize(st);
+  const cudaError_t fe = pooled ? pe : cudaFree(p);
+  return se != cudaSuccess ? se : fe;
 }
 
 // One device allocation per call, cut into buffers: the layout runs once to learn the size and once
@@ -979,8 +982,7 @@ cudaError_t fit_gemm_launch(const GemmArgs& g, int plan_rows, const GemmRoom& ro
 
 template <typename WT>
 cudaError_t run_in(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st, const int32_t* tokens, int n_seq, int seq_len,
-                   double* out_trace, double* out_fit, Buffers& B, int nb, int full, int n_sm, const GemmRoom& room, const GramPlan& gp,
-                   int n_slots) {
+                   std::vector<double>& sums, Buffers& B, int nb, int full, int n_sm, const GemmRoom& room, const GramPlan& gp, int n_slots) {
   const int L = g.n_layers, d = g.d_model, f = g.d_ffn, V = g.vocab, H = g.n_heads, hd = g.head_dim, T = seq_len - 1;
   const float scale = 1.0f / std::sqrt((float)hd);
   FIT_OK(cudaMemsetAsync(B.slots, 0, (size_t)L * kTensors * n_slots * sizeof(double), st));
@@ -1065,21 +1067,7 @@ cudaError_t run_in(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st,
   }
   finish_kernel<<<L * kTensors, 256, 0, st>>>(B.slots, n_slots, B.ms_part, B.out);
   FIT_OK(cudaGetLastError());
-  std::vector<double> h((size_t)L * kTensors * 2);  // per (layer, tensor): sum over the sequences of the squared norm, sum of theta^2
-  FIT_OK(cudaMemcpyAsync(h.data(), B.out, h.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-  FIT_OK(cudaStreamSynchronize(st));
-  for (int l = 0; l < L; ++l) {
-    double tr = 0.0, ft = 0.0;
-    for (int t = 0; t < kTensors; ++t) {
-      const double n = t < T_GATE ? (double)d * d : t < T_ATTN_NORM ? (double)f * d : (double)d;
-      const double Tt = h[((size_t)l * kTensors + t) * 2] / n_seq;
-      tr += Tt;
-      ft += Tt * (h[((size_t)l * kTensors + t) * 2 + 1] / n);
-    }
-    out_trace[l] = tr;
-    if (out_fit) out_fit[l] = ft;
-  }
-  return cudaSuccess;
+  return cudaMemcpyAsync(sums.data(), B.out, sums.size() * sizeof(double), cudaMemcpyDeviceToHost, st);
 }
 
 template <typename WT>
@@ -1118,9 +1106,24 @@ cudaError_t run(const sdfp_config& g, const sdfp_weights* w, cudaStream_t st, co
     FIT_OK(me);
     A.base = reinterpret_cast<unsigned char*>(p);
     lay();
-    const cudaError_t e = run_in<WT>(g, w, st, tokens, n_seq, seq_len, out_trace, out_fit, B, nb, full, n_sm, room, gp, n_slots);
+    const int L = g.n_layers;
+    std::vector<double> sums((size_t)L * kTensors * 2);  // per (layer, tensor): sum over the sequences of the squared norm, sum of theta^2
+    const cudaError_t e = run_in<WT>(g, w, st, tokens, n_seq, seq_len, sums, B, nb, full, n_sm, room, gp, n_slots);
     const cudaError_t fe = fit_free(p, A.used, st);
-    return e != cudaSuccess ? e : fe;
+    if (e != cudaSuccess || fe != cudaSuccess) return e != cudaSuccess ? e : fe;
+    const double d = g.d_model, f = g.d_ffn;
+    for (int l = 0; l < L; ++l) {
+      double tr = 0.0, ft = 0.0;
+      for (int t = 0; t < kTensors; ++t) {
+        const double n = t < T_GATE ? d * d : t < T_ATTN_NORM ? f * d : d;
+        const double Tt = sums[((size_t)l * kTensors + t) * 2] / n_seq;
+        tr += Tt;
+        ft += Tt * (sums[((size_t)l * kTensors + t) * 2 + 1] / n);
+      }
+      out_trace[l] = tr;
+      if (out_fit) out_fit[l] = ft;
+    }
+    return cudaSuccess;
   }
 }
 #undef FIT_OK
