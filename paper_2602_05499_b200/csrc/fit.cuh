@@ -787,7 +787,7 @@ constexpr int kFitRows = 512;  // calibration tokens that go through the stack t
 // tokens: 1.07 ms from the pool, 1.82 without; 4 layers d 4096, 2 x 64 tokens, 200 MB: 12.7 and 14.3).  The pool keeps what it has
 // handed out, at most kFitPoolKeep bytes, until sdfp_fit_release, until a context is destroyed or until one runs
 // out of memory.  A larger working set is allocated and freed by the call itself: the call takes tens
-// of milliseconds, and mapping that much through the pool costs more than cudaMalloc (1.2 GB: 17.8 and 7.7 ms a call).
+// of milliseconds, and mapping that much through the pool costs more than cudaMalloc (0.9 GB: 17.8 and 7.7 ms a call).
 constexpr unsigned long long kFitPoolKeep = 256ull << 20;
 constexpr int kFitPools = 64;
 struct FitPools {
