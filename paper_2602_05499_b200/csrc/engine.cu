@@ -22,6 +22,7 @@
 
 #include "../../include/sdfp.h"
 #include "attention.cuh"
+#include "cluster_pass.cuh"
 #include "common.cuh"
 #include "dense_attention.cuh"
 #include "fit.cuh"
@@ -47,6 +48,8 @@ struct LayerWeights {
   void* down = nullptr;  // packed [d, f]
   // the same matrices as tcgen05 operand images (dense path), null when that path is off
   void *um_qkv = nullptr, *um_wo = nullptr, *um_gu = nullptr, *um_down = nullptr;
+  // ... and in the layout of the cluster kernel (small decoders), null when that path is off
+  void *cl_qkv = nullptr, *cl_wo = nullptr, *cl_gu = nullptr, *cl_down = nullptr;
   float* attn_gain = nullptr;
   float* ffn_gain = nullptr;
 };
@@ -115,6 +118,14 @@ struct sdfp_ctx {
   int pass_slots[3] = {0, 0, 0};  // ring slots of the instantiation with 1 and with 2 column groups
   size_t pass_smem[3] = {0, 0, 0};  // dynamic shared memory of the instantiations with 1 and with 2 column groups
   int pass_grid = 0;
+  // small decoders: the passes of rounds, and whole greedy generations, inside one cluster (cluster_pass.cuh)
+  bool use_cluster = false;
+  ClLayout cl{};
+  ClStage *cl_prog_t = nullptr, *cl_prog_d = nullptr;  // device: the linear stages of the target and of the draft
+  int n_cl_t = 0, n_cl_d = 0;
+  int cl_first_t = 0, cl_first_d = 0;  // the norm their first stage reads the embedding through
+  void* cl_lm_head = nullptr;
+  float* cl_gains = nullptr;         // [2 n_layers + 1][d_model]
   // dense path on tcgen05 (bf16 tensor path): the prompt pass of every context, and every pass of
   // a context whose widest pass does not fit the whole-pass kernel
   bool use_dense = false;
@@ -442,7 +453,57 @@ int build_program(sdfp_ctx* c, bool draft, StageDesc** dev, StageShare** dev_sha
   return 0;
 }
 
+// The same for the cluster kernel.
+int build_cluster_program(sdfp_ctx* c, bool draft, ClStage** dev, int* n_all, int* first_gain) {
+  const sdfp_config& g = c->cfg;
+  const int d = g.d_model, f = g.d_ffn;
+  const KvCache& kv = (draft && !c->share_kv) ? c->cache_d : c->cache_t;
+  std::vector<ClStage> prog;
+  int resid = -1;  // the last stage that wrote the residual stream: it also leaves gain * h for the next norm
+  auto norm_gain = [&](int gain) {
+    if (resid >= 0)
+      prog[resid].gain_out = gain;
+    else
+      *first_gain = gain;
+  };
+  auto add = [&](const void* w, int kind, int n_pairs, int K, void* kc, void* vc) {
+    prog.push_back(ClStage{reinterpret_cast<const unsigned char*>(w), kc, vc, kind, n_pairs, K, 0, 0});
+  };
+  for (int l = 0; l < g.n_layers; ++l) {
+    const LayerWeights& lw = c->layers[l];
+    if (!draft || c->keep_attn[l]) {
+      norm_gain(2 * l);
+      add(lw.cl_qkv, CL_QKV, 3 * d / 2, d, kv.k[l], kv.v[l]);
+      add(lw.cl_wo, CL_O, d / 2, d, nullptr, nullptr);
+      resid = (int)prog.size() - 1;
+    }
+    if (!draft || c->keep_ffn[l]) {
+      norm_gain(2 * l + 1);
+      add(lw.cl_gu, CL_GATE_UP, f, d, nullptr, nullptr);
+      add(lw.cl_down, CL_DOWN, d / 2, f, nullptr, nullptr);
+      resid = (int)prog.size() - 1;
+    }
+  }
+  norm_gain(2 * g.n_layers);
+  add(c->cl_lm_head, CL_HEAD, g.vocab / 2, d, nullptr, nullptr);
+  for (size_t i = prog.size() - 1; i > 0; --i)
+    if (prog[i - 1].kind == CL_O) {
+      prog[i].after_kv = 1;
+      break;
+    }
+  if (*dev == nullptr)
+    if (int r = dev_alloc(c, dev, (size_t)4 * g.n_layers + 1)) return r;
+  CU_OK(c, cudaMemcpyAsync(*dev, prog.data(), prog.size() * sizeof(ClStage), cudaMemcpyHostToDevice, c->stream));
+  CU_OK(c, cudaStreamSynchronize(c->stream));  // prog is a local
+  *n_all = (int)prog.size();
+  return 0;
+}
+
 int build_programs(sdfp_ctx* c) {
+  if (c->use_cluster) {
+    if (int r = build_cluster_program(c, false, &c->cl_prog_t, &c->n_cl_t, &c->cl_first_t)) return r;
+    if (int r = build_cluster_program(c, true, &c->cl_prog_d, &c->n_cl_d, &c->cl_first_d)) return r;
+  }
   if (!c->use_pass) return 0;
   if (int r = build_program(c, false, &c->prog_t, &c->shares_t, &c->n_prog_t)) return r;
   return build_program(c, true, &c->prog_d, &c->shares_d, &c->n_prog_d);
@@ -563,6 +624,104 @@ cudaError_t run_pass(sdfp_ctx* c, bool draft, int rows, int rows_per_seq, bool w
   return hd128 ? launch_pass_t<2, 128, true>(c, pp) : launch_pass_t<2, 64, true>(c, pp);
 }
 
+// ---- the cluster kernel (rounds of small decoders) -----------------------------------------------
+
+using ClKernel = void (*)(const ClParams);
+ClKernel cluster_kernel(const sdfp_config& g) {
+  if (g.dtype == SDFP_BF16) return g.head_dim == 128 ? cluster_pass_kernel<__nv_bfloat16, 128> : cluster_pass_kernel<__nv_bfloat16, 64>;
+  return g.head_dim == 128 ? cluster_pass_kernel<float, 128> : cluster_pass_kernel<float, 64>;
+}
+
+cudaLaunchConfig_t cluster_launch_config(const sdfp_ctx* c, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(kClCtas);
+  lc.blockDim = dim3(kClThreads);
+  lc.dynamicSmemBytes = (size_t)c->cl.total;
+  lc.stream = c->stream;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = kClCtas;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  lc.attrs = attr;
+  lc.numAttrs = 1;
+  return lc;
+}
+
+// Whether the rounds of a context run in the cluster kernel, and with which layout.  Sixteen SMs do the arithmetic of a
+// pass, so the line lies where that takes as long as the stage boundaries it saves: bytes of a layer times sequences.  One
+// call of 40 + 32 tokens, 4 layers, FFN 2.7 d, vocabulary 4096, time on the other path over time here:
+//   bf16, draft length 2 to 8, one sequence: d 256 1.8, d 384 1.4, d 512 (6.3 MB) 1.25 to 1.3, d 640 0.97; two sequences
+//     d 256 1.4, d 320 (5 MB) 1.05 to 1.15, d 384 1.0 to 1.08; three, k = 4, d 256 (4.7 MB) 1.16, d 320 0.88; four, k = 2, d 256 (6.3 MB) 1.11
+//   fp32, the same: d 256 1.24 to 1.37, d 320 (5 MB) 1.06 to 1.19, d 384 0.97 to 1.08; two sequences, d 256 (6.3 MB) 0.92 to 1.02
+//   autoregressive (k_max 0), bf16: one sequence d 256 2.6, d 512 2.0, d 640 1.46, d 768 (14 MB) 1.15; two d 512 (12.6 MB) 1.46, d 640 0.92;
+//     eight d 256 (12.6 MB) 1.16, d 320 0.92; fp32: one d 256 2.0, d 512 (12.6 MB) 1.10; two d 384 (14 MB) 1.15; four d 256 (12.6 MB) 1.23
+bool cluster_wanted(sdfp_ctx* c, int widest) {
+  const sdfp_config& g = c->cfg;
+  if ((g.flags & SDFP_FLAG_NO_PASS_KERNEL) || (c->bf16 && !c->use_mma)) return false;
+  // every CTA has a share of every stage a layer is made of: the exchange between the stages relies on it
+  if (g.d_model < 8 * kClCtas || g.d_ffn < 4 * kClCtas || widest > kClMaxRows) return false;
+  const double layer_bytes = (4.0 * g.d_model * g.d_model + 3.0 * g.d_model * g.d_ffn) * (double)c->esz;
+  if (layer_bytes * g.max_batch > (g.k_max == 0 ? 13e6 : c->bf16 ? 6.4e6 : 5.2e6)) return false;
+  for (int rows = kClMaxRows; rows >= widest && c->cl.total <= 0; --rows)
+    c->cl = cluster_layout(g.d_model, g.d_ffn, g.n_heads, g.head_dim, g.n_layers, rows, g.max_seq, c->max_smem_optin);
+  if (c->cl.total <= 0) return false;
+  const ClKernel kernel = cluster_kernel(g);
+  int clusters = 0;
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t lc = cluster_launch_config(c, &attr);
+  const bool fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, c->max_smem_optin) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&clusters, kernel, &lc) == cudaSuccess && clusters >= 1;
+  cudaGetLastError();
+  return fits;
+}
+
+ClParams cluster_params(const sdfp_ctx* c) {
+  const sdfp_config& g = c->cfg;
+  ClParams p{};
+  p.prog_t = c->cl_prog_t;
+  p.prog_d = c->cl_prog_d;
+  p.n_t = c->n_cl_t;
+  p.n_d = c->n_cl_d;
+  p.first_gain_t = c->cl_first_t;
+  p.first_gain_d = c->cl_first_d;
+  p.gains = c->cl_gains;
+  p.n_gains = 2 * g.n_layers + 1;
+  p.d = g.d_model;
+  p.f = g.d_ffn;
+  p.heads = g.n_heads;
+  p.vocab = g.vocab;
+  p.max_seq = g.max_seq;
+  p.eps = g.rms_eps;
+  p.scale = 1.0f / std::sqrt((float)g.head_dim);
+  p.rope_cos = c->rope_cos;
+  p.rope_sin = c->rope_sin;
+  p.embed = c->embed;
+  p.lay = c->cl;
+  p.logits = c->logits;
+  p.gs = c->gs;
+  p.seq_tok = c->seq_tok;
+  p.draft_tok = c->draft_tok;
+  p.out_tok = c->out_tok;
+  p.stats = c->stats;
+  p.sync = c->psync;
+  return p;
+}
+
+cudaError_t launch_cluster(sdfp_ctx* c, const ClParams& p) {
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t lc = cluster_launch_config(c, &attr);
+  c->launches += 1;
+  return cudaLaunchKernelEx(&lc, cluster_kernel(c->cfg), p);
+}
+
+// One pass of a sampled round, to its logits
+cudaError_t run_cluster_pass(sdfp_ctx* c, const PassDesc& pd, bool draft) {
+  ClParams p = cluster_params(c);
+  p.pd = pd;
+  p.draft = draft ? 1 : 0;
+  return launch_cluster(c, p);
+}
+
 // ---- one forward pass ------------------------------------------------------------------
 
 // Rows of short prompts (at most one row block each) that share a sweep of the weights: beyond eight row
@@ -580,12 +739,28 @@ int enqueue_dense_pass(sdfp_ctx* c, const PassDesc& pd, bool draft, int rows, in
 
 enum Decide { DECIDE_NONE = 0, DECIDE_LOGITS = 1, DECIDE_ARGMAX = 2, DECIDE_SAMPLE_DRAFT = 3 };
 
+// the token decision on the logits of a pass
+int enqueue_decision(sdfp_ctx* c, const PassDesc& pd, int rows, int decide) {
+  if (decide == DECIDE_ARGMAX)
+    CU_OK(c, launch(c, argmax_kernel, dim3(rows), dim3(kArgmaxThreads), 0, (const float*)c->logits, c->cfg.vocab, pd, c->draft_tok,
+                    c->tgt_tok, c->row_argmax));
+  else if (decide == DECIDE_SAMPLE_DRAFT)
+    CU_OK(c, launch(c, sample_draft_kernel, dim3(rows), dim3(kSampleThreads), 0, (const float*)c->logits, c->cfg.vocab, pd,
+                    (const GenState*)c->gs, c->draft_tok, c->qprob, c->qsum));
+  return 0;
+}
+
 // rows: total rows; rows_per_seq for the attention grouping; n_chunks bounds the context.
 int enqueue_pass(sdfp_ctx* c, const PassDesc& pd, bool draft, int rows, int attn_rows_per_seq, int n_chunks,
                  int decide) {
   const sdfp_config& g = c->cfg;
   const int d = g.d_model, f = g.d_ffn;
   if (c->dense_decode) return enqueue_dense_pass(c, pd, draft, rows, attn_rows_per_seq, n_chunks, decide);
+  if (c->use_cluster && pd.kind != PASS_TOKENS && pd.kind != PASS_PROMPT) {  // a pass of a round
+    if (rows > c->cl.rows) return fail(c, SDFP_ESTATE, "a pass of %d rows reached the cluster kernel", rows);
+    CU_OK(c, run_cluster_pass(c, pd, draft));
+    return enqueue_decision(c, pd, rows, decide);
+  }
   if (c->bf16)
     CU_OK(c, launch(c, plan_embed_kernel<__nv_bfloat16>, dim3(rows), dim3(128), 0, pd, (const GenState*)c->gs,
                     (const int*)c->seq_tok, g.max_seq, (const int*)c->draft_tok, c->plan,
@@ -629,13 +804,7 @@ int enqueue_pass(sdfp_ctx* c, const PassDesc& pd, bool draft, int rows, int attn
     LinearCall lc{c->lm_head, c->h, d, rows, d, g.vocab / 2, c->final_gain, base_epi(c, EPI_LOGITS, c->logits, g.vocab)};
     CU_OK(c, run_linear(c, lc));
   }
-  if (decide == DECIDE_ARGMAX)
-    CU_OK(c, launch(c, argmax_kernel, dim3(rows), dim3(kArgmaxThreads), 0, (const float*)c->logits, g.vocab, pd,
-                    c->draft_tok, c->tgt_tok, c->row_argmax));
-  else if (decide == DECIDE_SAMPLE_DRAFT)
-    CU_OK(c, launch(c, sample_draft_kernel, dim3(rows), dim3(kSampleThreads), 0, (const float*)c->logits, g.vocab, pd,
-                    (const GenState*)c->gs, c->draft_tok, c->qprob, c->qsum));
-  return 0;
+  return enqueue_decision(c, pd, rows, decide);
 }
 
 // One forward pass of a context that decodes on the dense path: every linear layer is one launch of
@@ -709,19 +878,13 @@ int enqueue_dense_pass(sdfp_ctx* c, const PassDesc& pd, bool draft, int rows, in
   UmmaParams lm = dense_params(c, c->um_lm_head, c->um_xh, rows, RB, KBd, g.vocab / 2, base_epi(c, EPI_LOGITS, c->logits, g.vocab));
   normed(lm);
   CU_OK(c, launch_dense(c, lm));
-  if (decide == DECIDE_ARGMAX)
-    CU_OK(c, launch(c, argmax_kernel, dim3(rows), dim3(kArgmaxThreads), 0, (const float*)c->logits, g.vocab, pd, c->draft_tok,
-                    c->tgt_tok, c->row_argmax));
-  else if (decide == DECIDE_SAMPLE_DRAFT)
-    CU_OK(c, launch(c, sample_draft_kernel, dim3(rows), dim3(kSampleThreads), 0, (const float*)c->logits, g.vocab, pd,
-                    (const GenState*)c->gs, c->draft_tok, c->qprob, c->qsum));
-  return 0;
+  return enqueue_decision(c, pd, rows, decide);
 }
 
 int enqueue_round(sdfp_ctx* c, int k, int batch, bool sampled, int n_chunks) {
   PassDesc pd{};
   pd.n_seq = batch;
-  const bool fused = c->use_pass && !sampled;  // the lm-head leaves argmax partials; consumers finish them
+  const bool fused = c->use_pass && !c->use_cluster && !sampled;  // the lm-head leaves argmax partials; consumers finish them
   if (fused) {
     pd.amax_part = c->amax_part;
     pd.amax_groups = c->amax_groups;
@@ -748,7 +911,7 @@ int enqueue_round(sdfp_ctx* c, int k, int batch, bool sampled, int n_chunks) {
   pd.rows_per_seq = k + 1;
   if (int r = enqueue_pass(c, pd, false, (k + 1) * batch, k + 1, n_chunks, sampled ? DECIDE_LOGITS : DECIDE_ARGMAX))
     return r;
-  const int* pass_err = c->use_pass ? &c->psync->error : nullptr;
+  const int* pass_err = c->psync ? &c->psync->error : nullptr;
   if (sampled)
     CU_OK(c, launch(c, accept_sampled_kernel, dim3(1), dim3(kSampleThreads), 0, c->gs, (const float*)c->logits,
                     c->cfg.vocab, (const int*)c->draft_tok, (const float*)c->qprob, (const double*)c->qsum, c->seq_tok,
@@ -777,7 +940,7 @@ int pack_dense_image(sdfp_ctx* c, void** dst, PackSrc ps, int n_pairs, int K) {
 // kernels, `img` (may be null) for the dense path.  A context whose decode passes run on the dense
 // path reads only images: `dst` then points to the image as well.
 template <typename WT>
-int pack_matrix(sdfp_ctx* c, void** dst, void** img, PackSrc ps, int n_pairs, int K) {
+int pack_matrix(sdfp_ctx* c, void** dst, void** img, void** cl, PackSrc ps, int n_pairs, int K) {
   if (c->use_dense && img) {
     if (int r = pack_dense_image(c, img, ps, n_pairs, K)) return r;
     if (c->dense_decode) {
@@ -796,6 +959,12 @@ int pack_matrix(sdfp_ctx* c, void** dst, void** img, PackSrc ps, int n_pairs, in
   }
   CU_OK(c, cudaGetLastError());
   *dst = p;
+  if (c->use_cluster) {
+    if (int r = dev_alloc(c, &p, (size_t)n_pairs * 2 * cl_steps(K, sizeof(WT)) * ClElem<WT>::kStep)) return r;
+    pack_cluster_kernel<WT><<<1184, 256, 0, c->stream>>>(p, ps, n_pairs, K);
+    CU_OK(c, cudaGetLastError());
+    *cl = p;
+  }
   return 0;
 }
 
@@ -817,18 +986,25 @@ int load_weights(sdfp_ctx* c, const sdfp_weights* w) {
     if (!w->wq[l] || !w->wk[l] || !w->wv[l] || !w->wo[l] || !w->w_gate[l] || !w->w_up[l] || !w->w_down[l] ||
         !w->attn_norm[l] || !w->ffn_norm[l])
       return fail(c, SDFP_EINVAL, "layer %d has a NULL weight pointer", l);
-    if (int r = pack_matrix<WT>(c, &lw.qkv, &lw.um_qkv, PackSrc{w->wq[l], w->wk[l], w->wv[l], 0, H, hd}, 3 * d / 2, d)) return r;
-    if (int r = pack_matrix<WT>(c, &lw.wo, &lw.um_wo, PackSrc{w->wo[l], nullptr, nullptr, 2, H, hd}, d / 2, d)) return r;
-    if (int r = pack_matrix<WT>(c, &lw.gu, &lw.um_gu, PackSrc{w->w_gate[l], w->w_up[l], nullptr, 1, H, hd}, f, d)) return r;
-    if (int r = pack_matrix<WT>(c, &lw.down, &lw.um_down, PackSrc{w->w_down[l], nullptr, nullptr, 2, H, hd}, d / 2, f)) return r;
+    if (int r = pack_matrix<WT>(c, &lw.qkv, &lw.um_qkv, &lw.cl_qkv, PackSrc{w->wq[l], w->wk[l], w->wv[l], 0, H, hd}, 3 * d / 2, d)) return r;
+    if (int r = pack_matrix<WT>(c, &lw.wo, &lw.um_wo, &lw.cl_wo, PackSrc{w->wo[l], nullptr, nullptr, 2, H, hd}, d / 2, d)) return r;
+    if (int r = pack_matrix<WT>(c, &lw.gu, &lw.um_gu, &lw.cl_gu, PackSrc{w->w_gate[l], w->w_up[l], nullptr, 1, H, hd}, f, d)) return r;
+    if (int r = pack_matrix<WT>(c, &lw.down, &lw.um_down, &lw.cl_down, PackSrc{w->w_down[l], nullptr, nullptr, 2, H, hd}, d / 2, f)) return r;
     if (int r = widen_gain<WT>(c, &lw.attn_gain, w->attn_norm[l], d)) return r;
     if (int r = widen_gain<WT>(c, &lw.ffn_gain, w->ffn_norm[l], d)) return r;
   }
   // the prompt pass needs no logits: only contexts that decode on the dense path get an lm-head image
-  if (int r = pack_matrix<WT>(c, &c->lm_head, c->dense_decode ? &c->um_lm_head : nullptr,
+  if (int r = pack_matrix<WT>(c, &c->lm_head, c->dense_decode ? &c->um_lm_head : nullptr, &c->cl_lm_head,
                               PackSrc{w->lm_head, nullptr, nullptr, 2, H, hd}, g.vocab / 2, d))
     return r;
   if (int r = widen_gain<WT>(c, &c->final_gain, w->final_norm, d)) return r;
+  if (c->use_cluster) {
+    if (int r = dev_alloc(c, &c->cl_gains, (size_t)(2 * g.n_layers + 1) * d)) return r;
+    for (int i = 0; i <= 2 * g.n_layers; ++i) {
+      const float* src = i == 2 * g.n_layers ? c->final_gain : i & 1 ? c->layers[i / 2].ffn_gain : c->layers[i / 2].attn_gain;
+      CU_OK(c, cudaMemcpyAsync(c->cl_gains + (size_t)i * d, src, (size_t)d * 4, cudaMemcpyDeviceToDevice, c->stream));
+    }
+  }
   WT* e = nullptr;
   if (int r = dev_alloc(c, &e, (size_t)g.vocab * d)) return r;
   CU_OK(c, cudaMemcpyAsync(e, w->tok_embed, (size_t)g.vocab * d * sizeof(WT), cudaMemcpyDeviceToDevice, c->stream));
@@ -969,6 +1145,7 @@ extern "C" int sdfp_create(const sdfp_config* cfg, const sdfp_weights* w, void* 
   c->max_smem_optin = optin;
   c->use_dense = c->use_mma && !(g.flags & SDFP_FLAG_NO_DENSE);
   c->dense_decode = c->use_dense && !c->use_pass && !(g.flags & SDFP_FLAG_NO_PASS_KERNEL);
+  c->use_cluster = !c->dense_decode && cluster_wanted(c, widest);
   if (c->use_dense) {
     c->prompt_rows = std::min((int)kPromptRows, g.max_batch * std::min((int)kGroupedPrompt, g.max_seq));
     c->rows_cap = std::max(std::max((int)kMaxRows, g.max_seq), c->prompt_rows);
@@ -1070,15 +1247,16 @@ extern "C" int sdfp_create(const sdfp_config* cfg, const sdfp_weights* w, void* 
         return bail(r);
     }
   }
+  if (c->use_pass || c->use_cluster)
+    if ((r = dev_alloc(c, &c->psync, 1, true))) return bail(r);
   if (c->use_pass) {
-    if ((r = dev_alloc(c, &c->psync, 1, true)) ||
-        (r = dev_alloc(c, &c->split_partials, (size_t)c->pass_grid * kUnitTiles * 2 * 64, true)) ||
+    if ((r = dev_alloc(c, &c->split_partials, (size_t)c->pass_grid * kUnitTiles * 2 * 64, true)) ||
         (r = dev_alloc(c, &c->x_h, frag_image_len(g.d_model), true)) || (r = dev_alloc(c, &c->x_u, frag_image_len(g.d_ffn), true)) ||
         (r = dev_alloc(c, &c->ssq_part, (size_t)kSsqMaxGroups * kPassMaxRows, true)) ||
-        (r = dev_alloc(c, &c->amax_part, (size_t)((g.vocab / 16 + kUnitTiles - 1) / kUnitTiles) * kPassMaxRows, true)) ||
-        (r = build_programs(c)))
+        (r = dev_alloc(c, &c->amax_part, (size_t)((g.vocab / 16 + kUnitTiles - 1) / kUnitTiles) * kPassMaxRows, true)))
       return bail(r);
   }
+  if ((r = build_programs(c))) return bail(r);
   if (cudaMallocHost(reinterpret_cast<void**>(&c->pinned_flag), 64) != cudaSuccess) {
     c->err = "cudaMallocHost failed";
     return bail(SDFP_ENOMEM);
@@ -1141,6 +1319,9 @@ extern "C" int sdfp_set_draft_layers(sdfp_ctx* c, const uint8_t* keep_mask) {
 
 namespace {
 
+// rows one pass of this context carries
+int rows_per_pass(const sdfp_ctx* c) { return c->use_pass ? kPassMaxRows : kMaxRows; }
+
 int check_dense_error(sdfp_ctx* c) {
   if (!c->use_dense) return 0;
   int e = 0;
@@ -1160,13 +1341,13 @@ int check_dense_error(sdfp_ctx* c) {
 // A failed wait inside the pass kernel leaves its code in device memory; turn it into an error
 // and put the synchronisation words back to their initial state.
 int check_pass_error(sdfp_ctx* c) {
-  if (!c->use_pass) return 0;
+  if (!c->psync) return 0;
   PassSync ps{};
   CU_OK(c, cudaMemcpyAsync(&ps, c->psync, sizeof ps, cudaMemcpyDeviceToHost, c->stream));
   CU_OK(c, cudaStreamSynchronize(c->stream));
   if (ps.error == 0) return 0;
   cudaMemsetAsync(c->psync, 0, sizeof(PassSync), c->stream);
-  cudaMemsetAsync(c->split_partials, 0, (size_t)c->pass_grid * kUnitTiles * 2 * 64 * sizeof(ulonglong2), c->stream);
+  if (c->use_pass) cudaMemsetAsync(c->split_partials, 0, (size_t)c->pass_grid * kUnitTiles * 2 * 64 * sizeof(ulonglong2), c->stream);
   cudaStreamSynchronize(c->stream);
   static const char* const what[] = {"", "grid barrier", "weight slot never filled", "weight slot never freed",
                                      "partial sum of a split group never posted"};
@@ -1190,7 +1371,7 @@ int forward_logits_passes(sdfp_ctx* c, bool draft, const int32_t* tokens, int ro
 int forward_logits_passes_inner(sdfp_ctx* c, bool draft, const int32_t* tokens, int rows, int start, float* host_logits) {
   const sdfp_config& g = c->cfg;
   CU_OK(c, cudaMemcpyAsync(c->fwd_tok, tokens, (size_t)rows * 4, cudaMemcpyHostToDevice, c->stream));
-  const int per_pass = c->use_pass ? kPassMaxRows : kMaxRows;
+  const int per_pass = rows_per_pass(c);
   for (int off = 0; off < rows; off += per_pass) {
     const int cnt = std::min(per_pass, rows - off);
     PassDesc pd{};
@@ -1219,7 +1400,7 @@ namespace {
 // fill its cache: passes of the widest kind, of as many positions and then of as many sequences as
 // fit.  A row's numbers do not depend on the pass it sits in.
 int prefill_passes(sdfp_ctx* c, bool draft, int batch, int len) {
-  const int widest = c->use_pass ? kPassMaxRows : kMaxRows;
+  const int widest = rows_per_pass(c);
   for (int s = 0; s < len;) {
     // rows of a sequence: as many whole attention groups as fit, or what is left of the prompt
     const int left = std::min(widest, len - s), cnt = left > kAttnMaxR ? left / kAttnMaxR * kAttnMaxR : left;
@@ -1415,7 +1596,8 @@ extern "C" int sdfp_generate(sdfp_ctx* c, const int32_t* prompts, int32_t batch,
   const long long launches0 = c->launches;
   cudaGraphExec_t exec = nullptr;
   long long launches_per_round = 0;
-  if (c->use_graph) {
+  const bool in_one_launch = c->use_cluster && !sampled;  // the cluster kernel runs greedy rounds to the end
+  if (c->use_graph && !in_one_launch) {
     auto key = std::make_tuple((int)k, (int)batch, sampled ? 1 : 0, n_chunks);
     auto it = c->graphs.find(key);
     if (it == c->graphs.end()) {
@@ -1442,7 +1624,14 @@ extern "C" int sdfp_generate(sdfp_ctx* c, const int32_t* prompts, int32_t batch,
   }
   int rounds = 0;
   const int round_cap = max_new + 1;
-  while (rounds < round_cap) {
+  if (in_one_launch) {
+    ClParams cp = cluster_params(c);
+    cp.rounds = round_cap;
+    cp.first_rows = c->share_kv ? 1 : 2;
+    CU_OK(c, launch_cluster(c, cp));
+    CU_OK(c, cudaMemcpyAsync(&c->pinned_flag[2], &c->gs->round, 4, cudaMemcpyDeviceToHost, st));
+  }
+  while (!in_one_launch && rounds < round_cap) {
     if (exec) {
       CU_OK(c, cudaGraphLaunch(exec, st));
       c->launches += launches_per_round;
@@ -1457,6 +1646,7 @@ extern "C" int sdfp_generate(sdfp_ctx* c, const int32_t* prompts, int32_t batch,
   CU_OK(c, cudaEventRecord(c->ev[2], st));
   if (int r = check_pass_error(c)) return r;
   if (int r = check_dense_error(c)) return r;
+  if (in_one_launch) rounds = c->pinned_flag[2];  // the check above has waited for the copy
 
   // results
   std::vector<int> lens(kMaxBatch);

@@ -1,0 +1,86 @@
+"""Rounds of small decoders inside one thread-block cluster (csrc/cluster_pass.cuh) at the edges of its shares, steps and splits."""
+import numpy as np
+import pytest
+
+import synth_inputs as si
+from gpu_common import check_stream_against_oracle, make_pair
+from oracle import sdfp_oracle as orc
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("heads,head_dim,ffn,vocab,dtype,prompt,k", [
+    (2, 64, 64, 16, "f32", 1, 3),        # the smallest shares: four pairs per CTA, CTAs without a token of the vocabulary; a draft row in front of the text
+    (2, 64, 64, 16, "bf16", 300, 4),     # ... K of half a step; four CTAs per head
+    (3, 128, 528, 400, "f32", 200, 4),   # shares of different size, a ragged last K step, CTAs without a head; blocks of four keys
+    (3, 128, 1040, 400, "bf16", 60, 8),  # ... 9 rows: a second sweep of the weights
+    (7, 64, 1200, 272, "bf16", 90, 0),   # several steps and batches of pairs per warp
+    (17, 64, 80, 272, "bf16", 20, 0),    # more heads than CTAs
+])
+def test_greedy_rounds_at_the_edges(heads, head_dim, ffn, vocab, dtype, prompt, k):
+    """One launch for all rounds; every token is the oracle's choice given the tokens before it (near-ties of bf16 within
+    1e-2 as everywhere; fp32 within 1e-3, five times the logit error that 1e-4 in 2-norm can put on one of these vocabularies),
+    and speculative and autoregressive decoding agree."""
+    shape = si.ModelShape("edge", 3, heads * head_dim, heads, head_dim, ffn, vocab, dtype=dtype)
+    eng, m, _ = make_pair(shape, (1,), max_seq=prompt + 40 + k, k_max=k, random_gains=True)
+    try:
+        text = si.make_prompts(vocab, 1, prompt, seed=31)
+        out = eng.sdfp_generate(text, k, 36)
+        assert out.timing["kernel_launches"] == 1 and len(out.tokens[0]) == 36
+        assert eng.sdfp_generate(text, 0, 36).tokens == out.tokens
+        check_stream_against_oracle(m, text[0].tolist(), out.tokens[0], gap_tol=1e-3 if dtype == "f32" else 1e-2)
+        if k and dtype == "f32":
+            ref = orc.spec_generate(orc.CachedLM(m, max_seq=prompt + 60), orc.CachedLM(m, orc.keep_layers(3, (1,)), max_seq=prompt + 60),
+                                    text[0].tolist(), k, 36)
+            if ref.tokens == out.tokens[0]:  # no near-tie among them: the same drafts were accepted
+                assert [int(a) for a in out.stats[:, 0, 1]] == [r.accepted for r in ref.rounds]
+    finally:
+        eng.close()
+
+
+@pytest.mark.parametrize("dtype,batch,k,prompt", [("f32", 1, 4, 1), ("bf16", 3, 4, 70), ("bf16", 4, 2, 9), ("bf16", 8, 0, 2), ("f32", 4, 0, 33)])
+def test_rounds_of_a_batch(dtype, batch, k, prompt):
+    """speculative == autoregressive == one sequence alone, with the draft's own cache and with the target's; the sequences are
+    teacher-forced with the oracle; sampled decoding with the full model as its own draft accepts everything."""
+    shape = si.TINY if dtype == "f32" else si.TINY_BF16
+    eng, m, _ = make_pair(shape, (1, 2), max_seq=prompt + 40, max_batch=batch, k_max=k)
+    try:
+        prompts = si.make_prompts(m.vocab, batch, prompt, seed=50 + batch)
+        out = eng.sdfp_generate(prompts, k, 24)
+        assert out.timing["kernel_launches"] == 1
+        ar = eng.sdfp_generate(prompts, 0, 24)
+        assert ar.tokens == out.tokens and all(len(t) == 24 for t in out.tokens)
+        assert np.array_equal(out.stats[:, :, 2].sum(axis=0), np.full(batch, 24))
+        solo = eng.sdfp_generate(prompts[-1:], k, 24)
+        assert solo.tokens[0] == out.tokens[-1]
+        for b in (0, batch - 1):
+            check_stream_against_oracle(m, prompts[b].tolist(), out.tokens[b])
+        if k:
+            eng.sdfp_set_draft_kv_sharing(True)
+            assert eng.sdfp_generate(prompts, k, 24).tokens == out.tokens
+            eng.sdfp_set_draft_kv_sharing(False)
+            eng.sdfp_set_draft_layers(np.ones(shape.n_layers, dtype=np.uint8))
+            s = eng.sdfp_generate(prompts, k, 20, temperature=1.0, seed=5)
+            assert (s.stats[:-1, 0, 1] == k).all()
+    finally:
+        eng.close()
+
+
+def test_an_end_token():
+    """A sequence that ends early stays where it is while the other goes on; calls behind it start afresh."""
+    eng, m, _ = make_pair(si.TINY_BF16, (1, 2), max_seq=64, max_batch=2, k_max=4)
+    prompts = si.make_prompts(m.vocab, 2, 12, seed=77)
+    free = eng.sdfp_generate(prompts, 4, 30)
+    eng.close()
+    eos = free.tokens[0][7]
+    eng, _, _ = make_pair(si.TINY_BF16, (1, 2), max_seq=64, max_batch=2, k_max=4, eos_id=int(eos))
+    try:
+        for k in (4, 0):
+            out = eng.sdfp_generate(prompts, k, 30)
+            assert out.timing["kernel_launches"] == 1
+            for b in range(2):
+                want = free.tokens[b]
+                cut = want.index(eos) + 1 if eos in want else len(want)
+                assert out.tokens[b] == want[:cut]
+    finally:
+        eng.close()
