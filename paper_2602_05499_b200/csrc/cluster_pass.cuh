@@ -12,17 +12,18 @@
 //     goes through L2 but weights and the K/V cache.  From the last send to the last arrival 300 clocks pass.
 //   * The buffers need no second copy: a CTA writes into another's buffer only when it holds the complete output of a stage
 //     that the other contributed to after its last read of that buffer.  Every CTA has a share of every stage of a layer.
-//   * Weights: a warp owns output pairs and walks K with its lanes; two steps are in registers or on their way, the first
-//     before the wait for the activations.
+//   * Weights: a warp owns output pairs and walks K with its lanes; the first step is on its way before the wait for the
+//     activations.
 //   * The residual stream, the next norm's input and the SwiGLU output of all rows live in every CTA's shared
 //     memory in fp32; products are fp32 FMAs on exact activations.
 //   * K/V: the rows of the running pass are taken from shared memory, older keys from the cache in global memory,
 //     which the CTA that makes an entry also writes.
 // What bounds it now is instructions, about 14 000 a warp and pass at 4 layers d 256, six clocks each with two warps on a
-// scheduler (ncu): 16 warps, weights through a ring filled by a producer warp, all eight lanes groups of a warp on K, and
-// mma.sync for bf16 were built and were slower at one row (64, 82, 65 and 59 us a pass against 38).  In us a pass, 4 layers, bf16, autoregressive, this kernel
-// and the whole-pass kernel: d 256 38 and 126, d 384 52 and 136, d 512 60 and 142; fp32 and one launch per operation: 43 and 101,
-// 58 and 110, 99 and 114.  The line to the other paths is at cluster_wanted in engine.cu.
+// scheduler (ncu): 16 warps, weights through a ring filled by a producer warp, eight lanes on K and the others on pairs or rows, and
+// mma.sync for bf16 were built and were slower at one row (58, 82, 65 and 59 us a pass against 36); four and
+// sixteen warps take 10 to 30 % longer than eight.  In us a pass, 4 layers, bf16, autoregressive, this kernel
+// and the whole-pass kernel: d 256 37 and 126, d 384 50 and 136, d 512 59 and 142; fp32 and one launch per operation: 42 and 101,
+// 57 and 110, 97 and 114.  The line to the other paths is at cluster_wanted in engine.cu.
 //
 // Batch invariance: a (row, feature) sum runs over K in an order fixed by the matrix, a (row, head) softmax over
 // 4- or 8-key blocks dealt to the warps by absolute key index; neither depends on the rows of the pass.
@@ -264,29 +265,30 @@ __device__ __forceinline__ void cl_fma(float& t, const uint4& w, const float4& x
 __device__ __forceinline__ int cl_feature(int pair) { return ((pair >> 3) << 4) + (pair & 7); }  // the first of a pair's features, its second is 8 further
 
 // A warp's pairs lie behind one another in memory.  It takes P of them through RT rows at a time (more rows take another
-// sweep of the weights, from L2); D K steps of weights are in registers or on their way, the first before the wait for
-// the activations.  A sum is made in the same order whatever P and RT: K steps in order by each lane, the lanes in the xor tree.
-template <typename WT, int RT, int P, int D>
+// sweep of the weights, from L2); a K step of weights is in registers or on its way, the first before the wait for the
+// activations.  (Two to four steps ahead, in as many copies of the loop's body, were slower: tiny decoders by 4 %.)  A sum is made
+// in the same order whatever P and RT: K steps in order by each lane, the lanes in the xor tree.
+template <typename WT, int RT, int P>
 __device__ __forceinline__ void cl_dots(const ClParams& p, const ClDots& a, ClShared* sh) {
   constexpr bool BF = sizeof(WT) == 2;
   constexpr int N = RT * P * 2, CH = N < 16 ? N : 16;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_w = RT == 1 ? (a.np + kClWarps - 1) / kClWarps : (a.np / 2 + kClWarps - 1) / kClWarps * 2;  // pairs per warp
-  const int first = warp * n_w, cnt = max(0, min(n_w, a.np - first)), total = (cnt + P - 1) / P * a.steps;
+  const int first = warp * n_w, cnt = max(0, min(n_w, a.np - first));
   const int pair_len = a.steps * (kClUnit / 16);
 #pragma unroll 1
   for (int r0 = 0; r0 < a.R; r0 += RT) {
     const int rows = RT == 1 ? 1 : min(RT, a.R - r0);
     const uint4* w = reinterpret_cast<const uint4*>(a.W) + (size_t)first * pair_len + lane;
     int ask_pairs = cnt, ask_steps = a.steps;  // pairs from the next request's on, steps left of them
-    uint4 raw[D][P][2];
-    auto ask = [&](uint4 (&r)[P][2]) {
+    uint4 raw[P][2];
+    auto ask = [&]() {
       if (ask_pairs <= 0) return;
 #pragma unroll
       for (int j = 0; j < P; ++j)
         if (j < ask_pairs) {
-          r[j][0] = __ldg(w + j * pair_len);
-          r[j][1] = __ldg(w + j * pair_len + 32);
+          raw[j][0] = __ldg(w + j * pair_len);
+          raw[j][1] = __ldg(w + j * pair_len + 32);
         }
       w += kClUnit / 16;
       if (--ask_steps == 0) {
@@ -295,81 +297,70 @@ __device__ __forceinline__ void cl_dots(const ClParams& p, const ClDots& a, ClSh
         w += (P - 1) * pair_len;
       }
     };
-#pragma unroll
-    for (int i = 0; i < D; ++i) ask(raw[i]);
+    ask();
     if (r0 == 0) cl_begin(p, a, sh);
     const float* const x = cl_at<float>(a.x) + r0 * a.K + lane * 4;
     const int room = a.K - lane * 4;
-    float acc[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) acc[i] = 0.f;
-    int s = 0, c0 = 0, at = 0;  // step, its first column, first pair of the running P
 #pragma unroll 1
-    for (int q = 0; q < total; q += D) {
+    for (int at = 0; at < cnt; at += P) {  // first pair of the running P
+      float acc[N];
 #pragma unroll
-      for (int u = 0; u < D; ++u) {
-        if (q + u < total) {
-          const bool in0 = c0 < room, in1 = BF && c0 + 128 < room;
+      for (int i = 0; i < N; ++i) acc[i] = 0.f;
+#pragma unroll 1
+      for (int c0 = 0; c0 < a.K; c0 += ClElem<WT>::kStep) {
+        const bool in0 = c0 < room, in1 = BF && c0 + 128 < room;
 #pragma unroll
-          for (int i = 0; i < RT; ++i) {
-            if (RT == 1 || i < rows) {
-              float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;
-              if (in0) x0 = *reinterpret_cast<const float4*>(x + i * a.K + c0);
-              if (in1) x1 = *reinterpret_cast<const float4*>(x + i * a.K + c0 + 128);
+        for (int i = 0; i < RT; ++i) {
+          if (RT == 1 || i < rows) {
+            float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;
+            if (in0) x0 = *reinterpret_cast<const float4*>(x + i * a.K + c0);
+            if (in1) x1 = *reinterpret_cast<const float4*>(x + i * a.K + c0 + 128);
 #pragma unroll
-              for (int j = 0; j < P; ++j)
-                if (RT > 1 || j < cnt - at) {
-                  cl_fma<WT>(acc[(i * P + j) * 2], raw[u][j][0], x0, x1);
-                  cl_fma<WT>(acc[(i * P + j) * 2 + 1], raw[u][j][1], x0, x1);
-                }
-            }
+            for (int j = 0; j < P; ++j)
+              if (RT > 1 || j < cnt - at) {
+                cl_fma<WT>(acc[(i * P + j) * 2], raw[j][0], x0, x1);
+                cl_fma<WT>(acc[(i * P + j) * 2 + 1], raw[j][1], x0, x1);
+              }
           }
-          ask(raw[u]);
-          c0 += ClElem<WT>::kStep;
-          if (++s == a.steps) {
-            // lane groups end up with one (row, pair, half) each; both halves of a pair in the lane that uses them
+        }
+        ask();
+      }
+        // lane groups end up with one (row, pair, half) each; both halves of a pair in the lane that uses them
 #pragma unroll
-            for (int g = 0; g < N; g += CH) {
-              if (g / (2 * P) < rows) {
-                float v[CH];
+        for (int g = 0; g < N; g += CH) {
+          if (g / (2 * P) < rows) {
+            float v[CH];
 #pragma unroll
-                for (int i = 0; i < CH; ++i) v[i] = acc[g + i];
-                float v0 = warp_sum_scatter<CH>(v);
-                float v1 = __shfl_xor_sync(0xffffffffu, v0, 32 / CH);
-                const int pi = (g + lane / (32 / CH)) >> 1, row = r0 + pi / P, pl = first + at + pi % P;
-                if (lane % (64 / CH) == 0 && row < a.R && at + pi % P < cnt) {
-                  if (!a.head) {
-                    float* o = cl_at<float>(a.stg) + row * a.np + pl;
-                    o[0] = v0;
-                    o[a.R * a.np] = v1;
-                  } else {
-                    const int f0 = cl_feature(a.p0 + pl);
-                    const float inv = sh->inv[row];
-                    v0 *= inv;
-                    v1 *= inv;
-                    if (a.logits != nullptr) {
-                      float* o = a.logits + (size_t)row * p.vocab + f0;
-                      o[0] = v0;
-                      o[8] = v1;
-                    } else {  // only this lane touches its place
-                      float2* best = cl_at<float2>(p.lay.best) + row * 32 + warp * 4 + pi % P;
-                      const float2 o = *best;
-                      const bool second = v1 > v0;
-                      const float bv = second ? v1 : v0;
-                      const int bi = second ? f0 + 8 : f0;
-                      if (bv > o.x || (bv == o.x && bi < __float_as_int(o.y))) *best = make_float2(bv, __int_as_float(bi));
-                    }
-                  }
+            for (int i = 0; i < CH; ++i) v[i] = acc[g + i];
+            float v0 = warp_sum_scatter<CH>(v);
+            float v1 = __shfl_xor_sync(0xffffffffu, v0, 32 / CH);
+            const int pi = (g + lane / (32 / CH)) >> 1, row = r0 + pi / P, pl = first + at + pi % P;
+            if (lane % (64 / CH) == 0 && row < a.R && at + pi % P < cnt) {
+              if (!a.head) {
+                float* o = cl_at<float>(a.stg) + row * a.np + pl;
+                o[0] = v0;
+                o[a.R * a.np] = v1;
+              } else {
+                const int f0 = cl_feature(a.p0 + pl);
+                const float inv = sh->inv[row];
+                v0 *= inv;
+                v1 *= inv;
+                if (a.logits != nullptr) {
+                  float* o = a.logits + (size_t)row * p.vocab + f0;
+                  o[0] = v0;
+                  o[8] = v1;
+                } else {  // only this lane touches its place
+                  float2* best = cl_at<float2>(p.lay.best) + row * 4 * kClWarps + warp * 4 + pi % P;
+                  const float2 o = *best;
+                  const bool second = v1 > v0;
+                  const float bv = second ? v1 : v0;
+                  const int bi = second ? f0 + 8 : f0;
+                  if (bv > o.x || (bv == o.x && bi < __float_as_int(o.y))) *best = make_float2(bv, __int_as_float(bi));
                 }
               }
             }
-#pragma unroll
-            for (int i = 0; i < N; ++i) acc[i] = 0.f;
-            s = c0 = 0;
-            at += P;
           }
         }
-      }
     }
   }
 }
@@ -871,7 +862,9 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
         rope[i * 32 + ev.lane] = cs[i];
         rope[hp + i * 32 + ev.lane] = sn[i];
       }
-      if (loop) cl_at<float2>(p.lay.best)[row * 32 + ev.lane] = make_float2(-INFINITY, __int_as_float(0x7fffffff));
+      if (loop)
+#pragma unroll
+        for (int c = ev.lane; c < 4 * kClWarps; c += 32) cl_at<float2>(p.lay.best)[row * 4 * kClWarps + c] = make_float2(-INFINITY, __int_as_float(0x7fffffff));
     }
     cl_sync();
 
@@ -903,11 +896,11 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
       // the pass's keys and values, before anything of the next pass is sent: their writers, long done, in a stage whose last warps have the least to do
       if (t.after_kv && tid >= kClThreads - ((R * sh->mine[CL_QKV].nq + 31) & ~31)) __threadfence();
       if (R == 1)
-        cl_dots<WT, 1, 4, 2>(p, a, sh);
+        cl_dots<WT, 1, 4>(p, a, sh);
       else if (R <= 4)
-        cl_dots<WT, 4, 2, 2>(p, a, sh);
+        cl_dots<WT, 4, 2>(p, a, sh);
       else
-        cl_dots<WT, 8, 2, 2>(p, a, sh);
+        cl_dots<WT, 8, 2>(p, a, sh);
       if (a.head) break;
       cl_sync();  // the sums are there
       const bool live = !cl_aborted(sh);
@@ -932,9 +925,16 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
     if (!cl_aborted(sh))
 #pragma unroll 1
       for (int row = ev.warp; row < R; row += kClWarps) {
-        const float2 c = cl_at<float2>(p.lay.best)[row * 32 + ev.lane];
-        float bv = c.x;
-        int bi = __float_as_int(c.y);
+        float bv = -INFINITY;
+        int bi = 0x7fffffff;
+#pragma unroll
+        for (int e = ev.lane; e < 4 * kClWarps; e += 32) {
+          const float2 c = cl_at<float2>(p.lay.best)[row * 4 * kClWarps + e];
+          if (c.x > bv || (c.x == bv && __float_as_int(c.y) < bi)) {
+            bv = c.x;
+            bi = __float_as_int(c.y);
+          }
+        }
         cl_best_of_lanes<32>(bv, bi);
         if (ev.lane < kClCtas) cl_send2(ev.dst + p.lay.tok + (rank * R + row) * 8, bv, __int_as_float(bi), cl_bar_of(p, ev.dst, CL_BAR_TOK));
       }
@@ -1115,7 +1115,7 @@ inline ClLayout cluster_layout(int d, int f, int heads, int hd, int n_layers, in
   take(y.stg, 8LL * y.stg_floats);
   take(y.rope, 4LL * rows * hd);
   take(y.tok, 8LL * kClCtas * rows);
-  take(y.best, 8LL * rows * 32);
+  take(y.best, 32LL * rows * kClWarps);
   take(y.tab, (long long)sizeof(ClTab) * 2 * (4 * n_layers + 1));
   take(y.shared, (long long)sizeof(ClShared));
   y.total = at <= max_smem ? at : 0;

@@ -125,6 +125,8 @@ struct sdfp_ctx {
   int n_cl_t = 0, n_cl_d = 0;
   int cl_first_t = 0, cl_first_d = 0;  // the norm their first stage reads the embedding through
   void* cl_lm_head = nullptr;
+  unsigned char* cl_weights = nullptr;  // all matrices in its layout
+  size_t cl_used = 0;
   float* cl_gains = nullptr;         // [2 n_layers + 1][d_model]
   // dense path on tcgen05 (bf16 tensor path): the prompt pass of every context, and every pass of
   // a context whose widest pass does not fit the whole-pass kernel
@@ -936,6 +938,11 @@ int pack_dense_image(sdfp_ctx* c, void** dst, PackSrc ps, int n_pairs, int K) {
   return 0;
 }
 
+template <typename WT>
+size_t cluster_matrix_bytes(int n_pairs, int K) {
+  return (size_t)n_pairs * cl_steps(K, (int)sizeof(WT)) * kClUnit;
+}
+
 // A matrix in the layout(s) this context's kernels read: `dst` for the whole-pass / per-operation
 // kernels, `img` (may be null) for the dense path.  A context whose decode passes run on the dense
 // path reads only images: `dst` then points to the image as well.
@@ -959,11 +966,11 @@ int pack_matrix(sdfp_ctx* c, void** dst, void** img, void** cl, PackSrc ps, int 
   }
   CU_OK(c, cudaGetLastError());
   *dst = p;
-  if (c->use_cluster) {
-    if (int r = dev_alloc(c, &p, (size_t)n_pairs * 2 * cl_steps(K, sizeof(WT)) * ClElem<WT>::kStep)) return r;
-    pack_cluster_kernel<WT><<<1184, 256, 0, c->stream>>>(p, ps, n_pairs, K);
+  if (c->use_cluster) {  // (one allocation for all of them: cudaMalloc takes as long as the packing of a small matrix)
+    *cl = c->cl_weights + c->cl_used;
+    c->cl_used += cluster_matrix_bytes<WT>(n_pairs, K);
+    pack_cluster_kernel<WT><<<1184, 256, 0, c->stream>>>(reinterpret_cast<WT*>(*cl), ps, n_pairs, K);
     CU_OK(c, cudaGetLastError());
-    *cl = p;
   }
   return 0;
 }
@@ -981,6 +988,11 @@ int load_weights(sdfp_ctx* c, const sdfp_weights* w) {
   const sdfp_config& g = c->cfg;
   const int d = g.d_model, f = g.d_ffn, H = g.n_heads, hd = g.head_dim;
   c->layers.resize(g.n_layers);
+  if (c->use_cluster) {
+    const size_t layer = cluster_matrix_bytes<WT>(3 * d / 2, d) + cluster_matrix_bytes<WT>(d / 2, d) + cluster_matrix_bytes<WT>(f, d) +
+                         cluster_matrix_bytes<WT>(d / 2, f);
+    if (int r = dev_alloc(c, &c->cl_weights, layer * g.n_layers + cluster_matrix_bytes<WT>(g.vocab / 2, d))) return r;
+  }
   for (int l = 0; l < g.n_layers; ++l) {
     LayerWeights& lw = c->layers[l];
     if (!w->wq[l] || !w->wk[l] || !w->wv[l] || !w->wo[l] || !w->w_gate[l] || !w->w_up[l] || !w->w_down[l] ||
