@@ -18,7 +18,7 @@
 //     memory in fp32; products are fp32 FMAs on exact activations.
 //   * K/V: the rows of the running pass are taken from shared memory, older keys from the cache in global memory,
 //     which the CTA that makes an entry also writes.
-// What bounds it now is instructions, about 14 000 a warp and pass at 4 layers d 256, six clocks each with two warps on a
+// What bounds it now is instructions, 10 700 a warp and pass at 4 layers d 256, six to seven clocks each with two warps on a
 // scheduler (ncu): 16 warps, weights through a ring filled by a producer warp, eight lanes on K and the others on pairs or rows, and
 // mma.sync for bf16 were built and were slower at one row (58, 82, 65 and 59 us a pass against 36); four and
 // sixteen warps take 10 to 30 % longer than eight.  In us a pass, 4 layers, bf16, autoregressive, this kernel
@@ -325,42 +325,42 @@ __device__ __forceinline__ void cl_dots(const ClParams& p, const ClDots& a, ClSh
         }
         ask();
       }
-        // lane groups end up with one (row, pair, half) each; both halves of a pair in the lane that uses them
+      // lane groups end up with one (row, pair, half) each; both halves of a pair in the lane that uses them
 #pragma unroll
-        for (int g = 0; g < N; g += CH) {
-          if (g / (2 * P) < rows) {
-            float v[CH];
+      for (int g = 0; g < N; g += CH) {
+        if (g / (2 * P) < rows) {
+          float v[CH];
 #pragma unroll
-            for (int i = 0; i < CH; ++i) v[i] = acc[g + i];
-            float v0 = warp_sum_scatter<CH>(v);
-            float v1 = __shfl_xor_sync(0xffffffffu, v0, 32 / CH);
-            const int pi = (g + lane / (32 / CH)) >> 1, row = r0 + pi / P, pl = first + at + pi % P;
-            if (lane % (64 / CH) == 0 && row < a.R && at + pi % P < cnt) {
-              if (!a.head) {
-                float* o = cl_at<float>(a.stg) + row * a.np + pl;
+          for (int i = 0; i < CH; ++i) v[i] = acc[g + i];
+          float v0 = warp_sum_scatter<CH>(v);
+          float v1 = __shfl_xor_sync(0xffffffffu, v0, 32 / CH);
+          const int pi = (g + lane / (32 / CH)) >> 1, row = r0 + pi / P, pl = first + at + pi % P;
+          if (lane % (64 / CH) == 0 && row < a.R && at + pi % P < cnt) {
+            if (!a.head) {
+              float* o = cl_at<float>(a.stg) + row * a.np + pl;
+              o[0] = v0;
+              o[a.R * a.np] = v1;
+            } else {
+              const int f0 = cl_feature(a.p0 + pl);
+              const float inv = sh->inv[row];
+              v0 *= inv;
+              v1 *= inv;
+              if (a.logits != nullptr) {
+                float* o = a.logits + (size_t)row * p.vocab + f0;
                 o[0] = v0;
-                o[a.R * a.np] = v1;
-              } else {
-                const int f0 = cl_feature(a.p0 + pl);
-                const float inv = sh->inv[row];
-                v0 *= inv;
-                v1 *= inv;
-                if (a.logits != nullptr) {
-                  float* o = a.logits + (size_t)row * p.vocab + f0;
-                  o[0] = v0;
-                  o[8] = v1;
-                } else {  // only this lane touches its place
-                  float2* best = cl_at<float2>(p.lay.best) + row * 4 * kClWarps + warp * 4 + pi % P;
-                  const float2 o = *best;
-                  const bool second = v1 > v0;
-                  const float bv = second ? v1 : v0;
-                  const int bi = second ? f0 + 8 : f0;
-                  if (bv > o.x || (bv == o.x && bi < __float_as_int(o.y))) *best = make_float2(bv, __int_as_float(bi));
-                }
+                o[8] = v1;
+              } else {  // only this lane touches its place
+                float2* best = cl_at<float2>(p.lay.best) + row * 4 * kClWarps + warp * 4 + pi % P;
+                const float2 o = *best;
+                const bool second = v1 > v0;
+                const float bv = second ? v1 : v0;
+                const int bi = second ? f0 + 8 : f0;
+                if (bv > o.x || (bv == o.x && bi < __float_as_int(o.y))) *best = make_float2(bv, __int_as_float(bi));
               }
             }
           }
         }
+      }
     }
   }
 }
