@@ -1,33 +1,37 @@
-// Rounds of a small decoder inside ONE thread-block cluster of sixteen CTAs: the whole greedy generation loop (Algorithm 1,
+// Rounds of small decoders inside ONE thread-block cluster of sixteen CTAs: the whole greedy generation loop (Algorithm 1,
 // Stage B: k draft passes, verification, accept, commit) in one launch, or one pass of a sampled round.
 //
 // What bounds a small decoder is not its bytes but the chain of dependent stages, five a layer: spread over 148
 // SMs a stage boundary is a grid-wide exchange through L2 (about 5 us in the whole-pass kernel, about 4 us as one
 // launch per operation), for a fraction of a microsecond of work.  Sixteen SMs of one cluster hand their results on
 // through distributed shared memory instead:
-//   * Every linear stage gives each CTA an equal share of the output features.  The finished sums are gathered in shared
-//     memory; behind one barrier of the CTA a half-warp takes four pairs at a time, a lane sends the result to each of the
-//     sixteen CTAs with st.async, and the bytes complete a transaction count on an mbarrier of the receiver, which starts
-//     its next stage when all shares have landed.  No barrier over the cluster stands between stages, and nothing
-//     goes through L2 but weights and the K/V cache.  From the last send to the last arrival 300 clocks pass.
+//   * Every linear stage gives each CTA an equal share of the output features.  The finished values are gathered in shared
+//     memory; a half-warp takes four columns at a time, a lane sends them to each of the sixteen CTAs with st.async, and
+//     the bytes complete a transaction count on an mbarrier of the receiver, which starts its next stage when all
+//     shares have landed.  No barrier over the cluster stands between stages, and nothing goes through L2 but
+//     weights and the K/V cache.
 //   * The buffers need no second copy: a CTA writes into another's buffer only when it holds the complete output of a stage
 //     that the other contributed to after its last read of that buffer.  Every CTA has a share of every stage of a layer.
-//   * Weights: a warp owns output pairs and walks K with its lanes; the first step is on its way before the wait for the
-//     activations.
-//   * The residual stream, the next norm's input and the SwiGLU output of all rows live in every CTA's shared
-//     memory in fp32; products are fp32 FMAs on exact activations.
-//   * K/V: the rows of the running pass are taken from shared memory, older keys from the cache in global memory,
-//     which the CTA that makes an entry also writes.
-// What bounds it now is instructions, 10 700 a warp and pass at 4 layers d 256, six to seven clocks each with two warps on a
-// scheduler (ncu): 16 warps, weights through a ring filled by a producer warp, eight lanes on K and the others on pairs or rows, and
-// mma.sync for bf16 were built and were slower at one row (58, 82, 65 and 59 us a pass against 36); four and
-// sixteen warps take 10 to 30 % longer than eight.  In us a pass, 4 layers, bf16, autoregressive, this kernel
-// and the whole-pass kernel: d 256 37 and 126, d 384 50 and 136, d 512 59 and 142; fp32 and one launch per operation: 42 and 101,
-// 57 and 110, 97 and 114.  The line to the other paths is at cluster_wanted in engine.cu.
+//   * Weights are read where the context's other kernels read them; the first ones are on their way before the wait for
+//     the activations.
+//   * K/V: the rows of the running pass are taken from shared memory, older keys from the cache in global memory.  The
+//     CTA that reads a key in later passes is the one that appends it, so no pass waits for another CTA's cache entries.
+//   * Loops are left rolled: every instruction of a pass is met once per layer, and straight code that does not stay in the
+//     instruction cache is fetched from L2, eight instructions at a time.
 //
-// Batch invariance: a (row, feature) sum runs over K in an order fixed by the matrix, a (row, head) softmax over
-// 4- or 8-key blocks dealt to the warps by absolute key index; neither depends on the rows of the pass.
+// The results are, bit for bit, those of the path the context's other passes take (prompts, sdfp_forward_logits): the
+// whole-pass kernel for bf16, one kernel per operation for fp32.  A text goes on the same whether it was decoded in one
+// call or in several, and the logits a caller asks for are those that chose the tokens.  So the order of every sum is theirs:
+//   * bf16: the tiles and units of pass_kernel.cuh on mma.sync, hi + lo; a warp is a k-class, and a sum is made of the classes of a
+//     piece in order, then of the pieces in the order in which the whole-pass kernel's CTAs post them (StageShare).
+//     Which units a warp multiplies is written down once, on the host (ClEntry).
+//   * fp32: a warp owns output pairs and walks K with its lanes, as linear_fma_kernel does, on rows normalised before.
+//   * Attention in chunks of 64 keys: bf16 eight splits of the chunks with a running maximum each, added in split order
+//     (pass_kernel.cuh); fp32 every chunk by itself, added in chunk order (attention.cuh).
+//   * Squares of the residual rows: per 128 features, then over the groups (bf16); lanes over the row (fp32).
 #pragma once
+
+#include <vector>
 
 #include "attention.cuh"
 #include "common.cuh"
@@ -38,46 +42,75 @@
 namespace sdfp {
 
 constexpr int kClCtas = 16, kClWarps = 8, kClThreads = kClWarps * 32;
+static_assert(kClWarps == kClasses, "a warp is a k-class of the whole-pass kernel");
 constexpr int kClMaxRows = 16;
-constexpr int kClUnit = 1024;  // bytes of one K step of an output pair: 512 of either feature
+constexpr int kClTeam = 128;     // threads that work on an attention item
+constexpr int kClAttnRows = 8;   // rows of a sequence it takes together
+constexpr int kClTiles = 4;      // bf16: tiles a warp multiplies together
+constexpr int kClAhead = 8;      // bf16: units of weights (512 bytes a warp) in half of its ring
 
-enum ClBar { CL_BAR_H = 0, CL_BAR_U = 1, CL_BAR_QKV = 2, CL_BAR_X = 3, CL_BAR_TOK = 4, CL_BARS = 5 };
-enum ClKind { CL_QKV = 0, CL_O = 1, CL_GATE_UP = 2, CL_DOWN = 3, CL_HEAD = 4 };
+enum ClBar { CL_BAR_H = 0, CL_BAR_U = 1, CL_BAR_QKV = 2, CL_BAR_PART = 3, CL_BAR_X = 4, CL_BAR_TOK = 5, CL_BARS = 6 };
+enum ClKind { CL_QKV = 0, CL_O = 1, CL_GATE_UP = 2, CL_DOWN = 3, CL_HEAD = 4, CL_KINDS = 5 };
 
-template <typename WT>
-struct ClElem {
-  static constexpr int kLane = 16 / (int)sizeof(WT);  // columns in a lane's sixteen bytes
-  static constexpr int kStep = 32 * kLane;            // columns of a K step: 256 of bf16, 128 of fp32
-};
-__host__ __device__ __forceinline__ int cl_steps(int K, int elem_bytes) {
-  const int step = 512 / elem_bytes;
-  return (K + step - 1) / step;
+// Shares of the output features: pairs are dealt in fours, so that a share is sent sixteen bytes at a time, and in eights, the
+// row tile of the MMA, where every CTA gets one (a tile cut between two CTAs is multiplied by both).
+__host__ __device__ __forceinline__ int cl_deal(int n_pairs, int elem_bytes) { return elem_bytes == 2 && n_pairs >= 8 * kClCtas ? 8 : 4; }
+__host__ __device__ __forceinline__ int cl_first_pair(int n_pairs, int cta, int elem_bytes) {
+  const int deal = cl_deal(n_pairs, elem_bytes);
+  return (int)((long long)(n_pairs / deal) * cta / kClCtas) * deal;
 }
-// first pair of a CTA's share: pairs are dealt in fours, so that a share is sent sixteen bytes at a time
-__host__ __device__ __forceinline__ int cl_first_pair(int n_pairs, int cta) { return (n_pairs / 4) * cta / kClCtas * 4; }
-__host__ __device__ __forceinline__ int cl_max_pairs(int n_pairs) { return (n_pairs / 4 + kClCtas - 1) / kClCtas * 4; }
+__host__ __device__ __forceinline__ int cl_max_pairs(int n_pairs, int elem_bytes) {
+  const int deal = cl_deal(n_pairs, elem_bytes);
+  return (n_pairs / deal + kClCtas - 1) / kClCtas * deal;
+}
+__host__ __device__ __forceinline__ int cl_pairs_of(int kind, int d, int f, int vocab) {
+  return kind == CL_QKV ? 3 * d / 2 : kind == CL_GATE_UP ? f : kind == CL_HEAD ? vocab / 2 : d / 2;
+}
+
+// What a CTA does of the matrices of one kind: the same in every layer, made on the host
+struct ClMine {
+  int p0, np;             // its pairs
+  int tile_width;         // bf16: tiles multiplied together, 1, 2 or 4
+  int round0, n_rounds;   // its sums fit the staging buffer in one or more rounds
+  int entry0, n_entries;  // bf16: list of warp w = entries entry0 + w * n_entries ...
+  int pad;
+};
+struct ClRound {
+  int quad0, n_quads;  // fours of pairs that are finished in this round
+  unsigned magic;      // i / n_quads == i * magic >> 20 for the few hundred vectors of a round
+  int tile0, np;       // bf16: its first tile, and the pieces a sum is made of
+  int n_entries;       // bf16: of each warp
+  int pad[2];
+};
+struct ClEntry {       // bf16: one k-tile of a warp, for up to kClTiles neighbouring tiles
+  int w;               // the first tile's unit, in uint4 from the matrix's start
+  short kt, slot;      // k-tile, -1: none; slot >= 0: the sums are complete and go to this place, a tile's np places apart
+  unsigned char n_tiles, wrap, np, pad;  // from tile `wrap` on they lie in the next group
+  int pad2;
+};
+static_assert(sizeof(ClMine) == 32 && sizeof(ClRound) == 32 && sizeof(ClEntry) == 16, "copied in sixteen bytes");
 
 struct ClStage {  // a linear stage of a program; the attention follows a QKV stage without an entry of its own
-  const unsigned char* W;  // [pair][step][1 KB], see pack_cluster_kernel
-  void *kcache, *vcache;   // CL_QKV
-  int kind, n_pairs, K;
-  int gain_out;            // CL_O, CL_DOWN: which norm reads the residual stream next
-  int after_kv;            // the first stage behind the last CL_O
+  const unsigned char* W;
+  void *kcache, *vcache;  // CL_QKV
+  int kind, K;
+  int gain;               // fp32: the norm in front of this stage (-1: none); bf16, CL_O and CL_DOWN: the norm that reads the residual stream next
+  int pad;
 };
 
 struct ClTab {  // the same for this CTA, in shared memory
-  const unsigned char* W;  // its first pair
+  const unsigned char* W;  // bf16: the matrix, fp32: its first pair
   void *kcache, *vcache;
-  int kind, np, steps, gain_out;
-  int x, K, bar, row_bytes;  // its activations: where, columns, the barrier that brings them and their bytes per row
-  int norm, p0;
-  int after_kv;              // the first stage behind the last attention's O-projection
+  const float* gain;       // fp32: of the norm in front
+  int kind, K, gain_out;
+  int x, bar, row_bytes;   // its activations: where, the barrier that brings them and their bytes per row
+  int norm;
 };
 
 // Shared-memory layout, worked out on the host (bytes from the start)
 struct ClLayout {
-  int rows, splits, heads_per_cta, resid_np, stg_floats;
-  int h, y, part, xp, xml, xo, u, qkv, gain, hres, stg, rope, tok, best, tab, shared, total;
+  int rows, splits, heads_per_cta, resid_np, part_slots;
+  int h, y, part, team, team_bytes, xo, u, qkv, gain, hres, stg, red, ring, rope, tok, best, tab, plan, plan_rounds, plan_entries, plan_bytes, shared, total;
 };
 
 struct ClParams {
@@ -85,12 +118,13 @@ struct ClParams {
   const ClStage* prog_d;
   int n_t, n_d;              // stages to run of either
   int first_gain_t, first_gain_d;
-  const float* gains;        // [n_gains][d]
+  const float* const* gains;  // [n_gains] -> [d]
   int n_gains;
   int d, f, heads, vocab, max_seq;
   float eps, scale;
   const float *rope_cos, *rope_sin;
   const void* embed;
+  const unsigned char* plan;  // [CTA][plan_bytes]
   ClLayout lay;
   // what to run: greedy rounds until everything is finished, or one pass
   int rounds;                // > 0: at most this many greedy rounds
@@ -106,20 +140,15 @@ struct ClParams {
   PassSync* sync;
 };
 
-struct ClMine {  // this CTA's share of a kind of matrix
-  int p0, np, nq;
-  unsigned magic;  // i / nq == i * magic >> 20 for the few hundred vectors of a share
-};
-
 struct ClShared {
   uint64_t bar[CL_BARS];
-  ClMine mine[5];     // by ClKind
   int abort;
   unsigned long long wait_limit_ns;
   unsigned sabotage;  // bytes the next wait expects in vain (PassSync::bar_extra)
   float inv[kClMaxRows];
   int pos[kClMaxRows];
   int amax[kClMaxRows];
+  float att_m[2][kClAttnRows], att_l[2][kClAttnRows], att_a[2][kClAttnRows];  // attention rows of a team
   // state of the sequences
   int n[kMaxBatch], n_new[kMaxBatch], done[kMaxBatch];
   int last[kMaxBatch][2];  // the last two committed tokens
@@ -151,6 +180,9 @@ __device__ __forceinline__ void cl_send2(uint32_t dst, float x, float y, uint32_
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(dst), "f"(x), "f"(y), "r"(bar)
                : "memory");
 }
+__device__ __forceinline__ void cl_send1(uint32_t dst, float v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(dst), "r"(__float_as_uint(v)), "r"(bar) : "memory");
+}
 __device__ __forceinline__ void cl_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -163,8 +195,7 @@ __device__ __forceinline__ bool cl_try_wait(uint32_t bar, unsigned parity) {
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ void cl_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kClThreads) : "memory"); }  // the compute warps
-// ... and the same answer to "has anything failed" for all of them
+// a barrier of the CTA that gives everybody the same answer to "has anything failed"
 __device__ __forceinline__ bool cl_agree_ok(const int* abort_flag) {
   const int seen = *reinterpret_cast<const volatile int*>(abort_flag);
   unsigned any;
@@ -206,99 +237,169 @@ __device__ __forceinline__ void cl_wait(ClShared* sh, PassSync* sync, int which,
   __syncwarp();
 }
 
-// ---- dot products of a stage ------------------------------------------------------------------------------------
-struct ClDots {
-  const unsigned char* W;    // this CTA's pairs
-  int np, x, K, steps;       // its pairs; activations (offset of [row][K]) and matrix
-  int R;
-  int bar;                   // what brings the activations (ClBar), -1: nothing to wait for
-  unsigned bytes, parity;
-  bool norm;                 // the rows' norms are wanted
-  bool head;                 // lm-head: logits [row][vocab] or, without, the best of each (row, warp, place in the warp)
-  int stg;                   // out: [half][row][np] sums
-  int p0;
-  float* logits;
-};
-
-// Everything that has to be there before the first product
-__device__ __forceinline__ void cl_begin(const ClParams& p, const ClDots& a, ClShared* sh) {
-  if (a.bar >= 0) cl_wait(sh, p.sync, a.bar, a.bytes, a.parity);
-  if (a.norm) {  // the factors are needed behind the dot products only: the last warps, which have the fewest pairs, work them out
-    const int lane = threadIdx.x & 31;
-#pragma unroll 1
-    for (int row = kClWarps - 1 - (threadIdx.x >> 5); row < a.R; row += kClWarps) {
-      const float* h = cl_at<float>(p.lay.h) + row * p.d;
-      float s = 0.f;
-#pragma unroll 2
-      for (int c = lane * 4; c < p.d; c += 128) {
-        const float4 v = *reinterpret_cast<const float4*>(h + c);
-        s = fmaf(v.x, v.x, s);
-        s = fmaf(v.y, v.y, s);
-        s = fmaf(v.z, v.z, s);
-        s = fmaf(v.w, v.w, s);
-      }
-      s = warp_sum(s);
-      if (lane == 0) sh->inv[row] = rsqrtf(s * (1.0f / (float)p.d) + p.eps);
-    }
-  }
-  if (a.head) cl_sync();  // the logits are scaled where they are made
-}
-
-template <typename WT>
-__device__ __forceinline__ void cl_fma(float& t, const uint4& w, const float4& x0, const float4& x1) {
-  if (sizeof(WT) == 2) {
-    t = fmaf(__uint_as_float(w.x << 16), x0.x, t);
-    t = fmaf(__uint_as_float(w.x & 0xffff0000u), x0.y, t);
-    t = fmaf(__uint_as_float(w.y << 16), x0.z, t);
-    t = fmaf(__uint_as_float(w.y & 0xffff0000u), x0.w, t);
-    t = fmaf(__uint_as_float(w.z << 16), x1.x, t);
-    t = fmaf(__uint_as_float(w.z & 0xffff0000u), x1.y, t);
-    t = fmaf(__uint_as_float(w.w << 16), x1.z, t);
-    t = fmaf(__uint_as_float(w.w & 0xffff0000u), x1.w, t);
-  } else {
-    t = fmaf(__uint_as_float(w.x), x0.x, t);
-    t = fmaf(__uint_as_float(w.y), x0.y, t);
-    t = fmaf(__uint_as_float(w.z), x0.z, t);
-    t = fmaf(__uint_as_float(w.w), x0.w, t);
+// the better of two (value, index), ties to the lower index
+__device__ __forceinline__ void cl_better(float& bv, int& bi, float v, int i) {
+  if (v > bv || (v == bv && i < bi)) {
+    bv = v;
+    bi = i;
   }
 }
+template <int n>
+__device__ __forceinline__ void cl_best_of_lanes(float& bv, int& bi) {  // over n neighbouring lanes
+#pragma unroll
+  for (int o = n / 2; o > 0; o >>= 1) cl_better(bv, bi, __shfl_xor_sync(0xffffffffu, bv, o), __shfl_xor_sync(0xffffffffu, bi, o));
+}
+
 __device__ __forceinline__ int cl_feature(int pair) { return ((pair >> 3) << 4) + (pair & 7); }  // the first of a pair's features, its second is 8 further
 
-// A warp's pairs lie behind one another in memory.  It takes P of them through RT rows at a time (more rows take another
-// sweep of the weights, from L2); a K step of weights is in registers or on its way, the first before the wait for the
-// activations.  (Two to four steps ahead, in as many copies of the loop's body, were slower: tiny decoders by 4 %.)  A sum is made
-// in the same order whatever P and RT: K steps in order by each lane, the lanes in the xor tree.
-template <typename WT, int RT, int P>
-__device__ __forceinline__ void cl_dots(const ClParams& p, const ClDots& a, ClShared* sh) {
-  constexpr bool BF = sizeof(WT) == 2;
-  constexpr int N = RT * P * 2, CH = N < 16 ? N : 16;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_w = RT == 1 ? (a.np + kClWarps - 1) / kClWarps : (a.np / 2 + kClWarps - 1) / kClWarps * 2;  // pairs per warp
-  const int first = warp * n_w, cnt = max(0, min(n_w, a.np - first));
-  const int pair_len = a.steps * (kClUnit / 16);
+// Activations between the stages, sixteen bytes per four columns.  fp32: [row][K].  bf16: [eight columns][row][two columns] of
+// {hi, lo}, so that a lane of the MMA reads the two halves of its fragment of sixteen columns as two 64-bit words without conflicts.
+template <typename WT>
+__device__ __forceinline__ int cl_x_off(int K, int R, int row, int col) {  // bytes to columns col .. col + 3
+  return sizeof(WT) == 2 ? (((col >> 3) * R + row) * 4 + ((col & 7) >> 1)) * 8 : (row * K + col) * 4;
+}
+template <typename WT>
+__device__ __forceinline__ float4 cl_x_pack(const float4& x) {
+  if (sizeof(WT) == 4) return x;
+  uint32_t h0, h1, l0, l1;
+  split_pack(x.x, x.y, h0, l0);
+  split_pack(x.z, x.w, h1, l1);
+  return make_float4(__uint_as_float(h0), __uint_as_float(l0), __uint_as_float(h1), __uint_as_float(l1));
+}
+// (rounded products: the whole-pass kernel splits values that exist as such)
+__device__ __forceinline__ float4 cl_mul(const float4& a, const float4& b) {
+  return make_float4(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y), __fmul_rn(a.z, b.z), __fmul_rn(a.w, b.w));
+}
+
+struct ClEnv {
+  ClShared* sh;
+  const ClMine* mine;     // by ClKind
+  const ClRound* rounds;
+  const ClEntry* entries;
+  int tid, warp, lane, rank;
+  int R, rps;          // rows of the pass, rows per sequence; sequence b has cache slot b
+  uint32_t self, dst;  // shared memory of this CTA (as an address of the cluster's), of CTA tid mod 16: what goes to all CTAs is sent by a thread each
+};
+__device__ __forceinline__ uint32_t cl_bar_of(const ClParams& p, uint32_t cta, int which) {
+  return cta + p.lay.shared + (int)offsetof(ClShared, bar) + which * 8;
+}
+
+// ---- dot products of a stage ------------------------------------------------------------------------------------
+struct ClDots {
+  const unsigned char* W;
+  int kind, K, x;            // activations: where they are
+  int bar;                   // what brings them (ClBar), -1: nothing to wait for
+  unsigned bytes, parity;
+  bool norm;                 // the rows' norms are wanted
+  const float* gain;         // fp32: of that norm
+  float* logits;             // CL_HEAD: logits [row][vocab] or, without, the best of each (row, place)
+};
+
+// fp32: the rows' norms are applied here, for this CTA's own use; gains are asked for before the wait
+struct ClGain {
+  float4 g[2];
+  __device__ __forceinline__ void load(const float* gain, int d, int lane) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      g[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i * 128 + lane * 4 < d) g[i] = __ldg(reinterpret_cast<const float4*>(gain + i * 128 + lane * 4));
+    }
+  }
+};
+__device__ __forceinline__ void cl_norm_rows(const ClParams& p, const ClEnv& ev, const float* gain, const ClGain& cg) {
 #pragma unroll 1
-  for (int r0 = 0; r0 < a.R; r0 += RT) {
-    const int rows = RT == 1 ? 1 : min(RT, a.R - r0);
-    const uint4* w = reinterpret_cast<const uint4*>(a.W) + (size_t)first * pair_len + lane;
-    int ask_pairs = cnt, ask_steps = a.steps;  // pairs from the next request's on, steps left of them
+  for (int row = ev.warp; row < ev.R; row += kClWarps) {
+    const float* h = cl_at<float>(p.lay.h) + row * p.d;
+    float* y = cl_at<float>(p.lay.y) + row * p.d;
+    float s = 0.f;
+#pragma unroll 2
+    for (int c = ev.lane * 4; c < p.d; c += 128) {
+      const float4 v = *reinterpret_cast<const float4*>(h + c);
+      s = fmaf(v.x, v.x, s);
+      s = fmaf(v.y, v.y, s);
+      s = fmaf(v.z, v.z, s);
+      s = fmaf(v.w, v.w, s);
+    }
+    const float r = rsqrtf(warp_sum(s) / (float)p.d + p.eps);
+#pragma unroll 2
+    for (int i = 0; i * 128 + ev.lane * 4 < p.d; ++i) {
+      const int c = i * 128 + ev.lane * 4;
+      const float4 g = i == 0 ? cg.g[0] : i == 1 ? cg.g[1] : __ldg(reinterpret_cast<const float4*>(gain + c));
+      float4 v = *reinterpret_cast<const float4*>(h + c);
+      v.x = v.x * r * g.x;
+      v.y = v.y * r * g.y;
+      v.z = v.z * r * g.z;
+      v.w = v.w * r * g.w;
+      *reinterpret_cast<float4*>(y + c) = v;
+    }
+  }
+  __syncthreads();
+}
+
+// bf16: 1 / rms of the rows, needed behind the dot products only.  Per 128 features the squares of a pair, of the pair 32
+// further, the xor tree; then the groups.
+__device__ __forceinline__ void cl_row_scales(const ClParams& p, const ClEnv& ev) {
+  const int pairs = p.d / 2;
+#pragma unroll 1
+  for (int row = kClWarps - 1 - ev.warp; row < ev.R; row += kClWarps) {
+    const float* sq = cl_at<float>(p.lay.h) + row * pairs;
+    float part = 0.f;
+#pragma unroll 2
+    for (int g = 0; g < (pairs + 63) / 64; ++g) {
+      const int i = g * 64 + ev.lane;
+      const float v = warp_sum((i < pairs ? sq[i] : 0.f) + (i + 32 < pairs ? sq[i + 32] : 0.f));
+      if (ev.lane == (g & 31)) part += v;
+    }
+    const float s = warp_sum(part);
+    if (ev.lane == 0) ev.sh->inv[row] = rsqrtf(s / (float)p.d + p.eps);
+  }
+}
+
+// fp32.  A warp's pairs lie behind one another in memory, [pair][half][K].  It takes P of them through RT rows at a time (more
+// rows take another sweep of the weights, from L2); a K step of weights is in registers or on its way, the first before the
+// wait for the activations.  A sum is made in the same order whatever P and RT: K steps in order by each lane, the lanes in the xor tree.
+template <int RT, int P>
+__device__ __forceinline__ void cl_dots_f32(const ClParams& p, const ClEnv& ev, const ClDots& a) {
+  constexpr int N = RT * P * 2, CH = N < 16 ? N : 16;
+  const int warp = ev.warp, lane = ev.lane, R = ev.R;
+  const ClMine& me = ev.mine[a.kind];
+  const int np = me.np;
+  const int n_w = RT == 1 ? (np + kClWarps - 1) / kClWarps : (np / 2 + kClWarps - 1) / kClWarps * 2;  // pairs per warp
+  const int first = warp * n_w, cnt = max(0, min(n_w, np - first));
+  const int half_len = a.K / 4;  // in uint4
+#pragma unroll 1
+  for (int r0 = 0; r0 < R; r0 += RT) {
+    const int rows = RT == 1 ? 1 : min(RT, R - r0);
+    const uint4* w = reinterpret_cast<const uint4*>(a.W) + (size_t)first * 2 * half_len + lane;
+    int ask_pairs = cnt, ask_c = lane * 4;  // pairs from the next request's on, its column
     uint4 raw[P][2];
+#pragma unroll
+    for (int j = 0; j < P; ++j) raw[j][0] = raw[j][1] = make_uint4(0u, 0u, 0u, 0u);
     auto ask = [&]() {
       if (ask_pairs <= 0) return;
+      const bool in = ask_c < a.K;
 #pragma unroll
       for (int j = 0; j < P; ++j)
-        if (j < ask_pairs) {
-          raw[j][0] = __ldg(w + j * pair_len);
-          raw[j][1] = __ldg(w + j * pair_len + 32);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (!in) raw[j][h] = make_uint4(0u, 0u, 0u, 0u);
+          if (in && j < ask_pairs) raw[j][h] = __ldg(w + (2 * j + h) * half_len);
         }
-      w += kClUnit / 16;
-      if (--ask_steps == 0) {
-        ask_steps = a.steps;
+      w += 32;
+      ask_c += 128;
+      if (ask_c - lane * 4 >= a.K) {
+        w += 2 * P * half_len - (ask_c / 128) * 32;
+        ask_c = lane * 4;
         ask_pairs -= P;
-        w += (P - 1) * pair_len;
       }
     };
     ask();
-    if (r0 == 0) cl_begin(p, a, sh);
+    if (r0 == 0) {
+      ClGain cg;
+      if (a.norm) cg.load(a.gain, p.d, lane);
+      if (a.bar >= 0) cl_wait(ev.sh, p.sync, a.bar, a.bytes, a.parity);
+      if (a.norm) cl_norm_rows(p, ev, a.gain, cg);
+    }
     const float* const x = cl_at<float>(a.x) + r0 * a.K + lane * 4;
     const int room = a.K - lane * 4;
 #pragma unroll 1
@@ -307,19 +408,24 @@ __device__ __forceinline__ void cl_dots(const ClParams& p, const ClDots& a, ClSh
 #pragma unroll
       for (int i = 0; i < N; ++i) acc[i] = 0.f;
 #pragma unroll 1
-      for (int c0 = 0; c0 < a.K; c0 += ClElem<WT>::kStep) {
-        const bool in0 = c0 < room, in1 = BF && c0 + 128 < room;
+      for (int c0 = 0; c0 < a.K; c0 += 128) {
+        const bool in = c0 < room;
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
           if (RT == 1 || i < rows) {
-            float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;
-            if (in0) x0 = *reinterpret_cast<const float4*>(x + i * a.K + c0);
-            if (in1) x1 = *reinterpret_cast<const float4*>(x + i * a.K + c0 + 128);
+            float4 xv = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (in) xv = *reinterpret_cast<const float4*>(x + i * a.K + c0);
 #pragma unroll
             for (int j = 0; j < P; ++j)
               if (RT > 1 || j < cnt - at) {
-                cl_fma<WT>(acc[(i * P + j) * 2], raw[j][0], x0, x1);
-                cl_fma<WT>(acc[(i * P + j) * 2 + 1], raw[j][1], x0, x1);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  float& t = acc[(i * P + j) * 2 + h];
+                  t = fmaf(__uint_as_float(raw[j][h].x), xv.x, t);
+                  t = fmaf(__uint_as_float(raw[j][h].y), xv.y, t);
+                  t = fmaf(__uint_as_float(raw[j][h].z), xv.z, t);
+                  t = fmaf(__uint_as_float(raw[j][h].w), xv.w, t);
+                }
               }
           }
         }
@@ -332,30 +438,26 @@ __device__ __forceinline__ void cl_dots(const ClParams& p, const ClDots& a, ClSh
           float v[CH];
 #pragma unroll
           for (int i = 0; i < CH; ++i) v[i] = acc[g + i];
-          float v0 = warp_sum_scatter<CH>(v);
-          float v1 = __shfl_xor_sync(0xffffffffu, v0, 32 / CH);
+          const float v0 = warp_sum_scatter<CH>(v);
+          const float v1 = __shfl_xor_sync(0xffffffffu, v0, 32 / CH);
           const int pi = (g + lane / (32 / CH)) >> 1, row = r0 + pi / P, pl = first + at + pi % P;
-          if (lane % (64 / CH) == 0 && row < a.R && at + pi % P < cnt) {
-            if (!a.head) {
-              float* o = cl_at<float>(a.stg) + row * a.np + pl;
+          if (lane % (64 / CH) == 0 && row < R && at + pi % P < cnt) {
+            if (a.kind != CL_HEAD) {
+              float* o = cl_at<float>(p.lay.stg) + row * np + pl;
               o[0] = v0;
-              o[a.R * a.np] = v1;
+              o[R * np] = v1;
             } else {
-              const int f0 = cl_feature(a.p0 + pl);
-              const float inv = sh->inv[row];
-              v0 *= inv;
-              v1 *= inv;
+              const int f0 = cl_feature(me.p0 + pl);
               if (a.logits != nullptr) {
                 float* o = a.logits + (size_t)row * p.vocab + f0;
                 o[0] = v0;
                 o[8] = v1;
-              } else {  // only this lane touches its place
+              } else {  // only this lane touches its place; a NaN loses against everything, by itself
                 float2* best = cl_at<float2>(p.lay.best) + row * 4 * kClWarps + warp * 4 + pi % P;
-                const float2 o = *best;
-                const bool second = v1 > v0;
-                const float bv = second ? v1 : v0;
-                const int bi = second ? f0 + 8 : f0;
-                if (bv > o.x || (bv == o.x && bi < __float_as_int(o.y))) *best = make_float2(bv, __int_as_float(bi));
+                float2 o = *best;
+                if (v0 > o.x || (v0 == o.x && f0 < __float_as_int(o.y))) o = make_float2(v0, __int_as_float(f0));
+                if (v1 > o.x || (v1 == o.x && f0 + 8 < __float_as_int(o.y))) o = make_float2(v1, __int_as_float(f0 + 8));
+                *best = o;
               }
             }
           }
@@ -365,355 +467,547 @@ __device__ __forceinline__ void cl_dots(const ClParams& p, const ClDots& a, ClSh
   }
 }
 
-// the CTAs that hold a head: CTA c has heads c, c + 16, ...; with fewer heads than CTAs, `splits` CTAs share one
-__device__ __forceinline__ int cl_heads_of(int cta, int heads, int splits) {
-  if (heads >= kClCtas) return (heads - cta + kClCtas - 1) / kClCtas;
-  return cta < heads * splits ? 1 : 0;
-}
-
-struct ClEnv {
-  ClShared* sh;
-  int warp, lane, rank;
-  int R, rps;          // rows of the pass, rows per sequence; sequence b has cache slot b
-  uint32_t self, dst;  // shared memory of this CTA (as an address of the cluster's), of CTA tid mod 16: what goes to all CTAs is sent by a thread each
-  int stg;             // where the sums of the running stage are: two places in turn, a slow warp may still read the other
-  int hres;            // residual rows of this CTA's features: likewise two places in turn
-};
-__device__ __forceinline__ uint32_t cl_bar_of(const ClParams& p, uint32_t cta, int which) {
-  return cta + p.lay.shared + (int)offsetof(ClShared, bar) + which * 8;
-}
-__device__ __forceinline__ float4 cl_scale(float4 v, float s) { return make_float4(v.x * s, v.y * s, v.z * s, v.w * s); }
-
-// ---- epilogues: four pairs of a row at a time, behind one barrier of the CTA ------------------------------------------
-// Rotary embedding, cache entries, and q, k, v to the CTAs that work on the head; a thread per vector
-template <typename WT, int HD>
-__device__ __forceinline__ void cl_finish_qkv(const ClParams& p, const ClEnv& ev, const ClTab& t, bool send) {
-  constexpr int hp = HD / 2;
-  const ClMine me = ev.sh->mine[CL_QKV];
-  const float4* s0 = cl_at<float4>(ev.stg);
-  const float4* s1 = s0 + ev.R * me.nq;
-  const int per = p.d >> 1;
+// bf16: the weights of a stage on their way to a warp, through a ring of two halves in shared memory.  Every lane copies what it
+// will use itself, so nothing but its own wait stands between the copy and the use.
+struct ClRing {
+  const uint4* W;       // the matrix, this lane's part
+  const ClEntry* ent;   // this warp's list
+  int buf, steps, step, per, wrap_jump;  // halves in all and asked for so far, entries of a half
+  __device__ __forceinline__ void ask() {
+    if (step < steps) {
+      const ClEntry* e = ent + step * per;
+      uint32_t to = buf + (step & 1) * (kClAhead * 512);
 #pragma unroll 1
-  for (int i = kClThreads - 1 - threadIdx.x; i < ev.R * me.nq; i += kClThreads) {
-    const int row = (int)((unsigned)i * me.magic >> 20), pair = me.p0 + 4 * (i - row * me.nq);
-    const int which = pair >= 2 * per ? 2 : pair >= per ? 1 : 0, rem = pair - which * per, head = rem / hp, d0 = rem % hp;
-    const int pos = ev.sh->pos[row];
-    const float inv = ev.sh->inv[row];
-    float4 a = cl_scale(s0[i], inv), b = cl_scale(s1[i], inv);
-    if (which < 2) {
-      const float* rp = cl_at<float>(p.lay.rope) + row * 2 * hp + d0;
-      const float4 c = *reinterpret_cast<const float4*>(rp), s = *reinterpret_cast<const float4*>(rp + hp);
-      const float4 r = make_float4(a.x * c.x - b.x * s.x, a.y * c.y - b.y * s.y, a.z * c.z - b.z * s.z, a.w * c.w - b.w * s.w);
-      b = make_float4(b.x * c.x + a.x * s.x, b.y * c.y + a.y * s.y, b.z * c.z + a.z * s.z, b.w * c.w + a.w * s.w);
-      a = r;
+      for (int u = 0; u < per; ++u, to += kClAhead * 512 / per) {
+        const int4 v = *reinterpret_cast<const int4*>(e + u);
+        const uint4* w = W + v.x;
+        if ((short)v.y >= 0)
+#pragma unroll
+          for (int t = 0; t < kClTiles; ++t)
+            if (t < (v.z & 255)) cp_async16_to(to + t * 512, w + t * 32 + (t >= ((v.z >> 8) & 255) ? wrap_jump : 0));
+      }
+      ++step;
     }
-    if (which > 0) {
-      WT* dst = reinterpret_cast<WT*>(which == 1 ? t.kcache : t.vcache) + (((size_t)(row / ev.rps) * p.heads + head) * p.max_seq + pos) * HD + d0;
-      if constexpr (sizeof(WT) == 2) {  // the rows of this pass see what the cache will hold
-        const __nv_bfloat162 a0 = __floats2bfloat162_rn(a.x, a.y), a1 = __floats2bfloat162_rn(a.z, a.w);
-        const __nv_bfloat162 b0 = __floats2bfloat162_rn(b.x, b.y), b1 = __floats2bfloat162_rn(b.z, b.w);
-        if (pos >= 0) {
-          *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&a0), *reinterpret_cast<const uint32_t*>(&a1));
-          *reinterpret_cast<uint2*>(dst + hp) = make_uint2(*reinterpret_cast<const uint32_t*>(&b0), *reinterpret_cast<const uint32_t*>(&b1));
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  static __device__ __forceinline__ void cp_async16_to(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+  }
+};
+
+// One half of the ring.  CG: column groups of eight rows.  The accumulators go on from half to half; complete sums are left as
+// [place][class][row of the tile][two rows of the pass] of 128 bits, as a lane holds them: {half 0 of rows 2 q and 2 q + 1, half 1 of the same}.
+template <int CG>
+__device__ __forceinline__ void cl_mma_half(const ClParams& p, const ClEnv& ev, const ClDots& a, const ClEntry* e, int per, uint32_t from,
+                                            float (&acc)[kClTiles][CG][4]) {
+  const int g = ev.lane >> 2, q = ev.lane & 3, R = ev.R, Q = (R + 1) / 2;
+  const uint2* const x = cl_at<uint2>(a.x) + g * 4 + q;
+  int4 v = *reinterpret_cast<const int4*>(e);
+#pragma unroll 1
+  for (int u = 0; u < per; ++u, from += kClAhead * 512 / per) {
+    const int n = v.z & 255, kt = (short)v.y, slot = v.y >> 16, np = (v.z >> 16) & 255;
+    if (u + 1 < per) v = *reinterpret_cast<const int4*>(e + u + 1);
+    if (kt >= 0) {
+      uint2 b0[CG], b1[CG];
+#pragma unroll
+      for (int c = 0; c < CG; ++c) {
+        b0[c] = b1[c] = make_uint2(0u, 0u);
+        if (c * 8 + g < R) {
+          b0[c] = x[kt * 8 * R + c * 32];
+          b1[c] = x[kt * 8 * R + c * 32 + 4 * R];
         }
-        a = make_float4(__low2float(a0), __high2float(a0), __low2float(a1), __high2float(a1));
-        b = make_float4(__low2float(b0), __high2float(b0), __low2float(b1), __high2float(b1));
-      } else if (pos >= 0) {
-        *reinterpret_cast<float4*>(dst) = a;
-        *reinterpret_cast<float4*>(dst + hp) = b;
+      }
+#pragma unroll
+      for (int t = 0; t < kClTiles; ++t)
+        if (t < n) {
+          uint4 w;
+          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "r"(from + t * 512) : "memory");
+#pragma unroll
+          for (int c = 0; c < CG; ++c) {
+            mma_bf16_16816(acc[t][c], w, b0[c].x, b1[c].x);
+            mma_bf16_16816(acc[t][c], w, b0[c].y, b1[c].y);
+          }
+        }
+    }
+    if (slot >= 0) {
+      float4* o = cl_at<float4>(p.lay.red) + ((slot * kClasses + ev.warp) * 8 + g) * Q + q;
+#pragma unroll
+      for (int t = 0; t < kClTiles; ++t)
+#pragma unroll
+        for (int c = 0; c < CG; ++c) {
+          if (t < n && c * 4 + q < Q) o[t * np * kClasses * 8 * Q + c * 4] = make_float4(acc[t][c][0], acc[t][c][1], acc[t][c][2], acc[t][c][3]);
+          acc[t][c][0] = acc[t][c][1] = acc[t][c][2] = acc[t][c][3] = 0.f;
+        }
+    }
+  }
+}
+
+// bf16: both halves of a pair, each the classes of a piece in order, then the pieces
+__device__ __forceinline__ float2 cl_sum_pair(const ClParams& p, const ClRound& rd, int R, int row, int pair) {
+  const int Q = (R + 1) / 2, step = kClasses * 32 * Q;  // words of a place
+  const float* s = cl_at<float>(p.lay.red) + ((pair >> 3) - rd.tile0) * rd.np * step + ((pair & 7) * Q + (row >> 1)) * 4 + (row & 1);
+  float2 v = make_float2(0.f, 0.f);
+#pragma unroll 1
+  for (int i = 0; i < rd.np; ++i, s += step) {
+    float2 t = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < kClasses; ++c) {
+      t.x += s[c * 32 * Q];
+      t.y += s[c * 32 * Q + 2];
+    }
+    v = i == 0 ? t : make_float2(v.x + t.x, v.y + t.y);
+  }
+  return v;
+}
+
+// bf16 lm-head, one round: logits, or a thread's best of its row's pairs (a thread keeps to one row)
+__device__ __forceinline__ void cl_head_round(const ClParams& p, const ClEnv& ev, const ClMine& me, const ClRound& rd, float* logits, int row_log, float& bv, int& bi) {
+  const int row = ev.tid >> row_log;
+  if (row >= ev.R) return;
+  const float inv = ev.sh->inv[row];
+#pragma unroll 1
+  for (int j = ev.tid & ((1 << row_log) - 1); j < 4 * rd.n_quads; j += 1 << row_log) {
+    const int pair = me.p0 + 4 * rd.quad0 + j, f0 = cl_feature(pair);
+    const float2 s = cl_sum_pair(p, rd, ev.R, row, pair);
+    const float v0 = s.x * inv, v1 = s.y * inv;
+    if (logits != nullptr) {
+      float* o = logits + (size_t)row * p.vocab + f0;
+      o[0] = v0;
+      o[8] = v1;
+    } else {  // the whole-pass kernel compares a pair's halves first: a NaN in front hides the other
+      const float v = v1 > v0 ? v1 : v0;
+      const int fi = v1 > v0 ? f0 + 8 : f0;
+      if (v > bv || (v == bv && fi < bi)) {
+        bv = v;
+        bi = fi;
       }
     }
-    if (!send) continue;
-    const int hl = p.heads >= kClCtas ? head / kClCtas : 0;
-    const int off = p.lay.qkv + (((hl * 3 + which) * ev.R + row) * HD + d0) * 4;
+  }
+}
+
+// ---- epilogues: the values of a round, a thread per (row, pair), then behind a barrier their sending -------------------------
+template <typename WT, int HD>
+__device__ __forceinline__ void cl_values(const ClParams& p, const ClEnv& ev, const ClMine& me, const ClRound& rd, int kind) {
+  constexpr bool BF = sizeof(WT) == 2;
+  constexpr int hp = HD / 2;
+#pragma unroll 1
+  for (int i = ev.tid; i < 4 * ev.R * rd.n_quads; i += kClThreads) {
+    const int v = i >> 2, row = (int)((unsigned)v * rd.magic >> 20), pl = 4 * (rd.quad0 + v - row * rd.n_quads) + (i & 3), pair = me.p0 + pl;
+    float* o = cl_at<float>(p.lay.stg) + row * me.np + pl;
+    float2 s = BF ? cl_sum_pair(p, rd, ev.R, row, pair) : make_float2(o[0], o[ev.R * me.np]);
+    if (BF && (kind == CL_QKV || kind == CL_GATE_UP)) {
+      const float inv = ev.sh->inv[row];
+      s.x *= inv;
+      s.y *= inv;
+    }
+    if (kind == CL_QKV) {  // rotary embedding of q and k
+      if (pair < p.d) {
+        const float* rp = cl_at<float>(p.lay.rope) + row * 2 * hp + pair % hp;
+        const float c = rp[0], n = rp[hp];
+        const float r = s.x * c - s.y * n;
+        s.y = s.y * c + s.x * n;
+        s.x = r;
+      }
+    } else if (kind == CL_GATE_UP) {
+      s.x = __fmul_rn(s.x / (1.0f + __expf(-s.x)), s.y);
+    } else {  // new residual rows
+      float* own = cl_at<float>(p.lay.hres) + row * p.lay.resid_np + pl;
+      const int half_len = p.lay.rows * p.lay.resid_np;
+      s.x = own[0] + s.x;
+      s.y = own[half_len] + s.y;
+      own[0] = s.x;
+      own[half_len] = s.y;
+    }
+    o[0] = s.x;
+    o[ev.R * me.np] = s.y;
+  }
+}
+
+// Quarters of a q row lie eight words further apart than they are long: threads that share a key read them without conflicts.
+template <int HD>
+struct ClQ {
+  static constexpr int kLd = HD + 32;  // floats of a row
+  static __device__ __forceinline__ int at(int d) { return d / (HD / 4) * (HD / 4 + 8) + d % (HD / 4); }
+};
+
+// q, k, v to the CTAs that work on the head, a thread per four columns
+template <typename WT, int HD>
+__device__ __forceinline__ void cl_send_qkv(const ClParams& p, const ClEnv& ev, const ClMine& me, const ClRound& rd) {
+  constexpr int hp = HD / 2;
+  const int per = p.d >> 1, rows_all = p.lay.heads_per_cta * ev.R, total = ev.R * rd.n_quads;
+#pragma unroll 1
+  for (int i = ev.tid; i < 2 * total; i += kClThreads) {
+    const int half = i >= total ? 1 : 0, v = i - half * total;
+    const int row = (int)((unsigned)v * rd.magic >> 20), quad = rd.quad0 + v - row * rd.n_quads, pair = me.p0 + 4 * quad;
+    const int which = pair >= 2 * per ? 2 : pair >= per ? 1 : 0, rem = pair - which * per, head = rem / hp, d0 = rem % hp + half * hp;
+    const float4 x = cl_at<float4>(p.lay.stg)[(half * ev.R + row) * (me.np / 4) + quad];
+    const int hr = (p.heads >= kClCtas ? head / kClCtas : 0) * ev.R + row;
+    const int to = which == 0 ? p.lay.qkv + (hr * ClQ<HD>::kLd + ClQ<HD>::at(d0)) * 4
+                              : p.lay.qkv + rows_all * ClQ<HD>::kLd * 4 + (((which - 1) * rows_all + hr) * HD + d0) * (int)sizeof(WT);
+    const __nv_bfloat162 x0 = __floats2bfloat162_rn(x.x, x.y), x1 = __floats2bfloat162_rn(x.z, x.w);  // as the cache will hold them
 #pragma unroll 1
     for (int s = 0, cta = p.heads >= kClCtas ? head % kClCtas : head; s < p.lay.splits; ++s, cta += p.heads) {
-      const uint32_t to = cl_map(ev.self, cta), bar = cl_bar_of(p, to, CL_BAR_QKV);
-      cl_send4(to + off, a, bar);
-      cl_send4(to + off + hp * 4, b, bar);
+      const uint32_t dst = cl_map(ev.self, cta), bar = cl_bar_of(p, dst, CL_BAR_QKV);
+      if (which == 0 || sizeof(WT) == 4)
+        cl_send4(dst + to, x, bar);
+      else
+        cl_send2(dst + to, __uint_as_float(*reinterpret_cast<const uint32_t*>(&x0)), __uint_as_float(*reinterpret_cast<const uint32_t*>(&x1)), bar);
     }
   }
 }
 
-// (what goes to all CTAs: a half-warp per vector, a lane per CTA)
-__device__ __forceinline__ void cl_finish_gate_up(const ClParams& p, const ClEnv& ev) {
-  const ClMine me = ev.sh->mine[CL_GATE_UP];
-  const float4* s0 = cl_at<float4>(ev.stg);
-  const float4* s1 = s0 + ev.R * me.nq;
-  const uint32_t bar = cl_bar_of(p, ev.dst, CL_BAR_U);
-  auto f = [](float g, float u) { return g / (1.0f + __expf(-g)) * u; };
+// What goes to all CTAs: a half-warp per four columns, a lane per CTA.  SwiGLU: u.  Residual rows: fp32 as they are; bf16 times the
+// next norm's gain, and the squares of the pairs.
+template <typename WT>
+__device__ __forceinline__ void cl_send_all(const ClParams& p, const ClEnv& ev, const ClMine& me, const ClRound& rd, int kind, int gain_out) {
+  const float* gain = cl_at<float>(p.lay.gain) + gain_out * 2 * p.lay.resid_np;
+  const uint32_t bar = cl_bar_of(p, ev.dst, kind == CL_GATE_UP ? CL_BAR_U : CL_BAR_H);
 #pragma unroll 1
-  for (int i = threadIdx.x >> 4; i < ev.R * me.nq; i += kClThreads / 16) {
-    const int row = (int)((unsigned)i * me.magic >> 20), j = me.p0 + 4 * (i - row * me.nq);
-    const float inv = ev.sh->inv[row];
-    const float4 g = cl_scale(s0[i], inv), u = cl_scale(s1[i], inv);
-    cl_send4(ev.dst + p.lay.u + (row * p.f + j) * 4, make_float4(f(g.x, u.x), f(g.y, u.y), f(g.z, u.z), f(g.w, u.w)), bar);
+  for (int i = ev.tid >> 4; i < ev.R * rd.n_quads; i += kClThreads / 16) {
+    const int row = (int)((unsigned)i * rd.magic >> 20), quad = rd.quad0 + i - row * rd.n_quads, pair = me.p0 + 4 * quad;
+    const float4* s = cl_at<float4>(p.lay.stg) + row * (me.np / 4) + quad;
+    const float4 a = s[0];
+    if (kind == CL_GATE_UP) {
+      cl_send4(ev.dst + p.lay.u + cl_x_off<WT>(p.f, ev.R, row, pair), cl_x_pack<WT>(a), bar);
+      continue;
+    }
+    const float4 b = s[ev.R * (me.np / 4)];
+    const int f0 = cl_feature(pair);
+    if (sizeof(WT) == 4) {
+      cl_send4(ev.dst + p.lay.h + (row * p.d + f0) * 4, a, bar);
+      cl_send4(ev.dst + p.lay.h + (row * p.d + f0 + 8) * 4, b, bar);
+    } else {
+      const float4 ga = *reinterpret_cast<const float4*>(gain + 4 * quad), gb = *reinterpret_cast<const float4*>(gain + p.lay.resid_np + 4 * quad);
+      cl_send4(ev.dst + p.lay.y + cl_x_off<WT>(p.d, ev.R, row, f0), cl_x_pack<WT>(cl_mul(a, ga)), bar);
+      cl_send4(ev.dst + p.lay.y + cl_x_off<WT>(p.d, ev.R, row, f0 + 8), cl_x_pack<WT>(cl_mul(b, gb)), bar);
+      cl_send4(ev.dst + p.lay.h + (row * (p.d / 2) + pair) * 4,
+               make_float4(fmaf(a.x, a.x, b.x * b.x), fmaf(a.y, a.y, b.y * b.y), fmaf(a.z, a.z, b.z * b.z), fmaf(a.w, a.w, b.w * b.w)), bar);
+    }
   }
-}
-
-// new residual rows, and the same times the next norm's gain
-__device__ __forceinline__ void cl_finish_resid(const ClParams& p, ClEnv& ev, const ClTab& t) {
-  const ClMine me = ev.sh->mine[CL_O];
-  const int half_len = p.lay.rows * p.lay.resid_np;
-  const int next = p.lay.hres + (ev.hres == p.lay.hres ? half_len * 8 : 0);
-  const float4* sum = cl_at<float4>(ev.stg);
-  const uint32_t bar = cl_bar_of(p, ev.dst, CL_BAR_H);
-  const float* gain = cl_at<float>(p.lay.gain) + t.gain_out * 2 * p.lay.resid_np;
-#pragma unroll 1
-  for (int i = threadIdx.x >> 4; i < 2 * ev.R * me.nq; i += kClThreads / 16) {
-    const int rr = (int)((unsigned)i * me.magic >> 20), half = rr >= ev.R ? 1 : 0, row = rr - half * ev.R;
-    const int pl = 4 * (i - rr * me.nq), at = half * half_len + row * p.lay.resid_np + pl;
-    const float4 v = sum[i], o = *reinterpret_cast<const float4*>(cl_at<float>(ev.hres) + at);
-    const float4 g = *reinterpret_cast<const float4*>(gain + half * p.lay.resid_np + pl);
-    const float4 n = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
-    if ((threadIdx.x & 15) == 0) *reinterpret_cast<float4*>(cl_at<float>(next) + at) = n;
-    const int off = (row * p.d + cl_feature(me.p0 + pl) + half * 8) * 4;
-    cl_send4(ev.dst + p.lay.y + off, make_float4(n.x * g.x, n.y * g.y, n.z * g.z, n.w * g.w), bar);
-    cl_send4(ev.dst + p.lay.h + off, n, bar);
-  }
-  ev.hres = next;
 }
 
 // ---- attention ------------------------------------------------------------------------------------------------
-// The keys of a (row, head) in blocks of KPB, dealt by absolute index over `splits` CTAs and their eight warps:
-// block kb belongs to place kb mod (8 splits) = warp * splits + split.  LPK lanes hold a key, sixteen dimensions each;
-// every lane group keeps its own running maximum, the groups are combined at the end.
+// A head's keys in chunks of 64, dealt to places: bf16 chunk c to place c mod 8, which walks its chunks with a running maximum;
+// fp32 every chunk a place.  Place j belongs to CTA j mod `splits` of the head's; a team of four warps takes one (head,
+// sequence, place) at a time, up to eight rows of the sequence together.  What a row leaves in a place (sum, maximum, output)
+// goes to the head's first CTA, which adds the places in order and sends the result to everybody.
 template <typename WT, int HD>
 struct ClAttn {
-  static constexpr int LPK = HD / 16, KPB = 32 / LPK, V = ClElem<WT>::kLane, NV = 16 / V;
-  uint4 rk[NV], rv[NV];  // a block as it lies in the cache
-  __device__ __forceinline__ void load(const WT* gk, const WT* gv, int key, int dl, bool in) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      rk[j] = rv[j] = make_uint4(0u, 0u, 0u, 0u);
-      if (in) {
-        rk[j] = __ldcg(reinterpret_cast<const uint4*>(gk + (size_t)key * HD + (j * LPK + dl) * V));
-        rv[j] = __ldcg(reinterpret_cast<const uint4*>(gv + (size_t)key * HD + (j * LPK + dl) * V));
-      }
-    }
-  }
-  static __device__ __forceinline__ void widen(const uint4 (&r)[NV], float (&o)[16]) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      const uint32_t w[4] = {r[j].x, r[j].y, r[j].z, r[j].w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (sizeof(WT) == 2) {
-          o[j * V + 2 * e] = __uint_as_float(w[e] << 16);
-          o[j * V + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-        } else {
-          o[j * V + e] = __uint_as_float(w[e]);
-        }
-      }
-    }
-  }
+  static constexpr bool BF = sizeof(WT) == 2;
+  static constexpr int C = kAttnChunk, PARTS = BF ? 4 : 2, QD = HD / PARTS;  // threads per key, dimensions of each
+  static constexpr int VPR = HD * (int)sizeof(WT) / 16;                      // 16-byte vectors of a row
+  static constexpr int KLD = HD + 16 / (int)sizeof(WT);                      // elements of a key row, padded
+  static constexpr int OH = BF ? 2 : 1;                                      // halves of a chunk's keys summed by themselves
+  static constexpr int OT = HD * OH > kClTeam ? HD * OH / kClTeam : 1;       // (dimension, half) of a thread
+  static constexpr int PLD = HD + 4;                                         // floats of a row in a place: output, maximum, sum
+  static __device__ __forceinline__ int places(int pos) { return pos < 0 ? 0 : BF ? min(kAttnSplits, pos / C + 1) : pos / C + 1; }
 };
+__host__ __device__ constexpr int cl_team_bytes(int hd, int elem_bytes) {
+  return kAttnChunk * (hd * elem_bytes + 16) + kAttnChunk * hd * elem_bytes + kClAttnRows * kAttnChunk * 4;
+}
+static_assert(kAttnChunk * (64 * 2 + 16) >= kClAttnRows * 64 * 4, "halves are added where the keys were");
+__device__ __forceinline__ void cl_team_sync(int team) { asm volatile("bar.sync %0, %1;" ::"r"(2 + team), "n"(kClTeam) : "memory"); }
 
-// row r of sequence b; `blk` holds the place's first block as far as it lies in the cache, if `loaded`
-template <typename WT, int HD>
-__device__ __forceinline__ void cl_attend(const ClParams& p, const ClEnv& ev, const WT* gk, const WT* gv, int hl, int b, int r, int place, int split,
-                                          ClAttn<WT, HD>& blk, bool loaded) {
+template <typename WT, int HD, int RM>
+__device__ __forceinline__ void cl_attend(const ClParams& p, const ClEnv& ev, const WT* gk, const WT* gv, int hl, int b, int first_row, int place, bool& waited,
+                                          unsigned qkv_bytes, unsigned parity) {
   using A = ClAttn<WT, HD>;
-  constexpr int LPK = A::LPK, KPB = A::KPB, V = A::V, NV = A::NV;
-  const int lane = ev.lane, kl = lane / LPK, dl = lane % LPK, R = ev.R, rps = ev.rps;
-  const int row = b * rps + r, pos = ev.sh->pos[row];
-  const int S = p.lay.splits, first = place * S + split;
-  if (first * KPB > pos) return;  // also a row that carries nothing
-  const int p_last = ev.sh->pos[b * rps + rps - 1], base_pos = max(0, p_last - rps + 1);
-  const float* q = cl_at<float>(p.lay.qkv) + (hl * 3 * R + row) * HD;
-  const float* sk = cl_at<float>(p.lay.qkv) + (hl * 3 + 1) * R * HD;
-  const float* sv = sk + R * HD;
-  float m = -INFINITY, l = 0.f, o[16];
+  constexpr bool BF = A::BF;
+  constexpr int C = A::C;
+  const int team = ev.tid / kClTeam, tt = ev.tid % kClTeam, w4 = tt >> 5, lane = ev.lane;
+  const int R = ev.R, row0 = b * ev.rps + first_row, rps = RM == 1 ? 1 : min(RM, ev.rps - first_row), rows_all = p.lay.heads_per_cta * R;
+  const int max_pos = ev.sh->pos[row0 + rps - 1];
+  // positions of a sequence's rows follow one another, and with them the keys that are not in the cache
+  const int new_pos = ev.sh->pos[b * ev.rps + ev.rps - 1] - ev.rps + 1, base_pos = max(0, new_pos);
+  WT* sK = cl_at<WT>(p.lay.team + team * p.lay.team_bytes);
+  WT* sV = sK + C * A::KLD;
+  float* sS = reinterpret_cast<float*>(sV + C * HD);  // [row][C]
+  float* sO = reinterpret_cast<float*>(sK);           // at the end: [row][HD]
+  const float* sq = cl_at<float>(p.lay.qkv) + (hl * R + row0) * ClQ<HD>::kLd;
+  const WT* nk = reinterpret_cast<const WT*>(cl_at<float>(p.lay.qkv) + rows_all * ClQ<HD>::kLd) + (hl * R + b * ev.rps) * HD;  // keys of this pass
+  const WT* nv = nk + rows_all * HD;
+  float* s_m = ev.sh->att_m[team];
+  float* s_l = ev.sh->att_l[team];
+  float* s_a = ev.sh->att_a[team];
+  float o[A::OT][RM];
 #pragma unroll
-  for (int e = 0; e < 16; ++e) o[e] = 0.f;
+  for (int u = 0; u < A::OT; ++u)
+#pragma unroll
+    for (int i = 0; i < RM; ++i) o[u][i] = 0.f;
+  if (tt < rps) {
+    s_m[tt] = -INFINITY;
+    s_l[tt] = 0.f;
+  }
 #pragma unroll 1
-  for (int kb = first; kb * KPB <= pos; kb += kClWarps * S) {
-    const int key = kb * KPB + kl;
-    if (!loaded) blk.load(gk, gv, key, dl, key < base_pos);
-    loaded = false;
-    float k[16], v[16];
-    A::widen(blk.rk, k);
-    A::widen(blk.rv, v);
-    if (key >= base_pos && key <= pos) {
-      const int kr = b * rps + rps - 1 - (p_last - key);
+  for (int c = place; c * C <= max_pos; c += BF ? kAttnSplits : 1 << 24) {
+    const int key0 = c * C, n_keys = min(C, max_pos + 1 - key0);  // keys any row can see
+    // what lies in the cache is asked for before the rows of the pass are there
+    const int n_old = min(n_keys, base_pos - key0);
+#pragma unroll 2
+    for (int v = tt; v < n_old * A::VPR; v += kClTeam) {
+      cp_async16(sK + v / A::VPR * A::KLD + v % A::VPR * (16 / (int)sizeof(WT)), reinterpret_cast<const uint4*>(gk + (size_t)key0 * HD) + v);
+      cp_async16(reinterpret_cast<uint4*>(sV) + v, reinterpret_cast<const uint4*>(gv + (size_t)key0 * HD) + v);
+    }
+    if (!waited) {
+      cl_wait(ev.sh, p.sync, CL_BAR_QKV, qkv_bytes, parity);
+      waited = true;
+    }
+#pragma unroll 1
+    for (int v = max(0, n_old) * A::VPR + tt; v < n_keys * A::VPR; v += kClTeam) {
+      const int from = (key0 - new_pos) * A::VPR + v;
+      *reinterpret_cast<uint4*>(sK + v / A::VPR * A::KLD + v % A::VPR * (16 / (int)sizeof(WT))) = reinterpret_cast<const uint4*>(nk)[from];
+      reinterpret_cast<uint4*>(sV)[v] = reinterpret_cast<const uint4*>(nv)[from];
+    }
+    cp_async_wait_all();
+    cl_team_sync(team);
+    // scores
+#pragma unroll 1
+    for (int key = tt / A::PARTS; key < C; key += kClTeam / A::PARTS) {
+      const int part = tt % A::PARTS;
+      const WT* kr = sK + key * A::KLD + part * A::QD;
+      const float* q = sq + ClQ<HD>::at(part * A::QD);
+      float acc[RM];
 #pragma unroll
-      for (int j = 0; j < NV; ++j)
+      for (int i = 0; i < RM; ++i) acc[i] = 0.f;
+      if (key < n_keys) {
+#pragma unroll(RM == 1 ? 4 : 1)
+        for (int e = 0; e < A::QD; e += 4) {
+          const float4 k = load4(kr + e);
+          const float* qe = q + e + e / (HD / 4) * 8;
 #pragma unroll
-        for (int e = 0; e < V; e += 4) {
-          const int dim = (j * LPK + dl) * V + e;
-          const float4 x = *reinterpret_cast<const float4*>(sk + kr * HD + dim), c = *reinterpret_cast<const float4*>(sv + kr * HD + dim);
-          k[j * V + e] = x.x, k[j * V + e + 1] = x.y, k[j * V + e + 2] = x.z, k[j * V + e + 3] = x.w;
-          v[j * V + e] = c.x, v[j * V + e + 1] = c.y, v[j * V + e + 2] = c.z, v[j * V + e + 3] = c.w;
+          for (int i = 0; i < RM; ++i)
+            if (RM == 1 || i < rps) {
+              const float4 qv = *reinterpret_cast<const float4*>(qe + i * ClQ<HD>::kLd);
+              acc[i] = fmaf(k.x, qv.x, acc[i]);
+              acc[i] = fmaf(k.y, qv.y, acc[i]);
+              acc[i] = fmaf(k.z, qv.z, acc[i]);
+              acc[i] = fmaf(k.w, qv.w, acc[i]);
+            }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+        if (RM == 1 || i < rps) {
+          float s = acc[i];
+#pragma unroll
+          for (int w = 1; w < A::PARTS; w <<= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
+          if (part == 0) sS[i * C + key] = s * p.scale;
         }
     }
-    float s4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int j = 0; j < NV; ++j)
-#pragma unroll
-      for (int e = 0; e < V; e += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(q + (j * LPK + dl) * V + e);
-        s4[0] = fmaf(x.x, k[j * V + e], s4[0]);
-        s4[1] = fmaf(x.y, k[j * V + e + 1], s4[1]);
-        s4[2] = fmaf(x.z, k[j * V + e + 2], s4[2]);
-        s4[3] = fmaf(x.w, k[j * V + e + 3], s4[3]);
+    cl_team_sync(team);
+    // softmax of the chunk, a warp per row
+#pragma unroll 1
+    for (int i = w4; i < rps; i += kClTeam / 32) {
+      const int n = min(C, ev.sh->pos[row0 + i] + 1 - key0);
+      if (n <= 0) {  // the row sees nothing here
+        if (lane == 0) s_a[i] = 1.f;
+        sS[i * C + lane] = 0.f;
+        sS[i * C + lane + 32] = 0.f;
+        continue;
       }
-    float s = (s4[0] + s4[1]) + (s4[2] + s4[3]);
-#pragma unroll
-    for (int w = 1; w < LPK; w <<= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
-    s = key <= pos ? s * p.scale : -INFINITY;
-    const float mn = fmaxf(m, s), ms = mn == -INFINITY ? 0.f : mn;
-    const float a = __expf(m - ms), pr = __expf(s - ms);
-    m = mn;
-    l = fmaf(l, a, pr);
-#pragma unroll
-    for (int e = 0; e < 16; ++e) o[e] = fmaf(pr, v[e], o[e] * a);
-  }
-  constexpr int LEFT = 16 / KPB;  // dimensions a lane ends up with
-  float mx = m;
-#pragma unroll
-  for (int w = LPK; w < 32; w <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
-  const float fac = __expf(m - mx);  // the first block has a key the row sees: mx is finite
-  l *= fac;
-#pragma unroll
-  for (int w = LPK; w < 32; w <<= 1) l += __shfl_xor_sync(0xffffffffu, l, w);
-#pragma unroll
-  for (int e = 0; e < 16; ++e) o[e] *= fac;
-  int at = 0;  // first of the lane's sixteen values
-#pragma unroll
-  for (int w = 16, n = 8; w >= LPK; w >>= 1, n >>= 1) {
-    const bool up = (lane & w) != 0;
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-      if (e < n) {
-        const float keep = up ? o[e + n] : o[e], give = up ? o[e] : o[e + n];
-        o[e] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+      const float s0 = lane < n ? sS[i * C + lane] : -INFINITY, s1 = lane + 32 < n ? sS[i * C + lane + 32] : -INFINITY;
+      const float m_old = s_m[i], m_new = fmaxf(m_old, warp_max(fmaxf(s0, s1)));
+      const float p0 = lane < n ? __expf(s0 - m_new) : 0.f, p1 = lane + 32 < n ? __expf(s1 - m_new) : 0.f;
+      sS[i * C + lane] = p0;
+      sS[i * C + lane + 32] = p1;
+      const float sum = warp_sum(p0 + p1);
+      if (lane == 0) {
+        const float alpha = __expf(m_old - m_new);  // 0 on the row's first chunk
+        s_a[i] = alpha;
+        s_m[i] = m_new;
+        s_l[i] = BF ? fmaf(s_l[i], alpha, sum) : sum;
       }
-    at += up ? n : 0;
-  }
-  float* dst = cl_at<float>(p.lay.part) + ((hl * R + row) * kClWarps + place) * (HD + 4);
-  const int dim = ((at / V) * LPK + dl) * V + at % V;
+    }
+    cl_team_sync(team);
+    // output, keys in order
 #pragma unroll
-  for (int e = 0; e < LEFT; e += 2) *reinterpret_cast<float2*>(dst + dim + e) = make_float2(o[e], o[e + 1]);
-  if (lane == 0) *reinterpret_cast<float2*>(dst + HD) = make_float2(mx, l);
+    for (int u = 0; u < A::OT; ++u) {
+      const int id = tt + u * kClTeam, d = id % HD, half = id / HD;
+      if (half < A::OH) {
+        if (BF)
+#pragma unroll
+          for (int i = 0; i < RM; ++i)
+            if (RM == 1 || i < rps) o[u][i] *= s_a[i];
+        const int lo = half * (C / A::OH), hi = min(n_keys, lo + C / A::OH);
+        int k = lo;
+#pragma unroll(RM == 1 ? 2 : 1)
+        for (; k + 4 <= hi; k += 4) {
+          float v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[e] = to_f32(sV[(k + e) * HD + d]);
+#pragma unroll
+          for (int i = 0; i < RM; ++i)
+            if (RM == 1 || i < rps) {
+              const float4 p4 = *reinterpret_cast<const float4*>(sS + i * C + k);
+              o[u][i] = fmaf(p4.x, v[0], o[u][i]);
+              o[u][i] = fmaf(p4.y, v[1], o[u][i]);
+              o[u][i] = fmaf(p4.z, v[2], o[u][i]);
+              o[u][i] = fmaf(p4.w, v[3], o[u][i]);
+            }
+        }
+#pragma unroll 1
+        for (; k < hi; ++k) {
+          const float v = to_f32(sV[k * HD + d]);
+#pragma unroll
+          for (int i = 0; i < RM; ++i)
+            if (RM == 1 || i < rps) o[u][i] = fmaf(sS[i * C + k], v, o[u][i]);
+        }
+      }
+    }
+    cl_team_sync(team);  // the buffers are free again
+  }
+  // first + second half of the keys
+  if constexpr (A::OH == 2 && A::OT == 1) {
+    if (tt >= HD)
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+        if (RM == 1 || i < rps) sO[i * HD + tt - HD] = o[0][i];
+    cl_team_sync(team);
+    if (tt < HD)
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+        if (RM == 1 || i < rps) o[0][i] += sO[i * HD + tt];
+  } else if constexpr (A::OH == 2) {
+#pragma unroll
+    for (int i = 0; i < RM; ++i) o[0][i] += o[A::OT - 1][i];
+  }
+  // ... to the head's first CTA
+  const bool here = p.lay.splits == 1 || ev.rank < p.heads, live = !cl_aborted(ev.sh);
+  const uint32_t owner = cl_map(ev.self, here ? ev.rank : ev.rank % p.heads), bar = cl_bar_of(p, owner, CL_BAR_PART);
+#pragma unroll
+  for (int i = 0; i < RM; ++i) {
+    if ((RM > 1 && i >= rps) || place >= A::places(ev.sh->pos[row0 + i])) continue;
+    const int at = p.lay.part + ((hl * R + row0 + i) * p.lay.part_slots + place) * A::PLD * 4;
+    if (tt < HD) {
+      if (here)
+        *cl_at<float>(at + tt * 4) = o[0][i];
+      else if (live)
+        cl_send1(owner + at + tt * 4, o[0][i], bar);
+    }
+    if (tt == i) {
+      if (here)
+        *cl_at<float2>(at + HD * 4) = make_float2(s_m[i], s_l[i]);
+      else if (live)
+        cl_send2(owner + at + HD * 4, s_m[i], s_l[i], bar);
+    }
+  }
+  cl_team_sync(team);  // the rows' state is used by the next item
 }
 
-// Attention of this CTA's heads and the sending of its outcome.  One CTA per head sends the output, several per head
-// their unnormalised sums and (max, sum).
+// The places of a row and head in order, four dimensions
 template <typename WT, int HD>
-__device__ __forceinline__ void cl_attention(const ClParams& p, const ClEnv& ev, const ClTab& t, int nh, unsigned parity) {
-  using A = ClAttn<WT, HD>;
-  const int S = p.lay.splits, R = ev.R, rps = ev.rps;
-  const bool many = p.heads >= kClCtas;
-  const int split = many ? 0 : ev.rank / p.heads;
-  const int head0 = many ? ev.rank : ev.rank - split * p.heads;
-  auto cache_at = [&](void* base, int hl, int b) {
-    return reinterpret_cast<const WT*>(base) + ((size_t)b * p.heads + head0 + hl * kClCtas) * p.max_seq * HD;
-  };
-  const int n_seq = R / rps;
-  A blk;
-  {  // the first block of this warp's first place, as far as it lies in the cache: asked for before the wait
-    const int p_last = ev.sh->pos[rps - 1], key = (ev.warp * S + split) * A::KPB + ev.lane / A::LPK;
-    blk.load(cache_at(t.kcache, 0, 0), cache_at(t.vcache, 0, 0), key, ev.lane % A::LPK, key < max(0, p_last - rps + 1));
+__device__ __forceinline__ float4 cl_fold(const float* q, int n, int dim) {
+  constexpr int LD = ClAttn<WT, HD>::PLD;
+  constexpr bool BF = ClAttn<WT, HD>::BF;
+  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (n <= 0) return o;
+  float mx = -INFINITY, l = 0.f;
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    const float2 ml = *reinterpret_cast<const float2*>(q + j * LD + HD);
+    if (!BF || ml.y > 0.f) mx = fmaxf(mx, ml.x);
   }
-  cl_wait(ev.sh, p.sync, CL_BAR_QKV, (unsigned)(nh * 3 * R * HD * 4), parity);
-  int turn = ev.warp;  // short contexts fill only the first places: other warps take them in every item
-  bool loaded = true;
+  auto weight = [&](const float2& ml) { return !BF || ml.y > 0.f ? __expf(ml.x - mx) : 0.f; };
+  auto add = [&](int j, float w) {
+    const float4 v = *reinterpret_cast<const float4*>(q + j * LD + dim);
+    o.x = fmaf(v.x, w, o.x);
+    o.y = fmaf(v.y, w, o.y);
+    o.z = fmaf(v.z, w, o.z);
+    o.w = fmaf(v.w, w, o.w);
+  };
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    const float2 ml = *reinterpret_cast<const float2*>(q + j * LD + HD);
+    const float w = weight(ml);
+    l = fmaf(ml.y, w, l);
+    if (!BF) add(j, w);
+  }
+  if (BF) {  // as FoldStats: the sum goes into the weights
+    const float inv_l = l > 0.f ? 1.0f / l : 0.f;
+#pragma unroll 1
+    for (int j = 0; j < n; ++j) add(j, weight(*reinterpret_cast<const float2*>(q + j * LD + HD)) * inv_l);
+    return o;
+  }
+  const float inv_l = 1.0f / l;
+  return make_float4(o.x * inv_l, o.y * inv_l, o.z * inv_l, o.w * inv_l);
+}
+
+// Attention of this CTA's heads, its cache entries, and the sending of the outcome
+template <typename WT, int HD>
+__device__ __forceinline__ void cl_attention(const ClParams& p, const ClEnv& ev, const ClTab& t, int nh, unsigned& phases) {
+  using A = ClAttn<WT, HD>;
+  const int S = p.lay.splits, R = ev.R, rps = ev.rps, n_seq = R / rps;
+  const bool many = p.heads >= kClCtas;
+  const int split = many ? 0 : ev.rank / p.heads, head0 = many ? ev.rank : ev.rank - split * p.heads;
+  auto phase = [&](int which) {
+    const unsigned par = (phases >> which) & 1u;
+    phases ^= 1u << which;
+    return par;
+  };
+  auto cache_at = [&](void* base, int hl, int b) {
+    return reinterpret_cast<WT*>(base) + ((size_t)b * p.heads + head0 + hl * kClCtas) * p.max_seq * HD;
+  };
+  const unsigned qkv_bytes = (unsigned)(nh * R * (HD * 4 + 2 * HD * (int)sizeof(WT))), parity = phase(CL_BAR_QKV);
+  const int team = ev.tid / kClTeam;
+  bool waited = false;
+  int turn = 0;
 #pragma unroll 1
   for (int hl = 0; hl < nh; ++hl)
 #pragma unroll 1
     for (int b = 0; b < n_seq; ++b) {
-      const WT *gk = cache_at(t.kcache, hl, b), *gv = cache_at(t.vcache, hl, b);
+      const int n = A::places(ev.sh->pos[b * rps + rps - 1]);
 #pragma unroll 1
-      for (int r0 = 0; r0 < rps; ++r0) {
-        cl_attend<WT, HD>(p, ev, gk, gv, hl, b, r0, turn & (kClWarps - 1), split, blk, loaded);
-        turn += 3;
-        loaded = false;
+      for (int place = split; place < n; place += S) {
+        if ((turn++ & 1) != team) continue;
+        const WT *gk = cache_at(t.kcache, hl, b), *gv = cache_at(t.vcache, hl, b);
+        if (rps == 1)
+          cl_attend<WT, HD, 1>(p, ev, gk, gv, hl, b, 0, place, waited, qkv_bytes, parity);
+        else
+#pragma unroll 1
+          for (int r0 = 0; r0 < rps; r0 += kClAttnRows) cl_attend<WT, HD, kClAttnRows>(p, ev, gk, gv, hl, b, r0, place, waited, qkv_bytes, parity);
       }
     }
-  cl_sync();
-  // the places of every row, in order
-  float* stg = cl_at<float>(ev.stg);  // [hl][row][HD], behind it [hl][row][2]
+  if (!waited) cl_wait(ev.sh, p.sync, CL_BAR_QKV, qkv_bytes, parity);
+  __syncthreads();
+  if (split == 0) {
+    if (S > 1) {  // what the head's other CTAs send
+      int n = 0;
 #pragma unroll 1
-  for (int e = ev.warp * 32 + ev.lane; e < nh * R * HD; e += kClThreads) {
-    const int hr = e / HD, dim = e % HD, row = nh == 1 ? hr : hr % R;
+      for (int row = 0; row < R; ++row) {
+        const int places = A::places(ev.sh->pos[row]);
+        n += places - (places + S - 1) / S;
+      }
+      if (n > 0) cl_wait(ev.sh, p.sync, CL_BAR_PART, (unsigned)(n * (HD + 2) * 4), phase(CL_BAR_PART));
+    }
+    if (!cl_aborted(ev.sh)) {
+      const uint32_t bar = cl_bar_of(p, ev.dst, CL_BAR_X);
+#pragma unroll 1
+      for (int i = ev.tid >> 4; i < nh * R * (HD / 4); i += kClThreads / 16) {
+        const int hr = i / (HD / 4), dim = (i % (HD / 4)) * 4, hl = nh == 1 ? 0 : hr / R, row = hr - hl * R;
+        const float4 o = cl_fold<WT, HD>(cl_at<float>(p.lay.part) + hr * p.lay.part_slots * A::PLD, A::places(ev.sh->pos[row]), dim);
+        cl_send4(ev.dst + p.lay.xo + cl_x_off<WT>(p.d, R, row, (head0 + hl * kClCtas) * HD + dim), cl_x_pack<WT>(o), bar);
+      }
+    }
+  }
+  // the rows' keys and values into the cache, by the CTA that reads them there
+  const int rows_all = p.lay.heads_per_cta * R;
+  const WT* kv = reinterpret_cast<const WT*>(cl_at<float>(p.lay.qkv) + rows_all * ClQ<HD>::kLd);
+#pragma unroll 1
+  for (int i = ev.tid; i < 2 * nh * R * A::VPR; i += kClThreads) {
+    const int hr2 = i / A::VPR, v = i % A::VPR, which = hr2 >= nh * R ? 1 : 0, hr = hr2 - which * nh * R, hl = nh == 1 ? 0 : hr / R, row = hr - hl * R;
     const int pos = ev.sh->pos[row];
-    const int blocks = pos < 0 ? 0 : pos / A::KPB + 1;  // ... that the row sees; this CTA's places among them:
-    const int na = blocks > split ? min(kClWarps, (blocks - split + S - 1) / S) : 0;
-    const float* q = cl_at<float>(p.lay.part) + hr * kClWarps * (HD + 4);
-    float mx = -INFINITY, l = 0.f, o = 0.f;
-    float2 ml[kClWarps];
-    float v[kClWarps];
-#pragma unroll
-    for (int w = 0; w < kClWarps; ++w) {
-      ml[w] = make_float2(-INFINITY, 0.f);
-      v[w] = 0.f;
-      if (w < na) {
-        ml[w] = *reinterpret_cast<const float2*>(q + w * (HD + 4) + HD);
-        v[w] = q[w * (HD + 4) + dim];
-      }
-    }
-#pragma unroll
-    for (int w = 0; w < kClWarps; ++w) mx = fmaxf(mx, ml[w].x);
-#pragma unroll
-    for (int w = 0; w < kClWarps; ++w)
-      if (w < na) {
-        const float a = __expf(ml[w].x - mx);
-        l = fmaf(ml[w].y, a, l);
-        o = fmaf(v[w], a, o);
-      }
-    if (S == 1)
-      o *= l > 0.f ? 1.0f / l : 0.f;
-    else if (dim == 0)
-      *reinterpret_cast<float2*>(stg + nh * R * HD + hr * 2) = make_float2(mx, l);
-    stg[e] = o;
+    if (pos < 0) continue;
+    const int chunk = pos / A::C, place = A::BF ? chunk % kAttnSplits : chunk;
+    if (place % S != split) continue;
+    reinterpret_cast<uint4*>(cache_at(which ? t.vcache : t.kcache, hl, row / rps) + (size_t)pos * HD)[v] =
+        reinterpret_cast<const uint4*>(kv + (which * rows_all + hr) * HD)[v];
   }
-  cl_sync();
-  if (cl_aborted(ev.sh)) return;
-  const uint32_t bar = cl_bar_of(p, ev.dst, CL_BAR_X);
-  const uint32_t base = ev.dst + (S == 1 ? p.lay.xo : p.lay.xp + split * R * p.d * 4);
-#pragma unroll 1
-  for (int i = threadIdx.x >> 4; i < nh * R * (HD / 4); i += kClThreads / 16) {
-    const int hr = i / (HD / 4), dim = (i % (HD / 4)) * 4, hl = nh == 1 ? 0 : hr / R, row = hr - hl * R;
-    cl_send4(base + (row * p.d + (head0 + hl * kClCtas) * HD + dim) * 4, reinterpret_cast<const float4*>(stg)[i], bar);
-  }
-  if (S > 1)
-#pragma unroll 1
-    for (int row = threadIdx.x >> 4; row < R; row += kClThreads / 16) {  // fewer heads than CTAs: one head here
-      const float2 ml = *reinterpret_cast<const float2*>(stg + R * HD + row * 2);
-      cl_send2(ev.dst + p.lay.xml + ((split * R + row) * p.heads + head0) * 8, ml.x, ml.y, bar);
-    }
 }
 
-// splits > 1: the attention output from the CTAs' partial softmaxes, in split order
-template <int HD>
-__device__ __forceinline__ void cl_fold_splits(const ClParams& p, const ClEnv& ev) {
-  const int S = p.lay.splits, R = ev.R;
-  const float2* ml = cl_at<float2>(p.lay.xml);
-  const float* xp = cl_at<float>(p.lay.xp);
-  const int quads = p.d / 4;
-#pragma unroll 1
-  for (int e = ev.warp * 32 + ev.lane; e < R * quads; e += kClThreads) {
-    const int row = R == 1 ? 0 : e / quads, col = (e - row * quads) * 4, head = col / HD;
-    float mx = -INFINITY, l = 0.f;
-#pragma unroll 1
-    for (int s = 0; s < S; ++s) {
-      const float2 v = ml[(s * R + row) * p.heads + head];
-      if (v.y > 0.f) mx = fmaxf(mx, v.x);
-    }
-    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-    for (int s = 0; s < S; ++s) {
-      const float2 v = ml[(s * R + row) * p.heads + head];
-      const float a = v.y > 0.f ? __expf(v.x - mx) : 0.f;
-      const float4 x = *reinterpret_cast<const float4*>(xp + (s * R + row) * p.d + col);
-      l = fmaf(v.y, a, l);
-      o.x = fmaf(x.x, a, o.x);
-      o.y = fmaf(x.y, a, o.y);
-      o.z = fmaf(x.z, a, o.z);
-      o.w = fmaf(x.w, a, o.w);
-    }
-    *reinterpret_cast<float4*>(cl_at<float>(p.lay.xo) + row * p.d + col) = cl_scale(o, l > 0.f ? 1.0f / l : 0.f);
-  }
+// the CTAs that hold a head: CTA c has heads c, c + 16, ...; with fewer heads than CTAs, `splits` CTAs share one
+__device__ __forceinline__ int cl_heads_of(int cta, int heads, int splits) {
+  if (heads >= kClCtas) return (heads - cta + kClCtas - 1) / kClCtas;
+  return cta < heads * splits ? 1 : 0;
 }
 
 // What a pass's row carries
@@ -732,20 +1026,6 @@ __device__ __forceinline__ void cl_plan_row(const ClShared* sh, int kind, int st
   } else {
     pos = n - 1 + i;
     tok = i == 0 ? sh->last[b][1] : sh->drafts[b][i - 1];
-  }
-}
-
-// the better of (value, index) over `n` neighbouring lanes, ties to the lower index
-template <int n>
-__device__ __forceinline__ void cl_best_of_lanes(float& bv, int& bi) {
-#pragma unroll
-  for (int o = n / 2; o > 0; o >>= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ov > bv || (ov == bv && oi < bi)) {
-      bv = ov;
-      bi = oi;
-    }
   }
 }
 
@@ -795,26 +1075,23 @@ __device__ __forceinline__ void cl_commit(const ClParams& p, ClShared* sh, int b
   }
 }
 
-template <typename WT, int HD>
+template <typename WT, int HD, int CG>
 __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, const ClTab* tab_t, const ClTab* tab_d, int rank, bool loop, int batch, int k) {
+  constexpr bool BF = sizeof(WT) == 2;
   const int tid = threadIdx.x;
   ClEnv ev{};
   ev.sh = sh;
+  ev.mine = cl_at<ClMine>(p.lay.plan);
+  ev.rounds = cl_at<ClRound>(p.lay.plan_rounds);
+  ev.entries = cl_at<ClEntry>(p.lay.plan_entries);
+  ev.tid = tid;
   ev.warp = tid >> 5;
   ev.lane = tid & 31;
   ev.rank = rank;
   ev.self = smem_u32(cl_smem);
   ev.dst = cl_map(ev.self, tid & (kClCtas - 1));
-  ev.stg = p.lay.stg;
-  ev.hres = p.lay.hres;
-  auto other_stg = [&] { ev.stg = 2 * p.lay.stg + p.lay.stg_floats * 4 - ev.stg; };
   const int my_heads = cl_heads_of(rank, p.heads, p.lay.splits);
   unsigned phases = 0;
-  auto phase = [&](int which) {
-    const unsigned par = (phases >> which) & 1u;
-    phases ^= 1u << which;
-    return par;
-  };
 
 #pragma unroll 1
   for (int pass = 0;; pass = pass == k ? 0 : pass + 1) {  // loop mode: the number in the round, k = verification
@@ -828,55 +1105,66 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
     const int n_stages = draft ? p.n_d : p.n_t;
 
     // ---- tokens, embedding, rotary factors: warp r does rows r and r + 8 ----
+    {
+      const float* gain = p.gains[draft ? p.first_gain_d : p.first_gain_t];
 #pragma unroll 1
-    for (int row = ev.warp; row < R; row += kClWarps) {
-      int tok, pos;
-      cl_plan_row(sh, kind, loop ? pass : p.pd.step, ev.rps, row, tok, pos);
-      if (ev.lane == 0) sh->pos[row] = pos;
-      const WT* e = reinterpret_cast<const WT*>(p.embed) + (size_t)tok * p.d;
-      const float* gain = p.gains + (size_t)(draft ? p.first_gain_d : p.first_gain_t) * p.d;
-      float* h = cl_at<float>(p.lay.h) + row * p.d;
-      float* y = cl_at<float>(p.lay.y) + row * p.d;
-      float* own = cl_at<float>(ev.hres) + row * p.lay.resid_np;
-      const int q0 = sh->mine[CL_O].p0, q1 = q0 + sh->mine[CL_O].np;
-      constexpr int hp = HD / 2;
-      const int at = max(pos, 0) * hp;
-      float cs[hp / 32], sn[hp / 32];
+      for (int row = ev.warp; row < R; row += kClWarps) {
+        int tok, pos;
+        cl_plan_row(sh, kind, loop ? pass : p.pd.step, ev.rps, row, tok, pos);
+        if (ev.lane == 0) sh->pos[row] = pos;
+        const WT* e = reinterpret_cast<const WT*>(p.embed) + (size_t)tok * p.d;
+        float* own = cl_at<float>(p.lay.hres) + row * p.lay.resid_np;
+        const int q0 = ev.mine[CL_O].p0, q1 = q0 + ev.mine[CL_O].np;
+        constexpr int hp = HD / 2;
+        const int at = max(pos, 0) * hp;
+        float cs[hp / 32], sn[hp / 32];
 #pragma unroll
-      for (int i = 0; i < hp / 32; ++i) {
-        cs[i] = __ldg(p.rope_cos + at + i * 32 + ev.lane);
-        sn[i] = __ldg(p.rope_sin + at + i * 32 + ev.lane);
-      }
+        for (int i = 0; i < hp / 32; ++i) {
+          cs[i] = __ldg(p.rope_cos + at + i * 32 + ev.lane);
+          sn[i] = __ldg(p.rope_sin + at + i * 32 + ev.lane);
+        }
+        float total = 0.f;
 #pragma unroll 2
-      for (int c = ev.lane * 4; c < p.d; c += 128) {
-        const float4 v = pos >= 0 ? load4(e + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 g = __ldg(reinterpret_cast<const float4*>(gain + c));
-        *reinterpret_cast<float4*>(h + c) = v;
-        *reinterpret_cast<float4*>(y + c) = make_float4(v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w);
-        const int pair = (c >> 4) * 8 + (c & 7);  // of the first of these four features
-        if (pair >= q0 && pair < q1) *reinterpret_cast<float4*>(own + ((c >> 3) & 1) * p.lay.rows * p.lay.resid_np + pair - q0) = v;
-      }
-      float* rope = cl_at<float>(p.lay.rope) + row * 2 * hp;
+        for (int c0 = 0; c0 < p.d; c0 += 128) {
+          const int c = c0 + ev.lane * 4;
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (c < p.d) {
+            if (pos >= 0) v = load4(e + c);
+            if (BF) {
+              const float4 g = __ldg(reinterpret_cast<const float4*>(gain + c));
+              *reinterpret_cast<float4*>(cl_smem + p.lay.y + cl_x_off<WT>(p.d, R, row, c)) = cl_x_pack<WT>(make_float4(v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w));
+            } else {
+              *reinterpret_cast<float4*>(cl_at<float>(p.lay.h) + row * p.d + c) = v;
+            }
+            const int pair = (c >> 4) * 8 + (c & 7);  // of the first of these four features
+            if (pair >= q0 && pair < q1) *reinterpret_cast<float4*>(own + ((c >> 3) & 1) * p.lay.rows * p.lay.resid_np + pair - q0) = v;
+          }
+          if (BF) {  // a row's squares as the whole-pass kernel's first stage adds them: by 128 columns, the blocks in order
+            float s = fmaf(v.x, v.x, 0.f);
+            s = fmaf(v.y, v.y, s);
+            s = fmaf(v.z, v.z, s);
+            s = fmaf(v.w, v.w, s);
+            total += warp_sum(s);
+          }
+        }
+        if (BF && ev.lane == 0) sh->inv[row] = rsqrtf(total / (float)p.d + p.eps);
+        float* rope = cl_at<float>(p.lay.rope) + row * 2 * hp;
 #pragma unroll
-      for (int i = 0; i < hp / 32; ++i) {
-        rope[i * 32 + ev.lane] = cs[i];
-        rope[hp + i * 32 + ev.lane] = sn[i];
+        for (int i = 0; i < hp / 32; ++i) {
+          rope[i * 32 + ev.lane] = cs[i];
+          rope[hp + i * 32 + ev.lane] = sn[i];
+        }
+        if (loop) cl_at<float2>(p.lay.best)[row * 4 * kClWarps + ev.lane] = make_float2(-INFINITY, __int_as_float(0x7fffffff));
       }
-      if (loop)
-#pragma unroll
-        for (int c = ev.lane; c < 4 * kClWarps; c += 32) cl_at<float2>(p.lay.best)[row * 4 * kClWarps + c] = make_float2(-INFINITY, __int_as_float(0x7fffffff));
     }
-    cl_sync();
+    __syncthreads();
 
 #pragma unroll 1
     for (int s = 0; s < n_stages; ++s) {
       const ClTab t = tab[s];
       ClDots a{};
       a.W = t.W;
-      a.np = t.np;
-      a.R = R;
-      a.steps = t.steps;
-      a.stg = ev.stg;
+      a.kind = t.kind;
       a.x = t.x;
       a.K = t.K;
       a.bar = s > 0 ? t.bar : -1;  // the first stage's are the embedding
@@ -884,61 +1172,100 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
       a.parity = (phases >> t.bar) & 1u;
       if (s > 0) phases ^= 1u << t.bar;
       a.norm = t.norm != 0;
-      a.head = t.kind == CL_HEAD;
-      a.p0 = t.p0;
+      a.gain = t.gain;
       a.logits = loop ? nullptr : p.logits;
-      if (p.lay.splits > 1 && t.kind == CL_O) {
-        cl_wait(sh, p.sync, CL_BAR_X, a.bytes, a.parity);
-        cl_fold_splits<HD>(p, ev);
-        cl_sync();
-        a.bar = -1;
-      }
-      // the pass's keys and values, before anything of the next pass is sent: their writers, long done, in a stage whose last warps have the least to do
-      if (t.after_kv && tid >= kClThreads - ((R * sh->mine[CL_QKV].nq + 31) & ~31)) __threadfence();
-      if (R == 1)
-        cl_dots<WT, 1, 4>(p, a, sh);
-      else if (R <= 4)
-        cl_dots<WT, 4, 2>(p, a, sh);
-      else
-        cl_dots<WT, 8, 2>(p, a, sh);
-      if (a.head) break;
-      cl_sync();  // the sums are there
-      const bool live = !cl_aborted(sh);
-      if (t.kind == CL_QKV) {
-        cl_finish_qkv<WT, HD>(p, ev, t, live);
-        if (my_heads > 0) {
-          other_stg();
-          cl_attention<WT, HD>(p, ev, t, my_heads, phase(CL_BAR_QKV));
+      const ClMine& me = ev.mine[t.kind];
+      const bool is_head = t.kind == CL_HEAD;
+      if constexpr (BF) {
+        ClRing ring;
+        ring.W = reinterpret_cast<const uint4*>(a.W) + ev.lane;
+        ring.ent = ev.entries + me.entry0 + ev.warp * me.n_entries;
+        ring.buf = (int)ev.self + p.lay.ring + ev.warp * (2 * kClAhead * 512) + ev.lane * 16;
+        ring.per = kClAhead / me.tile_width;
+        ring.steps = me.n_entries / ring.per;
+        ring.step = 0;
+        ring.wrap_jump = (a.K / 16 - 1) * 256;  // to the next group's unit of the same k-tile, which starts with its first tile
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) ring.ask();
+        if (a.bar >= 0) cl_wait(sh, p.sync, a.bar, a.bytes, a.parity);
+        // lm-head: 256 threads over the rows, a power of two of them each
+        const int row_log = R <= 1 ? 8 : R <= 2 ? 7 : R <= 4 ? 6 : R <= 8 ? 5 : 4;
+        float bv = -INFINITY;
+        int bi = 0x7fffffff, done = 0;
+        float acc[kClTiles][CG][4];
+#pragma unroll
+        for (int i = 0; i < kClTiles; ++i)
+#pragma unroll
+          for (int c = 0; c < CG; ++c) acc[i][c][0] = acc[i][c][1] = acc[i][c][2] = acc[i][c][3] = 0.f;
+#pragma unroll 1
+        for (int r = 0; r < me.n_rounds; ++r) {
+          const ClRound& rd = ev.rounds[me.round0 + r];
+#pragma unroll 1
+          for (int end = done + rd.n_entries / ring.per; done < end; ++done) {
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            cl_mma_half<CG>(p, ev, a, ring.ent + done * ring.per, ring.per, ring.buf + (done & 1) * (kClAhead * 512), acc);
+            ring.ask();
+          }
+          if (a.norm && a.bar >= 0 && r == 0) cl_row_scales(p, ev);  // (the first stage's were made with the embedding)
+          __syncthreads();  // the sums are there
+          if (is_head) {
+            cl_head_round(p, ev, me, rd, a.logits, row_log, bv, bi);
+          } else {
+            cl_values<WT, HD>(p, ev, me, rd, t.kind);
+            __syncthreads();
+            if (cl_aborted(sh)) {
+            } else if (t.kind == CL_QKV) {
+              cl_send_qkv<WT, HD>(p, ev, me, rd);
+            } else {
+              cl_send_all<WT>(p, ev, me, rd, t.kind, t.gain_out);
+            }
+          }
+          if (r + 1 < me.n_rounds) __syncthreads();
         }
-      } else if (live) {
-        if (t.kind == CL_GATE_UP)
-          cl_finish_gate_up(p, ev);
+        if (is_head && loop) {
+          if (me.n_rounds == 0) __syncthreads();
+#pragma unroll 1
+          for (int o = min(16, 1 << (row_log - 1)); o > 0; o >>= 1) cl_better(bv, bi, __shfl_xor_sync(0xffffffffu, bv, o), __shfl_xor_sync(0xffffffffu, bi, o));
+          const int lanes = min(32, 1 << row_log), in_row = tid & ((1 << row_log) - 1), row = tid >> row_log;
+          if (row < R && in_row % lanes == 0) cl_at<float2>(p.lay.best)[row * 4 * kClWarps + in_row / lanes] = make_float2(bv, __int_as_float(bi));
+        }
+      } else {
+        if (R == 1)
+          cl_dots_f32<1, 4>(p, ev, a);
+        else if (R <= 4)
+          cl_dots_f32<4, 2>(p, ev, a);
         else
-          cl_finish_resid(p, ev, t);
+          cl_dots_f32<8, 2>(p, ev, a);
+        if (!is_head) {
+          const ClRound& rd = ev.rounds[me.round0];
+          __syncthreads();  // the sums are there
+          cl_values<WT, HD>(p, ev, me, rd, t.kind);
+          __syncthreads();
+          if (cl_aborted(sh)) {
+          } else if (t.kind == CL_QKV) {
+            cl_send_qkv<WT, HD>(p, ev, me, rd);
+          } else {
+            cl_send_all<WT>(p, ev, me, rd, t.kind, t.gain_out);
+          }
+        }
       }
-      other_stg();
+      if (t.kind == CL_QKV && my_heads > 0) cl_attention<WT, HD>(p, ev, t, my_heads, phases);
     }
     if (!loop) break;
 
     // ---- greedy decision: best of the CTA, then of the cluster ----
-    cl_sync();
+    __syncthreads();
     if (!cl_aborted(sh))
 #pragma unroll 1
       for (int row = ev.warp; row < R; row += kClWarps) {
-        float bv = -INFINITY;
-        int bi = 0x7fffffff;
-#pragma unroll
-        for (int e = ev.lane; e < 4 * kClWarps; e += 32) {
-          const float2 c = cl_at<float2>(p.lay.best)[row * 4 * kClWarps + e];
-          if (c.x > bv || (c.x == bv && __float_as_int(c.y) < bi)) {
-            bv = c.x;
-            bi = __float_as_int(c.y);
-          }
-        }
+        const float2 c = cl_at<float2>(p.lay.best)[row * 4 * kClWarps + ev.lane];
+        float bv = c.x;
+        int bi = __float_as_int(c.y);
         cl_best_of_lanes<32>(bv, bi);
         if (ev.lane < kClCtas) cl_send2(ev.dst + p.lay.tok + (rank * R + row) * 8, bv, __int_as_float(bi), cl_bar_of(p, ev.dst, CL_BAR_TOK));
       }
-    cl_wait(sh, p.sync, CL_BAR_TOK, (unsigned)(kClCtas * R * 8), phase(CL_BAR_TOK));
+    cl_wait(sh, p.sync, CL_BAR_TOK, (unsigned)(kClCtas * R * 8), (phases >> CL_BAR_TOK) & 1u);
+    phases ^= 1u << CL_BAR_TOK;
 #pragma unroll 1
     for (int row = ev.warp; row < R; row += kClWarps) {
       const float2 c = cl_at<float2>(p.lay.tok)[(ev.lane & (kClCtas - 1)) * R + row];
@@ -947,7 +1274,7 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
       cl_best_of_lanes<kClCtas>(bv, bi);
       if (ev.lane == 0) sh->amax[row] = min(max(bi, 0), p.vocab - 1);
     }
-    cl_sync();
+    __syncthreads();
     if (tid < 32) {
       if (verify)
         cl_commit(p, sh, batch, k, rank == 0, tid);
@@ -956,7 +1283,7 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
     }
     if (!cl_agree_ok(&sh->abort) || (verify && (sh->all_done || sh->round >= p.rounds))) break;
   }
-  cl_sync();
+  __syncthreads();
   if (loop && rank == 0) {
     if (tid < batch) {
       p.gs->n[tid] = sh->n[tid];
@@ -971,7 +1298,8 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
   }
 }
 
-template <typename WT, int HD>
+// CG: column groups of eight rows (bf16); all passes of a context take the same
+template <typename WT, int HD, int CG>
 __global__ void __launch_bounds__(kClThreads, 1) cluster_pass_kernel(const __grid_constant__ ClParams p) {
   ClShared* sh = cl_at<ClShared>(p.lay.shared);
   ClTab* tab_t = cl_at<ClTab>(p.lay.tab);
@@ -979,44 +1307,33 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_pass_kernel(const __gri
   const int tid = threadIdx.x, rank = (int)cl_rank();
   const bool loop = p.rounds > 0;
   const int batch = loop ? p.gs->batch : p.pd.n_seq, k = loop ? p.gs->k : 0;
-  constexpr int n_threads = kClThreads;
 
-  // ---- set-up: this CTA's shares, stage tables, the gains of its features, state ----
+  // ---- set-up: this CTA's plan, stage tables, the gains of its features, state ----
 #pragma unroll 1
-  for (int i = tid; i < p.n_t + p.n_d; i += n_threads) {
+  for (int i = tid; i < p.lay.plan_bytes / 16; i += kClThreads)
+    cl_at<uint4>(p.lay.plan)[i] = __ldg(reinterpret_cast<const uint4*>(p.plan + (size_t)rank * p.lay.plan_bytes) + i);
+#pragma unroll 1
+  for (int i = tid; i < p.n_t + p.n_d; i += kClThreads) {
     const ClStage s = i < p.n_t ? p.prog_t[i] : p.prog_d[i - p.n_t];
-    const int p0 = cl_first_pair(s.n_pairs, rank);
     ClTab& t = tab_t[i];
     t.kind = s.kind;
-    t.np = cl_first_pair(s.n_pairs, rank + 1) - p0;
-    t.steps = cl_steps(s.K, (int)sizeof(WT));
-    t.gain_out = s.gain_out;
-    t.p0 = p0;
-    t.norm = s.kind == CL_QKV || s.kind == CL_GATE_UP || s.kind == CL_HEAD;
-    t.x = s.kind == CL_O ? p.lay.xo : s.kind == CL_DOWN ? p.lay.u : p.lay.y;
     t.K = s.K;
+    t.norm = s.kind == CL_QKV || s.kind == CL_GATE_UP || s.kind == CL_HEAD;
+    t.gain = sizeof(WT) == 4 && t.norm ? p.gains[s.gain] : nullptr;
+    t.gain_out = s.gain;
+    t.x = s.kind == CL_O ? p.lay.xo : s.kind == CL_DOWN ? p.lay.u : p.lay.y;
     t.bar = s.kind == CL_O ? CL_BAR_X : s.kind == CL_DOWN ? CL_BAR_U : CL_BAR_H;
-    t.row_bytes = s.kind == CL_O ? p.lay.splits * (p.d * 4 + (p.lay.splits > 1 ? p.heads * 8 : 0)) : s.kind == CL_DOWN ? p.f * 4 : 2 * p.d * 4;
-    t.after_kv = s.after_kv;
+    t.row_bytes = s.kind == CL_DOWN ? p.f * 4 : s.kind == CL_O || sizeof(WT) == 4 ? p.d * 4 : p.d * 6;
     t.kcache = s.kcache;
     t.vcache = s.vcache;
-    t.W = s.W + (size_t)p0 * t.steps * kClUnit;
+    t.W = s.W + (sizeof(WT) == 4 ? (size_t)cl_first_pair(cl_pairs_of(s.kind, p.d, p.f, p.vocab), rank, 4) * 2 * s.K * 4 : 0);
   }
-  if (tid >= 96 && tid < 101) {
-    const int kind = tid - 96;
-    const int n_pairs = kind == CL_QKV ? 3 * p.d / 2 : kind == CL_GATE_UP ? p.f : kind == CL_HEAD ? p.vocab / 2 : p.d / 2;
-    ClMine& m = sh->mine[kind];
-    m.p0 = cl_first_pair(n_pairs, rank);
-    m.np = cl_first_pair(n_pairs, rank + 1) - m.p0;
-    m.nq = m.np / 4;
-    m.magic = m.nq > 0 ? (1u << 20) / m.nq + 1u : 0u;
-  }
-  {
-    const int p0 = cl_first_pair(p.d / 2, rank), np = cl_first_pair(p.d / 2, rank + 1) - p0, ld = 2 * p.lay.resid_np;
+  if (sizeof(WT) == 2) {
+    const int p0 = cl_first_pair(p.d / 2, rank, 2), np = cl_first_pair(p.d / 2, rank + 1, 2) - p0, ld = 2 * p.lay.resid_np;
 #pragma unroll 1
-    for (int i = tid; i < p.n_gains * 2 * np; i += n_threads) {
+    for (int i = tid; i < p.n_gains * 2 * np; i += kClThreads) {
       const int g = i / (2 * np), r = i - g * 2 * np, half = r >= np ? 1 : 0, pl = r - half * np, pair = p0 + pl;
-      cl_at<float>(p.lay.gain)[g * ld + half * p.lay.resid_np + pl] = __ldg(p.gains + (size_t)g * p.d + ((pair >> 3) << 4) + (pair & 7) + half * 8);
+      cl_at<float>(p.lay.gain)[g * ld + half * p.lay.resid_np + pl] = __ldg(p.gains[g] + cl_feature(pair) + half * 8);
     }
   }
   if (tid < CL_BARS) mbar_init(&sh->bar[tid], 1);
@@ -1048,7 +1365,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_pass_kernel(const __gri
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   cl_cluster_sync();  // barriers exist everywhere before anything is sent, and the CTA's tables are written
 
-  cl_compute<WT, HD>(p, sh, tab_t, tab_d, rank, loop, batch, k);
+  cl_compute<WT, HD, CG>(p, sh, tab_t, tab_d, rank, loop, batch, k);
 
   // In normal operation everything that was sent has been waited for.  After a wait that ran out something may still
   // be on its way to a CTA of the cluster: give it far longer than it takes before any CTA leaves.
@@ -1061,62 +1378,205 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_pass_kernel(const __gri
   cl_cluster_sync();
 }
 
-// ---- packing: [pair][K step][half][512 bytes] -------------------------------------------------------------------
-// A lane's sixteen bytes of a step: fp32 columns 4 lane .. +3; bf16 columns 4 lane .. +3 and 128 + 4 lane .. +3, so that
-// the matching activations are two conflict-free 128-bit reads.  Columns beyond K are zero.
-template <typename WT>
-__global__ void pack_cluster_kernel(WT* __restrict__ dst, PackSrc ps, int n_pairs, int K) {
-  constexpr int V = ClElem<WT>::kLane, STEP = ClElem<WT>::kStep;
-  const int steps = cl_steps(K, (int)sizeof(WT));
-  const size_t total = (size_t)n_pairs * 2 * steps * STEP;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int in = (int)(e % STEP);
-    const size_t rest = e / STEP;  // [pair][step][half]
-    const int r = (int)(rest & 1), s = (int)((rest >> 1) % steps), pair = (int)((rest >> 1) / steps);
-    const int lane = in / V, j = in % V;
-    const int c = s * STEP + (j >> 2) * 128 + lane * 4 + (j & 3);
-    dst[e] = c < K ? pack_src_row<WT>(ps, pair, r, K)[c] : WT(0.0f);
+// ---- host -------------------------------------------------------------------------------------------------------
+// What every CTA does of the five kinds of matrices, [CTA][stride].  bf16: the units of a group of 128 features are cut
+// as the whole-pass kernel's CTAs share them (stage_shares), and dealt to the classes from the beginning of each CTA's range.
+struct ClPlan {
+  std::vector<unsigned char> bytes;
+  int rounds_at = 0, entries_at = 0, stride = 0;
+  int most_places = 0;  // places the sums of a layer's stage take when it is finished in one round
+  int most_cuts = 1;    // pieces of a sum
+  int most_quads = 0;   // fours of pairs in a round
+};
+
+inline ClPlan cluster_plan(int d, int f, int vocab, int elem_bytes, int pass_grid, int place_slots) {
+  struct Cut {
+    int kt0, len, cls0;
+    bool operator==(const Cut& o) const { return kt0 == o.kt0 && len == o.len && cls0 == o.cls0; }
+  };
+  struct Batch {  // up to kClTiles neighbouring tiles that are cut alike
+    int tile, n, np;
+  };
+  struct Cta {
+    ClMine mine[CL_KINDS];
+    std::vector<ClRound> rounds;
+    std::vector<ClEntry> entries;
+  };
+  std::vector<Cta> ctas(kClCtas);
+  ClPlan out;
+  for (int kind = 0; kind < CL_KINDS; ++kind) {
+    const int n_pairs = cl_pairs_of(kind, d, f, vocab);
+    const int K = kind == CL_DOWN ? f : d, KT = K / 16, NT = n_pairs / 8, n_groups = (NT + kUnitTiles - 1) / kUnitTiles;
+    std::vector<std::vector<Cut>> cuts;
+    if (elem_bytes == 2) {
+      std::vector<StageShare> shares(pass_grid);
+      stage_shares(shares.data(), n_groups, KT, pass_grid);
+      cuts.resize(n_groups);
+      for (const StageShare& s : shares)
+        for (int u = 0; u < s.n;) {
+          const int grp = (s.ub + u) / KT, kt0 = (s.ub + u) % KT, len = std::min(s.n - u, KT - kt0);
+          cuts[grp].push_back(Cut{kt0, len, u % kClasses});
+          u += len;
+        }
+    }
+    for (int rank = 0; rank < kClCtas; ++rank) {
+      Cta& c = ctas[rank];
+      ClMine& m = c.mine[kind];
+      m = ClMine{};
+      m.p0 = cl_first_pair(n_pairs, rank, elem_bytes);
+      m.np = cl_first_pair(n_pairs, rank + 1, elem_bytes) - m.p0;
+      m.round0 = (int)c.rounds.size();
+      m.entry0 = (int)c.entries.size();
+      m.tile_width = 1;
+      auto add_round = [&](int pair0, int pair1) -> ClRound& {
+        ClRound r{};
+        r.quad0 = (pair0 - m.p0) / 4;
+        r.n_quads = (pair1 - pair0) / 4;
+        r.magic = r.n_quads > 0 ? (1u << 20) / (unsigned)r.n_quads + 1u : 0u;
+        out.most_quads = std::max(out.most_quads, r.n_quads);
+        c.rounds.push_back(r);
+        m.n_rounds += 1;
+        return c.rounds.back();
+      };
+      if (elem_bytes != 2) {
+        add_round(m.p0, m.p0 + m.np);
+        continue;
+      }
+      if (m.np == 0) continue;
+      std::vector<Batch> batches;
+      const int t1 = (m.p0 + m.np + 7) / 8;
+      int places = 0, width = 1;
+      for (int t = m.p0 / 8; t < t1;) {
+        const std::vector<Cut>& cut = cuts[t / kUnitTiles];
+        const int np = (int)cut.size(), most = std::max(1, std::min((int)kClTiles, place_slots / np));
+        int n = 1;
+        while (n < most && t + n < t1 && cuts[(t + n) / kUnitTiles] == cut) ++n;
+        batches.push_back(Batch{t, n, np});
+        out.most_cuts = std::max(out.most_cuts, np);
+        width = std::max(width, n);
+        places += n * np;
+        t += n;
+      }
+      if (kind != CL_HEAD) out.most_places = std::max(out.most_places, places);
+      m.tile_width = width == 3 ? 4 : width;
+      const int per = kClAhead / m.tile_width;
+      std::vector<std::vector<ClEntry>> lists(kClasses);
+      for (size_t b = 0; b < batches.size();) {
+        size_t e = b;
+        int tiles = 0;  // ... of the round
+        while (e < batches.size() && batches[e].np == batches[b].np && (e == b || (tiles + batches[e].n) * batches[b].np <= place_slots)) tiles += batches[e++].n;
+        const int tile0 = batches[b].tile;
+        ClRound& r = add_round(std::max(m.p0, tile0 * 8), std::min(m.p0 + m.np, (tile0 + tiles) * 8));
+        r.tile0 = tile0;
+        r.np = batches[b].np;
+        const size_t begin = lists[0].size();
+        size_t longest = 0;
+        for (int cls = 0; cls < kClasses; ++cls) {
+          for (size_t i = b; i < e; ++i) {
+            const Batch& bt = batches[i];
+            const int grp = bt.tile / kUnitTiles, in = bt.tile % kUnitTiles;
+            for (int pc = 0; pc < bt.np; ++pc) {
+              const Cut& cut = cuts[grp][pc];
+              ClEntry en{};
+              en.n_tiles = (unsigned char)bt.n;
+              en.wrap = (unsigned char)(kUnitTiles - in);
+              en.np = (unsigned char)bt.np;
+              en.kt = -1;
+              const int slot = (bt.tile - tile0) * bt.np + pc, first = (cls - cut.cls0 + kClasses) % kClasses;
+              for (int j = first; j < cut.len; j += kClasses) {
+                en.kt = (short)(cut.kt0 + j);
+                en.w = (grp * KT + en.kt) * (kUnitBytes / 16) + in * 32;
+                en.slot = j + kClasses < cut.len ? -1 : (short)slot;
+                lists[cls].push_back(en);
+              }
+              if (first >= cut.len) {  // nothing to add: the place is zero
+                en.slot = (short)slot;
+                lists[cls].push_back(en);
+              }
+            }
+          }
+          longest = std::max(longest, lists[cls].size());
+        }
+        longest = begin + (longest - begin + per - 1) / per * per;
+        ClEntry none{};
+        none.kt = none.slot = -1;
+        for (auto& l : lists) l.resize(longest, none);
+        r.n_entries = (int)(longest - begin);
+        b = e;
+      }
+      m.n_entries = (int)lists[0].size();
+      for (const auto& l : lists) c.entries.insert(c.entries.end(), l.begin(), l.end());
+    }
   }
+  size_t rounds = 0, entries = 0;
+  for (const Cta& c : ctas) {
+    rounds = std::max(rounds, c.rounds.size());
+    entries = std::max(entries, c.entries.size());
+  }
+  out.rounds_at = CL_KINDS * (int)sizeof(ClMine);
+  out.entries_at = out.rounds_at + (int)(rounds * sizeof(ClRound));
+  out.stride = out.entries_at + (int)(entries * sizeof(ClEntry));
+  out.bytes.assign((size_t)out.stride * kClCtas, 0);
+  for (int rank = 0; rank < kClCtas; ++rank) {
+    unsigned char* at = out.bytes.data() + (size_t)rank * out.stride;
+    const Cta& c = ctas[rank];
+    std::copy_n(reinterpret_cast<const unsigned char*>(c.mine), sizeof c.mine, at);
+    std::copy_n(reinterpret_cast<const unsigned char*>(c.rounds.data()), c.rounds.size() * sizeof(ClRound), at + out.rounds_at);
+    std::copy_n(reinterpret_cast<const unsigned char*>(c.entries.data()), c.entries.size() * sizeof(ClEntry), at + out.entries_at);
+  }
+  return out;
 }
 
-// ---- host -------------------------------------------------------------------------------------------------------
 // The layout for passes of up to `rows` rows; total = 0 when it does not fit
-inline ClLayout cluster_layout(int d, int f, int heads, int hd, int n_layers, int rows, int max_seq, int max_smem) {
+inline ClLayout cluster_layout(int d, int f, int heads, int hd, int n_layers, int rows, int max_seq, int elem_bytes, int place_slots, const ClPlan& plan,
+                               int max_smem) {
   ClLayout y{};
+  const bool bf16 = elem_bytes == 2;
   y.rows = rows;
-  const int key_block = 32 / (hd / 16);
+  const int chunks = (max_seq + kAttnChunk - 1) / kAttnChunk;
+  y.part_slots = bf16 ? std::min((int)kAttnSplits, chunks) : chunks;
   y.heads_per_cta = (heads + kClCtas - 1) / kClCtas;
-  // CTAs per head: as many as the longest context gives a block to every warp of, one when one does
-  y.splits = heads >= kClCtas ? 1 : std::max(1, std::min(kClCtas / heads, std::min(4, (max_seq + kClWarps * key_block - 1) / (kClWarps * key_block))));
-  y.resid_np = cl_max_pairs(d / 2);
+  y.splits = heads >= kClCtas ? 1 : std::min(kClCtas / heads, y.part_slots);  // CTAs per head
+  y.resid_np = cl_max_pairs(d / 2, elem_bytes);
   int at = 0;
   auto take = [&](int& off, long long bytes) {
     off = at;
     at = (int)std::min<long long>(1 << 30, ((long long)at + bytes + 127) / 128 * 128);
   };
-  take(y.h, 4LL * rows * d);
+  const long long hpr = (long long)y.heads_per_cta * rows;
+  take(y.h, (bf16 ? 2LL : 4LL) * rows * d);
   take(y.y, 4LL * rows * d);
-  // u lies over the attention's partial sums and output: it is written when every CTA has taken the O-projection's input
-  // in, and read before any CTA sends attention output of the next layer
+  // u lies over what the attention receives and sends: it is written when every CTA has taken the O-projection's input in, and
+  // read before any CTA sends anything of the next layer's attention
   const int u0 = at;
-  take(y.part, 4LL * rows * y.heads_per_cta * kClWarps * (hd + 4));
-  take(y.xp, y.splits > 1 ? 4LL * y.splits * rows * d : 0);
-  take(y.xml, y.splits > 1 ? 8LL * y.splits * rows * heads : 0);
+  take(y.part, 4LL * hpr * y.part_slots * (hd + 4));
   take(y.xo, 4LL * rows * d);
   const int att_end = at;
   at = u0;
   take(y.u, 4LL * rows * f);
   at = std::max(at, att_end);
-  take(y.qkv, 12LL * rows * y.heads_per_cta * hd);
-  take(y.gain, 8LL * (2 * n_layers + 1) * y.resid_np);
-  take(y.hres, 16LL * rows * y.resid_np);
-  const int share = std::max(2 * std::max(cl_max_pairs(3 * d / 2), cl_max_pairs(f)), y.heads_per_cta * (hd + 4));  // values of a row
-  y.stg_floats = rows * share;
-  take(y.stg, 8LL * y.stg_floats);
+  take(y.qkv, hpr * ((hd + 32) * 4 + 2 * hd * elem_bytes));
+  take(y.gain, bf16 ? 8LL * (2 * n_layers + 1) * y.resid_np : 0);
+  take(y.hres, 8LL * rows * y.resid_np);
+  take(y.stg, 8LL * rows * std::max(cl_max_pairs(3 * d / 2, elem_bytes), cl_max_pairs(f, elem_bytes)));
+  // the attention's keys and values lie over the weights on their way and the sums: it starts behind the barrier that ends the
+  // QKV stage's, and ends with one before the O-projection's begin
+  const int w0 = at;
+  y.team_bytes = cl_team_bytes(hd, elem_bytes);
+  take(y.team, 2LL * y.team_bytes);
+  const int team_end = at;
+  at = w0;
+  take(y.ring, bf16 ? kClWarps * 2LL * kClAhead * 512 : 0);
+  take(y.red, bf16 ? (long long)place_slots * kClasses * 8 * ((rows + 1) / 2) * 16 : 0);
+  at = std::max(at, team_end);
   take(y.rope, 4LL * rows * hd);
   take(y.tok, 8LL * kClCtas * rows);
   take(y.best, 32LL * rows * kClWarps);
   take(y.tab, (long long)sizeof(ClTab) * 2 * (4 * n_layers + 1));
+  take(y.plan, plan.stride);
+  y.plan_rounds = y.plan + plan.rounds_at;
+  y.plan_entries = y.plan + plan.entries_at;
+  y.plan_bytes = plan.stride;
   take(y.shared, (long long)sizeof(ClShared));
   y.total = at <= max_smem ? at : 0;
   return y;

@@ -48,8 +48,6 @@ struct LayerWeights {
   void* down = nullptr;  // packed [d, f]
   // the same matrices as tcgen05 operand images (dense path), null when that path is off
   void *um_qkv = nullptr, *um_wo = nullptr, *um_gu = nullptr, *um_down = nullptr;
-  // ... and in the layout of the cluster kernel (small decoders), null when that path is off
-  void *cl_qkv = nullptr, *cl_wo = nullptr, *cl_gu = nullptr, *cl_down = nullptr;
   float* attn_gain = nullptr;
   float* ffn_gain = nullptr;
 };
@@ -121,13 +119,12 @@ struct sdfp_ctx {
   // small decoders: the passes of rounds, and whole greedy generations, inside one cluster (cluster_pass.cuh)
   bool use_cluster = false;
   ClLayout cl{};
-  ClStage *cl_prog_t = nullptr, *cl_prog_d = nullptr;  // device: the linear stages of the target and of the draft
+  ClPlan cl_plan;                      // what each of its CTAs does of the matrices
+  unsigned char* cl_mem = nullptr;     // device: the plan, the gains' addresses, the programs
+  ClStage *cl_prog_t = nullptr, *cl_prog_d = nullptr;  // in there: the linear stages of the target and of the draft
+  const float** cl_gains = nullptr;    // in there: [2 n_layers + 1]
   int n_cl_t = 0, n_cl_d = 0;
   int cl_first_t = 0, cl_first_d = 0;  // the norm their first stage reads the embedding through
-  void* cl_lm_head = nullptr;
-  unsigned char* cl_weights = nullptr;  // all matrices in its layout
-  size_t cl_used = 0;
-  float* cl_gains = nullptr;         // [2 n_layers + 1][d_model]
   // dense path on tcgen05 (bf16 tensor path): the prompt pass of every context, and every pass of
   // a context whose widest pass does not fit the whole-pass kernel
   bool use_dense = false;
@@ -456,56 +453,77 @@ int build_program(sdfp_ctx* c, bool draft, StageDesc** dev, StageShare** dev_sha
 }
 
 // The same for the cluster kernel.
-int build_cluster_program(sdfp_ctx* c, bool draft, ClStage** dev, int* n_all, int* first_gain) {
+std::vector<ClStage> cluster_program(const sdfp_ctx* c, bool draft, int* first_gain) {
   const sdfp_config& g = c->cfg;
-  const int d = g.d_model, f = g.d_ffn;
+  const int d = g.d_model;
   const KvCache& kv = (draft && !c->share_kv) ? c->cache_d : c->cache_t;
   std::vector<ClStage> prog;
-  int resid = -1;  // the last stage that wrote the residual stream: it also leaves gain * h for the next norm
-  auto norm_gain = [&](int gain) {
-    if (resid >= 0)
-      prog[resid].gain_out = gain;
-    else
+  int resid = -1;  // the last stage that wrote the residual stream
+  // the norm in front of the next stage: fp32 applies it there; bf16 where its rows are made, by that stage or with the embedding
+  auto norm = [&](int gain) {
+    if (resid < 0)
       *first_gain = gain;
+    else if (c->bf16)
+      prog[resid].gain = gain;
+    return c->bf16 ? -1 : gain;
   };
-  auto add = [&](const void* w, int kind, int n_pairs, int K, void* kc, void* vc) {
-    prog.push_back(ClStage{reinterpret_cast<const unsigned char*>(w), kc, vc, kind, n_pairs, K, 0, 0});
+  auto add = [&](const void* w, int kind, int K, int gain, void* kc, void* vc) {
+    prog.push_back(ClStage{reinterpret_cast<const unsigned char*>(w), kc, vc, kind, K, gain, 0});
+    if (kind == CL_O || kind == CL_DOWN) resid = (int)prog.size() - 1;
   };
   for (int l = 0; l < g.n_layers; ++l) {
     const LayerWeights& lw = c->layers[l];
     if (!draft || c->keep_attn[l]) {
-      norm_gain(2 * l);
-      add(lw.cl_qkv, CL_QKV, 3 * d / 2, d, kv.k[l], kv.v[l]);
-      add(lw.cl_wo, CL_O, d / 2, d, nullptr, nullptr);
-      resid = (int)prog.size() - 1;
+      add(lw.qkv, CL_QKV, d, norm(2 * l), kv.k[l], kv.v[l]);
+      add(lw.wo, CL_O, d, -1, nullptr, nullptr);
     }
     if (!draft || c->keep_ffn[l]) {
-      norm_gain(2 * l + 1);
-      add(lw.cl_gu, CL_GATE_UP, f, d, nullptr, nullptr);
-      add(lw.cl_down, CL_DOWN, d / 2, f, nullptr, nullptr);
-      resid = (int)prog.size() - 1;
+      add(lw.gu, CL_GATE_UP, d, norm(2 * l + 1), nullptr, nullptr);
+      add(lw.down, CL_DOWN, g.d_ffn, -1, nullptr, nullptr);
     }
   }
-  norm_gain(2 * g.n_layers);
-  add(c->cl_lm_head, CL_HEAD, g.vocab / 2, d, nullptr, nullptr);
-  for (size_t i = prog.size() - 1; i > 0; --i)
-    if (prog[i - 1].kind == CL_O) {
-      prog[i].after_kv = 1;
-      break;
-    }
-  if (*dev == nullptr)
-    if (int r = dev_alloc(c, dev, (size_t)4 * g.n_layers + 1)) return r;
-  CU_OK(c, cudaMemcpyAsync(*dev, prog.data(), prog.size() * sizeof(ClStage), cudaMemcpyHostToDevice, c->stream));
-  CU_OK(c, cudaStreamSynchronize(c->stream));  // prog is a local
-  *n_all = (int)prog.size();
+  add(c->lm_head, CL_HEAD, d, norm(2 * g.n_layers), nullptr, nullptr);
+  return prog;
+}
+
+// Everything the cluster kernel reads besides weights, in one allocation and one copy.  Later only the draft's program changes.
+int build_cluster_programs(sdfp_ctx* c) {
+  const sdfp_config& g = c->cfg;
+  const size_t n_gains = 2 * (size_t)g.n_layers + 1, most = 4 * (size_t)g.n_layers + 1;
+  const size_t gains_at = (c->cl_plan.bytes.size() + 15) / 16 * 16, t_at = gains_at + (n_gains * sizeof(float*) + 15) / 16 * 16;
+  const size_t d_at = t_at + most * sizeof(ClStage), all = d_at + most * sizeof(ClStage);
+  const std::vector<ClStage> draft = cluster_program(c, true, &c->cl_first_d);
+  c->n_cl_d = (int)draft.size();
+  if (c->cl_mem != nullptr) {
+    CU_OK(c, cudaMemcpyAsync(c->cl_prog_d, draft.data(), draft.size() * sizeof(ClStage), cudaMemcpyHostToDevice, c->stream));
+    CU_OK(c, cudaStreamSynchronize(c->stream));  // draft is a local
+    return 0;
+  }
+  const std::vector<ClStage> target = cluster_program(c, false, &c->cl_first_t);
+  c->n_cl_t = (int)target.size();
+  std::vector<const float*> gains(n_gains);
+  for (int l = 0; l < g.n_layers; ++l) {
+    gains[2 * l] = c->layers[l].attn_gain;
+    gains[2 * l + 1] = c->layers[l].ffn_gain;
+  }
+  gains.back() = c->final_gain;
+  std::vector<unsigned char> mem(all, 0);
+  memcpy(mem.data(), c->cl_plan.bytes.data(), c->cl_plan.bytes.size());
+  memcpy(mem.data() + gains_at, gains.data(), n_gains * sizeof(float*));
+  memcpy(mem.data() + t_at, target.data(), target.size() * sizeof(ClStage));
+  memcpy(mem.data() + d_at, draft.data(), draft.size() * sizeof(ClStage));
+  if (int r = dev_alloc(c, &c->cl_mem, all)) return r;
+  c->cl_gains = reinterpret_cast<const float**>(c->cl_mem + gains_at);
+  c->cl_prog_t = reinterpret_cast<ClStage*>(c->cl_mem + t_at);
+  c->cl_prog_d = reinterpret_cast<ClStage*>(c->cl_mem + d_at);
+  CU_OK(c, cudaMemcpyAsync(c->cl_mem, mem.data(), all, cudaMemcpyHostToDevice, c->stream));
+  CU_OK(c, cudaStreamSynchronize(c->stream));  // mem is a local
   return 0;
 }
 
 int build_programs(sdfp_ctx* c) {
-  if (c->use_cluster) {
-    if (int r = build_cluster_program(c, false, &c->cl_prog_t, &c->n_cl_t, &c->cl_first_t)) return r;
-    if (int r = build_cluster_program(c, true, &c->cl_prog_d, &c->n_cl_d, &c->cl_first_d)) return r;
-  }
+  if (c->use_cluster)
+    if (int r = build_cluster_programs(c)) return r;
   if (!c->use_pass) return 0;
   if (int r = build_program(c, false, &c->prog_t, &c->shares_t, &c->n_prog_t)) return r;
   return build_program(c, true, &c->prog_d, &c->shares_d, &c->n_prog_d);
@@ -629,9 +647,11 @@ cudaError_t run_pass(sdfp_ctx* c, bool draft, int rows, int rows_per_seq, bool w
 // ---- the cluster kernel (rounds of small decoders) -----------------------------------------------
 
 using ClKernel = void (*)(const ClParams);
-ClKernel cluster_kernel(const sdfp_config& g) {
-  if (g.dtype == SDFP_BF16) return g.head_dim == 128 ? cluster_pass_kernel<__nv_bfloat16, 128> : cluster_pass_kernel<__nv_bfloat16, 64>;
-  return g.head_dim == 128 ? cluster_pass_kernel<float, 128> : cluster_pass_kernel<float, 64>;
+ClKernel cluster_kernel(const sdfp_ctx* c) {
+  const bool hd128 = c->cfg.head_dim == 128;
+  if (!c->bf16) return hd128 ? cluster_pass_kernel<float, 128, 1> : cluster_pass_kernel<float, 64, 1>;
+  if (c->cl.rows <= 8) return hd128 ? cluster_pass_kernel<__nv_bfloat16, 128, 1> : cluster_pass_kernel<__nv_bfloat16, 64, 1>;
+  return hd128 ? cluster_pass_kernel<__nv_bfloat16, 128, 2> : cluster_pass_kernel<__nv_bfloat16, 64, 2>;
 }
 
 cudaLaunchConfig_t cluster_launch_config(const sdfp_ctx* c, cudaLaunchAttribute* attr) {
@@ -658,15 +678,20 @@ cudaLaunchConfig_t cluster_launch_config(const sdfp_ctx* c, cudaLaunchAttribute*
 //     eight d 256 (12.6 MB) 1.16, d 320 0.92; fp32: one d 256 2.0, d 512 (12.6 MB) 1.10; two d 384 (14 MB) 1.15; four d 256 (12.6 MB) 1.23
 bool cluster_wanted(sdfp_ctx* c, int widest) {
   const sdfp_config& g = c->cfg;
-  if ((g.flags & SDFP_FLAG_NO_PASS_KERNEL) || (c->bf16 && !c->use_mma)) return false;
+  if ((g.flags & SDFP_FLAG_NO_PASS_KERNEL) || (c->bf16 && !c->use_pass)) return false;  // (bf16: the sums are the whole-pass kernel's)
   // every CTA has a share of every stage a layer is made of: the exchange between the stages relies on it
   if (g.d_model < 8 * kClCtas || g.d_ffn < 4 * kClCtas || widest > kClMaxRows) return false;
   const double layer_bytes = (4.0 * g.d_model * g.d_model + 3.0 * g.d_model * g.d_ffn) * (double)c->esz;
   if (layer_bytes * g.max_batch > (g.k_max == 0 ? 13e6 : c->bf16 ? 6.4e6 : 5.2e6)) return false;
-  for (int rows = kClMaxRows; rows >= widest && c->cl.total <= 0; --rows)
-    c->cl = cluster_layout(g.d_model, g.d_ffn, g.n_heads, g.head_dim, g.n_layers, rows, g.max_seq, c->max_smem_optin);
+  // the sums of a layer's stage in one round where shared memory has room for them
+  const ClPlan whole = cluster_plan(g.d_model, g.d_ffn, g.vocab, (int)c->esz, c->pass_grid, 1 << 14);
+  for (int places = std::max(8, whole.most_places);; places = std::max(places / 2, whole.most_cuts)) {
+    c->cl_plan = cluster_plan(g.d_model, g.d_ffn, g.vocab, (int)c->esz, c->pass_grid, places);
+    c->cl = cluster_layout(g.d_model, g.d_ffn, g.n_heads, g.head_dim, g.n_layers, widest, g.max_seq, (int)c->esz, places, c->cl_plan, c->max_smem_optin);
+    if (c->cl.total > 0 || !c->bf16 || places <= whole.most_cuts) break;
+  }
   if (c->cl.total <= 0) return false;
-  const ClKernel kernel = cluster_kernel(g);
+  const ClKernel kernel = cluster_kernel(c);
   int clusters = 0;
   cudaLaunchAttribute attr;
   const cudaLaunchConfig_t lc = cluster_launch_config(c, &attr);
@@ -698,6 +723,7 @@ ClParams cluster_params(const sdfp_ctx* c) {
   p.rope_cos = c->rope_cos;
   p.rope_sin = c->rope_sin;
   p.embed = c->embed;
+  p.plan = c->cl_mem;
   p.lay = c->cl;
   p.logits = c->logits;
   p.gs = c->gs;
@@ -713,7 +739,7 @@ cudaError_t launch_cluster(sdfp_ctx* c, const ClParams& p) {
   cudaLaunchAttribute attr;
   const cudaLaunchConfig_t lc = cluster_launch_config(c, &attr);
   c->launches += 1;
-  return cudaLaunchKernelEx(&lc, cluster_kernel(c->cfg), p);
+  return cudaLaunchKernelEx(&lc, cluster_kernel(c), p);
 }
 
 // One pass of a sampled round, to its logits
@@ -938,16 +964,11 @@ int pack_dense_image(sdfp_ctx* c, void** dst, PackSrc ps, int n_pairs, int K) {
   return 0;
 }
 
-template <typename WT>
-size_t cluster_matrix_bytes(int n_pairs, int K) {
-  return (size_t)n_pairs * cl_steps(K, (int)sizeof(WT)) * kClUnit;
-}
-
 // A matrix in the layout(s) this context's kernels read: `dst` for the whole-pass / per-operation
 // kernels, `img` (may be null) for the dense path.  A context whose decode passes run on the dense
 // path reads only images: `dst` then points to the image as well.
 template <typename WT>
-int pack_matrix(sdfp_ctx* c, void** dst, void** img, void** cl, PackSrc ps, int n_pairs, int K) {
+int pack_matrix(sdfp_ctx* c, void** dst, void** img, PackSrc ps, int n_pairs, int K) {
   if (c->use_dense && img) {
     if (int r = pack_dense_image(c, img, ps, n_pairs, K)) return r;
     if (c->dense_decode) {
@@ -966,12 +987,6 @@ int pack_matrix(sdfp_ctx* c, void** dst, void** img, void** cl, PackSrc ps, int 
   }
   CU_OK(c, cudaGetLastError());
   *dst = p;
-  if (c->use_cluster) {  // (one allocation for all of them: cudaMalloc takes as long as the packing of a small matrix)
-    *cl = c->cl_weights + c->cl_used;
-    c->cl_used += cluster_matrix_bytes<WT>(n_pairs, K);
-    pack_cluster_kernel<WT><<<1184, 256, 0, c->stream>>>(reinterpret_cast<WT*>(*cl), ps, n_pairs, K);
-    CU_OK(c, cudaGetLastError());
-  }
   return 0;
 }
 
@@ -988,35 +1003,23 @@ int load_weights(sdfp_ctx* c, const sdfp_weights* w) {
   const sdfp_config& g = c->cfg;
   const int d = g.d_model, f = g.d_ffn, H = g.n_heads, hd = g.head_dim;
   c->layers.resize(g.n_layers);
-  if (c->use_cluster) {
-    const size_t layer = cluster_matrix_bytes<WT>(3 * d / 2, d) + cluster_matrix_bytes<WT>(d / 2, d) + cluster_matrix_bytes<WT>(f, d) +
-                         cluster_matrix_bytes<WT>(d / 2, f);
-    if (int r = dev_alloc(c, &c->cl_weights, layer * g.n_layers + cluster_matrix_bytes<WT>(g.vocab / 2, d))) return r;
-  }
   for (int l = 0; l < g.n_layers; ++l) {
     LayerWeights& lw = c->layers[l];
     if (!w->wq[l] || !w->wk[l] || !w->wv[l] || !w->wo[l] || !w->w_gate[l] || !w->w_up[l] || !w->w_down[l] ||
         !w->attn_norm[l] || !w->ffn_norm[l])
       return fail(c, SDFP_EINVAL, "layer %d has a NULL weight pointer", l);
-    if (int r = pack_matrix<WT>(c, &lw.qkv, &lw.um_qkv, &lw.cl_qkv, PackSrc{w->wq[l], w->wk[l], w->wv[l], 0, H, hd}, 3 * d / 2, d)) return r;
-    if (int r = pack_matrix<WT>(c, &lw.wo, &lw.um_wo, &lw.cl_wo, PackSrc{w->wo[l], nullptr, nullptr, 2, H, hd}, d / 2, d)) return r;
-    if (int r = pack_matrix<WT>(c, &lw.gu, &lw.um_gu, &lw.cl_gu, PackSrc{w->w_gate[l], w->w_up[l], nullptr, 1, H, hd}, f, d)) return r;
-    if (int r = pack_matrix<WT>(c, &lw.down, &lw.um_down, &lw.cl_down, PackSrc{w->w_down[l], nullptr, nullptr, 2, H, hd}, d / 2, f)) return r;
+    if (int r = pack_matrix<WT>(c, &lw.qkv, &lw.um_qkv, PackSrc{w->wq[l], w->wk[l], w->wv[l], 0, H, hd}, 3 * d / 2, d)) return r;
+    if (int r = pack_matrix<WT>(c, &lw.wo, &lw.um_wo, PackSrc{w->wo[l], nullptr, nullptr, 2, H, hd}, d / 2, d)) return r;
+    if (int r = pack_matrix<WT>(c, &lw.gu, &lw.um_gu, PackSrc{w->w_gate[l], w->w_up[l], nullptr, 1, H, hd}, f, d)) return r;
+    if (int r = pack_matrix<WT>(c, &lw.down, &lw.um_down, PackSrc{w->w_down[l], nullptr, nullptr, 2, H, hd}, d / 2, f)) return r;
     if (int r = widen_gain<WT>(c, &lw.attn_gain, w->attn_norm[l], d)) return r;
     if (int r = widen_gain<WT>(c, &lw.ffn_gain, w->ffn_norm[l], d)) return r;
   }
   // the prompt pass needs no logits: only contexts that decode on the dense path get an lm-head image
-  if (int r = pack_matrix<WT>(c, &c->lm_head, c->dense_decode ? &c->um_lm_head : nullptr, &c->cl_lm_head,
+  if (int r = pack_matrix<WT>(c, &c->lm_head, c->dense_decode ? &c->um_lm_head : nullptr,
                               PackSrc{w->lm_head, nullptr, nullptr, 2, H, hd}, g.vocab / 2, d))
     return r;
   if (int r = widen_gain<WT>(c, &c->final_gain, w->final_norm, d)) return r;
-  if (c->use_cluster) {
-    if (int r = dev_alloc(c, &c->cl_gains, (size_t)(2 * g.n_layers + 1) * d)) return r;
-    for (int i = 0; i <= 2 * g.n_layers; ++i) {
-      const float* src = i == 2 * g.n_layers ? c->final_gain : i & 1 ? c->layers[i / 2].ffn_gain : c->layers[i / 2].attn_gain;
-      CU_OK(c, cudaMemcpyAsync(c->cl_gains + (size_t)i * d, src, (size_t)d * 4, cudaMemcpyDeviceToDevice, c->stream));
-    }
-  }
   WT* e = nullptr;
   if (int r = dev_alloc(c, &e, (size_t)g.vocab * d)) return r;
   CU_OK(c, cudaMemcpyAsync(e, w->tok_embed, (size_t)g.vocab * d * sizeof(WT), cudaMemcpyDeviceToDevice, c->stream));
@@ -1157,7 +1160,6 @@ extern "C" int sdfp_create(const sdfp_config* cfg, const sdfp_weights* w, void* 
   c->max_smem_optin = optin;
   c->use_dense = c->use_mma && !(g.flags & SDFP_FLAG_NO_DENSE);
   c->dense_decode = c->use_dense && !c->use_pass && !(g.flags & SDFP_FLAG_NO_PASS_KERNEL);
-  c->use_cluster = !c->dense_decode && cluster_wanted(c, widest);
   if (c->use_dense) {
     c->prompt_rows = std::min((int)kPromptRows, g.max_batch * std::min((int)kGroupedPrompt, g.max_seq));
     c->rows_cap = std::max(std::max((int)kMaxRows, g.max_seq), c->prompt_rows);
@@ -1194,6 +1196,7 @@ extern "C" int sdfp_create(const sdfp_config* cfg, const sdfp_weights* w, void* 
       return bail(SDFP_ECUDA);
     }
   }
+  c->use_cluster = cluster_wanted(c, widest);
   if (cudaError_t ke = configure_kernels(c)) {
     c->err = std::string("kernel configuration failed: ") + cudaGetErrorString(ke);
     return bail(SDFP_ECUDA);

@@ -66,6 +66,46 @@ def test_rounds_of_a_batch(dtype, batch, k, prompt):
         eng.close()
 
 
+@pytest.mark.parametrize("heads,head_dim,ffn,vocab,dtype,batch,k,new", [
+    (2, 64, 64, 16, "f32", 1, 3, 90),       # draft rows in front of the text, two chunks of keys
+    (4, 64, 688, 528, "f32", 1, 8, 40),     # nine rows
+    (3, 128, 528, 400, "f32", 2, 0, 150),
+    (2, 64, 64, 16, "bf16", 1, 3, 90),      # k-classes and CTAs without a unit, half a tile per CTA
+    (4, 64, 688, 528, "bf16", 1, 8, 40),    # two column groups; sums in three pieces
+    (4, 64, 688, 2048, "bf16", 2, 2, 140),
+    (3, 128, 1040, 400, "bf16", 1, 5, 70),
+    (8, 64, 1376, 4096, "bf16", 1, 0, 600),  # ten chunks: the first splits walk two
+])
+def test_rounds_have_the_bits_of_the_other_passes(heads, head_dim, ffn, vocab, dtype, batch, k, new):
+    """Keys and values that rounds leave in either cache, the tokens they choose and the counts they accept are those of the
+    kernels that run prompts and sdfp_forward_logits: logits behind a generated text are, bit for bit, the ones of the same
+    text fed from its first token, and every token is the first largest of its row.  A text goes on the same in a second call."""
+    shape = si.ModelShape("bits", 4, heads * head_dim, heads, head_dim, ffn, vocab, dtype=dtype)
+    eng, m, _ = make_pair(shape, (1, 2), max_seq=new + k + 8, max_batch=batch, k_max=k, random_gains=True)
+    try:
+        first = si.make_prompts(vocab, batch, 1, seed=61)
+        out = eng.sdfp_generate(first, k, new)
+        assert out.timing["kernel_launches"] == 1
+        text = first[0].tolist() + list(out.tokens[0])
+        tail = 12  # (behind a round the caches hold all keys in front of the last token)
+        for draft in ([False, True] if k else [False]):
+            got = eng.sdfp_forward_logits(text[-tail:-1], len(text) - tail, draft=draft)
+            whole = np.concatenate([eng.sdfp_forward_logits(text[i:i + 80], i, draft=draft) for i in range(0, len(text) - 1, 80)])[:len(text) - 1]
+            assert np.array_equal(got.view(np.uint32), whole[-tail + 1:].view(np.uint32))
+            if not draft:
+                assert text[1:] == [int(np.argmax(row)) for row in whole]
+        if batch == 1:
+            half = new // 2
+            if dtype == "f32" or half + 1 <= 16:  # (longer bf16 prompts run on the tcgen05 path)
+                on = eng.sdfp_generate(np.asarray([text[:1 + half]], dtype=np.int32), k, new - half)
+                assert on.tokens[0] == out.tokens[0][half:]
+        if k:  # drafted tokens are the draft's first largest
+            eng.sdfp_set_draft_layers(np.ones(shape.n_layers, dtype=np.uint8))
+            assert (eng.sdfp_generate(first, k, 20).stats[:-1, :, 1] == k).all()
+    finally:
+        eng.close()
+
+
 def test_an_end_token():
     """A sequence that ends early stays where it is while the other goes on; calls behind it start afresh."""
     eng, m, _ = make_pair(si.TINY_BF16, (1, 2), max_seq=64, max_batch=2, k_max=4)
