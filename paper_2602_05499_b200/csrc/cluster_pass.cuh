@@ -47,7 +47,7 @@ constexpr int kClMaxRows = 16;
 constexpr int kClTeam = 128;     // threads that work on an attention item
 constexpr int kClAttnRows = 8;   // rows of a sequence it takes together
 constexpr int kClTiles = 4;      // bf16: tiles a warp multiplies together
-constexpr int kClAhead = 8;      // bf16: units of weights (512 bytes a warp) in half of its ring
+constexpr int kClRing = 16;      // bf16: units of weights (512 bytes) a warp has on their way
 
 enum ClBar { CL_BAR_H = 0, CL_BAR_U = 1, CL_BAR_QKV = 2, CL_BAR_PART = 3, CL_BAR_X = 4, CL_BAR_TOK = 5, CL_BARS = 6 };
 enum ClKind { CL_QKV = 0, CL_O = 1, CL_GATE_UP = 2, CL_DOWN = 3, CL_HEAD = 4, CL_KINDS = 5 };
@@ -79,13 +79,12 @@ struct ClRound {
   int quad0, n_quads;  // fours of pairs that are finished in this round
   unsigned magic;      // i / n_quads == i * magic >> 20 for the few hundred vectors of a round
   int tile0, np;       // bf16: its first tile, and the pieces a sum is made of
-  int n_entries;       // bf16: of each warp
-  int pad[2];
+  int pad[3];
 };
 struct ClEntry {       // bf16: one k-tile of a warp, for up to kClTiles neighbouring tiles
   int w;               // the first tile's unit, in uint4 from the matrix's start
   short kt, slot;      // k-tile, -1: none; slot >= 0: the sums are complete and go to this place, a tile's np places apart
-  unsigned char n_tiles, wrap, np, pad;  // from tile `wrap` on they lie in the next group
+  unsigned char n_tiles, wrap, np, last;  // from tile `wrap` on they lie in the next group; last: of the round, 2: of all
   int pad2;
 };
 static_assert(sizeof(ClMine) == 32 && sizeof(ClRound) == 32 && sizeof(ClEntry) == 16, "copied in sixteen bytes");
@@ -236,6 +235,10 @@ __device__ __forceinline__ void cl_wait(ClShared* sh, PassSync* sync, int which,
   if (!cl_try_wait(bar, parity)) cl_poll(sh, sync, bar, parity);
   __syncwarp();
 }
+
+// The same value in all lanes, and known to be: in a loop that could run a different number of times in the lanes of a warp, every
+// shuffle first gathers the warp with a routine of a hundred clocks and more (a softmax row 2600 clocks, with this ${SM}).
+__device__ __forceinline__ int cl_uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 // the better of two (value, index), ties to the lower index
 __device__ __forceinline__ void cl_better(float& bv, int& bi, float v, int i) {
@@ -467,46 +470,55 @@ __device__ __forceinline__ void cl_dots_f32(const ClParams& p, const ClEnv& ev, 
   }
 }
 
-// bf16: the weights of a stage on their way to a warp, through a ring of two halves in shared memory.  Every lane copies what it
-// will use itself, so nothing but its own wait stands between the copy and the use.
+// bf16: the weights of a stage on their way to a warp, through a ring in shared memory.  Every lane copies what it will use
+// itself, so nothing but its own wait stands between the copy and the use.  An entry of the list is a group of copies; as many are
+// on their way as entries of the stage's width fill the ring.
 struct ClRing {
-  const uint4* W;       // the matrix, this lane's part
-  const ClEntry* ent;   // this warp's list
-  int buf, steps, step, per, wrap_jump;  // halves in all and asked for so far, entries of a half
+  const uint4* W;        // the matrix, this lane's part
+  const ClEntry* next;   // of this warp's list, null behind its end
+  int buf, at, width, wrap_jump;  // the ring, where in it the next entry goes, units of an entry
   __device__ __forceinline__ void ask() {
-    if (step < steps) {
-      const ClEntry* e = ent + step * per;
-      uint32_t to = buf + (step & 1) * (kClAhead * 512);
-#pragma unroll 1
-      for (int u = 0; u < per; ++u, to += kClAhead * 512 / per) {
-        const int4 v = *reinterpret_cast<const int4*>(e + u);
+    if (next != nullptr) {
+      const int4 v = *reinterpret_cast<const int4*>(next);
+      if ((short)v.y >= 0) {
         const uint4* w = W + v.x;
-        if ((short)v.y >= 0)
+        const int n = v.z & 255, wrap = (v.z >> 8) & 255;
 #pragma unroll
-          for (int t = 0; t < kClTiles; ++t)
-            if (t < (v.z & 255)) cp_async16_to(to + t * 512, w + t * 32 + (t >= ((v.z >> 8) & 255) ? wrap_jump : 0));
+        for (int t = 0; t < kClTiles; ++t)
+          if (t < n)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(buf + at + t * 512), "l"(w + t * 32 + (t >= wrap ? wrap_jump : 0)) : "memory");
       }
-      ++step;
+      next = (v.z >> 24) > 1 ? nullptr : next + 1;
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+    at = (at + width * 512) & (kClRing * 512 - 1);
   }
-  static __device__ __forceinline__ void cp_async16_to(uint32_t dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+  __device__ __forceinline__ void wait() const {  // for the oldest entry
+    if (width == 1)
+      asm volatile("cp.async.wait_group %0;" ::"n"(kClRing - 1) : "memory");
+    else if (width == 2)
+      asm volatile("cp.async.wait_group %0;" ::"n"(kClRing / 2 - 1) : "memory");
+    else
+      asm volatile("cp.async.wait_group %0;" ::"n"(kClRing / 4 - 1) : "memory");
   }
 };
 
-// One half of the ring.  CG: column groups of eight rows.  The accumulators go on from half to half; complete sums are left as
-// [place][class][row of the tile][two rows of the pass] of 128 bits, as a lane holds them: {half 0 of rows 2 q and 2 q + 1, half 1 of the same}.
+// The entries of a round.  CG: column groups of eight rows.  Complete sums are left as [place][class][row of the tile][two rows of
+// the pass] of 128 bits, as a lane holds them: {half 0 of rows 2 q and 2 q + 1, half 1 of the same}.
 template <int CG>
-__device__ __forceinline__ void cl_mma_half(const ClParams& p, const ClEnv& ev, const ClDots& a, const ClEntry* e, int per, uint32_t from,
-                                            float (&acc)[kClTiles][CG][4]) {
+__device__ __forceinline__ void cl_mma_round(const ClParams& p, const ClEnv& ev, int x_at, const ClEntry*& ent, ClRing& ring) {
   const int g = ev.lane >> 2, q = ev.lane & 3, R = ev.R, Q = (R + 1) / 2;
-  const uint2* const x = cl_at<uint2>(a.x) + g * 4 + q;
-  int4 v = *reinterpret_cast<const int4*>(e);
-#pragma unroll 1
-  for (int u = 0; u < per; ++u, from += kClAhead * 512 / per) {
-    const int n = v.z & 255, kt = (short)v.y, slot = v.y >> 16, np = (v.z >> 16) & 255;
-    if (u + 1 < per) v = *reinterpret_cast<const int4*>(e + u + 1);
+  const uint2* const x = cl_at<uint2>(x_at) + g * 4 + q;
+  float4* const red = cl_at<float4>(p.lay.red) + (ev.warp * 8 + g) * Q + q;
+  float acc[kClTiles][CG][4];
+#pragma unroll
+  for (int i = 0; i < kClTiles; ++i)
+#pragma unroll
+    for (int c = 0; c < CG; ++c) acc[i][c][0] = acc[i][c][1] = acc[i][c][2] = acc[i][c][3] = 0.f;
+  int4 v;
+  do {
+    v = *reinterpret_cast<const int4*>(ent++);
+    const int n = v.z & 255, kt = (short)v.y, slot = v.y >> 16;
     if (kt >= 0) {
       uint2 b0[CG], b1[CG];
 #pragma unroll
@@ -517,11 +529,12 @@ __device__ __forceinline__ void cl_mma_half(const ClParams& p, const ClEnv& ev, 
           b1[c] = x[kt * 8 * R + c * 32 + 4 * R];
         }
       }
+      ring.wait();
 #pragma unroll
       for (int t = 0; t < kClTiles; ++t)
         if (t < n) {
           uint4 w;
-          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "r"(from + t * 512) : "memory");
+          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "r"(ring.buf + ring.at + t * 512) : "memory");
 #pragma unroll
           for (int c = 0; c < CG; ++c) {
             mma_bf16_16816(acc[t][c], w, b0[c].x, b1[c].x);
@@ -529,17 +542,19 @@ __device__ __forceinline__ void cl_mma_half(const ClParams& p, const ClEnv& ev, 
           }
         }
     }
+    ring.ask();  // into the place just read
     if (slot >= 0) {
-      float4* o = cl_at<float4>(p.lay.red) + ((slot * kClasses + ev.warp) * 8 + g) * Q + q;
+      float4* o = red + slot * kClasses * 8 * Q;
+      const int step = ((v.z >> 16) & 255) * kClasses * 8 * Q;
 #pragma unroll
       for (int t = 0; t < kClTiles; ++t)
 #pragma unroll
         for (int c = 0; c < CG; ++c) {
-          if (t < n && c * 4 + q < Q) o[t * np * kClasses * 8 * Q + c * 4] = make_float4(acc[t][c][0], acc[t][c][1], acc[t][c][2], acc[t][c][3]);
+          if (t < n && c * 4 + q < Q) o[t * step + c * 4] = make_float4(acc[t][c][0], acc[t][c][1], acc[t][c][2], acc[t][c][3]);
           acc[t][c][0] = acc[t][c][1] = acc[t][c][2] = acc[t][c][3] = 0.f;
         }
     }
-  }
+  } while ((v.z >> 24) == 0);
 }
 
 // bf16: both halves of a pair, each the classes of a piece in order, then the pieces
@@ -714,7 +729,7 @@ __device__ __forceinline__ void cl_attend(const ClParams& p, const ClEnv& ev, co
   using A = ClAttn<WT, HD>;
   constexpr bool BF = A::BF;
   constexpr int C = A::C;
-  const int team = ev.tid / kClTeam, tt = ev.tid % kClTeam, w4 = tt >> 5, lane = ev.lane;
+  const int team = ev.warp / (kClTeam / 32), w4 = ev.warp % (kClTeam / 32), tt = ev.tid % kClTeam, lane = ev.lane;
   const int R = ev.R, row0 = b * ev.rps + first_row, rps = RM == 1 ? 1 : min(RM, ev.rps - first_row), rows_all = p.lay.heads_per_cta * R;
   const int max_pos = ev.sh->pos[row0 + rps - 1];
   // positions of a sequence's rows follow one another, and with them the keys that are not in the cache
@@ -798,7 +813,7 @@ __device__ __forceinline__ void cl_attend(const ClParams& p, const ClEnv& ev, co
     // softmax of the chunk, a warp per row
 #pragma unroll 1
     for (int i = w4; i < rps; i += kClTeam / 32) {
-      const int n = min(C, ev.sh->pos[row0 + i] + 1 - key0);
+      const int n = cl_uniform(min(C, ev.sh->pos[row0 + i] + 1 - key0));
       if (n <= 0) {  // the row sees nothing here
         if (lane == 0) s_a[i] = 1.f;
         sS[i * C + lane] = 0.f;
@@ -948,7 +963,7 @@ __device__ __forceinline__ void cl_attention(const ClParams& p, const ClEnv& ev,
     return reinterpret_cast<WT*>(base) + ((size_t)b * p.heads + head0 + hl * kClCtas) * p.max_seq * HD;
   };
   const unsigned qkv_bytes = (unsigned)(nh * R * (HD * 4 + 2 * HD * (int)sizeof(WT))), parity = phase(CL_BAR_QKV);
-  const int team = ev.tid / kClTeam;
+  const int team = ev.warp / (kClTeam / 32);
   bool waited = false;
   int turn = 0;
 #pragma unroll 1
@@ -1085,7 +1100,7 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
   ev.rounds = cl_at<ClRound>(p.lay.plan_rounds);
   ev.entries = cl_at<ClEntry>(p.lay.plan_entries);
   ev.tid = tid;
-  ev.warp = tid >> 5;
+  ev.warp = cl_uniform(tid >> 5);
   ev.lane = tid & 31;
   ev.rank = rank;
   ev.self = smem_u32(cl_smem);
@@ -1177,35 +1192,25 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
       const ClMine& me = ev.mine[t.kind];
       const bool is_head = t.kind == CL_HEAD;
       if constexpr (BF) {
+        const ClEntry* ent = ev.entries + me.entry0 + ev.warp * me.n_entries;
         ClRing ring;
         ring.W = reinterpret_cast<const uint4*>(a.W) + ev.lane;
-        ring.ent = ev.entries + me.entry0 + ev.warp * me.n_entries;
-        ring.buf = (int)ev.self + p.lay.ring + ev.warp * (2 * kClAhead * 512) + ev.lane * 16;
-        ring.per = kClAhead / me.tile_width;
-        ring.steps = me.n_entries / ring.per;
-        ring.step = 0;
+        ring.next = me.n_rounds > 0 ? ent : nullptr;
+        ring.buf = (int)ev.self + p.lay.ring + ev.warp * (kClRing * 512) + ev.lane * 16;
+        ring.at = 0;
+        ring.width = me.tile_width;
         ring.wrap_jump = (a.K / 16 - 1) * 256;  // to the next group's unit of the same k-tile, which starts with its first tile
 #pragma unroll 1
-        for (int i = 0; i < 2; ++i) ring.ask();
+        for (int i = 0; i < kClRing; i += ring.width) ring.ask();
         if (a.bar >= 0) cl_wait(sh, p.sync, a.bar, a.bytes, a.parity);
         // lm-head: 256 threads over the rows, a power of two of them each
         const int row_log = R <= 1 ? 8 : R <= 2 ? 7 : R <= 4 ? 6 : R <= 8 ? 5 : 4;
         float bv = -INFINITY;
-        int bi = 0x7fffffff, done = 0;
-        float acc[kClTiles][CG][4];
-#pragma unroll
-        for (int i = 0; i < kClTiles; ++i)
-#pragma unroll
-          for (int c = 0; c < CG; ++c) acc[i][c][0] = acc[i][c][1] = acc[i][c][2] = acc[i][c][3] = 0.f;
+        int bi = 0x7fffffff;
 #pragma unroll 1
         for (int r = 0; r < me.n_rounds; ++r) {
           const ClRound& rd = ev.rounds[me.round0 + r];
-#pragma unroll 1
-          for (int end = done + rd.n_entries / ring.per; done < end; ++done) {
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-            cl_mma_half<CG>(p, ev, a, ring.ent + done * ring.per, ring.per, ring.buf + (done & 1) * (kClAhead * 512), acc);
-            ring.ask();
-          }
+          cl_mma_round<CG>(p, ev, a.x, ent, ring);
           if (a.norm && a.bar >= 0 && r == 0) cl_row_scales(p, ev);  // (the first stage's were made with the embedding)
           __syncthreads();  // the sums are there
           if (is_head) {
@@ -1306,7 +1311,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_pass_kernel(const __gri
   ClTab* tab_d = tab_t + p.n_t;
   const int tid = threadIdx.x, rank = (int)cl_rank();
   const bool loop = p.rounds > 0;
-  const int batch = loop ? p.gs->batch : p.pd.n_seq, k = loop ? p.gs->k : 0;
+  const int batch = cl_uniform(loop ? p.gs->batch : p.pd.n_seq), k = cl_uniform(loop ? p.gs->k : 0);
 
   // ---- set-up: this CTA's plan, stage tables, the gains of its features, state ----
 #pragma unroll 1
@@ -1459,7 +1464,6 @@ inline ClPlan cluster_plan(int d, int f, int vocab, int elem_bytes, int pass_gri
       }
       if (kind != CL_HEAD) out.most_places = std::max(out.most_places, places);
       m.tile_width = width == 3 ? 4 : width;
-      const int per = kClAhead / m.tile_width;
       std::vector<std::vector<ClEntry>> lists(kClasses);
       for (size_t b = 0; b < batches.size();) {
         size_t e = b;
@@ -1469,9 +1473,7 @@ inline ClPlan cluster_plan(int d, int f, int vocab, int elem_bytes, int pass_gri
         ClRound& r = add_round(std::max(m.p0, tile0 * 8), std::min(m.p0 + m.np, (tile0 + tiles) * 8));
         r.tile0 = tile0;
         r.np = batches[b].np;
-        const size_t begin = lists[0].size();
-        size_t longest = 0;
-        for (int cls = 0; cls < kClasses; ++cls) {
+        for (int cls = 0; cls < kClasses; ++cls)
           for (size_t i = b; i < e; ++i) {
             const Batch& bt = batches[i];
             const int grp = bt.tile / kUnitTiles, in = bt.tile % kUnitTiles;
@@ -1495,17 +1497,14 @@ inline ClPlan cluster_plan(int d, int f, int vocab, int elem_bytes, int pass_gri
               }
             }
           }
-          longest = std::max(longest, lists[cls].size());
-        }
-        longest = begin + (longest - begin + per - 1) / per * per;
-        ClEntry none{};
-        none.kt = none.slot = -1;
-        for (auto& l : lists) l.resize(longest, none);
-        r.n_entries = (int)(longest - begin);
         b = e;
+        for (auto& l : lists) l.back().last = b < batches.size() ? 1 : 2;
       }
-      m.n_entries = (int)lists[0].size();
-      for (const auto& l : lists) c.entries.insert(c.entries.end(), l.begin(), l.end());
+      for (const auto& l : lists) m.n_entries = std::max(m.n_entries, (int)l.size());
+      for (auto& l : lists) {
+        l.resize(m.n_entries);
+        c.entries.insert(c.entries.end(), l.begin(), l.end());
+      }
     }
   }
   size_t rounds = 0, entries = 0;
@@ -1566,7 +1565,7 @@ inline ClLayout cluster_layout(int d, int f, int heads, int hd, int n_layers, in
   take(y.team, 2LL * y.team_bytes);
   const int team_end = at;
   at = w0;
-  take(y.ring, bf16 ? kClWarps * 2LL * kClAhead * 512 : 0);
+  take(y.ring, bf16 ? kClWarps * (long long)kClRing * 512 : 0);
   take(y.red, bf16 ? (long long)place_slots * kClasses * 8 * ((rows + 1) / 2) * 16 : 0);
   at = std::max(at, team_end);
   take(y.rope, 4LL * rows * hd);
