@@ -237,7 +237,7 @@ __device__ __forceinline__ void cl_wait(ClShared* sh, PassSync* sync, int which,
 }
 
 // The same value in all lanes, and known to be: in a loop that could run a different number of times in the lanes of a warp, every
-// shuffle first gathers the warp with a routine of a hundred clocks and more (a softmax row 2600 clocks, with this ${SM}).
+// shuffle first gathers the warp with a routine of a hundred clocks and more (a row's softmax took 2600 clocks instead of 600).
 __device__ __forceinline__ int cl_uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 // the better of two (value, index), ties to the lower index
@@ -366,7 +366,7 @@ __device__ __forceinline__ void cl_dots_f32(const ClParams& p, const ClEnv& ev, 
   constexpr int N = RT * P * 2, CH = N < 16 ? N : 16;
   const int warp = ev.warp, lane = ev.lane, R = ev.R;
   const ClMine& me = ev.mine[a.kind];
-  const int np = me.np;
+  const int np = cl_uniform(me.np);
   const int n_w = RT == 1 ? (np + kClWarps - 1) / kClWarps : (np / 2 + kClWarps - 1) / kClWarps * 2;  // pairs per warp
   const int first = warp * n_w, cnt = max(0, min(n_w, np - first));
   const int half_len = a.K / 4;  // in uint4
@@ -475,23 +475,35 @@ __device__ __forceinline__ void cl_dots_f32(const ClParams& p, const ClEnv& ev, 
 // on their way as entries of the stage's width fill the ring.
 struct ClRing {
   const uint4* W;        // the matrix, this lane's part
-  const ClEntry* next;   // of this warp's list, null behind its end
-  int buf, at, width, wrap_jump;  // the ring, where in it the next entry goes, units of an entry
+  const ClEntry* next;   // of this warp's list; the last one repeats itself
+  int4 v;                // *next
+  uint32_t buf;          // the ring
+  int at, width, wrap_jump;  // where in it the next entry goes, units of an entry
+  __device__ __forceinline__ void begin(const ClEntry* first) {
+    next = first;
+    get();
+    at = 0;
+  }
   __device__ __forceinline__ void ask() {
-    if (next != nullptr) {
-      const int4 v = *reinterpret_cast<const int4*>(next);
-      if ((short)v.y >= 0) {
-        const uint4* w = W + v.x;
-        const int n = v.z & 255, wrap = (v.z >> 8) & 255;
+    if ((short)v.y >= 0) {
+      const uint4* w = W + v.x;
+      const int n = v.z & 255, wrap = (v.z >> 8) & 255;
 #pragma unroll
-        for (int t = 0; t < kClTiles; ++t)
-          if (t < n)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(buf + at + t * 512), "l"(w + t * 32 + (t >= wrap ? wrap_jump : 0)) : "memory");
-      }
-      next = (v.z >> 24) > 1 ? nullptr : next + 1;
+      for (int t = 0; t < kClTiles; ++t)
+        if (t < n)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(buf + at + t * 512), "l"(w + t * 32 + (t >= wrap ? wrap_jump : 0)) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
     at = (at + width * 512) & (kClRing * 512 - 1);
+    if ((v.z >> 24) > 1)
+      v.y = -1;  // nothing any more
+    else
+      ++next, get();
+  }
+  __device__ __forceinline__ void get() {
+    v = *reinterpret_cast<const int4*>(next);
+    v.y = cl_uniform(v.y);
+    v.z = cl_uniform(v.z);
   }
   __device__ __forceinline__ void wait() const {  // for the oldest entry
     if (width == 1)
@@ -504,7 +516,8 @@ struct ClRing {
 };
 
 // The entries of a round.  CG: column groups of eight rows.  Complete sums are left as [place][class][row of the tile][two rows of
-// the pass] of 128 bits, as a lane holds them: {half 0 of rows 2 q and 2 q + 1, half 1 of the same}.
+// the pass] of 128 bits, as a lane holds them: {half 0 of rows 2 q and 2 q + 1, half 1 of the same}.  What an entry needs besides its
+// weights is read while the one in front of it is multiplied.
 template <int CG>
 __device__ __forceinline__ void cl_mma_round(const ClParams& p, const ClEnv& ev, int x_at, const ClEntry*& ent, ClRing& ring) {
   const int g = ev.lane >> 2, q = ev.lane & 3, R = ev.R, Q = (R + 1) / 2;
@@ -515,34 +528,47 @@ __device__ __forceinline__ void cl_mma_round(const ClParams& p, const ClEnv& ev,
   for (int i = 0; i < kClTiles; ++i)
 #pragma unroll
     for (int c = 0; c < CG; ++c) acc[i][c][0] = acc[i][c][1] = acc[i][c][2] = acc[i][c][3] = 0.f;
-  int4 v;
-  do {
-    v = *reinterpret_cast<const int4*>(ent++);
-    const int n = v.z & 255, kt = (short)v.y, slot = v.y >> 16;
-    if (kt >= 0) {
-      uint2 b0[CG], b1[CG];
+  uint2 b0[CG], b1[CG];
+  auto load_x = [&](int kt) {
 #pragma unroll
-      for (int c = 0; c < CG; ++c) {
-        b0[c] = b1[c] = make_uint2(0u, 0u);
-        if (c * 8 + g < R) {
-          b0[c] = x[kt * 8 * R + c * 32];
-          b1[c] = x[kt * 8 * R + c * 32 + 4 * R];
-        }
+    for (int c = 0; c < CG; ++c) {
+      b0[c] = b1[c] = make_uint2(0u, 0u);
+      if (kt >= 0 && c * 8 + g < R) {
+        b0[c] = x[kt * 8 * R + c * 32];
+        b1[c] = x[kt * 8 * R + c * 32 + 4 * R];
       }
+    }
+  };
+  int4 v = *reinterpret_cast<const int4*>(ent);
+  v.y = cl_uniform(v.y);
+  v.z = cl_uniform(v.z);
+  load_x((short)v.y);
+  for (;;) {
+    const int n = v.z & 255, slot = v.y >> 16, last = v.z >> 24;
+    int4 vn = *reinterpret_cast<const int4*>(ent + (last ? 0 : 1));
+    vn.y = cl_uniform(vn.y);
+    vn.z = cl_uniform(vn.z);
+    if ((short)v.y >= 0) {
       ring.wait();
+      uint4 w[kClTiles];
 #pragma unroll
       for (int t = 0; t < kClTiles; ++t)
-        if (t < n) {
-          uint4 w;
-          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "r"(ring.buf + ring.at + t * 512) : "memory");
+        if (t < n)
+          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                       : "=r"(w[t].x), "=r"(w[t].y), "=r"(w[t].z), "=r"(w[t].w)
+                       : "r"(ring.buf + ring.at + t * 512)
+                       : "memory");
+#pragma unroll
+      for (int t = 0; t < kClTiles; ++t)
+        if (t < n)
 #pragma unroll
           for (int c = 0; c < CG; ++c) {
-            mma_bf16_16816(acc[t][c], w, b0[c].x, b1[c].x);
-            mma_bf16_16816(acc[t][c], w, b0[c].y, b1[c].y);
+            mma_bf16_16816(acc[t][c], w[t], b0[c].x, b1[c].x);
+            mma_bf16_16816(acc[t][c], w[t], b0[c].y, b1[c].y);
           }
-        }
     }
     ring.ask();  // into the place just read
+    if (!last) load_x((short)vn.y);
     if (slot >= 0) {
       float4* o = red + slot * kClasses * 8 * Q;
       const int step = ((v.z >> 16) & 255) * kClasses * 8 * Q;
@@ -554,7 +580,10 @@ __device__ __forceinline__ void cl_mma_round(const ClParams& p, const ClEnv& ev,
           acc[t][c][0] = acc[t][c][1] = acc[t][c][2] = acc[t][c][3] = 0.f;
         }
     }
-  } while ((v.z >> 24) == 0);
+    ++ent;
+    if (last) break;
+    v = vn;
+  }
 }
 
 // bf16: both halves of a pair, each the classes of a piece in order, then the pieces
@@ -1195,20 +1224,22 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
         const ClEntry* ent = ev.entries + me.entry0 + ev.warp * me.n_entries;
         ClRing ring;
         ring.W = reinterpret_cast<const uint4*>(a.W) + ev.lane;
-        ring.next = me.n_rounds > 0 ? ent : nullptr;
-        ring.buf = (int)ev.self + p.lay.ring + ev.warp * (kClRing * 512) + ev.lane * 16;
-        ring.at = 0;
-        ring.width = me.tile_width;
+        ring.buf = ev.self + p.lay.ring + ev.warp * (kClRing * 512) + ev.lane * 16;
+        ring.width = cl_uniform(me.tile_width);
         ring.wrap_jump = (a.K / 16 - 1) * 256;  // to the next group's unit of the same k-tile, which starts with its first tile
+        const int n_rounds = cl_uniform(me.n_rounds);
+        if (n_rounds > 0) {
+          ring.begin(ent);
 #pragma unroll 1
-        for (int i = 0; i < kClRing; i += ring.width) ring.ask();
+          for (int i = 0; i < kClRing; i += ring.width) ring.ask();
+        }
         if (a.bar >= 0) cl_wait(sh, p.sync, a.bar, a.bytes, a.parity);
         // lm-head: 256 threads over the rows, a power of two of them each
         const int row_log = R <= 1 ? 8 : R <= 2 ? 7 : R <= 4 ? 6 : R <= 8 ? 5 : 4;
         float bv = -INFINITY;
         int bi = 0x7fffffff;
 #pragma unroll 1
-        for (int r = 0; r < me.n_rounds; ++r) {
+        for (int r = 0; r < n_rounds; ++r) {
           const ClRound& rd = ev.rounds[me.round0 + r];
           cl_mma_round<CG>(p, ev, a.x, ent, ring);
           if (a.norm && a.bar >= 0 && r == 0) cl_row_scales(p, ev);  // (the first stage's were made with the embedding)
@@ -1225,10 +1256,10 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
               cl_send_all<WT>(p, ev, me, rd, t.kind, t.gain_out);
             }
           }
-          if (r + 1 < me.n_rounds) __syncthreads();
+          if (r + 1 < n_rounds) __syncthreads();
         }
         if (is_head && loop) {
-          if (me.n_rounds == 0) __syncthreads();
+          if (n_rounds == 0) __syncthreads();
 #pragma unroll 1
           for (int o = min(16, 1 << (row_log - 1)); o > 0; o >>= 1) cl_better(bv, bi, __shfl_xor_sync(0xffffffffu, bv, o), __shfl_xor_sync(0xffffffffu, bi, o));
           const int lanes = min(32, 1 << row_log), in_row = tid & ((1 << row_log) - 1), row = tid >> row_log;
