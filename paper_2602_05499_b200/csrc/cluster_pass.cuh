@@ -478,23 +478,29 @@ struct ClRing {
   const ClEntry* next;   // of this warp's list; the last one repeats itself
   int4 v;                // *next
   uint32_t buf;          // the ring
-  int at, width, wrap_jump;  // where in it the next entry goes, units of an entry
+  int at, wrap_jump;     // where in it the next entry goes
   __device__ __forceinline__ void begin(const ClEntry* first) {
     next = first;
     get();
     at = 0;
   }
+  template <int TW>
+  __device__ __forceinline__ void fill() {
+#pragma unroll 1
+    for (int i = 0; i < kClRing; i += TW) ask<TW>();
+  }
+  template <int TW>  // the stage's width: tiles of an entry, at most
   __device__ __forceinline__ void ask() {
     if ((short)v.y >= 0) {
       const uint4* w = W + v.x;
       const int n = v.z & 255, wrap = (v.z >> 8) & 255;
 #pragma unroll
-      for (int t = 0; t < kClTiles; ++t)
-        if (t < n)
+      for (int t = 0; t < TW; ++t)
+        if (TW == 1 || t < n)
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(buf + at + t * 512), "l"(w + t * 32 + (t >= wrap ? wrap_jump : 0)) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    at = (at + width * 512) & (kClRing * 512 - 1);
+    at = (at + TW * 512) & (kClRing * 512 - 1);
     if ((v.z >> 24) > 1)
       v.y = -1;  // nothing any more
     else
@@ -505,27 +511,23 @@ struct ClRing {
     v.y = cl_uniform(v.y);
     v.z = cl_uniform(v.z);
   }
+  template <int TW>
   __device__ __forceinline__ void wait() const {  // for the oldest entry
-    if (width == 1)
-      asm volatile("cp.async.wait_group %0;" ::"n"(kClRing - 1) : "memory");
-    else if (width == 2)
-      asm volatile("cp.async.wait_group %0;" ::"n"(kClRing / 2 - 1) : "memory");
-    else
-      asm volatile("cp.async.wait_group %0;" ::"n"(kClRing / 4 - 1) : "memory");
+    asm volatile("cp.async.wait_group %0;" ::"n"(kClRing / TW - 1) : "memory");
   }
 };
 
 // The entries of a round.  CG: column groups of eight rows.  Complete sums are left as [place][class][row of the tile][two rows of
 // the pass] of 128 bits, as a lane holds them: {half 0 of rows 2 q and 2 q + 1, half 1 of the same}.  What an entry needs besides its
 // weights is read while the one in front of it is multiplied.
-template <int CG>
+template <int TW, int CG>
 __device__ __forceinline__ void cl_mma_round(const ClParams& p, const ClEnv& ev, int x_at, const ClEntry*& ent, ClRing& ring) {
   const int g = ev.lane >> 2, q = ev.lane & 3, R = ev.R, Q = (R + 1) / 2;
   const uint2* const x = cl_at<uint2>(x_at) + g * 4 + q;
   float4* const red = cl_at<float4>(p.lay.red) + (ev.warp * 8 + g) * Q + q;
-  float acc[kClTiles][CG][4];
+  float acc[TW][CG][4];
 #pragma unroll
-  for (int i = 0; i < kClTiles; ++i)
+  for (int i = 0; i < TW; ++i)
 #pragma unroll
     for (int c = 0; c < CG; ++c) acc[i][c][0] = acc[i][c][1] = acc[i][c][2] = acc[i][c][3] = 0.f;
   uint2 b0[CG], b1[CG];
@@ -549,34 +551,34 @@ __device__ __forceinline__ void cl_mma_round(const ClParams& p, const ClEnv& ev,
     vn.y = cl_uniform(vn.y);
     vn.z = cl_uniform(vn.z);
     if ((short)v.y >= 0) {
-      ring.wait();
-      uint4 w[kClTiles];
+      ring.wait<TW>();
+      uint4 w[TW];
 #pragma unroll
-      for (int t = 0; t < kClTiles; ++t)
-        if (t < n)
+      for (int t = 0; t < TW; ++t)
+        if (TW == 1 || t < n)
           asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
                        : "=r"(w[t].x), "=r"(w[t].y), "=r"(w[t].z), "=r"(w[t].w)
                        : "r"(ring.buf + ring.at + t * 512)
                        : "memory");
 #pragma unroll
-      for (int t = 0; t < kClTiles; ++t)
-        if (t < n)
+      for (int t = 0; t < TW; ++t)
+        if (TW == 1 || t < n)
 #pragma unroll
           for (int c = 0; c < CG; ++c) {
             mma_bf16_16816(acc[t][c], w[t], b0[c].x, b1[c].x);
             mma_bf16_16816(acc[t][c], w[t], b0[c].y, b1[c].y);
           }
     }
-    ring.ask();  // into the place just read
+    ring.ask<TW>();  // into the place just read
     if (!last) load_x((short)vn.y);
     if (slot >= 0) {
       float4* o = red + slot * kClasses * 8 * Q;
       const int step = ((v.z >> 16) & 255) * kClasses * 8 * Q;
 #pragma unroll
-      for (int t = 0; t < kClTiles; ++t)
+      for (int t = 0; t < TW; ++t)
 #pragma unroll
         for (int c = 0; c < CG; ++c) {
-          if (t < n && c * 4 + q < Q) o[t * step + c * 4] = make_float4(acc[t][c][0], acc[t][c][1], acc[t][c][2], acc[t][c][3]);
+          if ((TW == 1 || t < n) && c * 4 + q < Q) o[t * step + c * 4] = make_float4(acc[t][c][0], acc[t][c][1], acc[t][c][2], acc[t][c][3]);
           acc[t][c][0] = acc[t][c][1] = acc[t][c][2] = acc[t][c][3] = 0.f;
         }
     }
@@ -1119,6 +1121,66 @@ __device__ __forceinline__ void cl_commit(const ClParams& p, ClShared* sh, int b
   }
 }
 
+// bf16: a linear stage, dot products to sending
+template <int HD, int CG>
+__device__ __forceinline__ void cl_stage_bf16(const ClParams& p, const ClEnv& ev, const ClDots& a, const ClTab& t) {
+  const ClMine& me = ev.mine[a.kind];
+  const bool is_head = a.kind == CL_HEAD;
+  const int R = ev.R;
+  const ClEntry* ent = ev.entries + me.entry0 + ev.warp * me.n_entries;
+  ClRing ring;
+  ring.W = reinterpret_cast<const uint4*>(a.W) + ev.lane;
+  ring.buf = ev.self + p.lay.ring + ev.warp * (kClRing * 512) + ev.lane * 16;
+  ring.wrap_jump = (a.K / 16 - 1) * 256;  // to the next group's unit of the same k-tile, which starts with its first tile
+  const int n_rounds = cl_uniform(me.n_rounds), width = cl_uniform(me.tile_width);
+  if (n_rounds > 0) {
+    ring.begin(ent);
+    if (width == 1)
+      ring.fill<1>();
+    else if (width == 2)
+      ring.fill<2>();
+    else
+      ring.fill<4>();
+  }
+  if (a.bar >= 0) cl_wait(ev.sh, p.sync, a.bar, a.bytes, a.parity);
+  // lm-head: 256 threads over the rows, a power of two of them each
+  const int row_log = R <= 1 ? 8 : R <= 2 ? 7 : R <= 4 ? 6 : R <= 8 ? 5 : 4;
+  float bv = -INFINITY;
+  int bi = 0x7fffffff;
+#pragma unroll 1
+  for (int r = 0; r < n_rounds; ++r) {
+    const ClRound& rd = ev.rounds[me.round0 + r];
+    if (width == 1)
+      cl_mma_round<1, CG>(p, ev, a.x, ent, ring);
+    else if (width == 2)
+      cl_mma_round<2, CG>(p, ev, a.x, ent, ring);
+    else
+      cl_mma_round<4, CG>(p, ev, a.x, ent, ring);
+    if (a.norm && a.bar >= 0 && r == 0) cl_row_scales(p, ev);  // (the first stage's were made with the embedding)
+    __syncthreads();  // the sums are there
+    if (is_head) {
+      cl_head_round(p, ev, me, rd, a.logits, row_log, bv, bi);
+    } else {
+      cl_values<__nv_bfloat16, HD>(p, ev, me, rd, t.kind);
+      __syncthreads();
+      if (cl_aborted(ev.sh)) {
+      } else if (t.kind == CL_QKV) {
+        cl_send_qkv<__nv_bfloat16, HD>(p, ev, me, rd);
+      } else {
+        cl_send_all<__nv_bfloat16>(p, ev, me, rd, t.kind, t.gain_out);
+      }
+    }
+    if (r + 1 < n_rounds) __syncthreads();
+  }
+  if (is_head && a.logits == nullptr) {
+    if (n_rounds == 0) __syncthreads();
+#pragma unroll 1
+    for (int o = min(16, 1 << (row_log - 1)); o > 0; o >>= 1) cl_better(bv, bi, __shfl_xor_sync(0xffffffffu, bv, o), __shfl_xor_sync(0xffffffffu, bi, o));
+    const int lanes = min(32, 1 << row_log), in_row = ev.tid & ((1 << row_log) - 1), row = ev.tid >> row_log;
+    if (row < R && in_row % lanes == 0) cl_at<float2>(p.lay.best)[row * 4 * kClWarps + in_row / lanes] = make_float2(bv, __int_as_float(bi));
+  }
+}
+
 template <typename WT, int HD, int CG>
 __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, const ClTab* tab_t, const ClTab* tab_d, int rank, bool loop, int batch, int k) {
   constexpr bool BF = sizeof(WT) == 2;
@@ -1221,50 +1283,7 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
       const ClMine& me = ev.mine[t.kind];
       const bool is_head = t.kind == CL_HEAD;
       if constexpr (BF) {
-        const ClEntry* ent = ev.entries + me.entry0 + ev.warp * me.n_entries;
-        ClRing ring;
-        ring.W = reinterpret_cast<const uint4*>(a.W) + ev.lane;
-        ring.buf = ev.self + p.lay.ring + ev.warp * (kClRing * 512) + ev.lane * 16;
-        ring.width = cl_uniform(me.tile_width);
-        ring.wrap_jump = (a.K / 16 - 1) * 256;  // to the next group's unit of the same k-tile, which starts with its first tile
-        const int n_rounds = cl_uniform(me.n_rounds);
-        if (n_rounds > 0) {
-          ring.begin(ent);
-#pragma unroll 1
-          for (int i = 0; i < kClRing; i += ring.width) ring.ask();
-        }
-        if (a.bar >= 0) cl_wait(sh, p.sync, a.bar, a.bytes, a.parity);
-        // lm-head: 256 threads over the rows, a power of two of them each
-        const int row_log = R <= 1 ? 8 : R <= 2 ? 7 : R <= 4 ? 6 : R <= 8 ? 5 : 4;
-        float bv = -INFINITY;
-        int bi = 0x7fffffff;
-#pragma unroll 1
-        for (int r = 0; r < n_rounds; ++r) {
-          const ClRound& rd = ev.rounds[me.round0 + r];
-          cl_mma_round<CG>(p, ev, a.x, ent, ring);
-          if (a.norm && a.bar >= 0 && r == 0) cl_row_scales(p, ev);  // (the first stage's were made with the embedding)
-          __syncthreads();  // the sums are there
-          if (is_head) {
-            cl_head_round(p, ev, me, rd, a.logits, row_log, bv, bi);
-          } else {
-            cl_values<WT, HD>(p, ev, me, rd, t.kind);
-            __syncthreads();
-            if (cl_aborted(sh)) {
-            } else if (t.kind == CL_QKV) {
-              cl_send_qkv<WT, HD>(p, ev, me, rd);
-            } else {
-              cl_send_all<WT>(p, ev, me, rd, t.kind, t.gain_out);
-            }
-          }
-          if (r + 1 < n_rounds) __syncthreads();
-        }
-        if (is_head && loop) {
-          if (n_rounds == 0) __syncthreads();
-#pragma unroll 1
-          for (int o = min(16, 1 << (row_log - 1)); o > 0; o >>= 1) cl_better(bv, bi, __shfl_xor_sync(0xffffffffu, bv, o), __shfl_xor_sync(0xffffffffu, bi, o));
-          const int lanes = min(32, 1 << row_log), in_row = tid & ((1 << row_log) - 1), row = tid >> row_log;
-          if (row < R && in_row % lanes == 0) cl_at<float2>(p.lay.best)[row * 4 * kClWarps + in_row / lanes] = make_float2(bv, __int_as_float(bi));
-        }
+        cl_stage_bf16<HD, CG>(p, ev, a, t);
       } else {
         if (R == 1)
           cl_dots_f32<1, 4>(p, ev, a);
