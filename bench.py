@@ -213,7 +213,7 @@ def main():
     ap.add_argument("--workload", default="c2-7b-greedy-k4", choices=sorted(WORKLOADS))
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--share-kv", action="store_true", help="the draft attends the target's KV cache (no draft cache, no draft prompt pass)")
-    ap.add_argument("--flags", type=int, default=0, help="sdfp_config.flags (1 no graph, 2 no PDL, 4 FMA GEMM, 8 one kernel per operation instead of the whole-pass kernel)")
+    ap.add_argument("--flags", type=int, default=0, help="sdfp_config.flags (1 no graph, 2 no PDL, 4 FMA GEMM, 8 one kernel per operation instead of the whole-pass kernel, 32 small decoders without the cluster kernel)")
     args = ap.parse_args()
     rank = int(os.environ.get("RANK", "0"))
     local_rank = int(os.environ.get("LOCAL_RANK", "0"))

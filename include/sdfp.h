@@ -59,13 +59,15 @@ typedef enum { SDFP_F32 = 0, SDFP_BF16 = 1 } sdfp_dtype;
 #define SDFP_FLAG_NO_GRAPH 1u /* launch kernels directly instead of replaying CUDA graphs    */
 #define SDFP_FLAG_NO_PDL 2u   /* no programmatic dependent launch between consecutive kernels */
 #define SDFP_FLAG_FMA_GEMM 4u /* bf16 models: CUDA-core FMA GEMM instead of the tensor path  */
-#define SDFP_FLAG_NO_PASS_KERNEL 8u /* one kernel per operation: bf16 models without the persistent
-                                       whole-pass kernel, small models of either type without
-                                       the kernel that runs the rounds of sdfp_generate inside
-                                       one thread-block cluster                                */
+#define SDFP_FLAG_NO_PASS_KERNEL 8u /* bf16 models: one kernel per operation instead of the
+                                       persistent whole-pass kernel                            */
 #define SDFP_FLAG_NO_DENSE 16u      /* bf16 models: no tcgen05 path (the prompt goes through the
                                        decode kernels in chunks; contexts too wide for the
                                        whole-pass kernel run mma.sync kernels per operation)  */
+#define SDFP_FLAG_NO_CLUSTER 32u    /* small models: the rounds of sdfp_generate on the kernels of
+                                       every other pass (the whole-pass kernel, or one kernel per
+                                       operation) instead of inside one thread-block cluster; the
+                                       results have the same bits                              */
 
 /*
  * Model and capacity description.  The decoder is the LLaMA-2 architecture the

@@ -678,7 +678,7 @@ cudaLaunchConfig_t cluster_launch_config(const sdfp_ctx* c, cudaLaunchAttribute*
 //     eight d 256 (12.6 MB) 1.16, d 320 0.92; fp32: one d 256 2.0, d 512 (12.6 MB) 1.10; two d 384 (14 MB) 1.15; four d 256 (12.6 MB) 1.23
 bool cluster_wanted(sdfp_ctx* c, int widest) {
   const sdfp_config& g = c->cfg;
-  if ((g.flags & SDFP_FLAG_NO_PASS_KERNEL) || (c->bf16 && !c->use_pass)) return false;  // (bf16: the sums are the whole-pass kernel's)
+  if ((g.flags & SDFP_FLAG_NO_CLUSTER) || (c->bf16 && !c->use_pass)) return false;  // (bf16: the sums are the whole-pass kernel's)
   // every CTA has a share of every stage a layer is made of: the exchange between the stages relies on it
   if (g.d_model < 8 * kClCtas || g.d_ffn < 4 * kClCtas || widest > kClMaxRows) return false;
   const double layer_bytes = (4.0 * g.d_model * g.d_model + 3.0 * g.d_model * g.d_ffn) * (double)c->esz;

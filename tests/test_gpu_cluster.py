@@ -2,6 +2,7 @@
 import numpy as np
 import pytest
 
+import paper_2602_05499_b200 as pkg
 import synth_inputs as si
 from gpu_common import check_stream_against_oracle, make_pair
 from oracle import sdfp_oracle as orc
@@ -106,18 +107,37 @@ def test_rounds_have_the_bits_of_the_other_passes(heads, head_dim, ffn, vocab, d
         eng.close()
 
 
-def test_an_end_token():
+@pytest.mark.parametrize("shape", [si.TINY, si.TINY_BF16], ids=["f32", "bf16"])
+def test_the_flag_that_leaves_the_cluster_kernel_out(shape):
+    """Greedy and sampled rounds on the kernels of every other pass: the same tokens, statistics and, from the caches they leave, logits."""
+    prompts = si.make_prompts(shape.vocab, 2, 9, seed=67)
+    got = []
+    for flags in (0, pkg.FLAG_NO_CLUSTER):
+        eng, _, _ = make_pair(shape, (1, 2), max_seq=96, max_batch=1, k_max=5, flags=flags, random_gains=True)
+        greedy = eng.sdfp_generate(prompts[:1], 5, 70)
+        logits = [eng.sdfp_forward_logits(greedy.tokens[0][-9:], 70, draft=draft).view(np.uint32) for draft in (False, True)]
+        sampled = eng.sdfp_generate(prompts[1:], 5, 60, temperature=1.0, seed=9)
+        got.append((greedy, sampled, logits))
+        eng.close()
+    (a, sa, la), (b, sb, lb) = got
+    assert a.timing["kernel_launches"] == 1 < b.timing["kernel_launches"]
+    assert a.tokens == b.tokens and sa.tokens == sb.tokens and np.array_equal(a.stats, b.stats) and np.array_equal(sa.stats, sb.stats)
+    assert all(np.array_equal(x, y) for x, y in zip(la, lb))
+
+
+@pytest.mark.parametrize("flags", [0, pkg.FLAG_NO_CLUSTER], ids=["cluster", "whole-pass"])
+def test_an_end_token(flags):
     """A sequence that ends early stays where it is while the other goes on; calls behind it start afresh."""
-    eng, m, _ = make_pair(si.TINY_BF16, (1, 2), max_seq=64, max_batch=2, k_max=4)
+    eng, m, _ = make_pair(si.TINY_BF16, (1, 2), max_seq=64, max_batch=2, k_max=4, flags=flags)
     prompts = si.make_prompts(m.vocab, 2, 12, seed=77)
     free = eng.sdfp_generate(prompts, 4, 30)
     eng.close()
     eos = free.tokens[0][7]
-    eng, _, _ = make_pair(si.TINY_BF16, (1, 2), max_seq=64, max_batch=2, k_max=4, eos_id=int(eos))
+    eng, _, _ = make_pair(si.TINY_BF16, (1, 2), max_seq=64, max_batch=2, k_max=4, eos_id=int(eos), flags=flags)
     try:
         for k in (4, 0):
             out = eng.sdfp_generate(prompts, k, 30)
-            assert out.timing["kernel_launches"] == 1
+            assert (out.timing["kernel_launches"] == 1) == (flags == 0)
             for b in range(2):
                 want = free.tokens[b]
                 cut = want.index(eos) + 1 if eos in want else len(want)

@@ -146,14 +146,19 @@ def test_greedy_bf16(tiny_bf16):
     check_stream_against_oracle(m, prompt[0].tolist(), out.tokens[0])
 
 
-def test_graph_and_direct_launch_agree(tiny):
-    eng, m = tiny
-    prompt = si.make_prompts(m.vocab, 1, 16)
+@pytest.mark.parametrize("shape", [si.TINY, si.TINY_BF16], ids=["per-operation", "whole-pass"])
+def test_graph_and_direct_launch_agree(shape):
+    """Rounds replayed as a graph, launched directly and without programmatic dependent launch; and all of them inside one cluster."""
+    prompt = si.make_prompts(shape.vocab, 1, 16)
+    eng, _, _ = make_pair(shape, (1, 2))
     base = eng.sdfp_generate(prompt, 4, 40)
-    for flags in (pkg.FLAG_NO_GRAPH, pkg.FLAG_NO_PDL, pkg.FLAG_NO_GRAPH | pkg.FLAG_NO_PDL):
-        e2, _, _ = make_pair(si.TINY, (1, 2), flags=flags)
+    eng.close()
+    assert base.timing["kernel_launches"] == 1
+    for flags in (0, pkg.FLAG_NO_GRAPH, pkg.FLAG_NO_PDL, pkg.FLAG_NO_GRAPH | pkg.FLAG_NO_PDL):
+        e2, _, _ = make_pair(shape, (1, 2), flags=flags | pkg.FLAG_NO_CLUSTER)
         o2 = e2.sdfp_generate(prompt, 4, 40)
         e2.close()
+        assert o2.timing["kernel_launches"] > o2.n_rounds
         assert o2.tokens == base.tokens and np.array_equal(o2.stats, base.stats)
 
 
@@ -168,16 +173,18 @@ def test_run_to_run_determinism(tiny):
     assert np.array_equal(la.view(np.uint32), lb.view(np.uint32))
 
 
-def test_eos_stops_generation():
+@pytest.mark.parametrize("flags", [0, pkg.FLAG_NO_CLUSTER], ids=["cluster", "per-operation"])
+def test_eos_stops_generation(flags):
     shape = si.TINY
     prompt = si.make_prompts(shape.vocab, 1, 16)
-    eng, m, _ = make_pair(shape, (1, 2))
+    eng, m, _ = make_pair(shape, (1, 2), flags=flags)
     full = eng.sdfp_generate(prompt, 4, 40).tokens[0]
     eng.close()
     eos = full[17]
     first = full.index(eos)
-    eng, m, _ = make_pair(shape, (1, 2), eos_id=eos)
+    eng, m, _ = make_pair(shape, (1, 2), eos_id=eos, flags=flags)
     out = eng.sdfp_generate(prompt, 4, 40)
+    assert (out.timing["kernel_launches"] == 1) == (flags == 0)
     ar = eng.sdfp_generate(prompt, 0, 40)
     eng.close()
     assert out.tokens[0] == full[:first + 1] == ar.tokens[0]
@@ -355,13 +362,18 @@ def test_13b_shape_layers():
         eng.close()
 
 
-def test_batch_rows_are_independent_bf16():
-    """Three sequences with k = 4 are 15 rows: they run in the whole-pass kernel as three row
-    groups.  A sequence's tokens and acceptance counts must not depend on the others."""
-    eng, m, _ = make_pair(si.TINY_BF16, (1, 2), max_batch=3, k_max=4)
+@pytest.mark.parametrize("flags", [0, pkg.FLAG_NO_CLUSTER], ids=["cluster", "whole-pass"])
+def test_batch_rows_are_independent_bf16(flags):
+    """Three sequences with k = 4 are 15 rows: they run in the whole-pass kernel (or inside one cluster) as three
+    row groups.  A sequence's tokens and acceptance counts must not depend on the others, nor on a draft in the target's cache."""
+    eng, m, _ = make_pair(si.TINY_BF16, (1, 2), max_batch=3, k_max=4, flags=flags)
     try:
         prompts = si.make_prompts(m.vocab, 3, 24, seed=41)
         out = eng.sdfp_generate(prompts, 4, 40)
+        assert (out.timing["kernel_launches"] == 1) == (flags == 0)
+        eng.sdfp_set_draft_kv_sharing(True)
+        assert eng.sdfp_generate(prompts, 4, 40).tokens == out.tokens
+        eng.sdfp_set_draft_kv_sharing(False)
         ar = eng.sdfp_generate(prompts, 0, 40)
         assert out.tokens == ar.tokens
         for b in range(3):
