@@ -307,9 +307,12 @@ int sdfp_time_pass(sdfp_ctx *ctx, int32_t draft, int32_t rows, int32_t position,
 
 /*
  * Failure-path test hook (bf16 contexts whose passes run in the whole-pass kernel or on the
- * dense path; SDFP_ESTATE otherwise).  Section II-A's loop has no counterpart: this exercises
+ * dense path, and small models of either type whose rounds run inside one thread-block cluster;
+ * SDFP_ESTATE otherwise).  Section II-A's loop has no counterpart: this exercises
  * the library's own bounded waits.  Whole-pass kernel: after the call, the grid barriers of the
- * next pass expect one arrival more than the grid can provide.  Dense path: in the next
+ * next pass expect one arrival more than the grid can provide.  Rounds inside a cluster, if they
+ * are the next to run (an fp32 model's prompt and sdfp_forward_logits have no such wait and leave the
+ * hook armed): every CTA's first wait expects more bytes than are sent.  Dense path: in the next
  * sdfp_forward_logits or sdfp_forward_logits_static call (other entry points are not affected),
  * the CTAs of the linear kernels that hold the middle of a feature tile raise their "partial
  * sum posted" flags where nobody looks, so the CTA that finishes the tile waits for a post that

@@ -217,7 +217,7 @@ __device__ __noinline__ void cl_poll(ClShared* sh, PassSync* sync, uint32_t bar,
     if ((++spins & 15u) == 0) {
       if (cl_aborted(sh)) break;
       if (global_ns() - t0 > sh->wait_limit_ns) {
-        atomicCAS(&sync->error, 0, (int)PASS_ERR_GRID_BARRIER);
+        atomicCAS(&sync->error, 0, (int)PASS_ERR_CLUSTER);
         *reinterpret_cast<volatile int*>(&sh->abort) = 1;
         break;
       }
@@ -226,7 +226,7 @@ __device__ __noinline__ void cl_poll(ClShared* sh, PassSync* sync, uint32_t bar,
 }
 // Wait for a buffer the other CTAs fill.  Their bytes may have been counted before the barrier is told how many to expect.
 __device__ __forceinline__ void cl_wait(ClShared* sh, PassSync* sync, int which, unsigned bytes, unsigned parity) {
-  if (cl_aborted(sh)) return;  // a phase that never ended must not be armed again
+  if (__any_sync(0xffffffffu, cl_aborted(sh))) return;  // a phase that never ended must not be armed again; one answer for the warp
   if (threadIdx.x == kClThreads - 1) {
     mbar_arrive_expect_tx(&sh->bar[which], bytes + sh->sabotage);
     sh->sabotage = 0;
@@ -453,8 +453,7 @@ __device__ __forceinline__ void cl_dots_f32(const ClParams& p, const ClEnv& ev, 
               const int f0 = cl_feature(me.p0 + pl);
               if (a.logits != nullptr) {
                 float* o = a.logits + (size_t)row * p.vocab + f0;
-                o[0] = v0;
-                o[8] = v1;
+                if (!cl_aborted(ev.sh)) o[0] = v0, o[8] = v1;
               } else {  // only this lane touches its place; a NaN loses against everything, by itself
                 float2* best = cl_at<float2>(p.lay.best) + row * 4 * kClWarps + warp * 4 + pi % P;
                 float2 o = *best;
@@ -609,7 +608,7 @@ __device__ __forceinline__ float2 cl_sum_pair(const ClParams& p, const ClRound& 
 // bf16 lm-head, one round: logits, or a thread's best of its row's pairs (a thread keeps to one row)
 __device__ __forceinline__ void cl_head_round(const ClParams& p, const ClEnv& ev, const ClMine& me, const ClRound& rd, float* logits, int row_log, float& bv, int& bi) {
   const int row = ev.tid >> row_log;
-  if (row >= ev.R) return;
+  if (row >= ev.R || cl_aborted(ev.sh)) return;  // (what is read from the logits behind a failed wait are those of an earlier pass)
   const float inv = ev.sh->inv[row];
 #pragma unroll 1
   for (int j = ev.tid & ((1 << row_log) - 1); j < 4 * rd.n_quads; j += 1 << row_log) {
@@ -1057,7 +1056,7 @@ __device__ __forceinline__ int cl_heads_of(int cta, int heads, int splits) {
 }
 
 // What a pass's row carries
-__device__ __forceinline__ void cl_plan_row(const ClShared* sh, int kind, int step, int rps, int row, int& tok, int& pos) {
+__device__ __forceinline__ void cl_plan_row(const ClShared* sh, int kind, int step, int rps, int row, int vocab, int& tok, int& pos) {
   tok = 0;
   pos = -1;
   const int b = row / rps, i = row - b * rps;
@@ -1073,6 +1072,7 @@ __device__ __forceinline__ void cl_plan_row(const ClShared* sh, int kind, int st
     pos = n - 1 + i;
     tok = i == 0 ? sh->last[b][1] : sh->drafts[b][i - 1];
   }
+  tok = min(max(tok, 0), vocab - 1);  // (no token of a round whose logits were not numbers)
 }
 
 // accept (Eq. 2: draft token == target's argmax) and commit, one lane per sequence; every CTA keeps the state, CTA 0
@@ -1216,7 +1216,7 @@ __device__ __forceinline__ void cl_compute(const ClParams& p, ClShared* sh, cons
 #pragma unroll 1
       for (int row = ev.warp; row < R; row += kClWarps) {
         int tok, pos;
-        cl_plan_row(sh, kind, loop ? pass : p.pd.step, ev.rps, row, tok, pos);
+        cl_plan_row(sh, kind, loop ? pass : p.pd.step, ev.rps, row, p.vocab, tok, pos);
         if (ev.lane == 0) sh->pos[row] = pos;
         const WT* e = reinterpret_cast<const WT*>(p.embed) + (size_t)tok * p.d;
         float* own = cl_at<float>(p.lay.hres) + row * p.lay.resid_np;
@@ -1420,7 +1420,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_pass_kernel(const __gri
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   cl_cluster_sync();  // barriers exist everywhere before anything is sent, and the CTA's tables are written
 
-  cl_compute<WT, HD, CG>(p, sh, tab_t, tab_d, rank, loop, batch, k);
+  if (!cl_aborted(sh)) cl_compute<WT, HD, CG>(p, sh, tab_t, tab_d, rank, loop, batch, k);
 
   // In normal operation everything that was sent has been waited for.  After a wait that ran out something may still
   // be on its way to a CTA of the cluster: give it far longer than it takes before any CTA leaves.

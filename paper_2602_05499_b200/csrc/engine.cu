@@ -1365,9 +1365,9 @@ int check_pass_error(sdfp_ctx* c) {
   if (c->use_pass) cudaMemsetAsync(c->split_partials, 0, (size_t)c->pass_grid * kUnitTiles * 2 * 64 * sizeof(ulonglong2), c->stream);
   cudaStreamSynchronize(c->stream);
   static const char* const what[] = {"", "grid barrier", "weight slot never filled", "weight slot never freed",
-                                     "partial sum of a split group never posted"};
+                                     "partial sum of a split group never posted", "share of a stage never arrived in the cluster"};
   return fail(c, SDFP_ETIMEOUT, "pass kernel gave up a wait (%s); results of this call are invalid",
-              ps.error >= 1 && ps.error <= 4 ? what[ps.error] : "unknown");
+              ps.error >= 1 && ps.error <= 5 ? what[ps.error] : "unknown");
 }
 
 // Logits of `rows` tokens of sequence slot 0 at positions start.., in passes of as many rows as
@@ -1802,8 +1802,8 @@ extern "C" int sdfp_forward_logits_static(sdfp_ctx* c, int32_t draft, const int3
 extern "C" int sdfp_debug_expire_next_wait(sdfp_ctx* c, uint64_t wait_limit_ns) {
   if (!c) return SDFP_EINVAL;
   if (int r = check_device(c, "sdfp_debug_expire_next_wait")) return r;
-  if (!c->use_pass && !c->dense_decode)
-    return fail(c, SDFP_ESTATE, "sdfp_debug_expire_next_wait: this context uses neither the whole-pass kernel nor the dense path for its passes");
+  if (!c->psync && !c->dense_decode)
+    return fail(c, SDFP_ESTATE, "sdfp_debug_expire_next_wait: this context uses neither the whole-pass kernel nor the cluster kernel nor the dense path for its passes");
   if (wait_limit_ns < 1000000ull || wait_limit_ns > 2000000000ull)
     return fail(c, SDFP_EINVAL, "sdfp_debug_expire_next_wait: the limit must lie between 1 ms and 2 s");
   if (c->dense_decode) {  // the next sdfp_forward_logits[_static] call: see forward_logits_passes

@@ -107,7 +107,7 @@ __host__ __device__ __forceinline__ size_t frag_index(int kt, int row, int q) { 
 inline size_t frag_image_len(int K) { return (size_t)(K / 16) * 64; }  // in uint4
 
 // what a wait that gave up leaves in PassSync::error
-enum PassError { PASS_OK = 0, PASS_ERR_GRID_BARRIER = 1, PASS_ERR_SLOT_FULL = 2, PASS_ERR_SLOT_EMPTY = 3, PASS_ERR_SPLIT_FLAG = 4 };
+enum PassError { PASS_OK = 0, PASS_ERR_GRID_BARRIER = 1, PASS_ERR_SLOT_FULL = 2, PASS_ERR_SLOT_EMPTY = 3, PASS_ERR_SPLIT_FLAG = 4, PASS_ERR_CLUSTER = 5 };
 
 struct PassSync {                // one per context, in global memory, zero-initialised
   unsigned long long bar_count;  // grid-barrier arrivals of all launches so far: serial * grid when barrier `serial` is complete
@@ -115,8 +115,8 @@ struct PassSync {                // one per context, in global memory, zero-init
   int error;           // first PassError seen, sticky
   unsigned pad1[31];
   // Failure-path test hook, both zero in normal operation: every grid barrier expects this many
-  // arrivals more than the grid provides (so its wait can only run out), and waits give up after
-  // wait_limit_ns nanoseconds instead of the default (0 = default).
+  // arrivals more than the grid provides (so its wait can only run out; the cluster kernel's first waits
+  // expect a few bytes more than are sent), and waits give up after wait_limit_ns nanoseconds instead of the default (0 = default).
   unsigned long long bar_extra;
   unsigned long long wait_limit_ns;
   unsigned pad2[28];

@@ -1,4 +1,6 @@
 """Rounds of small decoders inside one thread-block cluster (csrc/cluster_pass.cuh) at the edges of its shares, steps and splits."""
+import time
+
 import numpy as np
 import pytest
 
@@ -103,6 +105,28 @@ def test_rounds_have_the_bits_of_the_other_passes(heads, head_dim, ffn, vocab, d
         if k:  # drafted tokens are the draft's first largest
             eng.sdfp_set_draft_layers(np.ones(shape.n_layers, dtype=np.uint8))
             assert (eng.sdfp_generate(first, k, 20).stats[:-1, :, 1] == k).all()
+    finally:
+        eng.close()
+
+
+@pytest.mark.parametrize("shape,prompt,temperature", [(si.TINY, 1, 0.0), (si.TINY, 30, 0.0), (si.TINY_BF16, 1, 0.0), (si.TINY_BF16, 24, 0.0), (si.TINY_BF16, 1, 1.0)])
+def test_a_wait_that_runs_out(shape, prompt, temperature):
+    """The cluster kernel's own waits, without faulting anything: every CTA's first one expects more bytes than are sent, with a 20 ms
+    limit.  (The prompts have no pass that would take the hook: one token, per-operation kernels, or long enough for the tcgen05
+    path.)  The CTAs walk to their end, the call comes back with SDFP_ETIMEOUT and the wait's name, the context works again."""
+    eng, _, _ = make_pair(shape, (1, 2), max_seq=96, max_batch=1, k_max=4)
+    try:
+        text = si.make_prompts(shape.vocab, 1, prompt, seed=91)
+        before = eng.sdfp_generate(text, 4, 24, temperature=temperature, seed=3)
+        for _ in range(2):
+            eng.sdfp_debug_expire_next_wait(20_000_000)
+            t0 = time.perf_counter()
+            with pytest.raises(pkg.SdfpError) as ei:
+                eng.sdfp_generate(text, 4, 24, temperature=temperature, seed=3)
+            assert time.perf_counter() - t0 < 1.0
+            assert ei.value.code == -5 and "in the cluster" in str(ei.value)
+            after = eng.sdfp_generate(text, 4, 24, temperature=temperature, seed=3)
+            assert after.tokens == before.tokens and np.array_equal(after.stats, before.stats)
     finally:
         eng.close()
 
