@@ -97,7 +97,7 @@ struct sdfp_ctx {
     cudaGraphExec_t exec;
     long long launches;
   };
-  std::map<std::tuple<int, int, int, int>, RoundGraph> graphs;  // (k, batch, sampled, n_chunks)
+  std::map<std::tuple<int, int, int, int>, RoundGraph> graphs;  // (k, batch, sampled + 2 in_cluster, n_chunks)
   long long launches = 0;
   Launcher L{};
 
@@ -118,6 +118,7 @@ struct sdfp_ctx {
   int pass_grid = 0;
   // small decoders: the passes of rounds, and whole greedy generations, inside one cluster (cluster_pass.cuh)
   bool use_cluster = false;
+  bool in_cluster = false;             // ... those of the running call (cluster_takes)
   ClLayout cl{};
   ClPlan cl_plan;                      // what each of its CTAs does of the matrices
   unsigned char* cl_mem = nullptr;     // device: the plan, the gains' addresses, the programs
@@ -668,21 +669,45 @@ cudaLaunchConfig_t cluster_launch_config(const sdfp_ctx* c, cudaLaunchAttribute*
   return lc;
 }
 
-// Whether the rounds of a context run in the cluster kernel, and with which layout.  Sixteen SMs do the arithmetic of a
-// pass, so the line lies where that takes as long as the stage boundaries it saves: bytes of a layer times sequences.  One
-// call of 40 + 32 tokens, 4 layers, FFN 2.7 d, vocabulary 4096, time on the other path over time here:
-//   bf16, draft length 2 to 8, one sequence: d 256 1.8, d 384 1.4, d 512 (6.3 MB) 1.25 to 1.3, d 640 0.97; two sequences
-//     d 256 1.4, d 320 (5 MB) 1.05 to 1.15, d 384 1.0 to 1.08; three, k = 4, d 256 (4.7 MB) 1.16, d 320 0.88; four, k = 2, d 256 (6.3 MB) 1.11
-//   fp32, the same: d 256 1.24 to 1.37, d 320 (5 MB) 1.06 to 1.19, d 384 0.97 to 1.08; two sequences, d 256 (6.3 MB) 0.92 to 1.02
-//   autoregressive (k_max 0), bf16: one sequence d 256 2.6, d 512 2.0, d 640 1.46, d 768 (14 MB) 1.15; two d 512 (12.6 MB) 1.46, d 640 0.92;
-//     eight d 256 (12.6 MB) 1.16, d 320 0.92; fp32: one d 256 2.0, d 512 (12.6 MB) 1.10; two d 384 (14 MB) 1.15; four d 256 (12.6 MB) 1.23
+// What sixteen SMs take longer for than all of them, over what the stage boundaries inside one cluster save, per layer and pass
+// of a call: below 1 the cluster kernel is about the faster one.  Megabytes of a layer's matrices, of its share of the lm-head and of
+// its keys and values at the end of the text, and sequences, in microseconds, fitted to 301 calls timed on both sides (4 layers,
+// head_dim 64, d 256 to 640, FFN 2.7 d, vocabulary 4096 and 32000, 64 to 2048 positions, draft length 0, 4 and 8, one to
+// eight sequences; us a round here, and time on the other path over it):
+//   bf16, one sequence, 64 positions, draft length 0 / 4 / 8: vocabulary 4096 d 256 61 / 238 / 435 (2.2 / 1.7 / 1.6), d 512 90 / 342 / 652
+//     (1.6 / 1.3 / 1.2), d 640 125 / 506 / - (1.24 / 0.92 / -); vocabulary 32000 d 256 97 / 423 / 835 (1.4 / 1.05 / 0.89), d 512 145 / 618 / - (1.02 / 0.76 / -)
+//   2048 positions, vocabulary 4096: d 256 87 / 393 / 720 (1.7 / 1.3 / 1.2), d 512 148 / 656 / - (1.16 / 0.82 / -)
+//   four sequences, draft length 0, 64 / 512 / 2048 positions: d 256 84 / 128 / 202 (1.6 / 1.07 / 0.80); two, draft length 4: 290 / 441 / 577 (1.5 / 1.03 / 0.94)
+//   fp32, one sequence, 64 positions: vocabulary 4096 d 256 55 / 252 / 456 (2.0 / 1.4 / 1.3), d 512 119 / 483 / 858 (1.03 / 0.80 / 0.76);
+//     vocabulary 32000 d 256 85 / 483 / 877 (1.5 / 0.86 / 0.81); 2048 positions, vocabulary 4096, d 256 97 / 505 / 920 (1.4 / 0.97 / 0.91)
+double cluster_cost(const sdfp_ctx* c, int k, int batch, int positions) {
+  const sdfp_config& g = c->cfg;
+  int kept = 0;
+  for (int l = 0; l < g.n_layers; ++l) kept += c->keep_attn[l] + c->keep_ffn[l];
+  const double mb = c->esz / 1e6, d = g.d_model, more = batch - 1, passes = 1.0 + k * kept / (2.0 * g.n_layers);
+  const double layer = (4.0 * d * d + 3.0 * d * g.d_ffn) * mb, kv = 2.0 * d * positions * mb;
+  const double head = (double)g.vocab * d * mb * (1.0 + k) / (g.n_layers * passes);
+  if (k == 0)
+    return c->bf16 ? (1.17 * layer + 1.11 * head + (2.3 + 3.4 * more) * kv + 1.7 * more) / 18.0
+                   : ((0.85 + 0.34 * more) * layer + (0.96 + 0.36 * more) * head + (1.5 + 2.7 * more) * kv + 1.7 * more) / 16.6;
+  return c->bf16 ? (0.97 * layer + (1.52 + 0.77 * more) * head + (3.1 + 3.9 * more) * kv + 0.5 * more) / 12.2
+                 : ((1.8 + 0.47 * more) * layer + (1.35 + 0.8 * more) * head + (2.8 + 3.2 * more) * kv + 5.6 * more) / 17.7;
+}
+
+// Whether the rounds of a call run in the cluster kernel.  The results have the same bits either way.  The line lies where 62 more
+// calls of other shapes (2 to 24 layers, head_dim 128, FFN 1 to 4 d) lose on neither side: of those greedy ones below 0.85 the slowest was as fast as the
+// other path, sampled ones, a launch per pass and its sampling kernel, had 1.25 and 1.31 of its speed at 0.46 and 0.49, 0.82 to 1.2 from 0.63 on.
+bool cluster_takes(const sdfp_ctx* c, int k, int batch, int positions, bool sampled) {
+  return c->use_cluster && cluster_cost(c, k, batch, positions) < (sampled ? 0.6 : 0.85);
+}
+
+// Whether a context has calls whose rounds run in the cluster kernel, and with which layout.
 bool cluster_wanted(sdfp_ctx* c, int widest) {
   const sdfp_config& g = c->cfg;
   if ((g.flags & SDFP_FLAG_NO_CLUSTER) || (c->bf16 && !c->use_pass)) return false;  // (bf16: the sums are the whole-pass kernel's)
   // every CTA has a share of every stage a layer is made of: the exchange between the stages relies on it
   if (g.d_model < 8 * kClCtas || g.d_ffn < 4 * kClCtas || widest > kClMaxRows) return false;
-  const double layer_bytes = (4.0 * g.d_model * g.d_model + 3.0 * g.d_model * g.d_ffn) * (double)c->esz;
-  if (layer_bytes * g.max_batch > (g.k_max == 0 ? 13e6 : c->bf16 ? 6.4e6 : 5.2e6)) return false;
+  if (cluster_cost(c, 0, 1, 64) >= 0.85 && cluster_cost(c, g.k_max, 1, 64) >= 0.85) return false;
   // the sums of a layer's stage in one round where shared memory has room for them
   const ClPlan whole = cluster_plan(g.d_model, g.d_ffn, g.vocab, (int)c->esz, c->pass_grid, 1 << 14);
   for (int places = std::max(8, whole.most_places);; places = std::max(places / 2, whole.most_cuts)) {
@@ -784,7 +809,7 @@ int enqueue_pass(sdfp_ctx* c, const PassDesc& pd, bool draft, int rows, int attn
   const sdfp_config& g = c->cfg;
   const int d = g.d_model, f = g.d_ffn;
   if (c->dense_decode) return enqueue_dense_pass(c, pd, draft, rows, attn_rows_per_seq, n_chunks, decide);
-  if (c->use_cluster && pd.kind != PASS_TOKENS && pd.kind != PASS_PROMPT) {  // a pass of a round
+  if (c->in_cluster && pd.kind != PASS_TOKENS && pd.kind != PASS_PROMPT) {  // a pass of a round
     if (rows > c->cl.rows) return fail(c, SDFP_ESTATE, "a pass of %d rows reached the cluster kernel", rows);
     CU_OK(c, run_cluster_pass(c, pd, draft));
     return enqueue_decision(c, pd, rows, decide);
@@ -912,7 +937,7 @@ int enqueue_dense_pass(sdfp_ctx* c, const PassDesc& pd, bool draft, int rows, in
 int enqueue_round(sdfp_ctx* c, int k, int batch, bool sampled, int n_chunks) {
   PassDesc pd{};
   pd.n_seq = batch;
-  const bool fused = c->use_pass && !c->use_cluster && !sampled;  // the lm-head leaves argmax partials; consumers finish them
+  const bool fused = c->use_pass && !c->in_cluster && !sampled;  // the lm-head leaves argmax partials; consumers finish them
   if (fused) {
     pd.amax_part = c->amax_part;
     pd.amax_groups = c->amax_groups;
@@ -1611,9 +1636,10 @@ extern "C" int sdfp_generate(sdfp_ctx* c, const int32_t* prompts, int32_t batch,
   const long long launches0 = c->launches;
   cudaGraphExec_t exec = nullptr;
   long long launches_per_round = 0;
-  const bool in_one_launch = c->use_cluster && !sampled;  // the cluster kernel runs greedy rounds to the end
+  c->in_cluster = cluster_takes(c, k, batch, prompt_len + max_new + k, sampled);
+  const bool in_one_launch = c->in_cluster && !sampled;  // the cluster kernel runs greedy rounds to the end
   if (c->use_graph && !in_one_launch) {
-    auto key = std::make_tuple((int)k, (int)batch, sampled ? 1 : 0, n_chunks);
+    auto key = std::make_tuple((int)k, (int)batch, (sampled ? 1 : 0) + (c->in_cluster ? 2 : 0), n_chunks);
     auto it = c->graphs.find(key);
     if (it == c->graphs.end()) {
       const long long l0 = c->launches;

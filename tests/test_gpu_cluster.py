@@ -149,6 +149,29 @@ def test_the_flag_that_leaves_the_cluster_kernel_out(shape):
     assert all(np.array_equal(x, y) for x, y in zip(la, lb))
 
 
+@pytest.mark.parametrize("d,vocab,dtype,max_seq,batch,k,inside", [
+    (256, 4096, "bf16", 96, 1, 4, True), (256, 4096, "f32", 96, 1, 4, True), (512, 4096, "bf16", 96, 1, 4, True),
+    (512, 32000, "bf16", 96, 1, 4, False),    # measured 0.76 of the whole-pass kernel's speed
+    (256, 32000, "f32", 96, 1, 4, False),     # 0.86
+    (256, 32000, "bf16", 96, 1, 0, True),     # 1.4
+    (512, 4096, "bf16", 2080, 1, 8, False),   # 0.78
+    (256, 4096, "bf16", 2080, 1, 8, True),    # 1.2
+    (256, 4096, "bf16", 2080, 4, 0, False),   # 0.80
+    (384, 4096, "f32", 2080, 1, 4, False),    # 0.65
+    (640, 4096, "bf16", 96, 1, 4, False),     # 0.92
+    (512, 4096, "f32", 96, 1, 0, True),       # 1.03
+])
+def test_which_decoders_run_inside_a_cluster(d, vocab, dtype, max_seq, batch, k, inside):
+    """The line takes the size of the vocabulary, the positions and the sequences of a call into account, not a layer's weights alone."""
+    shape = si.ModelShape("line", 4, d, d // 64, 64, 16 * int(d * 2.7 / 16), vocab, dtype=dtype)
+    eng, m, _ = make_pair(shape, (1, 2), max_seq=max_seq, max_batch=batch, k_max=k, draw_device="cuda:0")
+    try:
+        out = eng.sdfp_generate(si.make_prompts(vocab, batch, max_seq - 20, seed=5), k, 10)
+        assert (out.timing["kernel_launches"] == 1) == inside
+    finally:
+        eng.close()
+
+
 @pytest.mark.parametrize("flags", [0, pkg.FLAG_NO_CLUSTER], ids=["cluster", "whole-pass"])
 def test_an_end_token(flags):
     """A sequence that ends early stays where it is while the other goes on; calls behind it start afresh."""
