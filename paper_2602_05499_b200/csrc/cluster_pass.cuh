@@ -1436,12 +1436,14 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_pass_kernel(const __gri
 // ---- host -------------------------------------------------------------------------------------------------------
 // What every CTA does of the five kinds of matrices, [CTA][stride].  bf16: the units of a group of 128 features are cut
 // as the whole-pass kernel's CTAs share them (stage_shares), and dealt to the classes from the beginning of each CTA's range.
+// place_slots: places the sums of a round may take; 0: only work out what a plan needs.
 struct ClPlan {
   std::vector<unsigned char> bytes;
   int rounds_at = 0, entries_at = 0, stride = 0;
   int most_places = 0;  // places the sums of a layer's stage take when it is finished in one round
   int most_cuts = 1;    // pieces of a sum
-  int most_quads = 0;   // fours of pairs in a round
+  int most_quads = 0;   // fours of pairs in a round of a layer's stage
+  long long most_units = 0;  // bf16: of a matrix, in uint4
 };
 
 inline ClPlan cluster_plan(int d, int f, int vocab, int elem_bytes, int pass_grid, int place_slots) {
@@ -1458,13 +1460,16 @@ inline ClPlan cluster_plan(int d, int f, int vocab, int elem_bytes, int pass_gri
     std::vector<ClEntry> entries;
   };
   std::vector<Cta> ctas(kClCtas);
+  std::vector<std::vector<ClEntry>> lists(kClasses);
+  std::vector<Batch> batches;
+  std::vector<StageShare> shares(pass_grid);
   ClPlan out;
   for (int kind = 0; kind < CL_KINDS; ++kind) {
     const int n_pairs = cl_pairs_of(kind, d, f, vocab);
     const int K = kind == CL_DOWN ? f : d, KT = K / 16, NT = n_pairs / 8, n_groups = (NT + kUnitTiles - 1) / kUnitTiles;
     std::vector<std::vector<Cut>> cuts;
     if (elem_bytes == 2) {
-      std::vector<StageShare> shares(pass_grid);
+      out.most_units = std::max(out.most_units, (long long)n_groups * KT * (kUnitBytes / 16));
       stage_shares(shares.data(), n_groups, KT, pass_grid);
       cuts.resize(n_groups);
       for (const StageShare& s : shares)
@@ -1488,7 +1493,7 @@ inline ClPlan cluster_plan(int d, int f, int vocab, int elem_bytes, int pass_gri
         r.quad0 = (pair0 - m.p0) / 4;
         r.n_quads = (pair1 - pair0) / 4;
         r.magic = r.n_quads > 0 ? (1u << 20) / (unsigned)r.n_quads + 1u : 0u;
-        out.most_quads = std::max(out.most_quads, r.n_quads);
+        if (kind != CL_HEAD) out.most_quads = std::max(out.most_quads, r.n_quads);
         c.rounds.push_back(r);
         m.n_rounds += 1;
         return c.rounds.back();
@@ -1498,12 +1503,12 @@ inline ClPlan cluster_plan(int d, int f, int vocab, int elem_bytes, int pass_gri
         continue;
       }
       if (m.np == 0) continue;
-      std::vector<Batch> batches;
+      batches.clear();
       const int t1 = (m.p0 + m.np + 7) / 8;
       int places = 0, width = 1;
       for (int t = m.p0 / 8; t < t1;) {
         const std::vector<Cut>& cut = cuts[t / kUnitTiles];
-        const int np = (int)cut.size(), most = std::max(1, std::min((int)kClTiles, place_slots / np));
+        const int np = (int)cut.size(), most = place_slots > 0 ? std::max(1, std::min((int)kClTiles, place_slots / np)) : kClTiles;
         int n = 1;
         while (n < most && t + n < t1 && cuts[(t + n) / kUnitTiles] == cut) ++n;
         batches.push_back(Batch{t, n, np});
@@ -1514,7 +1519,8 @@ inline ClPlan cluster_plan(int d, int f, int vocab, int elem_bytes, int pass_gri
       }
       if (kind != CL_HEAD) out.most_places = std::max(out.most_places, places);
       m.tile_width = width == 3 ? 4 : width;
-      std::vector<std::vector<ClEntry>> lists(kClasses);
+      if (place_slots <= 0) continue;
+      for (auto& l : lists) l.clear();
       for (size_t b = 0; b < batches.size();) {
         size_t e = b;
         int tiles = 0;  // ... of the round
@@ -1627,7 +1633,12 @@ inline ClLayout cluster_layout(int d, int f, int heads, int hd, int n_layers, in
   y.plan_entries = y.plan + plan.entries_at;
   y.plan_bytes = plan.stride;
   take(y.shared, (long long)sizeof(ClShared));
-  y.total = at <= max_smem ? at : 0;
+  // what the kernel's fields hold: the bytes of a stage on an mbarrier (20 bits), a round's vectors divided by multiplication, places, pieces
+  // and k-tiles of an entry, units of a matrix; and the first norm's squares, added as sixteen warps of 128 columns do
+  const long long most_bytes = std::max({6LL * rows * d, 4LL * rows * f, hpr * (4 * hd + 2 * hd * elem_bytes), hpr * y.part_slots * (hd + 2) * 4, 8LL * kClCtas * rows});
+  const bool held = most_bytes < 1 << 20 && (long long)rows * plan.most_quads * plan.most_quads < 1 << 20 && place_slots < 1 << 15 && plan.most_cuts < 256 &&
+                    std::max(d, f) / 16 < 1 << 15 && plan.most_units < 1LL << 31 && d <= 2048;
+  y.total = held && at <= max_smem ? at : 0;
   return y;
 }
 

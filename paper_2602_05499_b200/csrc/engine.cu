@@ -709,7 +709,7 @@ bool cluster_wanted(sdfp_ctx* c, int widest) {
   if (g.d_model < 8 * kClCtas || g.d_ffn < 4 * kClCtas || widest > kClMaxRows) return false;
   if (cluster_cost(c, 0, 1, 64) >= 0.85 && cluster_cost(c, g.k_max, 1, 64) >= 0.85) return false;
   // the sums of a layer's stage in one round where shared memory has room for them
-  const ClPlan whole = cluster_plan(g.d_model, g.d_ffn, g.vocab, (int)c->esz, c->pass_grid, 1 << 14);
+  const ClPlan whole = cluster_plan(g.d_model, g.d_ffn, g.vocab, (int)c->esz, c->pass_grid, 0);
   for (int places = std::max(8, whole.most_places);; places = std::max(places / 2, whole.most_cuts)) {
     c->cl_plan = cluster_plan(g.d_model, g.d_ffn, g.vocab, (int)c->esz, c->pass_grid, places);
     c->cl = cluster_layout(g.d_model, g.d_ffn, g.n_heads, g.head_dim, g.n_layers, widest, g.max_seq, (int)c->esz, places, c->cl_plan, c->max_smem_optin);
