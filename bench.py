@@ -310,9 +310,14 @@ def main():
     peak, peak_src = measured_peak_gbs()
     per_kernel = {}
     mid = plen + n_new // 2                      # a context in the middle of the generation
-    uses_pass = (shape.dtype == "bf16" and not (args.flags & (pkg.FLAG_NO_PASS_KERNEL | pkg.FLAG_FMA_GEMM))
+    in_cluster = out.timing["kernel_launches"] == 1  # a small decoder: the whole generation was one launch of the cluster kernel
+    uses_pass = (not in_cluster and shape.dtype == "bf16" and not (args.flags & (pkg.FLAG_NO_PASS_KERNEL | pkg.FLAG_FMA_GEMM))
                  and batch * 9 <= 16)          # k_max = 8: wider contexts run one kernel per operation
-    if uses_pass:
+    if in_cluster:
+        dom_ms, dom_bytes = dec_ms / args.steps, (wbytes + kvbytes) // args.steps
+        dom_name = "cluster_pass_kernel (a whole generation: %d draft and %d target passes inside one cluster of 16 CTAs)" % (
+            draft_passes // args.steps, target_passes // args.steps)
+    elif uses_pass:
         for name, draft, rows in (("draft_pass@M=1", True, 1), ("draft_pass@M=2", True, 2),
                                   ("verify_pass@M=%d" % (k + 1), False, k + 1), ("ar_pass@M=1", False, 1)):
             ms, nbytes = eng.sdfp_time_pass(draft, rows, mid, 24)

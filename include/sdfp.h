@@ -301,6 +301,9 @@ int sdfp_time_linear(sdfp_ctx *ctx, int32_t which, int32_t rows, int32_t iters,
  * the lm-head, the K/V of those layers for positions 0..position+rows-1, and the K/V rows it
  * writes.  The token ids fed are 0; the K/V cache of slot 0 is overwritten from `position` on
  * (in Section II-A's terms: a timing-only verification pass whose result is discarded).
+ * A small model's rounds of sdfp_generate run in another kernel, inside one thread-block cluster (a
+ * greedy generation is then ONE launch in sdfp_timing.kernel_launches); what this times is the
+ * kernel of its prompts and of sdfp_forward_logits.
  */
 int sdfp_time_pass(sdfp_ctx *ctx, int32_t draft, int32_t rows, int32_t position, int32_t iters,
                    float *ms_per_launch, int64_t *bytes_per_launch);
