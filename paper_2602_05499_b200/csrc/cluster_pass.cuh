@@ -820,14 +820,13 @@ __device__ __forceinline__ void cl_attend(const ClParams& p, const ClEnv& ev, co
           const float4 k = load4(kr + e);
           const float* qe = q + e + e / (HD / 4) * 8;
 #pragma unroll
-          for (int i = 0; i < RM; ++i)
-            if (RM == 1 || i < rps) {
-              const float4 qv = *reinterpret_cast<const float4*>(qe + i * ClQ<HD>::kLd);
-              acc[i] = fmaf(k.x, qv.x, acc[i]);
-              acc[i] = fmaf(k.y, qv.y, acc[i]);
-              acc[i] = fmaf(k.z, qv.z, acc[i]);
-              acc[i] = fmaf(k.w, qv.w, acc[i]);
-            }
+          for (int i = 0; i < RM; ++i) {  // (rows the group does not have read something of this CTA's memory, and are not used)
+            const float4 qv = *reinterpret_cast<const float4*>(qe + i * ClQ<HD>::kLd);
+            acc[i] = fmaf(k.x, qv.x, acc[i]);
+            acc[i] = fmaf(k.y, qv.y, acc[i]);
+            acc[i] = fmaf(k.z, qv.z, acc[i]);
+            acc[i] = fmaf(k.w, qv.w, acc[i]);
+          }
         }
       }
 #pragma unroll
@@ -871,8 +870,7 @@ __device__ __forceinline__ void cl_attend(const ClParams& p, const ClEnv& ev, co
       if (half < A::OH) {
         if (BF)
 #pragma unroll
-          for (int i = 0; i < RM; ++i)
-            if (RM == 1 || i < rps) o[u][i] *= s_a[i];
+          for (int i = 0; i < RM; ++i) o[u][i] *= s_a[i];
         const int lo = half * (C / A::OH), hi = min(n_keys, lo + C / A::OH);
         int k = lo;
 #pragma unroll(RM == 1 ? 2 : 1)
@@ -881,21 +879,19 @@ __device__ __forceinline__ void cl_attend(const ClParams& p, const ClEnv& ev, co
 #pragma unroll
           for (int e = 0; e < 4; ++e) v[e] = to_f32(sV[(k + e) * HD + d]);
 #pragma unroll
-          for (int i = 0; i < RM; ++i)
-            if (RM == 1 || i < rps) {
-              const float4 p4 = *reinterpret_cast<const float4*>(sS + i * C + k);
-              o[u][i] = fmaf(p4.x, v[0], o[u][i]);
-              o[u][i] = fmaf(p4.y, v[1], o[u][i]);
-              o[u][i] = fmaf(p4.z, v[2], o[u][i]);
-              o[u][i] = fmaf(p4.w, v[3], o[u][i]);
-            }
+          for (int i = 0; i < RM; ++i) {
+            const float4 p4 = *reinterpret_cast<const float4*>(sS + i * C + k);
+            o[u][i] = fmaf(p4.x, v[0], o[u][i]);
+            o[u][i] = fmaf(p4.y, v[1], o[u][i]);
+            o[u][i] = fmaf(p4.z, v[2], o[u][i]);
+            o[u][i] = fmaf(p4.w, v[3], o[u][i]);
+          }
         }
 #pragma unroll 1
         for (; k < hi; ++k) {
           const float v = to_f32(sV[k * HD + d]);
 #pragma unroll
-          for (int i = 0; i < RM; ++i)
-            if (RM == 1 || i < rps) o[u][i] = fmaf(sS[i * C + k], v, o[u][i]);
+          for (int i = 0; i < RM; ++i) o[u][i] = fmaf(sS[i * C + k], v, o[u][i]);
         }
       }
     }
@@ -939,41 +935,49 @@ __device__ __forceinline__ void cl_attend(const ClParams& p, const ClEnv& ev, co
   cl_team_sync(team);  // the rows' state is used by the next item
 }
 
-// The places of a row and head in order, four dimensions
+// The weights of a row's places, left where their maxima and sums were: bf16 exp(m - max) / sum, as FoldStats; fp32 exp(m - max), and 1 / sum
+// beside the first
 template <typename WT, int HD>
-__device__ __forceinline__ float4 cl_fold(const float* q, int n, int dim) {
+__device__ __forceinline__ void cl_weigh(float* q, int n) {
   constexpr int LD = ClAttn<WT, HD>::PLD;
   constexpr bool BF = ClAttn<WT, HD>::BF;
-  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (n <= 0) return o;
   float mx = -INFINITY, l = 0.f;
 #pragma unroll 1
   for (int j = 0; j < n; ++j) {
     const float2 ml = *reinterpret_cast<const float2*>(q + j * LD + HD);
     if (!BF || ml.y > 0.f) mx = fmaxf(mx, ml.x);
   }
-  auto weight = [&](const float2& ml) { return !BF || ml.y > 0.f ? __expf(ml.x - mx) : 0.f; };
-  auto add = [&](int j, float w) {
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    const float2 ml = *reinterpret_cast<const float2*>(q + j * LD + HD);
+    const float w = !BF || ml.y > 0.f ? __expf(ml.x - mx) : 0.f;
+    l = fmaf(ml.y, w, l);
+    q[j * LD + HD] = w;
+  }
+  const float inv_l = !BF || l > 0.f ? 1.0f / l : 0.f;
+  if (BF)
+#pragma unroll 1
+    for (int j = 0; j < n; ++j) q[j * LD + HD] *= inv_l;
+  else
+    q[HD + 1] = inv_l;
+}
+// The places in order, four dimensions
+template <typename WT, int HD>
+__device__ __forceinline__ float4 cl_fold(const float* q, int n, int dim) {
+  constexpr int LD = ClAttn<WT, HD>::PLD;
+  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (n <= 0) return o;
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    const float w = q[j * LD + HD];
     const float4 v = *reinterpret_cast<const float4*>(q + j * LD + dim);
     o.x = fmaf(v.x, w, o.x);
     o.y = fmaf(v.y, w, o.y);
     o.z = fmaf(v.z, w, o.z);
     o.w = fmaf(v.w, w, o.w);
-  };
-#pragma unroll 1
-  for (int j = 0; j < n; ++j) {
-    const float2 ml = *reinterpret_cast<const float2*>(q + j * LD + HD);
-    const float w = weight(ml);
-    l = fmaf(ml.y, w, l);
-    if (!BF) add(j, w);
   }
-  if (BF) {  // as FoldStats: the sum goes into the weights
-    const float inv_l = l > 0.f ? 1.0f / l : 0.f;
-#pragma unroll 1
-    for (int j = 0; j < n; ++j) add(j, weight(*reinterpret_cast<const float2*>(q + j * LD + HD)) * inv_l);
-    return o;
-  }
-  const float inv_l = 1.0f / l;
+  if (ClAttn<WT, HD>::BF) return o;
+  const float inv_l = q[HD + 1];
   return make_float4(o.x * inv_l, o.y * inv_l, o.z * inv_l, o.w * inv_l);
 }
 
@@ -1007,6 +1011,8 @@ __device__ __forceinline__ void cl_attention(const ClParams& p, const ClEnv& ev,
         const WT *gk = cache_at(t.kcache, hl, b), *gv = cache_at(t.vcache, hl, b);
         if (rps == 1)
           cl_attend<WT, HD, 1>(p, ev, gk, gv, hl, b, 0, place, waited, qkv_bytes, parity);
+        else if (rps == 2)
+          cl_attend<WT, HD, 2>(p, ev, gk, gv, hl, b, 0, place, waited, qkv_bytes, parity);
         else
 #pragma unroll 1
           for (int r0 = 0; r0 < rps; r0 += kClAttnRows) cl_attend<WT, HD, kClAttnRows>(p, ev, gk, gv, hl, b, r0, place, waited, qkv_bytes, parity);
@@ -1024,6 +1030,11 @@ __device__ __forceinline__ void cl_attention(const ClParams& p, const ClEnv& ev,
       }
       if (n > 0) cl_wait(ev.sh, p.sync, CL_BAR_PART, (unsigned)(n * (HD + 2) * 4), phase(CL_BAR_PART));
     }
+    if (ev.tid < nh * R) {
+      const int row = nh == 1 ? ev.tid : ev.tid % R;
+      cl_weigh<WT, HD>(cl_at<float>(p.lay.part) + ev.tid * p.lay.part_slots * A::PLD, A::places(ev.sh->pos[row]));
+    }
+    __syncthreads();
     if (!cl_aborted(ev.sh)) {
       const uint32_t bar = cl_bar_of(p, ev.dst, CL_BAR_X);
 #pragma unroll 1
