@@ -191,3 +191,21 @@ def test_an_end_token(flags):
                 assert out.tokens[b] == want[:cut]
     finally:
         eng.close()
+
+
+def test_a_logit_that_is_not_a_number_hides_no_other():
+    """fp32, one row of the lm-head not numbers: its neighbour in the pair (eight rows on), often the largest, is still chosen, as on the
+    kernels of every other pass."""
+    shape = si.TINY
+    w = si.make_weights(shape, (1, 2))
+    w["lm_head"][0] = float("nan")
+    w["lm_head"][8] *= 40.0
+    got = []
+    for flags in (0, pkg.FLAG_NO_CLUSTER):
+        eng = pkg.Sdfp(shape, si.weights_to(w, "cuda:0"), max_seq=64, k_max=4, flags=flags)
+        eng.sdfp_set_draft_layers(si.keep_mask(shape.n_layers, (1, 2)))
+        outs = [eng.sdfp_generate(si.make_prompts(shape.vocab, 1, 5, seed=s), 4, 12) for s in range(4)]
+        assert all((o.timing["kernel_launches"] == 1) == (flags == 0) for o in outs)
+        got.append([o.tokens[0] for o in outs])
+        eng.close()
+    assert got[0] == got[1] and any(8 in t for t in got[0])
